@@ -33,6 +33,23 @@ struct WarpTeam {
   }
   // value held by member `src`
   __device__ __forceinline__ uint64_t bcast(uint64_t v, int src) const { return __shfl_sync(kFull, v, src); }
+  // 32-bit forms for counts of one trade: lane mask of the team's part of
+  // this warp, sum of counts (below 2^24) with the OR of flag bits 24..31,
+  // exclusive prefix sum, and the sum over the warps before this one
+  __device__ __forceinline__ unsigned lanes() const { return kFull; }
+  __device__ __forceinline__ uint32_t count_or(uint32_t cnt, uint32_t flags) const {
+    return __reduce_add_sync(kFull, cnt) | __reduce_or_sync(kFull, flags);
+  }
+  __device__ __forceinline__ uint32_t exscan32(uint32_t v) const {
+    uint32_t x = v;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const uint32_t y = __shfl_up_sync(kFull, x, o);
+      if (rank >= o) x += y;
+    }
+    return x - v;
+  }
+  __device__ __forceinline__ uint32_t warps_before(uint32_t) const { return 0u; }
 };
 
 // W consecutive lanes of a warp (W = 8 or 16): a warp holds 32 / W such
@@ -65,6 +82,26 @@ struct LaneTeam {
     return x - v;
   }
   __device__ __forceinline__ uint64_t bcast(uint64_t v, int src) const { return __shfl_sync(mask, v, src, W); }
+  // see WarpTeam; the flags travel as 5-bit counts above an 8-bit one, so one
+  // shuffle chain serves them all (counts of at most 4 W <= 64 entries)
+  __device__ __forceinline__ unsigned lanes() const { return mask; }
+  __device__ __forceinline__ uint32_t count_or(uint32_t cnt, uint32_t flags) const {
+    uint32_t v = cnt | ((flags >> 24 & 1u) << 8) | ((flags >> 25 & 1u) << 14) | ((flags >> 26 & 1u) << 20);
+#pragma unroll
+    for (int o = W / 2; o; o >>= 1) v += __shfl_xor_sync(mask, v, o, W);
+    return (v & 0xffu) | ((v & 0x3f00u) ? 1u << 24 : 0u) | ((v & 0xfc000u) ? 1u << 25 : 0u) |
+           ((v >> 20) ? 1u << 26 : 0u);
+  }
+  __device__ __forceinline__ uint32_t exscan32(uint32_t v) const {
+    uint32_t x = v;
+#pragma unroll
+    for (int o = 1; o < W; o <<= 1) {
+      const uint32_t y = __shfl_up_sync(mask, x, o, W);
+      if (rank >= o) x += y;
+    }
+    return x - v;
+  }
+  __device__ __forceinline__ uint32_t warps_before(uint32_t) const { return 0u; }
 };
 
 // A CTA of NT threads; `red` points at kRedSlots int64 slots of shared memory.
@@ -113,6 +150,36 @@ struct BlockTeam {
 #pragma unroll
     for (int o = 16; o; o >>= 1) before += __shfl_xor_sync(kFull, before, o);
     return x - v + before;
+  }
+  // see WarpTeam; one barrier each, through the same two buffers
+  __device__ __forceinline__ unsigned lanes() const { return kFull; }
+  __device__ __forceinline__ uint32_t count_or(uint32_t cnt, uint32_t flags) {
+    const int lane = rank & 31;
+    const uint32_t x = __reduce_add_sync(kFull, cnt) | __reduce_or_sync(kFull, flags);
+    uint32_t* part = reinterpret_cast<uint32_t*>(red + buf * NW);
+    if (lane == 0) part[rank >> 5] = x;
+    __syncthreads();
+    buf ^= 1;
+    const uint32_t p = lane < NW ? part[lane] : 0u;
+    return __reduce_add_sync(kFull, p & 0xffffffu) | (__reduce_or_sync(kFull, p) & 0xff000000u);
+  }
+  __device__ __forceinline__ uint32_t warps_before(uint32_t v) {   // v: the same in every lane of a warp
+    const int lane = rank & 31, w = rank >> 5;
+    uint32_t* part = reinterpret_cast<uint32_t*>(red + buf * NW);
+    if (lane == 0) part[w] = v;
+    __syncthreads();
+    buf ^= 1;
+    return __reduce_add_sync(kFull, lane < w ? part[lane] : 0u);
+  }
+  __device__ __forceinline__ uint32_t exscan32(uint32_t v) {
+    const int lane = rank & 31;
+    uint32_t x = v;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const uint32_t y = __shfl_up_sync(kFull, x, o);
+      if (lane >= o) x += y;
+    }
+    return x - v + warps_before(__shfl_sync(kFull, x, 31));
   }
 };
 
@@ -209,6 +276,36 @@ struct SubTeam {
 #pragma unroll
     for (int o = 16; o; o >>= 1) before += __shfl_xor_sync(kFull, before, o);
     return x - v + before;
+  }
+  // see WarpTeam; one barrier each, through the same two buffers
+  __device__ __forceinline__ unsigned lanes() const { return kFull; }
+  __device__ __forceinline__ uint32_t count_or(uint32_t cnt, uint32_t flags) {
+    const int lane = rank & 31;
+    const uint32_t x = __reduce_add_sync(kFull, cnt) | __reduce_or_sync(kFull, flags);
+    uint32_t* part = reinterpret_cast<uint32_t*>(red + buf * NW);
+    if (lane == 0) part[rank >> 5] = x;
+    sync();
+    buf ^= 1;
+    const uint32_t p = lane < NW ? part[lane] : 0u;
+    return __reduce_add_sync(kFull, p & 0xffffffu) | (__reduce_or_sync(kFull, p) & 0xff000000u);
+  }
+  __device__ __forceinline__ uint32_t warps_before(uint32_t v) {   // v: the same in every lane of a warp
+    const int lane = rank & 31, w = rank >> 5;
+    uint32_t* part = reinterpret_cast<uint32_t*>(red + buf * NW);
+    if (lane == 0) part[w] = v;
+    sync();
+    buf ^= 1;
+    return __reduce_add_sync(kFull, lane < w ? part[lane] : 0u);
+  }
+  __device__ __forceinline__ uint32_t exscan32(uint32_t v) {
+    const int lane = rank & 31;
+    uint32_t x = v;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const uint32_t y = __shfl_up_sync(kFull, x, o);
+      if (lane >= o) x += y;
+    }
+    return x - v + warps_before(__shfl_sync(kFull, x, 31));
   }
 };
 

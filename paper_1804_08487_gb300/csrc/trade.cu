@@ -847,10 +847,8 @@ __device__ void phase_a(Team& tm, const StepCtx& c, int64_t t, const WsA& w, Sel
 // bin.  Used by the first pass only: a trade whose dependency has not
 // published yet is deferred to the in-order pass.
 
-// per-entry meta word
-constexpr uint32_t kMSlot = 0x3FFFu;        // hash slot of the far trade (tables of at most 2^14 slots)
-constexpr uint32_t kMR = 1u << 14;          // entry sits in v's row
-constexpr uint32_t kMCol = 1u << 15;        // neighbour at the odd position 2s+1
+// per-entry meta word (the entry's row is i >= deg u, its column the low bit of y)
+constexpr uint32_t kMSlot = 0x7FFFu;        // hash slot of the far trade
 constexpr uint32_t kMUV = 1u << 16;         // the edge {u, v}
 constexpr uint32_t kMInD = 1u << 17;        // element of D
 constexpr uint32_t kMFlip = 1u << 18;       // the trade moves the edge to its other node
@@ -858,39 +856,59 @@ constexpr uint32_t kMValid = 1u << 19;      // an entry of the trade
 constexpr uint32_t kMMulti = 1u << 20;      // block of two or more edges
 constexpr int kMFarShift = 21;              // bits 21..31: top kFarBits bits of the far trade's key
 
-__host__ __device__ constexpr int hash_lg_c(int L) {
-  int lg = 1;
-  while ((1 << lg) < 2 * L) ++lg;
+__host__ __device__ constexpr int lg_ceil(int x) {
+  int lg = 0;
+  while ((1 << lg) < x) ++lg;
   return lg;
 }
 
 // One team's workspace: a base address and a compile-time layout for trades
-// of at most LMAX entries and 2^B histogram bins.
-template <int LMAX, int B>
+// of at most LMAX entries and 2^B histogram bins (four per member).
+//
+// The far-trade hash has two tables of (key, block word) pairs.  Table 1
+// (kH slots, at least 4 per entry) is never cleared: in one round every entry
+// stores its key and a zero block word into its home slot, whatever is there,
+// so after a barrier each home slot holds a key of this trade.  Only the
+// entries that find another key there (about 8 % at 4 to 8 slots per entry)
+// go to table 2 (kH2 >= LMAX slots, cleared per trade), by compare-and-swap.
+// Clearing the single 8-byte-per-slot table this replaces took 16 stores per
+// member; table 2 and the histogram take 3.
+template <int LMAX, int B, int CAND>
 struct RegWs {
   static_assert(B >= 5, "tables are cleared in 16-byte stores");
   static constexpr int kLmax = LMAX;
-  static constexpr int kH = 1 << hash_lg_c(2 * LMAX);   // at least 4 slots per entry
+  static constexpr int kCandCap = CAND;                 // candidates ranked directly
+  static constexpr int kH = 1 << lg_ceil(4 * LMAX);
+  static constexpr int kH2 = 1 << lg_ceil(LMAX);
+  static_assert(kH + kH2 <= int(kMSlot) + 1, "slot field");
   static constexpr size_t kCk = 0;                              // candidate keys
-  static constexpr size_t kCtb = kCk + kCand * 8;               // candidate tie-breaks
-  static constexpr size_t kSel = kCtb + kCand * 8;              // selection results shared by the team
+  static constexpr size_t kCtb = kCk + CAND * 8;                // candidate tie-breaks
+  static constexpr size_t kSel = kCtb + CAND * 8;               // selection results shared by the team
   static constexpr size_t kPw = kSel + ((sizeof(SelOut) + 15) & ~size_t(15));   // radix prefix (4 words)
   static constexpr size_t kNc = kPw + 16;                       // candidate count
-  static constexpr size_t kHk = kNc + 16;                       // hash slot keys (far trade + 1; 0 = empty)
-  static constexpr size_t kHist = kHk + size_t(kH) * 4;         // radix histogram
-  static constexpr size_t kHb = kHist + (size_t(1) << B) * 4;   // slot block bytes (see block_flags)
-  static constexpr size_t kBytes = (kHb + size_t(kH) * 4 + 15) & ~size_t(15);
-  static_assert(kHk % 16 == 0 && kHist % 16 == 0 && kHb % 16 == 0, "16-byte aligned tables");
+  static constexpr size_t kHist = kNc + 16;                     // radix histogram
+  static constexpr size_t kHk = kHist + (size_t(1) << B) * 4;   // slots: table 1, then table 2
+  static constexpr size_t kBytes = (kHk + size_t(kH + kH2) * 8 + 15) & ~size_t(15);
+  static_assert(kHk % 16 == 0 && kHist % 16 == 0, "16-byte aligned tables");
   char* base;
   __device__ __forceinline__ uint64_t* ck() const { return reinterpret_cast<uint64_t*>(base + kCk); }
   __device__ __forceinline__ uint64_t* ctb() const { return reinterpret_cast<uint64_t*>(base + kCtb); }
   __device__ __forceinline__ SelOut* sel() const { return reinterpret_cast<SelOut*>(base + kSel); }
   __device__ __forceinline__ uint32_t* pw() const { return reinterpret_cast<uint32_t*>(base + kPw); }
   __device__ __forceinline__ int32_t* ncand() const { return reinterpret_cast<int32_t*>(base + kNc); }
-  __device__ __forceinline__ uint32_t* hk() const { return reinterpret_cast<uint32_t*>(base + kHk); }
   __device__ __forceinline__ uint32_t* hist() const { return reinterpret_cast<uint32_t*>(base + kHist); }
-  __device__ __forceinline__ uint32_t* hb() const { return reinterpret_cast<uint32_t*>(base + kHb); }
+  __device__ __forceinline__ uint2* hs() const { return reinterpret_cast<uint2*>(base + kHk); }
 };
+
+// Slot of key (far trade + 1) in table 2 (mask + 1 slots at tab, more than
+// the keys it can get), starting the probe at p.
+__device__ __forceinline__ uint32_t h_claim2(uint2* tab, uint32_t mask, uint32_t key, uint32_t p) {
+  for (;;) {
+    const uint32_t cur = atomicCAS(&tab[p].x, 0u, key);
+    if (cur == 0u || cur == key) return p;
+    p = (p + 1u) & mask;
+  }
+}
 
 // A slot's block word holds one byte per edge of the 2x2 block matrix
 // (byte 2 rho + gamma: the trade's node rho adjacent to the far node
@@ -904,8 +922,8 @@ __device__ __forceinline__ uint32_t compact_bytes(uint32_t x) {   // x: bytes 0 
 __device__ __forceinline__ uint32_t block_flags(uint32_t w) {
   return compact_bytes(w & 0x01010101u) | (compact_bytes((w >> 1) & 0x01010101u) << 4);
 }
-__device__ __forceinline__ void block_mark(uint32_t* hb, uint32_t slot, int q, uint8_t v) {
-  reinterpret_cast<uint8_t*>(hb + slot)[q] = v;
+__device__ __forceinline__ void block_mark(uint2* hs, uint32_t slot, uint32_t q, uint8_t v) {
+  reinterpret_cast<uint8_t*>(&hs[slot].y)[q] = v;
 }
 
 // Trade t (nodes at t2u, t2u+1) depends on the earlier trade s through a
@@ -960,17 +978,12 @@ __device__ __forceinline__ bool sel_match(int q, const uint32_t* pw, uint64_t ke
   return true;
 }
 
-// The step-start positions (lo, hi) of an entry's edge.
-__device__ __forceinline__ void entry_lo_hi(uint32_t t2u, uint32_t m, uint32_t y, uint32_t* lo, uint32_t* hi) {
-  const uint32_t x = t2u + ((m & kMR) ? 1u : 0u);
-  *lo = min(x, y);
-  *hi = max(x, y);
-}
-
 template <class Team, int J, int B, bool kKeepKey, bool kOneSeed = false, class Ws>
 __device__ void phase_a_reg(Team& tm, const StepCtx& c, int64_t t, const Ws& w) {
-  static_assert(Team::N <= 2048 && Team::N * J < (1 << 20), "reduction fields: 20-bit count, 12-bit flags");
-  constexpr int NB = 1 << B;
+  constexpr int N = Team::N;
+  constexpr bool kWarp = N <= 32;   // the team is a warp or part of one
+  static_assert((1 << B) == 4 * N, "four histogram bins per member");
+  static_assert(N * J <= Ws::kLmax && N * J < (1 << 16), "16-bit placement counts");
   const TradeRows tr = trade_rows(c, t);
   const KeyCtx kc = key_ctx(c, t);
   const int du = tr.du, L = tr.du + tr.dv;
@@ -978,125 +991,96 @@ __device__ void phase_a_reg(Team& tm, const StepCtx& c, int64_t t, const Ws& w) 
   // the trade's work
   const int64_t ou = c.rp_next[__ldg(c.M + 2 * t)];
   const int64_t ov = tr.single ? 0 : c.rp_next[__ldg(c.M + 2 * t + 1)];
-  // at least 4 hash slots per entry, and about one first-digit bin per entry
-  const int lgH = max(5, 34 - __clz(max(L, 2) - 1));   // next power of two >= 4 L
-  const int H = 1 << lgH;
-  const int B0 = min(B, max(5, 32 - __clz(max(L - 1, 1))));
-  const int NB0 = 1 << B0;
   const uint32_t t32 = static_cast<uint32_t>(t), T32 = static_cast<uint32_t>(c.T);
   const uint32_t t2u = 2u * t32;
+  const unsigned lanes = tm.lanes();
+  const unsigned below_me = (1u << (threadIdx.x & 31)) - 1u;
+  const int lgL = 32 - __clz(max(L, 16) - 1);   // slots of table 2: the next power of two >= L (at least 16)
+  uint2* const hs = w.hs();
+  uint2* const hs2 = hs + Ws::kH;
   {
-    // clear the tables in 16-byte stores (H and NB0 are powers of two >= 32;
-    // the layout keeps every table 16-byte aligned)
     const uint4 z = make_uint4(0u, 0u, 0u, 0u);
-    uint4* hk4 = reinterpret_cast<uint4*>(w.hk());
-    uint4* hb4 = reinterpret_cast<uint4*>(w.hb());
-    uint4* hs4 = reinterpret_cast<uint4*>(w.hist());
-    for (int i = tm.rank; i < (H >> 2); i += Team::N) {
-      hk4[i] = z;
-      hb4[i] = z;
-    }
-    for (int i = tm.rank; i < (NB0 >> 2); i += Team::N) hs4[i] = z;
+    reinterpret_cast<uint4*>(w.hist())[tm.rank] = z;
+    uint4* h4 = reinterpret_cast<uint4*>(hs2);
+    for (int i = tm.rank; i < (1 << (lgL - 1)); i += N) h4[i] = z;
+    if (tm.rank == 0) *w.ncand() = 0;
   }
-  if (tm.rank == 0) *w.ncand() = 0;
-  tm.sync();
-  // entries into the hash: presence bit (row, column) in the far trade's slot
+  // entries and their home slots (at least 4 slots per entry): every entry
+  // stores its key there
   uint32_t y[J], mt[J], kt[J], kl[kKeepKey ? J : 1];
 #pragma unroll
   for (int j = 0; j < J; ++j) {
-    const int i = tm.rank + j * Team::N;
+    const int i = tm.rank + j * N;
     y[j] = 0;
     mt[j] = 0;
     kt[j] = 0;
     if (kKeepKey) kl[j] = 0;
-    if (i < L) {
-      const int32_t yy = __ldcg(c.col + tr.b0 + i);
-      const uint32_t r = i >= du ? 1u : 0u;
-      const uint32_t s = static_cast<uint32_t>(yy) >> 1;
-      uint32_t m = kMValid | (r ? kMR : 0u) | ((yy & 1) ? kMCol : 0u);
-      if (s == t32) m |= kMUV;
-      else m |= hslot(s, lgH);
-      y[j] = static_cast<uint32_t>(yy);
-      mt[j] = m;
-    }
+    if (i < L) y[j] = static_cast<uint32_t>(__ldcg(c.col + tr.b0 + i));
   }
-  // the hash (open addressing, far trade + 1 as key): every entry writes its
-  // key into its home slot if that is empty (a plain store); after a barrier
-  // it reads the slot back: its key (written by itself or by an entry of the
-  // same far trade) places it; the few entries whose slot another key won
-  // claim a further slot with a compare-and-swap.
-  {
-    uint32_t pend = 0;
 #pragma unroll
-    for (int j = 0; j < J; ++j)
-      if ((mt[j] & kMValid) && !(mt[j] & kMUV)) pend |= 1u << j;
-    // a warp or part of one repeats the plain round (its barriers are
-    // cheap) until every entry is placed; a larger team runs one round, then
-    // compare-and-swap
-    // (the first round's slots are all empty or written in this round, so
-    // its stores need no check).  An entry marks its edge in the slot's
-    // block word as soon as its slot is final.
-    constexpr bool kRounds = Team::N <= 32;
-    bool first = true;
-    for (;;) {
-#pragma unroll
-      for (int j = 0; j < J; ++j)
-        if ((pend >> j) & 1u) {
-          const uint32_t sl = mt[j] & kMSlot;
-          if (first || w.hk()[sl] == 0u) w.hk()[sl] = (y[j] >> 1) + 1u;
-        }
-      first = false;
-      tm.sync();
-      bool more = false;
-#pragma unroll
-      for (int j = 0; j < J; ++j)
-        if ((pend >> j) & 1u) {
-          const uint32_t sl = mt[j] & kMSlot;
-          const uint32_t key = (y[j] >> 1) + 1u;
-          const int q = 2 * ((mt[j] & kMR) ? 1 : 0) + ((mt[j] & kMCol) ? 1 : 0);
-          if (w.hk()[sl] == key) {
-            pend &= ~(1u << j);
-            block_mark(w.hb(), sl, q, 1);
-          } else if (kRounds) {
-            mt[j] = (mt[j] & ~kMSlot) | ((sl + 1u) & static_cast<uint32_t>(H - 1));
-            more = true;
-          } else {   // lost the slot to another key: claim one further on
-            const uint32_t sl2 = h_claim(w.hk(), static_cast<uint32_t>(H - 1), key, (sl + 1u) & (H - 1));
-            mt[j] = (mt[j] & ~kMSlot) | sl2;
-            block_mark(w.hb(), sl2, q, 1);
-          }
-        }
-      if (!kRounds || !tm.any(more)) break;
+  for (int j = 0; j < J; ++j) {
+    if (tm.rank + j * N >= L) continue;
+    const uint32_t s = y[j] >> 1;
+    if (s == t32) {
+      mt[j] = kMValid | kMUV;
+    } else {
+      const uint32_t sl = hslot(s, lgL + 2);
+      hs[sl] = make_uint2(s + 1u, 0u);
+      mt[j] = kMValid | sl;
     }
   }
   tm.sync();
+  // an entry whose key is in its slot marks its edge in the slot's block
+  // word; the others (another key won the slot) take a slot of table 2
+  uint32_t pend = 0;
+#pragma unroll
+  for (int j = 0; j < J; ++j) {
+    if (!(mt[j] & kMValid) || (mt[j] & kMUV)) continue;
+    const uint32_t sl = mt[j] & kMSlot;
+    const uint32_t q = (tm.rank + j * N >= du ? 2u : 0u) + (y[j] & 1u);
+    if (hs[sl].x == (y[j] >> 1) + 1u) block_mark(hs, sl, q, 1);
+    else pend |= 1u << j;
+  }
+  if (pend) {
+#pragma unroll
+    for (int j = 0; j < J; ++j)
+      if ((pend >> j) & 1u) {
+        const uint32_t s = y[j] >> 1;
+        const uint32_t q = (tm.rank + j * N >= du ? 2u : 0u) + (y[j] & 1u);
+        const uint32_t sl = Ws::kH + h_claim2(hs2, (1u << lgL) - 1u, s + 1u, (s * 0x85EBCA6Bu) >> (32 - lgL));
+        mt[j] = kMValid | sl;
+        block_mark(hs, sl, q, 1);
+      }
+  }
+  tm.sync();
   // block analysis, keys, histogram of the first radix digit
-  bool defer = false, has_dependents = false, any_multi = false;
-  int cnt_a = 0;
+  constexpr uint32_t kFlDefer = 1u << 24, kFlDep = 1u << 25, kFlMulti = 1u << 26;
+  uint32_t flags = 0, cnt_a = 0;
 #pragma unroll
   for (int j = 0; j < J; ++j) {
     uint32_t m = mt[j];
     if (!(m & kMValid) || (m & kMUV)) continue;
-    const int r = (m & kMR) ? 1 : 0;
-    const uint32_t colb = (m & kMCol) ? 1u : 0u;
+    const int r = tm.rank + j * N >= du ? 1 : 0;
     const uint32_t s = y[j] >> 1;
-    const uint32_t f = block_flags(w.hb()[m & kMSlot]) & 15u;
+    const uint32_t fw = hs[m & kMSlot].y;
     int other = 0;   // the other row is adjacent to this neighbour when t acts
-    if (f & (f - 1u)) {
+    if (fw & (fw - 1u)) {
       // a block of two or more edges: common neighbours and dependencies
       m |= kMMulti;
-      any_multi = true;
+      flags |= kFlMulti;
+      const uint32_t colb = y[j] & 1u;
+      const uint32_t f = block_flags(fw) & 15u;
       const int u0 = f & 1, u1 = (f >> 1) & 1, v0 = (f >> 2) & 1, v1 = (f >> 3) & 1;
       const int cu = u0 + u1, cv = v0 + v1;
-      if (!tr.single && s > t32 && s < T32 && (u0 + v0 == 1 || u1 + v1 == 1)) has_dependents = true;
-      int col_now = static_cast<int>(colb);
+      if (!tr.single && s > t32 && s < T32 && (u0 + v0 == 1 || u1 + v1 == 1)) flags |= kFlDep;
+      const int col_now = static_cast<int>(colb);
       other = r ? (col_now ? u1 : u0) : (col_now ? v1 : v0);
       if (!tr.single && s < t32 && (cu == 1 || cv == 1)) {
         // unpublished: a parallel pass leaves the trade to a later pass,
         // an in-order pass waits
         if (ld_acquire(c.done + s) != c.stamp &&
             !(c.wait && wait_published(c.done + s, c.err, c.stamp, c.wait_ns))) {
-          defer = true;
+          flags |= kFlDefer;
           mt[j] = m;
           continue;
         }
@@ -1105,128 +1089,122 @@ __device__ void phase_a_reg(Team& tm, const StepCtx& c, int64_t t, const Ws& w) 
     }
     // both trades' keys of this edge (step-start positions)
     const uint32_t x = t2u + r, yb = y[j];
-    const uint32_t lo = min(x, yb), hi = max(x, yb);
-    const EdgeKeys ek = edge_keys<kOneSeed>(c, kc, lo, hi);
-    const bool lo_mine = (lo >> 1) == t32;
-    const uint64_t own = lo_mine ? ek.lo_side : ek.hi_side;
-    const uint64_t far = lo_mine ? ek.hi_side : ek.lo_side;
-    kt[j] = static_cast<uint32_t>(own >> 32);
-    if (kKeepKey) kl[j] = static_cast<uint32_t>(own);
-    m |= static_cast<uint32_t>(far >> (64 - kFarBits)) << kMFarShift;
+    const EdgeKeys ek = edge_keys<kOneSeed>(c, kc, min(x, yb), max(x, yb));
+    const bool lo_mine = s > t32;   // the own end is the lower position
+    kt[j] = static_cast<uint32_t>((lo_mine ? ek.lo_side : ek.hi_side) >> 32);
+    if (kKeepKey) kl[j] = static_cast<uint32_t>(lo_mine ? ek.lo_side : ek.hi_side);
+    m |= (static_cast<uint32_t>((lo_mine ? ek.hi_side : ek.lo_side) >> 32) >> (32 - kFarBits)) << kMFarShift;
     if (!other && !tr.single) {
       m |= kMInD;
       cnt_a += (r == 0);
-      atomicAdd(&w.hist()[kt[j] >> (32 - B0)], 1u);
+      atomicAdd(&w.hist()[kt[j] >> (32 - B)], 1u);
     }
     mt[j] = m;
   }
-  // one reduction: |A_{u-v}| (bits 0..19) and, in 12-bit fields that hold a
-  // count over up to 1024 members, the members that saw a deferral, a later
-  // dependent trade, a multi-edge block
-  const int64_t tot = tm.sum(static_cast<int64_t>(cnt_a) | (static_cast<int64_t>(defer) << 20) |
-                             (static_cast<int64_t>(has_dependents) << 32) | (static_cast<int64_t>(any_multi) << 44));
-  if ((tot >> 20) & 0xfff) {
+  // one reduction: |A_{u-v}|, and whether any member saw a deferral, a later
+  // dependent trade, a multi-edge block (it also orders the histogram)
+  const uint32_t tot = tm.count_or(cnt_a, flags);
+  if (tot & kFlDefer) {
     if (tm.rank == 0) defer_trade(c, t, L);
     tm.sync();
     return;
   }
-  const int a = static_cast<int>(tot & 0xfffff);
-  const bool publish_fence = ((tot >> 32) & 0xfff) != 0;
-  const bool multi_any = ((tot >> 44) & 0xfff) != 0;
+  const uint32_t a = tot & 0xffffffu;
+  const bool publish_fence = (tot & kFlDep) != 0;
+  const bool multi_any = (tot & kFlMulti) != 0;
   const bool no_thr = tr.single || a == 0;   // u keeps nothing of D
+  if (kWarp) tm.sync();
   uint64_t tk = 0, tt = 0;
   if (!no_thr) {
-    // the bin of the first digit (top B0 key bits) that holds the a-th smallest element
-    constexpr int BPM = (NB + Team::N - 1) / Team::N;
+    // the bin of the first digit (top B key bits) that holds the a-th
+    // smallest element: four bins per member
+    uint32_t bin = 0, below = 0, cnt = 0;
     {
-      const int bpm0 = (NB0 + Team::N - 1) / Team::N;
-      const int b0 = tm.rank * bpm0;
-      int local = 0;
-#pragma unroll
-      for (int q = 0; q < BPM; ++q)
-        if (q < bpm0 && b0 + q < NB0) local += static_cast<int>(w.hist()[b0 + q]);
-      int run = static_cast<int>(tm.exscan(local));
-#pragma unroll
-      for (int q = 0; q < BPM; ++q) {
-        const int b = b0 + q;
-        if (q < bpm0 && b < NB0) {
-          const int hc = static_cast<int>(w.hist()[b]);
-          if (run < a && a <= run + hc) {
-            w.sel()->bin = b;
-            w.sel()->below = run;
-            w.sel()->cnt = hc;
-          }
-          run += hc;
+      const uint4 h = reinterpret_cast<const uint4*>(w.hist())[tm.rank];
+      const uint32_t c1 = h.x + h.y, c2 = c1 + h.z, c3 = c2 + h.w;
+      const uint32_t run = tm.exscan32(c3);
+      const uint32_t k = a - run;   // 1-based rank within the member's bins
+      const bool found = a > run && k <= c3;
+      uint32_t p = 3, pb = c2, pc = h.w;
+      if (k <= c2) { p = 2; pb = c1; pc = h.z; }
+      if (k <= c1) { p = 1; pb = h.x; pc = h.y; }
+      if (k <= h.x) { p = 0; pb = 0; pc = h.x; }
+      if (kWarp) {   // at most 128 entries: 8-bit fields
+        const uint32_t info = (4u * tm.rank + p) | ((run + pb) << 8) | (pc << 16);
+        const int src = __ffs(__ballot_sync(lanes, found) & lanes) - 1;
+        const uint32_t got = __shfl_sync(lanes, info, src);
+        bin = got & 0xffu;
+        below = (got >> 8) & 0xffu;
+        cnt = got >> 16;
+      } else {
+        if (found) {
+          w.sel()->bin = static_cast<int32_t>(4u * tm.rank + p);
+          w.sel()->below = static_cast<int32_t>(run + pb);
+          w.sel()->cnt = static_cast<int32_t>(pc);
         }
+        tm.sync();
+        bin = static_cast<uint32_t>(w.sel()->bin);
+        below = static_cast<uint32_t>(w.sel()->below);
+        cnt = static_cast<uint32_t>(w.sel()->cnt);
       }
     }
-    tm.sync();
-    int qbits = B0;             // top bits of the order fixed so far
-    int kk = a - w.sel()->below;  // rank sought among the elements sharing them
-    int cnt = w.sel()->cnt;
-    if (tm.rank == 0) {
-      w.pw()[0] = static_cast<uint32_t>(w.sel()->bin) << (32 - B0);
-      w.pw()[1] = w.pw()[2] = w.pw()[3] = 0u;
-    }
-    tm.sync();
-    // more elements share the prefix than the candidate list holds (or the
-    // list is disabled): further B-bit digits of (key, lo, hi)
-    while (cnt > c.cand_max) {
-      for (int i = tm.rank; i < NB; i += Team::N) w.hist()[i] = 0u;
+    int qbits = B;              // top bits of the order fixed so far
+    uint32_t kk = a - below;    // rank sought among the elements sharing them
+    const uint32_t cap = min(static_cast<uint32_t>(c.cand_max), static_cast<uint32_t>(Ws::kCandCap));
+    if (cnt > cap) {
+      // more elements share the prefix than the candidate list holds (or the
+      // list is disabled): further B-bit digits of (key, lo, hi)
       tm.sync();
-#pragma unroll
-      for (int j = 0; j < J; ++j) {
-        if (!(mt[j] & kMInD)) continue;
-        uint32_t lo, hi;
-        entry_lo_hi(t2u, mt[j], y[j], &lo, &hi);
-        const uint64_t key = kKeepKey ? ((static_cast<uint64_t>(kt[j]) << 32) | kl[j]) : own_key(kc, t, lo, hi);
-        if (sel_match(qbits, w.pw(), key, lo, hi)) atomicAdd(&w.hist()[sel_digit(qbits, B, key, lo, hi)], 1u);
+      if (tm.rank == 0) {
+        w.pw()[0] = bin << (32 - B);
+        w.pw()[1] = w.pw()[2] = w.pw()[3] = 0u;
       }
-      tm.sync();
-      {
-        const int b0 = tm.rank * BPM;
-        int local = 0;
+      while (cnt > cap) {
+        reinterpret_cast<uint4*>(w.hist())[tm.rank] = make_uint4(0u, 0u, 0u, 0u);
+        tm.sync();
 #pragma unroll
-        for (int q = 0; q < BPM; ++q)
-          if (b0 + q < NB) local += static_cast<int>(w.hist()[b0 + q]);
-        int run = static_cast<int>(tm.exscan(local));
-#pragma unroll
-        for (int q = 0; q < BPM; ++q) {
-          const int b = b0 + q;
-          if (b < NB) {
-            const int hc = static_cast<int>(w.hist()[b]);
-            if (run < kk && kk <= run + hc) {
-              w.sel()->bin = b;
-              w.sel()->below = run;
-              w.sel()->cnt = hc;
-            }
-            run += hc;
-          }
+        for (int j = 0; j < J; ++j) {
+          if (!(mt[j] & kMInD)) continue;
+          const uint32_t x = t2u + (tm.rank + j * N >= du ? 1u : 0u);
+          const uint32_t lo = min(x, y[j]), hi = max(x, y[j]);
+          const uint64_t key = kKeepKey ? ((static_cast<uint64_t>(kt[j]) << 32) | kl[j]) : own_key(kc, t, lo, hi);
+          if (sel_match(qbits, w.pw(), key, lo, hi)) atomicAdd(&w.hist()[sel_digit(qbits, B, key, lo, hi)], 1u);
         }
+        tm.sync();
+        const uint4 h = reinterpret_cast<const uint4*>(w.hist())[tm.rank];
+        const uint32_t hv[4] = {h.x, h.y, h.z, h.w};
+        uint32_t run = tm.exscan32(h.x + h.y + h.z + h.w);
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+          if (run < kk && kk <= run + hv[q]) {
+            w.sel()->bin = 4 * tm.rank + q;
+            w.sel()->below = static_cast<int32_t>(run);
+            w.sel()->cnt = static_cast<int32_t>(hv[q]);
+          }
+          run += hv[q];
+        }
+        tm.sync();
+        const uint32_t dig = static_cast<uint32_t>(w.sel()->bin);
+        kk -= static_cast<uint32_t>(w.sel()->below);
+        cnt = static_cast<uint32_t>(w.sel()->cnt);
+        if (tm.rank == 0) {   // append the digit to the prefix (it may straddle two words)
+          const int wd = qbits >> 5, off = qbits & 31;
+          const uint64_t d64 = static_cast<uint64_t>(dig) << (64 - B - off);
+          w.pw()[wd] |= static_cast<uint32_t>(d64 >> 32);
+          if (wd < 3) w.pw()[wd + 1] |= static_cast<uint32_t>(d64);
+        }
+        qbits += B;
+        tm.sync();
       }
-      tm.sync();
-      const uint32_t dig = static_cast<uint32_t>(w.sel()->bin);
-      kk -= w.sel()->below;
-      cnt = w.sel()->cnt;
-      tm.sync();
-      if (tm.rank == 0) {   // append the digit to the prefix (it may straddle two words)
-        const int wd = qbits >> 5, off = qbits & 31;
-        const uint64_t d64 = static_cast<uint64_t>(dig) << (64 - B - off);
-        w.pw()[wd] |= static_cast<uint32_t>(d64 >> 32);
-        if (wd < 3) w.pw()[wd + 1] |= static_cast<uint32_t>(d64);
-      }
-      qbits += B;
-      tm.sync();
     }
     // rank the few elements that share the prefix by their full order
 #pragma unroll
     for (int j = 0; j < J; ++j) {
-      if (!(mt[j] & kMInD)) continue;
-      if (qbits == B0 && (kt[j] >> (32 - B0)) != (w.pw()[0] >> (32 - B0))) continue;
-      uint32_t lo, hi;
-      entry_lo_hi(t2u, mt[j], y[j], &lo, &hi);
+      if (!(mt[j] & kMInD) || (kt[j] >> (32 - B)) != bin) continue;
+      const uint32_t x = t2u + (tm.rank + j * N >= du ? 1u : 0u);
+      const uint32_t lo = min(x, y[j]), hi = max(x, y[j]);
       const uint64_t key = kKeepKey ? ((static_cast<uint64_t>(kt[j]) << 32) | kl[j]) : own_key(kc, t, lo, hi);
-      if (qbits > B0 && !sel_match(qbits, w.pw(), key, lo, hi)) continue;
+      if (qbits > B && !sel_match(qbits, w.pw(), key, lo, hi)) continue;
       if (cnt == 1) {
         w.sel()->key = key;
         w.sel()->tb = tie_break(lo, hi);
@@ -1238,9 +1216,10 @@ __device__ void phase_a_reg(Team& tm, const StepCtx& c, int64_t t, const Ws& w) 
     }
     tm.sync();
     if (cnt > 1) {
-      for (int q = tm.rank; q < cnt; q += Team::N) {
-        int rk = 0;
-        for (int p = 0; p < cnt; ++p) rk += (w.ck()[p] < w.ck()[q] || (w.ck()[p] == w.ck()[q] && w.ctb()[p] < w.ctb()[q]));
+      for (uint32_t q = tm.rank; q < cnt; q += N) {
+        uint32_t rk = 0;
+        for (uint32_t p = 0; p < cnt; ++p)
+          rk += (w.ck()[p] < w.ck()[q] || (w.ck()[p] == w.ck()[q] && w.ctb()[p] < w.ctb()[q]));
         if (rk == kk - 1) {
           w.sel()->key = w.ck()[q];
           w.sel()->tb = w.ctb()[q];
@@ -1251,50 +1230,64 @@ __device__ void phase_a_reg(Team& tm, const StepCtx& c, int64_t t, const Ws& w) 
     tk = w.sel()->key;
     tt = w.sel()->tb;
   }
-  // own decisions: u keeps the elements at or below the threshold
+  // own decisions: u keeps the elements at or below the threshold; and how
+  // many entries of this warp land in u's and in v's new row
   const uint32_t tk32 = static_cast<uint32_t>(tk >> 32);
+  uint32_t to_v = 0, all = 0;
 #pragma unroll
   for (int j = 0; j < J; ++j) {
     const uint32_t m = mt[j];
-    if (!(m & kMInD)) continue;
-    const int r = (m & kMR) ? 1 : 0;
-    bool low;
-    if (no_thr) {
-      low = false;
-    } else if (kt[j] != tk32) {
-      low = kt[j] < tk32;
-    } else {
-      uint32_t lo, hi;
-      entry_lo_hi(t2u, m, y[j], &lo, &hi);
-      const uint64_t key = kKeepKey ? ((static_cast<uint64_t>(kt[j]) << 32) | kl[j]) : own_key(kc, t, lo, hi);
-      low = at_or_below(key, tie_break(lo, hi), tk, tt);
+    const bool r = tm.rank + j * N >= du;
+    bool side = r;
+    if (m & kMInD) {
+      bool low;
+      if (no_thr) {
+        low = false;
+      } else if (kt[j] != tk32) {
+        low = kt[j] < tk32;
+      } else {
+        const uint32_t x = t2u + (r ? 1u : 0u);
+        const uint32_t lo = min(x, y[j]), hi = max(x, y[j]);
+        const uint64_t key = kKeepKey ? ((static_cast<uint64_t>(kt[j]) << 32) | kl[j]) : own_key(kc, t, lo, hi);
+        low = at_or_below(key, tie_break(lo, hi), tk, tt);
+      }
+      side = !low;
+      if (side != r) {
+        mt[j] = m | kMFlip;
+        if (m & kMMulti) block_mark(hs, m & kMSlot, (r ? 2u : 0u) + (y[j] & 1u), 3);
+      }
     }
-    if ((low ? 0 : 1) != r) {
-      mt[j] = m | kMFlip;
-      if (m & kMMulti) block_mark(w.hb(), m & kMSlot, 2 * r + ((m & kMCol) ? 1 : 0), 3);
+    if (!kWarp) {
+      to_v += __popc(__ballot_sync(kFull, (m & kMValid) && side));
+      all += __popc(__ballot_sync(kFull, (m & kMValid) != 0));
     }
   }
   if (multi_any) tm.sync();
   // placement: each entry goes into the new row of its node after the trade
-  // (u's or v's row of step g+1) at a slot given by a scan over the team
-  int n0 = 0, n1 = 0;
-#pragma unroll
-  for (int j = 0; j < J; ++j) {
-    const uint32_t m = mt[j];
-    if (!(m & kMValid)) continue;
-    const int side = ((m & kMR) ? 1 : 0) ^ ((m & kMFlip) ? 1 : 0);
-    n0 += side == 0;
-    n1 += side;
+  // (u's or v's row of step g+1).  Slots follow (entry index j, lane), by
+  // ballots, so the stores of one instruction fill two runs.
+  uint32_t s0 = 0, s1 = 0;
+  if (!kWarp) {
+    const uint32_t pre = tm.warps_before((all - to_v) | (to_v << 16));
+    s0 = pre & 0xffffu;
+    s1 = pre >> 16;
   }
-  const int64_t pre = tm.exscan(static_cast<int64_t>(n0) | (static_cast<int64_t>(n1) << 32));
-  int s0 = static_cast<int>(pre & 0xffffffff), s1 = static_cast<int>(pre >> 32);
-  if (tm.rank == Team::N - 1 && (s0 + n0 != du || s1 + n1 != tr.dv)) latch(c.err, kErrRowLength);
+  int32_t* const ph_u = c.ph + ou;
+  int32_t* const ph_v = c.ph + ov;
+  uint16_t* const fb_u = c.fb + ou;
+  uint16_t* const fb_v = c.fb + ov;
 #pragma unroll
   for (int j = 0; j < J; ++j) {
     const uint32_t m = mt[j];
-    if (!(m & kMValid)) continue;
-    const int r = (m & kMR) ? 1 : 0;
+    const int r = tm.rank + j * N >= du ? 1 : 0;
     const int f = (m & kMFlip) ? 1 : 0;
+    const int side = r ^ f;
+    const unsigned bv = __ballot_sync(lanes, (m & kMValid) != 0) & lanes;
+    const unsigned b1 = __ballot_sync(lanes, (m & kMValid) && side) & lanes;
+    const uint32_t k = side ? s1 + __popc(b1 & below_me) : s0 + __popc((bv ^ b1) & below_me);
+    s0 += __popc(bv ^ b1);
+    s1 += __popc(b1);
+    if (!(m & kMValid)) continue;
     // will the far trade decide this edge?  (A single-edge block: yes,
     // unless the far node is the untraded one of an odd n, trade index T.)
     int in_far = 0;
@@ -1303,10 +1296,10 @@ __device__ void phase_a_reg(Team& tm, const StepCtx& c, int64_t t, const Ws& w) 
       if (!(m & kMMulti)) {
         in_far = s < T32;
       } else if (tr.single || s < t32) {
-        const uint32_t fl = block_flags(w.hb()[m & kMSlot]);
+        const uint32_t fl = block_flags(hs[m & kMSlot].y);
         in_far = __popc(r ? (fl & 12u) : (fl & 3u)) == 1;   // trade s acted before t: initial block
       } else if (s < T32) {   // block after t's own decisions: presence bits 0..3, flips 4..7
-        const uint32_t fl = block_flags(w.hb()[m & kMSlot]);
+        const uint32_t fl = block_flags(hs[m & kMSlot].y);
         const int myrow = r ^ f;
         int same = 0;
 #pragma unroll
@@ -1317,13 +1310,13 @@ __device__ void phase_a_reg(Team& tm, const StepCtx& c, int64_t t, const Ws& w) 
         in_far = (same == 1);
       }
     }
-    const int side = r ^ f;
-    const int k = side ? s1++ : s0++;
-    if (k >= (side ? tr.dv : du)) continue;   // counts checked above: never write outside the row
-    const int64_t slot = (side ? ov : ou) + k;
-    c.ph[slot] = static_cast<int32_t>(y[j]);
-    c.fb[slot] = static_cast<uint16_t>(f | (in_far ? (((m >> kMFarShift) << 1) | kFbInFar) : 0u));
+    if (k >= static_cast<uint32_t>(side ? tr.dv : du)) continue;   // checked below: never write outside the row
+    (side ? ph_v : ph_u)[k] = static_cast<int32_t>(y[j]);
+    (side ? fb_v : fb_u)[k] = static_cast<uint16_t>(f | (in_far ? (((m >> kMFarShift) << 1) | kFbInFar) : 0u));
   }
+  // the last warp's counts are the rows' lengths
+  if (tm.rank == N - 1 && (s0 != static_cast<uint32_t>(du) || s1 != static_cast<uint32_t>(tr.dv)))
+    latch(c.err, kErrRowLength);
   if (tm.rank == 0 && !tr.single) {
     c.thr_key[t] = tk;
     c.thr_tb[t] = tt;
@@ -1343,7 +1336,7 @@ __device__ void phase_a_reg(Team& tm, const StepCtx& c, int64_t t, const Ws& w) 
 constexpr int kWarpJ = 4;                       // entries per lane: trades up to 128 entries
 constexpr int kWarpB = 7;                       // first radix digit: 128 bins
 constexpr int kWarpWarps = 8;                   // warps per CTA
-using WarpWs = RegWs<32 * kWarpJ, kWarpB>;
+using WarpWs = RegWs<32 * kWarpJ, kWarpB, kCand>;
 
 // The smallest trades (L <= W J, W = 8 or 16) on teams of W lanes: 32 / W
 // trades per warp, so the per-trade work (clearing the tables, scans,
@@ -1352,7 +1345,7 @@ using WarpWs = RegWs<32 * kWarpJ, kWarpB>;
 template <int W>
 struct LaneCfg {
   static constexpr int B = W == 8 ? 5 : 6;   // ~1 first-digit bin per entry
-  using Ws = RegWs<W * kWarpJ, B>;
+  using Ws = RegWs<W * kWarpJ, B, 8>;   // a crowded bin (8 of the few entries) takes a further digit
   static constexpr int kTeams = 32 * kWarpWarps / W;   // teams per CTA
   static constexpr size_t kSmem = Ws::kBytes * kTeams;
 };
@@ -1389,7 +1382,7 @@ constexpr int kTeamJ = 4;
 template <int NT>
 struct TeamCfg {
   static constexpr int B = NT == 64 ? 8 : NT == 128 ? 9 : NT == 256 ? 10 : NT == 512 ? 11 : 12;   // ~1 bin per entry
-  using Ws = RegWs<NT * kTeamJ, B>;
+  using Ws = RegWs<NT * kTeamJ, B, kCand>;
   static constexpr int kMax = NT * kTeamJ;
 };
 template <int CT, int NT, bool kOneSeed>
@@ -2072,7 +2065,13 @@ int init_trade_kernels(Graph* h) {
                                   static_cast<int>(LaneCfg<8>::kSmem)));
   CB_CUDA(h, cudaFuncSetAttribute(k_phase_a_lanes<16>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                   static_cast<int>(LaneCfg<16>::kSmem)));
+  CB_CUDA(h, cudaFuncSetAttribute(k_phase_a_warp, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                  static_cast<int>(WarpWs::kBytes * kWarpWarps)));
+  CB_CUDA(h, cudaFuncSetAttribute(k_phase_a_list_warp, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                  static_cast<int>(WarpWs::kBytes * kWarpWarps)));
   // shared memory, not L1, limits how many CTAs of these kernels an SM holds
+  CB_CUDA(h, cudaFuncSetAttribute(k_phase_a_warp, cudaFuncAttributePreferredSharedMemoryCarveout,
+                                  cudaSharedmemCarveoutMaxShared));
   CB_CUDA(h, cudaFuncSetAttribute(k_phase_a_lanes<8>, cudaFuncAttributePreferredSharedMemoryCarveout,
                                   cudaSharedmemCarveoutMaxShared));
   CB_CUDA(h, cudaFuncSetAttribute(k_phase_a_lanes<16>, cudaFuncAttributePreferredSharedMemoryCarveout,
