@@ -1,4 +1,4 @@
-// Cooperative "teams" working on one trade or one row: part of a warp (8 or
+// Cooperative "teams" working on one trade or one row: part of a warp (4 to
 // 16 lanes, LaneTeam), a warp (WarpTeam), part of a CTA (64 to 512 threads
 // with a named barrier, SubTeam) or a whole CTA (BlockTeam).
 // The trade and row algorithms are written once against this interface; all
@@ -16,6 +16,8 @@ struct WarpTeam {
   __device__ __forceinline__ WarpTeam() : rank(threadIdx.x & 31) {}
   __device__ __forceinline__ void sync() const { __syncwarp(); }
   __device__ __forceinline__ bool any(bool p) const { return __any_sync(kFull, p); }
+  // does any team of this warp need a branch? (p is the same in every member)
+  __device__ __forceinline__ bool warp_any(bool p) const { return p; }
   __device__ __forceinline__ int64_t sum(int64_t v) const {
 #pragma unroll
     for (int o = 16; o; o >>= 1) v += __shfl_xor_sync(kFull, v, o);
@@ -52,43 +54,31 @@ struct WarpTeam {
   __device__ __forceinline__ uint32_t warps_before(uint32_t) const { return 0u; }
 };
 
-// W consecutive lanes of a warp (W = 8 or 16): a warp holds 32 / W such
-// teams, each on its own trade.  Synchronisation and shuffles name only the
-// team's lanes, so teams that diverge (different trip counts, an early
-// return) never wait for each other; while they run the same instructions,
-// one warp instruction serves all of them.
+// W consecutive lanes of a warp (W = 4, 8 or 16): a warp holds 32 / W such
+// teams, each on its own trade, in lockstep.  Every call names the whole
+// warp, so all teams must reach every call together (warp-uniform control
+// flow: a branch around a call is taken when any team needs it, see
+// warp_any).  Naming only a team's lanes instead let the teams drift apart,
+// and with a mask that the compiler does not know every vote and shuffle
+// costs a convergence check: 1736 warp instructions per round of four trades
+// against 1257 of a whole warp on one.
 template <int W>
 struct LaneTeam {
-  static_assert(W == 8 || W == 16, "lane teams of 8 or 16 lanes");
+  static_assert(W == 4 || W == 8 || W == 16, "lane teams of 4, 8 or 16 lanes");
   static constexpr int N = W;
   int rank;
   unsigned mask;
   __device__ __forceinline__ LaneTeam()
       : rank(threadIdx.x & (W - 1)), mask(((1u << W) - 1u) << ((threadIdx.x & 31) & ~(W - 1))) {}
-  __device__ __forceinline__ void sync() const { __syncwarp(mask); }
-  __device__ __forceinline__ bool any(bool p) const { return __any_sync(mask, p); }
-  __device__ __forceinline__ int64_t sum(int64_t v) const {
-#pragma unroll
-    for (int o = W / 2; o; o >>= 1) v += __shfl_xor_sync(mask, v, o, W);
-    return v;
-  }
-  __device__ __forceinline__ int64_t exscan(int64_t v) const {
-    int64_t x = v;
-#pragma unroll
-    for (int o = 1; o < W; o <<= 1) {
-      const int64_t y = __shfl_up_sync(mask, x, o, W);
-      if (rank >= o) x += y;
-    }
-    return x - v;
-  }
-  __device__ __forceinline__ uint64_t bcast(uint64_t v, int src) const { return __shfl_sync(mask, v, src, W); }
+  __device__ __forceinline__ void sync() const { __syncwarp(); }
+  __device__ __forceinline__ bool warp_any(bool p) const { return __any_sync(kFull, p); }
   // see WarpTeam; the flags travel as 5-bit counts above an 8-bit one, so one
   // shuffle chain serves them all (counts of at most 4 W <= 64 entries)
   __device__ __forceinline__ unsigned lanes() const { return mask; }
   __device__ __forceinline__ uint32_t count_or(uint32_t cnt, uint32_t flags) const {
     uint32_t v = cnt | ((flags >> 24 & 1u) << 8) | ((flags >> 25 & 1u) << 14) | ((flags >> 26 & 1u) << 20);
 #pragma unroll
-    for (int o = W / 2; o; o >>= 1) v += __shfl_xor_sync(mask, v, o, W);
+    for (int o = W / 2; o; o >>= 1) v += __shfl_xor_sync(kFull, v, o, W);
     return (v & 0xffu) | ((v & 0x3f00u) ? 1u << 24 : 0u) | ((v & 0xfc000u) ? 1u << 25 : 0u) |
            ((v >> 20) ? 1u << 26 : 0u);
   }
@@ -96,7 +86,7 @@ struct LaneTeam {
     uint32_t x = v;
 #pragma unroll
     for (int o = 1; o < W; o <<= 1) {
-      const uint32_t y = __shfl_up_sync(mask, x, o, W);
+      const uint32_t y = __shfl_up_sync(kFull, x, o, W);
       if (rank >= o) x += y;
     }
     return x - v;
@@ -151,6 +141,7 @@ struct BlockTeam {
     for (int o = 16; o; o >>= 1) before += __shfl_xor_sync(kFull, before, o);
     return x - v + before;
   }
+  __device__ __forceinline__ bool warp_any(bool p) const { return p; }
   // see WarpTeam; one barrier each, through the same two buffers
   __device__ __forceinline__ unsigned lanes() const { return kFull; }
   __device__ __forceinline__ uint32_t count_or(uint32_t cnt, uint32_t flags) {
@@ -277,6 +268,7 @@ struct SubTeam {
     for (int o = 16; o; o >>= 1) before += __shfl_xor_sync(kFull, before, o);
     return x - v + before;
   }
+  __device__ __forceinline__ bool warp_any(bool p) const { return p; }
   // see WarpTeam; one barrier each, through the same two buffers
   __device__ __forceinline__ unsigned lanes() const { return kFull; }
   __device__ __forceinline__ uint32_t count_or(uint32_t cnt, uint32_t flags) {

@@ -847,14 +847,22 @@ __device__ void phase_a(Team& tm, const StepCtx& c, int64_t t, const WsA& w, Sel
 // bin.  Used by the first pass only: a trade whose dependency has not
 // published yet is deferred to the in-order pass.
 
-// per-entry meta word (the entry's row is i >= deg u, its column the low bit of y)
-constexpr uint32_t kMSlot = 0x7FFFu;        // hash slot of the far trade
-constexpr uint32_t kMUV = 1u << 16;         // the edge {u, v}
-constexpr uint32_t kMInD = 1u << 17;        // element of D
-constexpr uint32_t kMFlip = 1u << 18;       // the trade moves the edge to its other node
-constexpr uint32_t kMValid = 1u << 19;      // an entry of the trade
-constexpr uint32_t kMMulti = 1u << 20;      // block of two or more edges
-constexpr int kMFarShift = 21;              // bits 21..31: top kFarBits bits of the far trade's key
+// Per entry a member keeps the neighbour position y, the top 32 bits of its
+// own key, and a word of the far trade's hash slot (bits 0..14) and the far
+// key's top kFarBits bits (from bit kMFarShift); per member, one bit per entry
+// j for what the entry is (valid, the edge {u, v}, in D, moved, in a
+// multi-edge block).
+constexpr uint32_t kMSlot = 0x7FFFu;
+constexpr int kMFarShift = 21;
+
+// a[j] for a j known at run time (a select chain: a stays in registers)
+template <int J>
+__device__ __forceinline__ uint32_t pick(const uint32_t (&a)[J], int j) {
+  uint32_t v = a[0];
+#pragma unroll
+  for (int k = 1; k < J; ++k) v = j == k ? a[k] : v;
+  return v;
+}
 
 __host__ __device__ constexpr int lg_ceil(int x) {
   int lg = 0;
@@ -978,15 +986,20 @@ __device__ __forceinline__ bool sel_match(int q, const uint32_t* pw, uint64_t ke
   return true;
 }
 
+// The common path is straight-line code over the J entries; everything that
+// few entries need (blocks of several edges, slots lost to another key, the
+// threshold bin's elements) runs in rolled loops over the member's bit masks,
+// so it exists once and stays out of the instruction cache's way.
 template <class Team, int J, int B, bool kKeepKey, bool kOneSeed = false, class Ws>
-__device__ void phase_a_reg(Team& tm, const StepCtx& c, int64_t t, const Ws& w) {
+__device__ void phase_a_reg(Team& tm, const StepCtx& c, int64_t t, const Ws& w, bool active = true) {
   constexpr int N = Team::N;
   constexpr bool kWarp = N <= 32;   // the team is a warp or part of one
-  static_assert((1 << B) == 4 * N, "four histogram bins per member");
-  static_assert(N * J <= Ws::kLmax && N * J < (1 << 16), "16-bit placement counts");
+  static_assert(J == 4 && (1 << B) == 4 * N, "four entries and four histogram bins per member");
+  static_assert(N * J == Ws::kLmax && N * J < (1 << 16), "16-bit placement counts");
+  constexpr int kLgH = lg_ceil(Ws::kH), kLgH2 = lg_ceil(Ws::kH2);
   const TradeRows tr = trade_rows(c, t);
   const KeyCtx kc = key_ctx(c, t);
-  const int du = tr.du, L = tr.du + tr.dv;
+  const int du = tr.du, L = active ? tr.du + tr.dv : 0;
   // the new rows' offsets, loaded now so their two dependent loads overlap
   // the trade's work
   const int64_t ou = c.rp_next[__ldg(c.M + 2 * t)];
@@ -995,127 +1008,137 @@ __device__ void phase_a_reg(Team& tm, const StepCtx& c, int64_t t, const Ws& w) 
   const uint32_t t2u = 2u * t32;
   const unsigned lanes = tm.lanes();
   const unsigned below_me = (1u << (threadIdx.x & 31)) - 1u;
-  const int lgL = 32 - __clz(max(L, 16) - 1);   // slots of table 2: the next power of two >= L (at least 16)
   uint2* const hs = w.hs();
   uint2* const hs2 = hs + Ws::kH;
   {
     const uint4 z = make_uint4(0u, 0u, 0u, 0u);
     reinterpret_cast<uint4*>(w.hist())[tm.rank] = z;
-    uint4* h4 = reinterpret_cast<uint4*>(hs2);
-    for (int i = tm.rank; i < (1 << (lgL - 1)); i += N) h4[i] = z;
+    uint4* h4 = reinterpret_cast<uint4*>(hs2);   // kH2 = 4 N slots of 8 bytes
+    h4[tm.rank] = z;
+    h4[tm.rank + N] = z;
     if (tm.rank == 0) *w.ncand() = 0;
   }
-  // entries and their home slots (at least 4 slots per entry): every entry
-  // stores its key there
+  // entries and their home slots: every entry stores its key there
   uint32_t y[J], mt[J], kt[J], kl[kKeepKey ? J : 1];
+  uint32_t hashed = 0, uv = 0;   // entries to other trades; the edge {u, v}
 #pragma unroll
   for (int j = 0; j < J; ++j) {
     const int i = tm.rank + j * N;
-    y[j] = 0;
-    mt[j] = 0;
-    kt[j] = 0;
-    if (kKeepKey) kl[j] = 0;
-    if (i < L) y[j] = static_cast<uint32_t>(__ldcg(c.col + tr.b0 + i));
+    y[j] = i < L ? static_cast<uint32_t>(__ldcg(c.col + tr.b0 + i)) : 0u;
   }
 #pragma unroll
   for (int j = 0; j < J; ++j) {
-    if (tm.rank + j * N >= L) continue;
     const uint32_t s = y[j] >> 1;
-    if (s == t32) {
-      mt[j] = kMValid | kMUV;
-    } else {
-      const uint32_t sl = hslot(s, lgL + 2);
-      hs[sl] = make_uint2(s + 1u, 0u);
-      mt[j] = kMValid | sl;
+    mt[j] = hslot(s, kLgH);
+    kt[j] = 0;
+    if (kKeepKey) kl[j] = 0;
+    if (tm.rank + j * N < L) {
+      if (s == t32) uv |= 1u << j;
+      else {
+        hashed |= 1u << j;
+        hs[mt[j]] = make_uint2(s + 1u, 0u);
+      }
     }
   }
+  uint32_t valid = hashed | uv;
+  // bit j: entry j sits in v's row
+  uint32_t in_v = 0;
+#pragma unroll
+  for (int j = 0; j < J; ++j) in_v |= (tm.rank + j * N >= du ? 1u : 0u) << j;
   tm.sync();
   // an entry whose key is in its slot marks its edge in the slot's block
   // word; the others (another key won the slot) take a slot of table 2
-  uint32_t pend = 0;
+  uint32_t lost = 0;
 #pragma unroll
   for (int j = 0; j < J; ++j) {
-    if (!(mt[j] & kMValid) || (mt[j] & kMUV)) continue;
-    const uint32_t sl = mt[j] & kMSlot;
-    const uint32_t q = (tm.rank + j * N >= du ? 2u : 0u) + (y[j] & 1u);
-    if (hs[sl].x == (y[j] >> 1) + 1u) block_mark(hs, sl, q, 1);
-    else pend |= 1u << j;
+    if (!((hashed >> j) & 1u)) continue;
+    const uint32_t q = 2u * ((in_v >> j) & 1u) + (y[j] & 1u);
+    if (hs[mt[j]].x == (y[j] >> 1) + 1u) block_mark(hs, mt[j], q, 1);
+    else lost |= 1u << j;
   }
-  if (pend) {
+  while (lost) {
+    const int j = __ffs(lost) - 1;
+    lost &= lost - 1u;
+    const uint32_t yj = pick(y, j), s = yj >> 1;
+    const uint32_t sl = Ws::kH + h_claim2(hs2, Ws::kH2 - 1u, s + 1u, (s * 0x85EBCA6Bu) >> (32 - kLgH2));
 #pragma unroll
-    for (int j = 0; j < J; ++j)
-      if ((pend >> j) & 1u) {
-        const uint32_t s = y[j] >> 1;
-        const uint32_t q = (tm.rank + j * N >= du ? 2u : 0u) + (y[j] & 1u);
-        const uint32_t sl = Ws::kH + h_claim2(hs2, (1u << lgL) - 1u, s + 1u, (s * 0x85EBCA6Bu) >> (32 - lgL));
-        mt[j] = kMValid | sl;
-        block_mark(hs, sl, q, 1);
-      }
+    for (int k = 0; k < J; ++k) mt[k] = j == k ? sl : mt[k];
+    block_mark(hs, sl, 2u * ((in_v >> j) & 1u) + (yj & 1u), 1);
   }
   tm.sync();
-  // block analysis, keys, histogram of the first radix digit
+  // blocks of two or more edges: common neighbours and dependencies
   constexpr uint32_t kFlDefer = 1u << 24, kFlDep = 1u << 25, kFlMulti = 1u << 26;
-  uint32_t flags = 0, cnt_a = 0;
+  uint32_t flags = 0, multi = 0;
+  uint32_t in_d = tr.single ? 0u : hashed;   // elements of D: the other row is not adjacent to the neighbour
 #pragma unroll
   for (int j = 0; j < J; ++j) {
-    uint32_t m = mt[j];
-    if (!(m & kMValid) || (m & kMUV)) continue;
-    const int r = tm.rank + j * N >= du ? 1 : 0;
-    const uint32_t s = y[j] >> 1;
-    const uint32_t fw = hs[m & kMSlot].y;
-    int other = 0;   // the other row is adjacent to this neighbour when t acts
-    if (fw & (fw - 1u)) {
-      // a block of two or more edges: common neighbours and dependencies
-      m |= kMMulti;
-      flags |= kFlMulti;
-      const uint32_t colb = y[j] & 1u;
-      const uint32_t f = block_flags(fw) & 15u;
-      const int u0 = f & 1, u1 = (f >> 1) & 1, v0 = (f >> 2) & 1, v1 = (f >> 3) & 1;
-      const int cu = u0 + u1, cv = v0 + v1;
-      if (!tr.single && s > t32 && s < T32 && (u0 + v0 == 1 || u1 + v1 == 1)) flags |= kFlDep;
-      const int col_now = static_cast<int>(colb);
-      other = r ? (col_now ? u1 : u0) : (col_now ? v1 : v0);
-      if (!tr.single && s < t32 && (cu == 1 || cv == 1)) {
-        // unpublished: a parallel pass leaves the trade to a later pass,
-        // an in-order pass waits
-        if (ld_acquire(c.done + s) != c.stamp &&
-            !(c.wait && wait_published(c.done + s, c.err, c.stamp, c.wait_ns))) {
-          flags |= kFlDefer;
-          mt[j] = m;
-          continue;
-        }
-        other = replay_other(c.thr_key, c.thr_tb, kc, t2u, s, f, r, static_cast<int>(colb));
+    const uint32_t fw = hs[mt[j]].y;
+    if (fw & (fw - 1u)) multi |= 1u << j;
+  }
+  multi &= hashed;
+  for (uint32_t left = multi; left;) {
+    const int j = __ffs(left) - 1;
+    left &= left - 1u;
+    flags |= kFlMulti;
+    const uint32_t yj = pick(y, j), s = yj >> 1;
+    const int r = (in_v >> j) & 1u, colb = yj & 1u;
+    const uint32_t f = block_flags(hs[pick(mt, j)].y) & 15u;
+    const int u0 = f & 1, u1 = (f >> 1) & 1, v0 = (f >> 2) & 1, v1 = (f >> 3) & 1;
+    const int cu = u0 + u1, cv = v0 + v1;
+    if (!tr.single && s > t32 && s < T32 && (u0 + v0 == 1 || u1 + v1 == 1)) flags |= kFlDep;
+    int other = r ? (colb ? u1 : u0) : (colb ? v1 : v0);   // the other row is adjacent when t acts
+    if (!tr.single && s < t32 && (cu == 1 || cv == 1)) {
+      // unpublished: a parallel pass leaves the trade to a later pass, an
+      // in-order pass waits
+      if (ld_acquire(c.done + s) != c.stamp && !(c.wait && wait_published(c.done + s, c.err, c.stamp, c.wait_ns))) {
+        flags |= kFlDefer;
+        break;
       }
+      other = replay_other(c.thr_key, c.thr_tb, kc, t2u, s, f, r, colb);
     }
-    // both trades' keys of this edge (step-start positions)
-    const uint32_t x = t2u + r, yb = y[j];
+    if (other) in_d &= ~(1u << j);
+  }
+  // both trades' keys of every edge (step-start positions), histogram of the
+  // first radix digit
+#pragma unroll
+  for (int j = 0; j < J; ++j) {
+    if (!((hashed >> j) & 1u)) continue;
+    const uint32_t x = t2u + ((in_v >> j) & 1u), yb = y[j];
     const EdgeKeys ek = edge_keys<kOneSeed>(c, kc, min(x, yb), max(x, yb));
-    const bool lo_mine = s > t32;   // the own end is the lower position
+    const bool lo_mine = x < yb;
     kt[j] = static_cast<uint32_t>((lo_mine ? ek.lo_side : ek.hi_side) >> 32);
     if (kKeepKey) kl[j] = static_cast<uint32_t>(lo_mine ? ek.lo_side : ek.hi_side);
-    m |= (static_cast<uint32_t>((lo_mine ? ek.hi_side : ek.lo_side) >> 32) >> (32 - kFarBits)) << kMFarShift;
-    if (!other && !tr.single) {
-      m |= kMInD;
-      cnt_a += (r == 0);
-      atomicAdd(&w.hist()[kt[j] >> (32 - B)], 1u);
-    }
-    mt[j] = m;
+    mt[j] |= (static_cast<uint32_t>((lo_mine ? ek.hi_side : ek.lo_side) >> 32) >> (32 - kFarBits)) << kMFarShift;
+    if ((in_d >> j) & 1u) atomicAdd(&w.hist()[kt[j] >> (32 - B)], 1u);
   }
   // one reduction: |A_{u-v}|, and whether any member saw a deferral, a later
-  // dependent trade, a multi-edge block (it also orders the histogram)
-  const uint32_t tot = tm.count_or(cnt_a, flags);
+  // dependent trade, a multi-edge block (a barrier of larger teams, so it
+  // also orders the histogram)
+  const uint32_t tot = tm.count_or(__popc(in_d & ~in_v), flags);
   if (tot & kFlDefer) {
     if (tm.rank == 0) defer_trade(c, t, L);
+    active = false;
+  }
+  if (!tm.warp_any(active)) {
     tm.sync();
     return;
   }
-  const uint32_t a = tot & 0xffffffu;
+  if (!active) valid = hashed = in_d = multi = 0;   // teams in lockstep: the others' trades go on
+  const uint32_t a = active ? tot & 0xffffffu : 0u;
   const bool publish_fence = (tot & kFlDep) != 0;
   const bool multi_any = (tot & kFlMulti) != 0;
   const bool no_thr = tr.single || a == 0;   // u keeps nothing of D
+  // the edge of entry j and its own key
+  auto edge_of = [&](int j, uint32_t* lo, uint32_t* hi) -> uint64_t {
+    const uint32_t x = t2u + ((in_v >> j) & 1u), yj = pick(y, j);
+    *lo = min(x, yj);
+    *hi = max(x, yj);
+    if constexpr (kKeepKey) return (static_cast<uint64_t>(pick(kt, j)) << 32) | pick(kl, j);
+    else return own_key(kc, t, *lo, *hi);
+  };
   if (kWarp) tm.sync();
   uint64_t tk = 0, tt = 0;
-  if (!no_thr) {
+  if (tm.warp_any(!no_thr)) {
     // the bin of the first digit (top B key bits) that holds the a-th
     // smallest element: four bins per member
     uint32_t bin = 0, below = 0, cnt = 0;
@@ -1131,11 +1154,11 @@ __device__ void phase_a_reg(Team& tm, const StepCtx& c, int64_t t, const Ws& w) 
       if (k <= h.x) { p = 0; pb = 0; pc = h.x; }
       if (kWarp) {   // at most 128 entries: 8-bit fields
         const uint32_t info = (4u * tm.rank + p) | ((run + pb) << 8) | (pc << 16);
-        const int src = __ffs(__ballot_sync(lanes, found) & lanes) - 1;
-        const uint32_t got = __shfl_sync(lanes, info, src);
+        const int src = __ffs(__ballot_sync(kFull, found) & lanes) - 1;
+        const uint32_t got = __shfl_sync(kFull, info, src & 31);
         bin = got & 0xffu;
         below = (got >> 8) & 0xffu;
-        cnt = got >> 16;
+        cnt = no_thr ? 0u : got >> 16;
       } else {
         if (found) {
           w.sel()->bin = static_cast<int32_t>(4u * tm.rank + p);
@@ -1151,7 +1174,7 @@ __device__ void phase_a_reg(Team& tm, const StepCtx& c, int64_t t, const Ws& w) 
     int qbits = B;              // top bits of the order fixed so far
     uint32_t kk = a - below;    // rank sought among the elements sharing them
     const uint32_t cap = min(static_cast<uint32_t>(c.cand_max), static_cast<uint32_t>(Ws::kCandCap));
-    if (cnt > cap) {
+    if (tm.warp_any(cnt > cap)) {
       // more elements share the prefix than the candidate list holds (or the
       // list is disabled): further B-bit digits of (key, lo, hi)
       tm.sync();
@@ -1159,15 +1182,15 @@ __device__ void phase_a_reg(Team& tm, const StepCtx& c, int64_t t, const Ws& w) 
         w.pw()[0] = bin << (32 - B);
         w.pw()[1] = w.pw()[2] = w.pw()[3] = 0u;
       }
-      while (cnt > cap) {
+      while (tm.warp_any(cnt > cap)) {
+        const bool need = cnt > cap;
         reinterpret_cast<uint4*>(w.hist())[tm.rank] = make_uint4(0u, 0u, 0u, 0u);
         tm.sync();
-#pragma unroll
-        for (int j = 0; j < J; ++j) {
-          if (!(mt[j] & kMInD)) continue;
-          const uint32_t x = t2u + (tm.rank + j * N >= du ? 1u : 0u);
-          const uint32_t lo = min(x, y[j]), hi = max(x, y[j]);
-          const uint64_t key = kKeepKey ? ((static_cast<uint64_t>(kt[j]) << 32) | kl[j]) : own_key(kc, t, lo, hi);
+        for (uint32_t left = need ? in_d : 0u; left;) {
+          const int j = __ffs(left) - 1;
+          left &= left - 1u;
+          uint32_t lo, hi;
+          const uint64_t key = edge_of(j, &lo, &hi);
           if (sel_match(qbits, w.pw(), key, lo, hi)) atomicAdd(&w.hist()[sel_digit(qbits, B, key, lo, hi)], 1u);
         }
         tm.sync();
@@ -1176,7 +1199,7 @@ __device__ void phase_a_reg(Team& tm, const StepCtx& c, int64_t t, const Ws& w) 
         uint32_t run = tm.exscan32(h.x + h.y + h.z + h.w);
 #pragma unroll
         for (int q = 0; q < 4; ++q) {
-          if (run < kk && kk <= run + hv[q]) {
+          if (need && run < kk && kk <= run + hv[q]) {
             w.sel()->bin = 4 * tm.rank + q;
             w.sel()->below = static_cast<int32_t>(run);
             w.sel()->cnt = static_cast<int32_t>(hv[q]);
@@ -1185,25 +1208,29 @@ __device__ void phase_a_reg(Team& tm, const StepCtx& c, int64_t t, const Ws& w) 
         }
         tm.sync();
         const uint32_t dig = static_cast<uint32_t>(w.sel()->bin);
-        kk -= static_cast<uint32_t>(w.sel()->below);
-        cnt = static_cast<uint32_t>(w.sel()->cnt);
-        if (tm.rank == 0) {   // append the digit to the prefix (it may straddle two words)
+        if (need) {
+          kk -= static_cast<uint32_t>(w.sel()->below);
+          cnt = static_cast<uint32_t>(w.sel()->cnt);
+        }
+        if (need && tm.rank == 0) {   // append the digit to the prefix (it may straddle two words)
           const int wd = qbits >> 5, off = qbits & 31;
           const uint64_t d64 = static_cast<uint64_t>(dig) << (64 - B - off);
           w.pw()[wd] |= static_cast<uint32_t>(d64 >> 32);
           if (wd < 3) w.pw()[wd + 1] |= static_cast<uint32_t>(d64);
         }
-        qbits += B;
+        if (need) qbits += B;
         tm.sync();
       }
     }
     // rank the few elements that share the prefix by their full order
+    uint32_t cand = 0;
 #pragma unroll
-    for (int j = 0; j < J; ++j) {
-      if (!(mt[j] & kMInD) || (kt[j] >> (32 - B)) != bin) continue;
-      const uint32_t x = t2u + (tm.rank + j * N >= du ? 1u : 0u);
-      const uint32_t lo = min(x, y[j]), hi = max(x, y[j]);
-      const uint64_t key = kKeepKey ? ((static_cast<uint64_t>(kt[j]) << 32) | kl[j]) : own_key(kc, t, lo, hi);
+    for (int j = 0; j < J; ++j) cand |= ((kt[j] >> (32 - B)) == bin ? 1u : 0u) << j;
+    for (cand = cnt ? cand & in_d : 0u; cand;) {
+      const int j = __ffs(cand) - 1;
+      cand &= cand - 1u;
+      uint32_t lo, hi;
+      const uint64_t key = edge_of(j, &lo, &hi);
       if (qbits > B && !sel_match(qbits, w.pw(), key, lo, hi)) continue;
       if (cnt == 1) {
         w.sel()->key = key;
@@ -1215,8 +1242,8 @@ __device__ void phase_a_reg(Team& tm, const StepCtx& c, int64_t t, const Ws& w) 
       }
     }
     tm.sync();
-    if (cnt > 1) {
-      for (uint32_t q = tm.rank; q < cnt; q += N) {
+    if (tm.warp_any(cnt > 1)) {
+      for (uint32_t q = tm.rank; cnt > 1 && q < cnt; q += N) {
         uint32_t rk = 0;
         for (uint32_t p = 0; p < cnt; ++p)
           rk += (w.ck()[p] < w.ck()[q] || (w.ck()[p] == w.ck()[q] && w.ctb()[p] < w.ctb()[q]));
@@ -1227,48 +1254,69 @@ __device__ void phase_a_reg(Team& tm, const StepCtx& c, int64_t t, const Ws& w) 
       }
       tm.sync();
     }
-    tk = w.sel()->key;
-    tt = w.sel()->tb;
+    if (!no_thr) {
+      tk = w.sel()->key;
+      tt = w.sel()->tb;
+    }
   }
-  // own decisions: u keeps the elements at or below the threshold; and how
-  // many entries of this warp land in u's and in v's new row
+  // own decisions: u keeps the elements at or below the threshold
   const uint32_t tk32 = static_cast<uint32_t>(tk >> 32);
-  uint32_t to_v = 0, all = 0;
+  uint32_t above = 0, equal = 0;
 #pragma unroll
   for (int j = 0; j < J; ++j) {
-    const uint32_t m = mt[j];
-    const bool r = tm.rank + j * N >= du;
-    bool side = r;
-    if (m & kMInD) {
-      bool low;
-      if (no_thr) {
-        low = false;
-      } else if (kt[j] != tk32) {
-        low = kt[j] < tk32;
-      } else {
-        const uint32_t x = t2u + (r ? 1u : 0u);
-        const uint32_t lo = min(x, y[j]), hi = max(x, y[j]);
-        const uint64_t key = kKeepKey ? ((static_cast<uint64_t>(kt[j]) << 32) | kl[j]) : own_key(kc, t, lo, hi);
-        low = at_or_below(key, tie_break(lo, hi), tk, tt);
-      }
-      side = !low;
-      if (side != r) {
-        mt[j] = m | kMFlip;
-        if (m & kMMulti) block_mark(hs, m & kMSlot, (r ? 2u : 0u) + (y[j] & 1u), 3);
-      }
-    }
-    if (!kWarp) {
-      to_v += __popc(__ballot_sync(kFull, (m & kMValid) && side));
-      all += __popc(__ballot_sync(kFull, (m & kMValid) != 0));
+    above |= (kt[j] > tk32 ? 1u : 0u) << j;
+    equal |= (kt[j] == tk32 ? 1u : 0u) << j;
+  }
+  if (no_thr) {
+    above = 0xfu;
+  } else {
+    for (equal &= in_d; equal;) {   // the threshold itself, and keys that share its top half
+      const int j = __ffs(equal) - 1;
+      equal &= equal - 1u;
+      uint32_t lo, hi;
+      const uint64_t key = edge_of(j, &lo, &hi);
+      if (!at_or_below(key, tie_break(lo, hi), tk, tt)) above |= 1u << j;
     }
   }
-  if (multi_any) tm.sync();
+  const uint32_t flip = (above ^ in_v) & in_d;   // elements that change node
+  const uint32_t side = in_v ^ flip;             // the row each entry lands in
+  if (tm.warp_any(multi_any)) {
+    for (uint32_t left = multi & flip; left;) {
+      const int j = __ffs(left) - 1;
+      left &= left - 1u;
+      block_mark(hs, pick(mt, j) & kMSlot, 2u * ((in_v >> j) & 1u) + (pick(y, j) & 1u), 3);
+    }
+    tm.sync();
+  }
+  // will the far trade decide the edge?  (A single-edge block: yes, unless
+  // the far node is the untraded one of an odd n, trade index T.)
+  uint32_t in_far = 0;
+#pragma unroll
+  for (int j = 0; j < J; ++j) in_far |= ((y[j] >> 1) < T32 ? 1u : 0u) << j;
+  in_far &= hashed;
+  for (uint32_t left = multi; left;) {
+    const int j = __ffs(left) - 1;
+    left &= left - 1u;
+    const uint32_t fl = block_flags(hs[pick(mt, j) & kMSlot].y), s = pick(y, j) >> 1;
+    int same = 0;
+    if (tr.single || s < t32) {   // trade s acted before t: initial block
+      same = __popc((in_v >> j) & 1u ? (fl & 12u) : (fl & 3u));
+    } else if (s < T32) {         // block after t's own decisions: presence bits 0..3, flips 4..7
+      const uint32_t row = (side >> j) & 1u;
+#pragma unroll
+      for (int q = 0; q < 4; ++q)
+        if ((fl >> q) & 1) same += (((q >> 1) ^ ((fl >> (4 + q)) & 1)) == row);
+    }
+    if (same != 1) in_far &= ~(1u << j);
+  }
   // placement: each entry goes into the new row of its node after the trade
   // (u's or v's row of step g+1).  Slots follow (entry index j, lane), by
   // ballots, so the stores of one instruction fill two runs.
   uint32_t s0 = 0, s1 = 0;
   if (!kWarp) {
-    const uint32_t pre = tm.warps_before((all - to_v) | (to_v << 16));
+    const uint32_t nv = __reduce_add_sync(kFull, __popc(valid & side));
+    const uint32_t nu = __reduce_add_sync(kFull, __popc(valid & ~side));
+    const uint32_t pre = tm.warps_before(nu | (nv << 16));
     s0 = pre & 0xffffu;
     s1 = pre >> 16;
   }
@@ -1278,46 +1326,22 @@ __device__ void phase_a_reg(Team& tm, const StepCtx& c, int64_t t, const Ws& w) 
   uint16_t* const fb_v = c.fb + ov;
 #pragma unroll
   for (int j = 0; j < J; ++j) {
-    const uint32_t m = mt[j];
-    const int r = tm.rank + j * N >= du ? 1 : 0;
-    const int f = (m & kMFlip) ? 1 : 0;
-    const int side = r ^ f;
-    const unsigned bv = __ballot_sync(lanes, (m & kMValid) != 0) & lanes;
-    const unsigned b1 = __ballot_sync(lanes, (m & kMValid) && side) & lanes;
-    const uint32_t k = side ? s1 + __popc(b1 & below_me) : s0 + __popc((bv ^ b1) & below_me);
-    s0 += __popc(bv ^ b1);
+    const bool mine = (valid >> j) & 1u, to_v = (side >> j) & 1u;
+    const unsigned b1 = __ballot_sync(kFull, mine && to_v) & lanes;
+    const unsigned b0 = __ballot_sync(kFull, mine && !to_v) & lanes;
+    const uint32_t k = (to_v ? s1 : s0) + __popc((to_v ? b1 : b0) & below_me);
+    s0 += __popc(b0);
     s1 += __popc(b1);
-    if (!(m & kMValid)) continue;
-    // will the far trade decide this edge?  (A single-edge block: yes,
-    // unless the far node is the untraded one of an odd n, trade index T.)
-    int in_far = 0;
-    if (!(m & kMUV)) {
-      const uint32_t s = y[j] >> 1;
-      if (!(m & kMMulti)) {
-        in_far = s < T32;
-      } else if (tr.single || s < t32) {
-        const uint32_t fl = block_flags(hs[m & kMSlot].y);
-        in_far = __popc(r ? (fl & 12u) : (fl & 3u)) == 1;   // trade s acted before t: initial block
-      } else if (s < T32) {   // block after t's own decisions: presence bits 0..3, flips 4..7
-        const uint32_t fl = block_flags(hs[m & kMSlot].y);
-        const int myrow = r ^ f;
-        int same = 0;
-#pragma unroll
-        for (int q = 0; q < 4; ++q) {
-          if (!((fl >> q) & 1)) continue;
-          same += (((q >> 1) ^ ((fl >> (4 + q)) & 1)) == myrow);
-        }
-        in_far = (same == 1);
-      }
+    if (mine && k < static_cast<uint32_t>(to_v ? tr.dv : du)) {   // checked below: never outside the row
+      (to_v ? ph_v : ph_u)[k] = static_cast<int32_t>(y[j]);
+      (to_v ? fb_v : fb_u)[k] = static_cast<uint16_t>(
+          ((flip >> j) & 1u) | ((in_far >> j) & 1u ? (((mt[j] >> kMFarShift) << 1) | kFbInFar) : 0u));
     }
-    if (k >= static_cast<uint32_t>(side ? tr.dv : du)) continue;   // checked below: never write outside the row
-    (side ? ph_v : ph_u)[k] = static_cast<int32_t>(y[j]);
-    (side ? fb_v : fb_u)[k] = static_cast<uint16_t>(f | (in_far ? (((m >> kMFarShift) << 1) | kFbInFar) : 0u));
   }
   // the last warp's counts are the rows' lengths
-  if (tm.rank == N - 1 && (s0 != static_cast<uint32_t>(du) || s1 != static_cast<uint32_t>(tr.dv)))
+  if (active && tm.rank == N - 1 && (s0 != static_cast<uint32_t>(du) || s1 != static_cast<uint32_t>(tr.dv)))
     latch(c.err, kErrRowLength);
-  if (tm.rank == 0 && !tr.single) {
+  if (active && tm.rank == 0 && !tr.single) {
     c.thr_key[t] = tk;
     c.thr_tb[t] = tt;
     c.thr_top[t] = static_cast<uint8_t>(tk >> 56);
@@ -1349,7 +1373,7 @@ struct LaneCfg {
   static constexpr int kTeams = 32 * kWarpWarps / W;   // teams per CTA
   static constexpr size_t kSmem = Ws::kBytes * kTeams;
 };
-template <int W>
+template <int W, bool kOneSeed>
 __global__ void __launch_bounds__(32 * kWarpWarps, 4) k_phase_a_lanes(StepCtx c, const int32_t* __restrict__ lists,
                                                                    const int64_t* __restrict__ ctr, int cls) {
   using Cfg = LaneCfg<W>;
@@ -1359,10 +1383,16 @@ __global__ void __launch_bounds__(32 * kWarpWarps, 4) k_phase_a_lanes(StepCtx c,
   LaneTeam<W> tm;
   const ClassList cl = class_list(lists, ctr, cls);
   const int64_t step = static_cast<int64_t>(gridDim.x) * Cfg::kTeams;
-  for (int64_t q = static_cast<int64_t>(blockIdx.x) * Cfg::kTeams + id; q < cl.len; q += step)
-    phase_a_reg<LaneTeam<W>, kWarpJ, Cfg::B, true>(tm, c, cl.list[q], w);
+  // a warp's teams run in lockstep, so its loop ends when none has a trade
+  const int first = id & ~(32 / W - 1);
+  for (int64_t q0 = static_cast<int64_t>(blockIdx.x) * Cfg::kTeams + first; q0 < cl.len; q0 += step) {
+    const int64_t q = q0 + (id - first);
+    const bool active = q < cl.len;
+    phase_a_reg<LaneTeam<W>, kWarpJ, Cfg::B, true, kOneSeed>(tm, c, cl.list[active ? q : q0], w, active);
+  }
 }
 
+template <bool kOneSeed>
 __global__ void __launch_bounds__(32 * kWarpWarps, 4) k_phase_a_warp(StepCtx c, const int32_t* __restrict__ lists,
                                                                   const int64_t* __restrict__ ctr, int cls) {
   extern __shared__ __align__(16) char wsm[];
@@ -1372,7 +1402,7 @@ __global__ void __launch_bounds__(32 * kWarpWarps, 4) k_phase_a_warp(StepCtx c, 
   const ClassList cl = class_list(lists, ctr, cls);
   const int64_t step = static_cast<int64_t>(gridDim.x) * kWarpWarps;
   for (int64_t q = static_cast<int64_t>(blockIdx.x) * kWarpWarps + wid; q < cl.len; q += step)
-    phase_a_reg<WarpTeam, kWarpJ, kWarpB, true>(tm, c, cl.list[q], w);
+    phase_a_reg<WarpTeam, kWarpJ, kWarpB, true, kOneSeed>(tm, c, cl.list[q], w);
 }
 
 // Phase A of larger trades: a CTA of CT threads holds CT / NT teams of NT
@@ -2038,9 +2068,21 @@ int init_seed_kernels(Graph* h) {
   CB_CUDA(h, cudaFuncSetAttribute(k_phase_a_team<kBigThreads, kBigThreads, kOneSeed>,
                                   cudaFuncAttributeMaxDynamicSharedMemorySize,
                                   static_cast<int>(team_smem<kBigThreads, kBigThreads>())));
-  // shared memory, not L1, limits how many CTAs of this kernel an SM holds
+  CB_CUDA(h, cudaFuncSetAttribute(k_phase_a_lanes<8, kOneSeed>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                  static_cast<int>(LaneCfg<8>::kSmem)));
+  CB_CUDA(h, cudaFuncSetAttribute(k_phase_a_lanes<16, kOneSeed>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                  static_cast<int>(LaneCfg<16>::kSmem)));
+  CB_CUDA(h, cudaFuncSetAttribute(k_phase_a_warp<kOneSeed>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                  static_cast<int>(WarpWs::kBytes * kWarpWarps)));
+  // shared memory, not L1, limits how many CTAs of these kernels an SM holds
   CB_CUDA(h, cudaFuncSetAttribute(k_phase_a_block<kMedThreads, kOneSeed>,
                                   cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared));
+  CB_CUDA(h, cudaFuncSetAttribute(k_phase_a_lanes<8, kOneSeed>, cudaFuncAttributePreferredSharedMemoryCarveout,
+                                  cudaSharedmemCarveoutMaxShared));
+  CB_CUDA(h, cudaFuncSetAttribute(k_phase_a_lanes<16, kOneSeed>, cudaFuncAttributePreferredSharedMemoryCarveout,
+                                  cudaSharedmemCarveoutMaxShared));
+  CB_CUDA(h, cudaFuncSetAttribute(k_phase_a_warp<kOneSeed>, cudaFuncAttributePreferredSharedMemoryCarveout,
+                                  cudaSharedmemCarveoutMaxShared));
   return CB_OK;
 }
 }  // namespace
@@ -2061,21 +2103,8 @@ int init_trade_kernels(Graph* h) {
   CB_CUDA(h, cudaFuncSetAttribute(k_phase_a_list<kBigThreads>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                   static_cast<int>(std::max(TeamCfg<kBigThreads>::Ws::kBytes,
                                                             ws_a_bytes(kSmemMaxCap)))));
-  CB_CUDA(h, cudaFuncSetAttribute(k_phase_a_lanes<8>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                  static_cast<int>(LaneCfg<8>::kSmem)));
-  CB_CUDA(h, cudaFuncSetAttribute(k_phase_a_lanes<16>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                  static_cast<int>(LaneCfg<16>::kSmem)));
-  CB_CUDA(h, cudaFuncSetAttribute(k_phase_a_warp, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                  static_cast<int>(WarpWs::kBytes * kWarpWarps)));
   CB_CUDA(h, cudaFuncSetAttribute(k_phase_a_list_warp, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                   static_cast<int>(WarpWs::kBytes * kWarpWarps)));
-  // shared memory, not L1, limits how many CTAs of these kernels an SM holds
-  CB_CUDA(h, cudaFuncSetAttribute(k_phase_a_warp, cudaFuncAttributePreferredSharedMemoryCarveout,
-                                  cudaSharedmemCarveoutMaxShared));
-  CB_CUDA(h, cudaFuncSetAttribute(k_phase_a_lanes<8>, cudaFuncAttributePreferredSharedMemoryCarveout,
-                                  cudaSharedmemCarveoutMaxShared));
-  CB_CUDA(h, cudaFuncSetAttribute(k_phase_a_lanes<16>, cudaFuncAttributePreferredSharedMemoryCarveout,
-                                  cudaSharedmemCarveoutMaxShared));
   return CB_OK;
 }
 
@@ -2212,14 +2241,14 @@ int super_step(Graph* h) {
     int r;
     if ((r = mark(0))) return r;
     if (h->lane_teams) {
-      k_phase_a_lanes<8><<<wgrid, 32 * kWarpWarps, LaneCfg<8>::kSmem, s>>>(c, L, cnt, 0);
+      k_phase_a_lanes<8, kOne><<<wgrid, 32 * kWarpWarps, LaneCfg<8>::kSmem, s>>>(c, L, cnt, 0);
       if ((r = launched()) || (r = mark(1))) return r;
-      k_phase_a_lanes<16><<<wgrid, 32 * kWarpWarps, LaneCfg<16>::kSmem, s>>>(c, L, cnt, 1);
+      k_phase_a_lanes<16, kOne><<<wgrid, 32 * kWarpWarps, LaneCfg<16>::kSmem, s>>>(c, L, cnt, 1);
       if ((r = launched()) || (r = mark(2))) return r;
     } else if ((r = mark(1)) || (r = mark(2))) {
       return r;
     }
-    k_phase_a_warp<<<wgrid, 32 * kWarpWarps, WarpWs::kBytes * kWarpWarps, s>>>(c, L, cnt, 2);
+    k_phase_a_warp<kOne><<<wgrid, 32 * kWarpWarps, WarpWs::kBytes * kWarpWarps, s>>>(c, L, cnt, 2);
     if ((r = launched()) || (r = mark(3))) return r;
     if (h->cta_paths) {
       k_phase_a_team<256, 64, kOne><<<mgrid, 256, team_smem<256, 64>(), s>>>(c, L, cnt, 3);
