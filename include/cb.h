@@ -233,10 +233,11 @@ int cb_timings(cb_handle h, double* ms, int count);
  *   "cand_max"  register paths: when at most this many elements share the
  *               threshold's leading key bits they are ranked directly,
  *               else more radix digits follow [32]; 1..32 (a test knob).
- *   "inorder_threads" CTA size of the pass that runs deferred trades in
- *               index order: 1024 (large trades in shared memory) or 256
- *               (four CTAs per SM; trades above block_max from global
- *               memory) [1024; 256 for cb_create_batch].
+ *   "inorder_threads" CTA size of the pass that completes the deferred
+ *               trades in index order: 1024 (large trades in shared memory)
+ *               or 256 (four CTAs per SM; trades above 1024 entries in
+ *               shared memory up to block_max, from global memory above)
+ *               [1024; 256 for cb_create_batch].
  *   "uniform_threads" CTA size of the executor of cb_uniform_trades: 256
  *               (two CTAs per SM), 512 or 1024 (more threads per hub trade,
  *               fewer trades at once) [1024].
@@ -245,6 +246,8 @@ int cb_timings(cb_handle h, double* ms, int count);
  *   "retry_passes" parallel passes over the deferred trades between the
  *               first pass and the in-order pass, each running every deferred
  *               trade whose dependencies have published by then [2]; 0..4.
+ *               Handles of fewer than 2^20 trades go straight to the in-order
+ *               pass, which is faster there.
  *   "relaxed"   1: relaxed global trades (Def. "Relaxed global trade",
  *               Appendix EM-GCB): super step g orders the nodes by
  *               h(x) = (a x + b) mod p, p the smallest prime >= n, with

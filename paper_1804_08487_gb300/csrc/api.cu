@@ -24,12 +24,6 @@ __global__ void k_degrees(int64_t n, const int64_t* __restrict__ rp, int32_t* __
   atomicMax(maxdeg, local);
 }
 
-__global__ void k_gather_deg(int64_t n, const int32_t* __restrict__ order, const int32_t* __restrict__ deg_id,
-                             int32_t* __restrict__ out) {
-  for (int64_t p = blockIdx.x * int64_t(blockDim.x) + threadIdx.x; p < n; p += int64_t(gridDim.x) * blockDim.x)
-    out[p] = deg_id[order[p]];
-}
-
 unsigned grid1d(int64_t work, int num_sms) {
   const int64_t want = (work + 255) / 256;
   return static_cast<unsigned>(std::max<int64_t>(1, std::min<int64_t>(want, int64_t(num_sms) * 16)));
@@ -66,9 +60,8 @@ void release(Graph* h) {
   free_uniform(h);
   free_presence(h);
   void* bufs[] = {h->deg_id, h->rp_id, h->order[0], h->order[1], h->rp[0], h->rp[1], h->col[0], h->col[1],
-                  h->pos_next, h->M, h->deg_next, h->stash, h->thr_key, h->thr_tb, h->thr_top, h->done,
-                  h->lists, h->dlist, h->Minv, h->cls_flag, h->cls_scan,
-                  h->counters, h->err,
+                  h->pos[0], h->pos[1], h->stash, h->thr_key, h->thr_tb, h->done,
+                  h->chunk_row, h->lists, h->def_list, h->def_bits, h->def_seg, h->counters, h->err,
                   h->ws_global, h->sort_ws, h->scan_ws, h->segs, h->seg_of, h->pairs, h->far_pack,
                   h->lcg_ab, h->lcg_gaps, h->swaps};
   if (h->stream)
@@ -220,14 +213,6 @@ void destroy_graph(Graph* h) {
   delete static_cast<cb_graph*>(h);
 }
 
-// Scratch int32: the trade classes' counts per 2048-trade chunk, then
-// (rebuild) the first row of each 2048-entry chunk plus one.
-int64_t cls_flag_count(int64_t ntasks, int64_t nnz) {
-  return std::max<int64_t>(kClasses * (ntasks / 2048 + 1), nnz / 2048 + 2);
-}
-// Scratch int64: the exclusive scan of those counts.
-int64_t cls_scan_count(int64_t ntasks) { return kClasses * (ntasks / 2048 + 1) + 1; }
-
 // Common part of handle creation.  On entry: n, nnz, the segment table (host
 // and device, seg_of for batches) and the id-space CSR (rp_id, col[0],
 // unsorted rows) are in place.  Validates, sizes the workspaces and lays the
@@ -255,18 +240,22 @@ int finish_create(Graph* h) {
     }
     h->maxdeg = static_cast<int64_t>(hm);
   }
-  h->sort_ws_bytes = perm_ws_bytes(std::max<int64_t>(n, 1), h->nbuckets);
+  int64_t slots = 0;
+  for (int i = 0; i < h->nseg; ++i) slots += int64_t(h->hsegs[i].cap) << h->hsegs[i].B;
+  h->sort_ws_bytes = perm_ws_bytes(h->nbuckets, std::max<int64_t>(slots, 1));
   h->scan_ws_bytes = scan_ws_bytes(std::max<int64_t>(n + 1, h->nbuckets + 1));
   if (dalloc(h, &h->order[0], n) || dalloc(h, &h->order[1], n) || dalloc(h, &h->rp[0], n + 1) || dalloc(h, &h->rp[1], n + 1) ||
-      dalloc(h, &h->pos_next, n) || dalloc(h, &h->M, n) || dalloc(h, &h->Minv, n) || dalloc(h, &h->deg_next, n) ||
-      dalloc(h, &h->stash, nnz) ||
+      dalloc(h, &h->chunk_row, nnz / kRowChunk + 2) || dalloc(h, &h->pos[0], n) || dalloc(h, &h->pos[1], n) || dalloc(h, &h->stash, nnz) ||
       dalloc(h, &h->thr_key, h->ntasks) || dalloc(h, &h->thr_tb, h->ntasks) || dalloc(h, &h->done, h->ntasks) ||
       dalloc(h, &h->far_pack, h->ntasks) ||
-      dalloc(h, &h->thr_top, h->ntasks) || dalloc(h, &h->lists, h->ntasks) || dalloc(h, &h->dlist, 2 * h->ntasks) ||
-      dalloc(h, &h->cls_flag, cls_flag_count(h->ntasks, nnz)) || dalloc(h, &h->cls_scan, cls_scan_count(h->ntasks)) ||
+      dalloc(h, &h->lists, kClasses * h->ntasks) || dalloc(h, &h->def_list, 3 * h->ntasks + 2) ||
+      dalloc(h, &h->def_bits, h->ntasks / 32 + 1) || dalloc(h, &h->def_seg, 3 * kDefSegs) ||
       dmalloc(h, &h->sort_ws, h->sort_ws_bytes) || dmalloc(h, &h->scan_ws, h->scan_ws_bytes))
     return fail(h, CB_ENOMEM, "device allocation failed");
   CB_CUDA(h, cudaMemsetAsync(h->done, 0, sizeof(uint32_t) * std::max<int64_t>(h->ntasks, 1), s));
+  CB_CUDA(h, cudaMemsetAsync(h->def_bits, 0, sizeof(uint32_t) * (h->ntasks / 32 + 1), s));
+  CB_CUDA(h, cudaMemsetAsync(h->def_seg, 0, sizeof(int32_t) * 3 * kDefSegs, s));
+  if ((rc = clear_perm_ws(h))) return rc;
   // the rebuild reads 8 placeholders (32 B) and 8 side words (16 B) per vector load
   if ((reinterpret_cast<uintptr_t>(h->col[0]) | reinterpret_cast<uintptr_t>(h->col[1])) % 16 ||
       reinterpret_cast<uintptr_t>(h->stash) % 16)
@@ -289,14 +278,12 @@ int finish_create(Graph* h) {
   // position-space layout of the first super step (rows are sets: no sort);
   // the step's adjacency lives in col[cur = 0]
   h->cur = 0;
-  if ((rc = compute_permutation(h, 0, -1, h->order[0], h->pos_next))) return rc;
-  if (n) k_gather_deg<<<grid1d(n, h->num_sms), 256, 0, s>>>(n, h->order[0], h->deg_id, h->deg_next);
-  CB_CUDA(h, cudaGetLastError());
-  ++h->launches;
-  CB_CUDA(h, exclusive_scan_i32(h->deg_next, h->rp[0], n, h->scan_ws, s, &h->launches));
+  if ((rc = compute_permutation(h, 0, -1, h->order[0], h->pos[0], h->rp[0], nullptr))) return rc;
   int32_t* pcol = idcol == h->col[0] ? h->col[1] : h->col[0];
-  if ((rc = relabel_rows(h, n, h->rp_id, idcol, h->order[0], h->pos_next, h->rp[0], pcol))) return rc;
+  if ((rc = relabel_rows(h, n, h->rp_id, idcol, h->order[0], h->pos[0], h->rp[0], pcol))) return rc;
   if (pcol != h->col[0]) std::swap(h->col[0], h->col[1]);
+  // the super steps' counters start at zero (creation used them as scratch)
+  CB_CUDA(h, cudaMemsetAsync(h->counters, 0, sizeof(int64_t) * (2 * kCounters + 1), s));
   return check_device_error(h);
 }
 
@@ -403,17 +390,12 @@ int set_relaxed(Graph* h, bool on) {
   }
   const int spare = 1 - h->cur;
   // node-id rows of the current graph into col[spare]
-  if ((rc = invert_permutation(h, h->order[h->cur], h->pos_next))) return rc;
-  if ((rc = permute_rows(h, n, h->rp[h->cur], h->col[h->cur], h->pos_next, h->order[h->cur], h->rp_id,
+  if ((rc = permute_rows(h, n, h->rp[h->cur], h->col[h->cur], h->pos[h->cur], h->order[h->cur], h->rp_id,
                          h->col[spare])))
     return rc;
   h->relaxed = on;
-  if ((rc = compute_permutation(h, 0, -1, h->order[h->cur], h->pos_next))) return rc;
-  if (n) k_gather_deg<<<grid1d(n, h->num_sms), 256, 0, s>>>(n, h->order[h->cur], h->deg_id, h->deg_next);
-  CB_CUDA(h, cudaGetLastError());
-  ++h->launches;
-  CB_CUDA(h, exclusive_scan_i32(h->deg_next, h->rp[h->cur], n, h->scan_ws, s, &h->launches));
-  if ((rc = relabel_rows(h, n, h->rp_id, h->col[spare], h->order[h->cur], h->pos_next, h->rp[h->cur],
+  if ((rc = compute_permutation(h, 0, -1, h->order[h->cur], h->pos[h->cur], h->rp[h->cur], nullptr))) return rc;
+  if ((rc = relabel_rows(h, n, h->rp_id, h->col[spare], h->order[h->cur], h->pos[h->cur], h->rp[h->cur],
                          h->col[h->cur])))
     return rc;
   h->pairs_step = ~0ull;
@@ -433,10 +415,10 @@ int64_t estimate_handle_bytes(int64_t n, int64_t nnz, int64_t maxdeg, int num_sm
   const int64_t ntasks = n / 2 + (n & 1);
   const int64_t nb = int64_t(1) << bucket_bits(n);
   int64_t b = 0;
-  b += sizeof(Seg) + 8 * (n + 1) + 4 * n + 2 * 4 * (nnz + kColPad) + 32 + 8 * kCounters;   // cb_create
-  b += 2 * 4 * n + 2 * 8 * (n + 1) + 4 * 4 * n + 2 * nnz;                                 // per node, side words
-  b += ntasks * (8 + 8 + 4 + 16 + 1 + 4 + 8) + 4 * cls_flag_count(ntasks, nnz) + 8 * cls_scan_count(ntasks) + 32;
-  b += static_cast<int64_t>(perm_ws_bytes(std::max<int64_t>(n, 1), nb) + scan_ws_bytes(std::max(n + 1, nb + 1)));
+  b += sizeof(Seg) + 8 * (n + 1) + 4 * n + 2 * 4 * (nnz + kColPad) + 32 + 8 * (2 * kCounters + 1);   // cb_create
+  b += 2 * 4 * n + 2 * 8 * (n + 1) + 2 * 4 * n + 2 * nnz + 4 * (nnz / kRowChunk + 2);                                 // per node, side words
+  b += ntasks * (8 + 8 + 4 + 16 + 4 * kClasses + 4 * 3) + ntasks / 8 + 4 * 3 * kDefSegs + 16;                                  // per trade
+  b += static_cast<int64_t>(perm_ws_bytes(nb, nb * bucket_space(n, bucket_bits(n))) + scan_ws_bytes(n + 1));
   const int64_t max_trade = 2 * maxdeg;
   if (max_trade > kBlockMaxDefault || maxdeg > 16384) {   // default block_max
     const size_t slice = trade_ws_slice_bytes(std::max<int64_t>(max_trade, 1));
@@ -503,11 +485,12 @@ int cb_create(int64_t n, const int64_t* row_ptr, const int32_t* col, uint64_t se
     S.m = nnz / 2;
     S.g = static_cast<uint32_t>(first_step);
     S.B = bucket_bits(n);
+    S.cap = static_cast<int32_t>(bucket_space(n, S.B));
     h->nbuckets = int64_t(1) << S.B;
   }
   cudaStream_t s = h->stream;
   if (dalloc(h, &h->segs, 1) || dalloc(h, &h->rp_id, n + 1) || dalloc(h, &h->deg_id, n) || dalloc(h, &h->col[0], nnz + kColPad) ||
-      dalloc(h, &h->col[1], nnz + kColPad) || dalloc(h, &h->err, 8) || dalloc(h, &h->counters, kCounters) ||
+      dalloc(h, &h->col[1], nnz + kColPad) || dalloc(h, &h->err, 8) || dalloc(h, &h->counters, 2 * kCounters + 1) ||
       !(h->host_counters = new (std::nothrow) int64_t[kCounters]))
     return bail(fail(h, CB_ENOMEM, "device allocation failed"));
   CB_CUDA(h, cudaMemsetAsync(h->err, 0, 8 * sizeof(int32_t), s));
@@ -562,7 +545,7 @@ int cb_create_batch(int32_t count, const int64_t* n, const int64_t* row_ptr, con
     return bail(fail(h, CB_ENOMEM, "host allocation failed"));
   }
   int64_t* eoff = rpo + count;
-  int64_t off = 0, r = 0, e = 0, base = 0, pairs = 0;
+  int64_t off = 0, r = 0, e = 0, base = 0, pairs = 0, slots = 0;
   bool bad = false;
   for (int32_t i = 0; i < count; ++i) {
     Seg& S = h->hsegs[i];
@@ -573,6 +556,9 @@ int cb_create_batch(int32_t count, const int64_t* n, const int64_t* row_ptr, con
     S.span = n[i] + (n[i] & 1);
     S.bucket_base = base;
     S.B = bucket_bits(S.span);
+    S.cap = static_cast<int32_t>(bucket_space(S.span, S.B));
+    S.slot_base = slots;
+    slots += int64_t(S.cap) << S.B;
     S.g = static_cast<uint32_t>(first_step);
     const int64_t z = rph[r + n[i]];
     bad |= rph[r] != 0 || z < 0 || (z & 1);
@@ -603,7 +589,7 @@ int cb_create_batch(int32_t count, const int64_t* n, const int64_t* row_ptr, con
   int64_t* d_rp_in = nullptr;
   int64_t* d_rpo = nullptr;
   if (dalloc(h, &h->segs, count) || dalloc(h, &h->seg_of, N) || dalloc(h, &h->rp_id, N + 1) || dalloc(h, &h->deg_id, N) ||
-      dalloc(h, &h->col[0], e + kColPad) || dalloc(h, &h->col[1], e + kColPad) || dalloc(h, &h->err, 8) || dalloc(h, &h->counters, kCounters) ||
+      dalloc(h, &h->col[0], e + kColPad) || dalloc(h, &h->col[1], e + kColPad) || dalloc(h, &h->err, 8) || dalloc(h, &h->counters, 2 * kCounters + 1) ||
       !(h->host_counters = new (std::nothrow) int64_t[kCounters]) || dalloc(h, &d_rp_in, nrp) ||
       dalloc(h, &d_rpo, 2 * static_cast<int64_t>(count))) {
     delete[] rpo;
@@ -777,31 +763,32 @@ int cb_permutation(cb_handle h, uint64_t g, int32_t* order_out, int mem_kind) {
   if (!h || !order_out || (mem_kind != CB_HOST && mem_kind != CB_DEVICE)) return fail(h, CB_EINVAL, "bad argument");
   if (g >= 0xfffffffeull) return fail(h, CB_ERANGE, "step too large");
   int rc;
-  // M is free between super steps
-  if ((rc = compute_permutation(h, 0, static_cast<int64_t>(g), h->M, nullptr))) return rc;
-  CB_CUDA(h, cudaMemcpyAsync(order_out, h->M, sizeof(int32_t) * h->n,
+  int32_t* const order = h->pos[1 - h->cur];   // free between super steps
+  if ((rc = compute_permutation(h, 0, static_cast<int64_t>(g), order, nullptr, nullptr, nullptr))) return rc;
+  CB_CUDA(h, cudaMemcpyAsync(order_out, order, sizeof(int32_t) * h->n,
                              mem_kind == CB_HOST ? cudaMemcpyDeviceToHost : cudaMemcpyDeviceToDevice, h->stream));
   return cb_sync(h);
 }
 
 int cb_stats(cb_handle h, int64_t* out, int count) {
   if (!h || !out || count < 0) return fail(h, CB_EINVAL, "bad argument");
-  // counters of the last super step (reset at the start of each one)
-  CB_CUDA(h, cudaMemcpyAsync(h->host_counters, h->counters, kCounters * sizeof(int64_t), cudaMemcpyDeviceToHost,
-                             h->stream));
+  // counters of the last super step: the set the next one does not use
+  CB_CUDA(h, cudaMemcpyAsync(h->host_counters, h->counters + (1 - h->cur) * kCounters, kCounters * sizeof(int64_t),
+                             cudaMemcpyDeviceToHost, h->stream));
   CB_CUDA(h, cudaStreamSynchronize(h->stream));
   const int64_t* hc = h->host_counters;
-  // pass r + 1 runs what pass r left deferred (the last: the in-order pass)
-  int64_t passes = 1;
-  for (int r = 0; r <= h->retry_passes; ++r) passes += hc[kCtrPassLeft + r] > 0;
+  const int retries = retry_passes_of(h);
+  auto left = [&](int r) { return hc[kCtrDef + 3 * r] + hc[kCtrDef + 3 * r + 1] + hc[kCtrDef + 3 * r + 2]; };
+  int64_t passes = 1;   // pass r + 1 runs what pass r left deferred (the last: the in-order pass)
+  for (int r = 0; r <= retries; ++r) passes += left(r) > 0;
   h->stats[0] = passes;
-  h->stats[1] = hc[kCtrPassLeft];
+  h->stats[1] = left(0);
   h->stats[2] = h->stats[3] = 0;
-  for (int k = 0; k < kClasses; ++k) h->stats[k < kWarpClasses ? 2 : 3] += hc[kCtrFirstLen + k];
+  for (int k = 0; k < kClasses; ++k) h->stats[k < kWarpClasses ? 2 : 3] += hc[kCtrClsLen + k];
   h->stats[4] = hc[kCtrGws];
-  h->stats[6] = hc[kCtrPassLeft + h->retry_passes];
+  h->stats[6] = left(retries);
   for (int k = 0; k < kClasses; ++k) {
-    h->stats[7 + k] = hc[kCtrFirstLen + k];
+    h->stats[7 + k] = hc[kCtrClsLen + k];
     h->stats[7 + kClasses + k] = hc[kCtrFirstEnt + k];
   }
   const int k = std::min(count, kStats);

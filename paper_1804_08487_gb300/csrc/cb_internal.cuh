@@ -33,24 +33,21 @@ constexpr int kBlockMaxCap = 2048;  // largest trade on the 256-thread path
 constexpr int kBlockMaxDefault = 1024;   // default of the "block_max" option
 constexpr int kSmemMaxCap = 8192;   // largest trade kept in shared memory on the 1024-thread path
 constexpr int kBlockThreads = 256;  // CTA size of the block path
-constexpr int kCounters = 96;       // device counters per handle
+constexpr int kCounters = 64;       // device counters of one super step (two sets per handle, used in turn)
 // Trade size classes of the threshold phase (one team size each) and the
 // device counters of a super step.
 constexpr int kClasses = 9;
 constexpr int kWarpClasses = 3;     // classes 0..2 run on warps or parts of a warp
 constexpr int kCtrClsLen = 0;       // [0, kClasses): trades per class
-constexpr int kCtrClsStart = 10;    // [10, 10 + kClasses): first entry of each class in the class lists
-constexpr int kCtrClaims = 19;      // chunks claimed by the in-order pass
-constexpr int kCtrFirstLen = 20;    // [20, 20 + kClasses): trades per class in the first pass
-constexpr int kCtrFirstEnt = 29;    // [29, 29 + kClasses): directed entries per class in the first pass
-constexpr int kCtrPassLeft = 40;    // [40, 40 + kRetryPassesMax + 2): trades left deferred after pass r
+constexpr int kCtrFirstEnt = 10;    // [10, 10 + kClasses): their directed entries
 constexpr int kRetryPassesMax = 4;
-constexpr int kCtrPassSmall = 48;   // [48, 54): of those, the small ones (listed from the front of the list)
-constexpr int kCtrPassBig = 56;     // [56, 62): the others (listed from the back)
-constexpr int kCtrListClaim = 64;   // [64, 64 + 3 kRetryPassesMax]: list positions claimed by the passes' kernels
-constexpr int kCtrListOk = 80;      // 1: the in-order pass runs on the sorted list of the last pass
-constexpr int kCtrListN = 81;       // the sorted list's length
-static_assert(40 + kRetryPassesMax + 2 <= 48 && 64 + 3 * kRetryPassesMax < 80, "counter layout");
+constexpr int kCtrDef = 24;         // [24 + 3 r, 27 + 3 r): trades that pass r deferred, by kind (r <= kRetryPassesMax)
+constexpr int kCtrFinished = 40;    // chunks of the in-order pass claimed
+constexpr int kCtrChunks = 41;      // its chunks
+constexpr int kCtrClaim = 42;       // [42 + 3 r, 45 + 3 r): trades of each list that retry pass r claimed
+static_assert(24 + 3 * (kRetryPassesMax + 1) <= 40 && 42 + 3 * kRetryPassesMax <= kCounters - 1, "counter layout");
+constexpr int kRowChunk = 2048;      // entries per sample of the entry -> row index
+constexpr int kDefSegs = 1024;      // most segments of the trades that deferred ones are counted in
 constexpr int kStats = 7 + 2 * kClasses;   // counters cb_stats reports
 constexpr int kTimings = 6 + kClasses;     // values cb_timings reports
 constexpr int kCtrGws = kCounters - 1;   // trades whose workspace is in global memory
@@ -71,8 +68,10 @@ struct Seg {
   int64_t bucket_base;   // first permutation bucket
   int64_t m;             // undirected edges
   int64_t pair_off;      // first exported pair
+  int64_t slot_base;     // first id of its permutation bucket space
   uint32_t g;            // super step (advanced on the device at the end of each step)
   int32_t B;             // permutation bucket bits
+  int32_t cap;           // ids one bucket holds
 };
 
 struct Graph {
@@ -102,22 +101,19 @@ struct Graph {
   int cur = 0;
   int32_t* order[2] = {nullptr, nullptr};  // node at each position
   int64_t* rp[2] = {nullptr, nullptr};     // position-space row offsets (n+1)
+  int32_t* chunk_row = nullptr;            // row of every kRowChunk-th entry of the offsets last computed
   int32_t* col[2] = {nullptr, nullptr};    // position-space rows, ascending
-  int32_t* pos_next = nullptr;             // position of each node id in step g+1
-  int32_t* M = nullptr;                    // step-g position -> step-(g+1) position
-  int32_t* Minv = nullptr;                 // step-(g+1) position -> step-g position
-  int32_t* deg_next = nullptr;             // degree by step-(g+1) position
+  int32_t* pos[2] = {nullptr, nullptr};    // position of each node (pos[1 - cur] is scratch between steps)
   uint16_t* stash = nullptr;               // per placed entry (step g+1 layout): bit0 own flip, bits 1.. far key prefix
   uint64_t* thr_key = nullptr;             // per trade: threshold key
-  uint8_t* thr_top = nullptr;              // per trade: top 6 bits of the threshold key
   uint64_t* thr_tb = nullptr;              // per trade: threshold tie-break (lo<<32|hi)
-  uint32_t* done = nullptr;                // per trade: 1 once the threshold is published (cleared per step)
+  uint32_t* done = nullptr;                // per trade: the step + 1 once its threshold is published
   int4* far_pack = nullptr;                // per trade: new positions of its nodes, threshold prefix (rebuild)
-  int32_t* lists = nullptr;                // trades of every size class, class after class, index order within
-  int32_t* dlist = nullptr;                // 2 ntasks: the trades each pass deferred, for the next one
-  int32_t* cls_flag = nullptr;             // scratch: per-chunk class counts, then the rebuild's chunk rows
-  int64_t* cls_scan = nullptr;             // scratch: their exclusive scan
-  int64_t* counters = nullptr;             // list lengths, deferred count, claims (kCounters)
+  int32_t* lists = nullptr;                // kClasses x ntasks: the trades of each size class
+  uint32_t* def_bits = nullptr;            // deferred trades, one bit each (zero between steps)
+  int32_t* def_seg = nullptr;              // their counts per kind and segment (zero between steps)
+  int32_t* def_list = nullptr;             // by kind for a retry pass; in index order with the chunks' first ones for the in-order pass
+  int64_t* counters = nullptr;             // two sets of kCounters, then the CTAs that ended the step
   int32_t* err = nullptr;                  // latched device error
   // workspaces
   void* ws_global = nullptr;               // global workspace for trades too big for smem
@@ -205,14 +201,17 @@ cudaError_t exclusive_scan_i32(const int32_t* in, int64_t* out, int64_t n, void*
                                int64_t* launches = nullptr);
 
 // permute.cu
-size_t perm_ws_bytes(int64_t n, int64_t nbuckets);
+struct ClassArgs;
+size_t perm_ws_bytes(int64_t nbuckets, int64_t slots);
 int bucket_bits(int64_t n);
-// order_out[p] = node at position p; pos_out[x] = position of x (may be null).
-// Each segment uses its device step counter + dg, or the step g_abs for all
-// when g_abs >= 0.
-int compute_permutation(Graph* h, uint32_t dg, int64_t g_abs, int32_t* order_out, int32_t* pos_out);
-// M, deg_next and rp[1-cur] for the step after the current one
-int prepare_next(Graph* h);
+int64_t bucket_space(int64_t span, int B);
+// order_out[p] = node at position p; pos_out[x] = position of x, rp_out[p] =
+// row offsets of that order (n + 1; either may be null).  Each segment uses
+// its device step counter + dg, or the step g_abs for all when g_abs >= 0.
+// classes (may be null): build the size-class lists of the current step too.
+int compute_permutation(Graph* h, uint32_t dg, int64_t g_abs, int32_t* order_out, int32_t* pos_out, int64_t* rp_out,
+                        const ClassArgs* classes);
+int clear_perm_ws(Graph* h);
 
 // rows.cu
 // dst row q <- src row rowmap[q] with values mapped through valmap (identity if null), ascending
@@ -227,7 +226,6 @@ int rows_sorted(Graph* h, const int64_t* rp, const int32_t* col, int64_t n, bool
 int relabel_rows(Graph* h, int64_t nrows, const int64_t* src_rp, const int32_t* src_col, const int32_t* rowmap,
                  const int32_t* valmap, const int64_t* dst_rp, int32_t* dst_col);
 int check_row_offsets(Graph* h, const int64_t* rp, int64_t n);
-int invert_permutation(Graph* h, const int32_t* order, int32_t* pos);
 // canonical pairs (x < y, sorted, local ids) of the current step into `pairs`
 // (2m int32, device); uses the spare adjacency buffer
 int export_sorted_pairs(Graph* h, int32_t* pairs);
@@ -238,6 +236,7 @@ int flush_timing(Graph* h, int set, bool add);   // wait for a recorded event se
 int init_trade_kernels(Graph* h);   // one-time kernel attributes (outside stream capture)
 int init_perm_kernels(Graph* h);
 size_t trade_ws_slice_bytes(int64_t max_trade);
+int retry_passes_of(const Graph* h);   // retry passes a super step launches
 
 // api.cu
 // stream-ordered device allocation counted in the handle's device bytes

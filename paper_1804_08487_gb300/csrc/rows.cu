@@ -272,11 +272,6 @@ __global__ void k_relabel(RowArgs a) {
   }
 }
 
-__global__ void k_invert(int64_t n, const int32_t* __restrict__ order, int32_t* __restrict__ pos) {
-  for (int64_t p = blockIdx.x * int64_t(blockDim.x) + threadIdx.x; p < n; p += int64_t(gridDim.x) * blockDim.x)
-    pos[order[p]] = static_cast<int32_t>(p);
-}
-
 // ---- canonical export: only the entries above the diagonal are sorted
 
 // cnt[x] = entries of (unsorted) row x greater than x
@@ -400,7 +395,7 @@ int validate_sorted_graph(Graph* h, const int64_t* rp, const int32_t* col, int64
   cudaStream_t s = h->stream;
   // scratch: low in a step buffer of n int32, its scan in rp[1] (n+1 int64),
   // none in use before the first super step; the partition in `grouped`
-  int32_t* low = h->M;
+  int32_t* low = h->pos[1];
   int64_t* grp = h->rp[1];
   int sh = 0;
   while (((n - 1) >> sh) >= kVBuckets) ++sh;
@@ -475,14 +470,6 @@ int check_row_offsets(Graph* h, const int64_t* rp, int64_t n) {
   return CB_OK;
 }
 
-int invert_permutation(Graph* h, const int32_t* order, int32_t* pos) {
-  if (h->n == 0) return CB_OK;
-  k_invert<<<grid_of(h->n, 256, h->num_sms), 256, 0, h->stream>>>(h->n, order, pos);
-  CB_CUDA(h, cudaGetLastError());
-  ++h->launches;
-  return CB_OK;
-}
-
 // Canonical pairs of the current step: id-space rows (unsorted), the count
 // above the diagonal per row, and each row's upper part sorted into place.
 int export_sorted_pairs(Graph* h, int32_t* pairs) {
@@ -490,11 +477,10 @@ int export_sorted_pairs(Graph* h, int32_t* pairs) {
   if (n == 0) return CB_OK;
   int rc;
   const int spare = 1 - h->cur;
-  if ((rc = invert_permutation(h, h->order[h->cur], h->pos_next))) return rc;
-  if ((rc = relabel_rows(h, n, h->rp[h->cur], h->col[h->cur], h->pos_next, h->order[h->cur], h->rp_id,
+  if ((rc = relabel_rows(h, n, h->rp[h->cur], h->col[h->cur], h->pos[h->cur], h->order[h->cur], h->rp_id,
                          h->col[spare])))
     return rc;
-  int32_t* cnt = h->deg_next;      // free between super steps
+  int32_t* cnt = h->pos[spare];    // free between super steps
   int64_t* off = h->rp[spare];
   cudaStream_t s = h->stream;
   const unsigned wgrid = grid_of(n * 32, 256, h->num_sms);

@@ -756,7 +756,6 @@ int uniform_trades(Graph* h, uint64_t count) {
     b->ctas = ctas;
   }
   // node id -> position of the current step
-  if ((rc = invert_permutation(h, h->order[h->cur], h->pos_next))) return rc;
   const unsigned g1 = grid_for_work(n, h->num_sms);
   uint64_t done = 0;
   while (done < count) {
@@ -764,7 +763,7 @@ int uniform_trades(Graph* h, uint64_t count) {
     const uint64_t first = h->uni_next + done;
     const unsigned gL = grid_for_work(L, h->num_sms);
     // the sequence in positions, its Suc lists and every slot's next trade
-    k_uni_draw<<<gL, 256, 0, s>>>(L, first, h->seed, n, h->pos_next, h->rp[h->cur], b->tp, b->dslot);
+    k_uni_draw<<<gL, 256, 0, s>>>(L, first, h->seed, n, h->pos[h->cur], h->rp[h->cur], b->tp, b->dslot);
     CB_CUDA(h, cudaGetLastError());
     CB_CUDA(h, cudaMemsetAsync(b->occ, 0, sizeof(int32_t) * n, s));
     k_uni_count<<<gL, 256, 0, s>>>(L, n, b->tp, b->occ, h->err);
