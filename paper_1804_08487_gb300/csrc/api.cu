@@ -21,7 +21,12 @@ __global__ void k_degrees(int64_t n, const int64_t* __restrict__ rp, int32_t* __
     deg[x] = static_cast<int32_t>(d);
     if (d > 0 && static_cast<unsigned long long>(d) > local) local = static_cast<unsigned long long>(d);
   }
-  atomicMax(maxdeg, local);
+#pragma unroll
+  for (int o = 16; o; o >>= 1) {
+    const unsigned long long v = __shfl_xor_sync(0xffffffffu, local, o);
+    local = v > local ? v : local;
+  }
+  if ((threadIdx.x & 31) == 0 && local) atomicMax(maxdeg, local);
 }
 
 unsigned grid1d(int64_t work, int num_sms) {
@@ -263,17 +268,25 @@ int finish_create(Graph* h) {
   if ((rc = size_trade_workspace(h))) return rc;
   // rows in id space, sorted (sorted input is used as it is), then validated:
   // simple and symmetric
-  bool sorted = false;
-  if ((rc = rows_sorted(h, h->rp_id, h->col[0], n, &sorted))) return rc;
   int32_t* idcol = h->col[0];
-  if (!sorted) {
-    if ((rc = permute_rows(h, n, h->rp_id, h->col[0], nullptr, nullptr, h->rp_id, h->col[1]))) return rc;
-    idcol = h->col[1];
-  }
-  if ((rc = validate_sorted_graph(h, h->rp_id, idcol, n, idcol == h->col[0] ? h->col[1] : h->col[0]))) return rc;
-  if ((rc = check_device_error(h))) {
-    h->last_error = "graph is not simple and symmetric";
-    return CB_EINVAL;
+  {
+    Validation v;
+    bool sorted = false;
+    rc = scan_rows(h, h->rp_id, idcol, n, &v, &sorted);
+    if (!rc && !sorted && !v.bad) {
+      rc = permute_rows(h, n, h->rp_id, h->col[0], nullptr, nullptr, h->rp_id, h->col[1]);
+      idcol = h->col[1];
+      if (!rc) rc = scan_rows(h, h->rp_id, idcol, n, &v, &sorted);
+    }
+    if (!rc && sorted && !v.bad)
+      rc = validate_sorted_graph(h, h->rp_id, idcol, n, &v, idcol == h->col[0] ? h->col[1] : h->col[0]);
+    free_validation(h, &v);
+    if (rc) return rc;
+    rc = check_device_error(h);
+    if (rc || !sorted || v.bad) {
+      h->last_error = "graph is not simple and symmetric";
+      return CB_EINVAL;
+    }
   }
   // position-space layout of the first super step (rows are sets: no sort);
   // the step's adjacency lives in col[cur = 0]
@@ -283,7 +296,7 @@ int finish_create(Graph* h) {
   if ((rc = relabel_rows(h, n, h->rp_id, idcol, h->order[0], h->pos[0], h->rp[0], pcol))) return rc;
   if (pcol != h->col[0]) std::swap(h->col[0], h->col[1]);
   // the super steps' counters start at zero (creation used them as scratch)
-  CB_CUDA(h, cudaMemsetAsync(h->counters, 0, sizeof(int64_t) * (2 * kCounters + 1), s));
+  CB_CUDA(h, cudaMemsetAsync(h->counters, 0, sizeof(int64_t) * (2 * kCounters + 4), s));
   return check_device_error(h);
 }
 
@@ -415,7 +428,7 @@ int64_t estimate_handle_bytes(int64_t n, int64_t nnz, int64_t maxdeg, int num_sm
   const int64_t ntasks = n / 2 + (n & 1);
   const int64_t nb = int64_t(1) << bucket_bits(n);
   int64_t b = 0;
-  b += sizeof(Seg) + 8 * (n + 1) + 4 * n + 2 * 4 * (nnz + kColPad) + 32 + 8 * (2 * kCounters + 1);   // cb_create
+  b += sizeof(Seg) + 8 * (n + 1) + 4 * n + 2 * 4 * (nnz + kColPad) + 32 + 8 * (2 * kCounters + 4);   // cb_create
   b += 2 * 4 * n + 2 * 8 * (n + 1) + 2 * 4 * n + 2 * nnz + 4 * (nnz / kRowChunk + 2);                                 // per node, side words
   b += ntasks * (8 + 8 + 4 + 16 + 4 * kClasses + 4 * 3) + ntasks / 8 + 4 * 3 * kDefSegs + 16;                                  // per trade
   b += static_cast<int64_t>(perm_ws_bytes(nb, nb * bucket_space(n, bucket_bits(n))) + scan_ws_bytes(n + 1));
@@ -490,7 +503,7 @@ int cb_create(int64_t n, const int64_t* row_ptr, const int32_t* col, uint64_t se
   }
   cudaStream_t s = h->stream;
   if (dalloc(h, &h->segs, 1) || dalloc(h, &h->rp_id, n + 1) || dalloc(h, &h->deg_id, n) || dalloc(h, &h->col[0], nnz + kColPad) ||
-      dalloc(h, &h->col[1], nnz + kColPad) || dalloc(h, &h->err, 8) || dalloc(h, &h->counters, 2 * kCounters + 1) ||
+      dalloc(h, &h->col[1], nnz + kColPad) || dalloc(h, &h->err, 8) || dalloc(h, &h->counters, 2 * kCounters + 4) ||
       !(h->host_counters = new (std::nothrow) int64_t[kCounters]))
     return bail(fail(h, CB_ENOMEM, "device allocation failed"));
   CB_CUDA(h, cudaMemsetAsync(h->err, 0, 8 * sizeof(int32_t), s));
@@ -589,7 +602,7 @@ int cb_create_batch(int32_t count, const int64_t* n, const int64_t* row_ptr, con
   int64_t* d_rp_in = nullptr;
   int64_t* d_rpo = nullptr;
   if (dalloc(h, &h->segs, count) || dalloc(h, &h->seg_of, N) || dalloc(h, &h->rp_id, N + 1) || dalloc(h, &h->deg_id, N) ||
-      dalloc(h, &h->col[0], e + kColPad) || dalloc(h, &h->col[1], e + kColPad) || dalloc(h, &h->err, 8) || dalloc(h, &h->counters, 2 * kCounters + 1) ||
+      dalloc(h, &h->col[0], e + kColPad) || dalloc(h, &h->col[1], e + kColPad) || dalloc(h, &h->err, 8) || dalloc(h, &h->counters, 2 * kCounters + 4) ||
       !(h->host_counters = new (std::nothrow) int64_t[kCounters]) || dalloc(h, &d_rp_in, nrp) ||
       dalloc(h, &d_rpo, 2 * static_cast<int64_t>(count))) {
     delete[] rpo;

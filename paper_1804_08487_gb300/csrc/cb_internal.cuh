@@ -217,11 +217,23 @@ int clear_perm_ws(Graph* h);
 // dst row q <- src row rowmap[q] with values mapped through valmap (identity if null), ascending
 int permute_rows(Graph* h, int64_t nrows, const int64_t* src_rp, const int32_t* src_col,
                  const int32_t* rowmap, const int32_t* valmap, const int64_t* dst_rp, int32_t* dst_col);
-// simple and symmetric, or kErrValidate latched; `grouped` is scratch of
-// row_ptr[n] int32 (not synchronising)
-int validate_sorted_graph(Graph* h, const int64_t* rp, const int32_t* col, int64_t n, int32_t* grouped);
-// *sorted = every row strictly increasing (synchronises)
-int rows_sorted(Graph* h, const int64_t* rp, const int32_t* col, int64_t n, bool* sorted);
+// Validation of the input: scan_rows checks ids and says whether every row is
+// strictly increasing (synchronises); validate_sorted_graph then checks the
+// symmetry of such rows and latches kErrValidate (not synchronising; `grouped`
+// is scratch of row_ptr[n] int32).
+struct Validation {
+  char* ws = nullptr;
+  size_t bytes = 0;
+  int sh = 0, nb = 0, ctas = 0;
+  int32_t* flags = nullptr;
+  int32_t* counts = nullptr;   // upper entries per (bucket, CTA)
+  int64_t* place = nullptr;    // their exclusive scan
+  void* scan = nullptr;
+  bool bad = false;            // an id out of range or a self loop
+};
+int scan_rows(Graph* h, const int64_t* rp, const int32_t* col, int64_t n, Validation* v, bool* sorted);
+int validate_sorted_graph(Graph* h, const int64_t* rp, const int32_t* col, int64_t n, Validation* v, int32_t* grouped);
+void free_validation(Graph* h, Validation* v);
 // like permute_rows without sorting (rows keep their order)
 int relabel_rows(Graph* h, int64_t nrows, const int64_t* src_rp, const int32_t* src_col, const int32_t* rowmap,
                  const int32_t* valmap, const int64_t* dst_rp, int32_t* dst_col);

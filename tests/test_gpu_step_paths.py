@@ -7,7 +7,7 @@ import pytest
 
 from oracle import Oracle
 from paper_1804_08487_gb300 import synth
-from paper_1804_08487_gb300.cb import Curveball, Ensemble
+from paper_1804_08487_gb300.cb import CB_EINVAL, CbError, Curveball, Ensemble
 
 pytestmark = pytest.mark.gpu
 
@@ -88,3 +88,64 @@ def test_dense_cores_through_the_in_order_pass(n, b, options):
         assert np.array_equal(c.edges(), o.edges())
     assert c.stats()["deferred"] > 0
     c.close()
+
+
+# rows of 32, 33, 256, 257, 1024, 1025 and more entries above the diagonal
+# (a warp on its tile, a warp on a listed row, 1024 threads, a global slice), a star
+# whose hub is the first or the last node, and an output buffer that is only
+# 4-byte aligned.
+@pytest.mark.parametrize("d", [1, 2, 31, 32, 33, 64, 65, 128, 129, 255, 256, 257, 511, 512, 513, 1023, 1024, 1025, 2049, 5000, 20000])
+@pytest.mark.parametrize("hub_last", [False, True])
+def test_export_of_long_rows(d, hub_last):
+    import torch
+    n = d + 40
+    rng = np.random.default_rng(d)
+    hub = n - 1 if hub_last else 0
+    leaves = np.setdiff1d(rng.permutation(n)[:d + 1], [hub])[:d]
+    extra = rng.integers(0, n, (30, 2))
+    e = {(min(hub, x), max(hub, x)) for x in leaves.tolist()} | {(min(a, b), max(a, b)) for a, b in extra.tolist() if a != b}
+    e = np.array(sorted(e), dtype=np.int64)
+    both = np.concatenate([e, e[:, ::-1]])
+    both = both[np.lexsort((both[:, 1], both[:, 0]))]
+    rp = np.concatenate([[0], np.cumsum(np.bincount(both[:, 0], minlength=n))]).astype(np.int64)
+    c = Curveball(rp, both[:, 1].astype(np.int32), 3)
+    assert np.array_equal(c.edges(), e)
+    c.global_trades(1)
+    o = Oracle(rp, both[:, 1].astype(np.int32), 3)
+    o.superstep(1)
+    buf = torch.zeros(2 * len(e) + 1, dtype=torch.int32, device="cuda")
+    c.edges(buf[1:])
+    assert np.array_equal(buf[1:].cpu().numpy().reshape(-1, 2), o.edges())
+    assert np.array_equal(c.edges(), o.edges())
+    c.close()
+
+
+# one wrong entry in an otherwise symmetric graph of many tiles and buckets:
+# an entry moved, repeated, out of range, a self loop, a missing mirror
+@pytest.mark.parametrize("n", [40, 5000, 70000])
+@pytest.mark.parametrize("what", ["moved", "repeated", "range", "negative", "loop", "mirror"])
+@pytest.mark.parametrize("shuffled", [False, True])
+def test_malformed_graphs_are_refused(n, what, shuffled):
+    g = synth.powerlaw_graph(n, 3, min(n // 3, 200), 2.0, 5)
+    rp, col = g.row_ptr, g.col.copy()
+    rng = np.random.default_rng(n)
+    if shuffled:
+        for x in range(0, n, 7):
+            rng.shuffle(col[rp[x]:rp[x + 1]])
+    x = int(rng.integers(n // 2, n))
+    i = int(rp[x]) + 1
+    row = set(col[rp[x]:rp[x + 1]].tolist())
+    if what == "moved" or what == "mirror":
+        y = next(v for v in range(n) if v not in row and v != x)
+        col[i] = y
+    elif what == "repeated":
+        col[i] = col[i - 1]
+    elif what == "range":
+        col[int(rp[x + 1]) - 1] = n
+    elif what == "negative":
+        col[int(rp[x])] = -1
+    else:
+        col[i] = x
+    with pytest.raises(CbError) as err:
+        Curveball(rp, col, 1)
+    assert err.value.code == CB_EINVAL
