@@ -3,6 +3,7 @@
 #include <algorithm>
 #include <cstring>
 #include <string>
+#include <type_traits>
 
 #include "cb_internal.cuh"
 
@@ -13,11 +14,13 @@ size_t trade_ws_slice_bytes(int64_t max_trade);
 namespace {
 thread_local std::string g_error;
 
+// Degrees, their maximum, and the offsets' checks.
 __global__ void k_degrees(int64_t n, const int64_t* __restrict__ rp, int32_t* __restrict__ deg,
-                          unsigned long long* __restrict__ maxdeg) {
+                          unsigned long long* __restrict__ maxdeg, int32_t* err) {
   unsigned long long local = 0;
   for (int64_t x = blockIdx.x * int64_t(blockDim.x) + threadIdx.x; x < n; x += int64_t(gridDim.x) * blockDim.x) {
     const int64_t d = rp[x + 1] - rp[x];
+    if (d < 0 || d >= n || (x == 0 && rp[0] != 0)) atomicCAS(err, 0, static_cast<int32_t>(kErrValidate));
     deg[x] = static_cast<int32_t>(d);
     if (d > 0 && static_cast<unsigned long long>(d) > local) local = static_cast<unsigned long long>(d);
   }
@@ -64,11 +67,7 @@ void release(Graph* h) {
   if (h->stream) cudaStreamSynchronize(h->stream);
   free_uniform(h);
   free_presence(h);
-  void* bufs[] = {h->deg_id, h->rp_id, h->order[0], h->order[1], h->rp[0], h->rp[1], h->col[0], h->col[1],
-                  h->pos[0], h->pos[1], h->stash, h->thr_key, h->thr_tb, h->done,
-                  h->chunk_row, h->lists, h->def_list, h->def_bits, h->def_seg, h->counters, h->err,
-                  h->ws_global, h->sort_ws, h->scan_ws, h->segs, h->seg_of, h->pairs, h->far_pack,
-                  h->lcg_ab, h->lcg_gaps, h->swaps};
+  void* bufs[] = {h->arena, h->ws_global, h->pairs, h->lcg_ab, h->lcg_gaps, h->swaps};
   if (h->stream)
     for (void* b : bufs) dfree(h, b);
   for (auto& x : h->step_exec)
@@ -218,75 +217,101 @@ void destroy_graph(Graph* h) {
   delete static_cast<cb_graph*>(h);
 }
 
-// Common part of handle creation.  On entry: n, nnz, the segment table (host
-// and device, seg_of for batches) and the id-space CSR (rp_id, col[0],
-// unsorted rows) are in place.  Validates, sizes the workspaces and lays the
-// graph out for its first super step.
-int finish_create(Graph* h) {
+// The arrays every handle has, in one allocation (n, nnz and the segments
+// are known): creating and releasing 25 arrays one by one cost more than the
+// kernels of a small graph's creation.  What has to start at zero comes first.
+int alloc_arrays(Graph* h) {
   const int64_t n = h->n, nnz = h->nnz;
-  cudaStream_t s = h->stream;
-  int rc;
   h->m = nnz / 2;
   h->T = n / 2;
   h->ntasks = h->T + (n & 1);
-  if ((rc = init_trade_kernels(h)) || (rc = init_perm_kernels(h))) return rc;
-  if ((rc = check_row_offsets(h, h->rp_id, n))) return rc;
-  {
-    unsigned long long* dmax = reinterpret_cast<unsigned long long*>(h->counters);
-    CB_CUDA(h, cudaMemsetAsync(dmax, 0, sizeof(unsigned long long), s));
-    if (n) k_degrees<<<grid1d(n, h->num_sms), 256, 0, s>>>(n, h->rp_id, h->deg_id, dmax);
-    CB_CUDA(h, cudaGetLastError());
-    ++h->launches;
-    unsigned long long hm = 0;
-    CB_CUDA(h, cudaMemcpyAsync(&hm, dmax, sizeof(hm), cudaMemcpyDeviceToHost, s));
-    if ((rc = check_device_error(h))) {
-      h->last_error = "row_ptr is not a valid CSR offset array (degrees in [0, n), ids in range)";
-      return CB_EINVAL;
-    }
-    h->maxdeg = static_cast<int64_t>(hm);
-  }
   int64_t slots = 0;
   for (int i = 0; i < h->nseg; ++i) slots += int64_t(h->hsegs[i].cap) << h->hsegs[i].B;
-  h->sort_ws_bytes = perm_ws_bytes(h->nbuckets, std::max<int64_t>(slots, 1));
-  h->scan_ws_bytes = scan_ws_bytes(std::max<int64_t>(n + 1, h->nbuckets + 1));
-  if (dalloc(h, &h->order[0], n) || dalloc(h, &h->order[1], n) || dalloc(h, &h->rp[0], n + 1) || dalloc(h, &h->rp[1], n + 1) ||
-      dalloc(h, &h->chunk_row, nnz / kRowChunk + 2) || dalloc(h, &h->pos[0], n) || dalloc(h, &h->pos[1], n) || dalloc(h, &h->stash, nnz) ||
-      dalloc(h, &h->thr_key, h->ntasks) || dalloc(h, &h->thr_tb, h->ntasks) || dalloc(h, &h->done, h->ntasks) ||
-      dalloc(h, &h->far_pack, h->ntasks) ||
-      dalloc(h, &h->lists, kClasses * h->ntasks) || dalloc(h, &h->def_list, 3 * h->ntasks + 2) ||
-      dalloc(h, &h->def_bits, h->ntasks / 32 + 1) || dalloc(h, &h->def_seg, 3 * kDefSegs) ||
-      dmalloc(h, &h->sort_ws, h->sort_ws_bytes) || dmalloc(h, &h->scan_ws, h->scan_ws_bytes))
-    return fail(h, CB_ENOMEM, "device allocation failed");
-  CB_CUDA(h, cudaMemsetAsync(h->done, 0, sizeof(uint32_t) * std::max<int64_t>(h->ntasks, 1), s));
-  CB_CUDA(h, cudaMemsetAsync(h->def_bits, 0, sizeof(uint32_t) * (h->ntasks / 32 + 1), s));
-  CB_CUDA(h, cudaMemsetAsync(h->def_seg, 0, sizeof(int32_t) * 3 * kDefSegs, s));
-  if ((rc = clear_perm_ws(h))) return rc;
-  // the rebuild reads 8 placeholders (32 B) and 8 side words (16 B) per vector load
-  if ((reinterpret_cast<uintptr_t>(h->col[0]) | reinterpret_cast<uintptr_t>(h->col[1])) % 16 ||
-      reinterpret_cast<uintptr_t>(h->stash) % 16)
-    return fail(h, CB_ECUDA, "device allocation not aligned for vector loads");
-  if ((rc = size_trade_workspace(h))) return rc;
+  const size_t sort_bytes = perm_ws_bytes(h->nbuckets, std::max<int64_t>(slots, 1));
+  const size_t scan_bytes = scan_ws_bytes(std::max<int64_t>(n + 1, h->nbuckets + 1));
+  size_t used = 0, zeroed = 0;
+  char* base = nullptr;
+  auto take = [&](auto** p, int64_t count) {
+    using T = std::remove_reference_t<decltype(**p)>;
+    *p = reinterpret_cast<T*>(base + used);
+    used += (sizeof(T) * static_cast<size_t>(std::max<int64_t>(count, 1)) + 255) & ~size_t(255);
+  };
+  auto layout = [&]() {
+    used = 0;
+    take(&h->err, 64);   // then the scratch, so that one copy reads both
+    take(&h->scratch, kScratch);
+    take(&h->counters, 2 * kCounters + 1);
+    take(&h->def_seg, 3 * kDefSegs);
+    take(&h->def_bits, h->ntasks / 32 + 1);
+    take(&h->done, h->ntasks);
+    zeroed = used + perm_zero_bytes(h->nbuckets);
+    take(&h->sort_ws, static_cast<int64_t>(sort_bytes));
+    take(&h->scan_ws, static_cast<int64_t>(scan_bytes));
+    take(&h->segs, h->nseg);
+    if (h->batch) take(&h->seg_of, n);
+    take(&h->rp_id, n + 1);
+    take(&h->deg_id, n);
+    take(&h->col[0], nnz + kColPad);
+    take(&h->col[1], nnz + kColPad);
+    for (int i = 0; i < 2; ++i) {
+      take(&h->order[i], n);
+      take(&h->pos[i], n);
+      take(&h->rp[i], n + 1);
+    }
+    take(&h->chunk_row, nnz / kRowChunk + 2);
+    take(&h->stash, nnz);
+    take(&h->thr_key, h->ntasks);
+    take(&h->thr_tb, h->ntasks);
+    take(&h->far_pack, h->ntasks);
+    take(&h->lists, kClasses * h->ntasks);
+    take(&h->def_list, 3 * h->ntasks + 2);
+  };
+  layout();
+  if (dmalloc(h, reinterpret_cast<void**>(&base), used)) return fail(h, CB_ENOMEM, "device allocation failed");
+  h->arena = base;
+  layout();
+  CB_CUDA(h, cudaMemsetAsync(base, 0, zeroed, h->stream));
+  return CB_OK;
+}
+
+// Common part of handle creation.  On entry: the arrays, the segment table
+// (host and device, seg_of for batches) and the id-space CSR (rp_id, col[0],
+// unsorted rows) are in place.  Validates, sizes the workspaces and lays the
+// graph out for its first super step.
+int finish_create(Graph* h) {
+  const int64_t n = h->n;
+  cudaStream_t s = h->stream;
+  int rc;
+  if ((rc = init_trade_kernels(h)) || (rc = init_perm_kernels(h))) return rc;
+  if (n)
+    k_degrees<<<grid1d(n, h->num_sms), 256, 0, s>>>(n, h->rp_id, h->deg_id,
+                                                    reinterpret_cast<unsigned long long*>(h->scratch), h->err);
+  CB_CUDA(h, cudaGetLastError());
+  ++h->launches;
   // rows in id space, sorted (sorted input is used as it is), then validated:
   // simple and symmetric
   int32_t* idcol = h->col[0];
   {
     Validation v;
-    bool sorted = false;
-    rc = scan_rows(h, h->rp_id, idcol, n, &v, &sorted);
-    if (!rc && !sorted && !v.bad) {
-      rc = permute_rows(h, n, h->rp_id, h->col[0], nullptr, nullptr, h->rp_id, h->col[1]);
+    auto give_up = [&](int code, const char* what) {
+      free_validation(h, &v);
+      if (what) h->last_error = what;
+      return code;
+    };
+    if ((rc = scan_rows(h, h->rp_id, idcol, n, &v))) return give_up(rc, nullptr);
+    if (v.err != kErrNone)
+      return give_up(CB_EINVAL, "row_ptr is not a valid CSR offset array (degrees in [0, n), ids in range)");
+    h->maxdeg = v.maxdeg;
+    if ((rc = size_trade_workspace(h))) return give_up(rc, nullptr);
+    if (v.unsorted && !v.bad) {
+      if ((rc = permute_rows(h, n, h->rp_id, h->col[0], nullptr, nullptr, h->rp_id, h->col[1]))) return give_up(rc, nullptr);
       idcol = h->col[1];
-      if (!rc) rc = scan_rows(h, h->rp_id, idcol, n, &v, &sorted);
+      if ((rc = scan_rows(h, h->rp_id, idcol, n, &v))) return give_up(rc, nullptr);
     }
-    if (!rc && sorted && !v.bad)
-      rc = validate_sorted_graph(h, h->rp_id, idcol, n, &v, idcol == h->col[0] ? h->col[1] : h->col[0]);
+    if (v.unsorted || v.bad || v.upper != v.lower) return give_up(CB_EINVAL, "graph is not simple and symmetric");
+    rc = validate_sorted_graph(h, h->rp_id, idcol, n, &v, idcol == h->col[0] ? h->col[1] : h->col[0]);
     free_validation(h, &v);
     if (rc) return rc;
-    rc = check_device_error(h);
-    if (rc || !sorted || v.bad) {
-      h->last_error = "graph is not simple and symmetric";
-      return CB_EINVAL;
-    }
   }
   // position-space layout of the first super step (rows are sets: no sort);
   // the step's adjacency lives in col[cur = 0]
@@ -295,9 +320,12 @@ int finish_create(Graph* h) {
   int32_t* pcol = idcol == h->col[0] ? h->col[1] : h->col[0];
   if ((rc = relabel_rows(h, n, h->rp_id, idcol, h->order[0], h->pos[0], h->rp[0], pcol))) return rc;
   if (pcol != h->col[0]) std::swap(h->col[0], h->col[1]);
-  // the super steps' counters start at zero (creation used them as scratch)
-  CB_CUDA(h, cudaMemsetAsync(h->counters, 0, sizeof(int64_t) * (2 * kCounters + 4), s));
-  return check_device_error(h);
+  // (the ids were in range, so the layout is safe to run on an asymmetric graph)
+  if ((rc = check_device_error(h)) == CB_ECHECK) {
+    h->last_error = "graph is not simple and symmetric";
+    return CB_EINVAL;
+  }
+  return rc;
 }
 
 void drop_graphs(Graph* h) {
@@ -428,7 +456,7 @@ int64_t estimate_handle_bytes(int64_t n, int64_t nnz, int64_t maxdeg, int num_sm
   const int64_t ntasks = n / 2 + (n & 1);
   const int64_t nb = int64_t(1) << bucket_bits(n);
   int64_t b = 0;
-  b += sizeof(Seg) + 8 * (n + 1) + 4 * n + 2 * 4 * (nnz + kColPad) + 32 + 8 * (2 * kCounters + 4);   // cb_create
+  b += sizeof(Seg) + 8 * (n + 1) + 4 * n + 2 * 4 * (nnz + kColPad) + 32 + 8 * (2 * kCounters + 1 + kScratch);   // cb_create
   b += 2 * 4 * n + 2 * 8 * (n + 1) + 2 * 4 * n + 2 * nnz + 4 * (nnz / kRowChunk + 2);                                 // per node, side words
   b += ntasks * (8 + 8 + 4 + 16 + 4 * kClasses + 4 * 3) + ntasks / 8 + 4 * 3 * kDefSegs + 16;                                  // per trade
   b += static_cast<int64_t>(perm_ws_bytes(nb, nb * bucket_space(n, bucket_bits(n))) + scan_ws_bytes(n + 1));
@@ -502,11 +530,8 @@ int cb_create(int64_t n, const int64_t* row_ptr, const int32_t* col, uint64_t se
     h->nbuckets = int64_t(1) << S.B;
   }
   cudaStream_t s = h->stream;
-  if (dalloc(h, &h->segs, 1) || dalloc(h, &h->rp_id, n + 1) || dalloc(h, &h->deg_id, n) || dalloc(h, &h->col[0], nnz + kColPad) ||
-      dalloc(h, &h->col[1], nnz + kColPad) || dalloc(h, &h->err, 8) || dalloc(h, &h->counters, 2 * kCounters + 4) ||
-      !(h->host_counters = new (std::nothrow) int64_t[kCounters]))
-    return bail(fail(h, CB_ENOMEM, "device allocation failed"));
-  CB_CUDA(h, cudaMemsetAsync(h->err, 0, 8 * sizeof(int32_t), s));
+  if (!(h->host_counters = new (std::nothrow) int64_t[kCounters])) return bail(fail(h, CB_ENOMEM, "host allocation failed"));
+  if ((rc = alloc_arrays(h))) return bail(rc);
   if ((rc = upload_segs(h))) return bail(rc);
   CB_CUDA(h, cudaMemcpyAsync(h->rp_id, row_ptr, sizeof(int64_t) * (n + 1), kind, s));
   if (nnz) CB_CUDA(h, cudaMemcpyAsync(h->col[0], col, sizeof(int32_t) * nnz, kind, s));
@@ -550,6 +575,7 @@ int cb_create_batch(int32_t count, const int64_t* n, const int64_t* row_ptr, con
     rph = rp_copy;
   }
   h->nseg = count;
+  h->batch = true;
   h->hsegs = new (std::nothrow) Seg[count];
   int64_t* rpo = new (std::nothrow) int64_t[2 * static_cast<size_t>(count)];
   if (!h->hsegs || !rpo) {
@@ -601,9 +627,8 @@ int cb_create_batch(int32_t count, const int64_t* n, const int64_t* row_ptr, con
   cudaStream_t s = h->stream;
   int64_t* d_rp_in = nullptr;
   int64_t* d_rpo = nullptr;
-  if (dalloc(h, &h->segs, count) || dalloc(h, &h->seg_of, N) || dalloc(h, &h->rp_id, N + 1) || dalloc(h, &h->deg_id, N) ||
-      dalloc(h, &h->col[0], e + kColPad) || dalloc(h, &h->col[1], e + kColPad) || dalloc(h, &h->err, 8) || dalloc(h, &h->counters, 2 * kCounters + 4) ||
-      !(h->host_counters = new (std::nothrow) int64_t[kCounters]) || dalloc(h, &d_rp_in, nrp) ||
+  rc = alloc_arrays(h);
+  if (rc || !(h->host_counters = new (std::nothrow) int64_t[kCounters]) || dalloc(h, &d_rp_in, nrp) ||
       dalloc(h, &d_rpo, 2 * static_cast<int64_t>(count))) {
     delete[] rpo;
     dfree(h, d_rp_in);
@@ -611,7 +636,7 @@ int cb_create_batch(int32_t count, const int64_t* n, const int64_t* row_ptr, con
     return bail(fail(h, CB_ENOMEM, "device allocation failed"));
   }
   const cudaMemcpyKind kind = mem_kind == CB_HOST ? cudaMemcpyHostToDevice : cudaMemcpyDeviceToDevice;
-  cudaError_t ce = cudaMemsetAsync(h->err, 0, 8 * sizeof(int32_t), s);
+  cudaError_t ce = cudaSuccess;
   if (ce == cudaSuccess)
     ce = cudaMemcpyAsync(h->segs, h->hsegs, sizeof(Seg) * count, cudaMemcpyHostToDevice, s);
   if (ce == cudaSuccess) ce = cudaMemcpyAsync(d_rpo, rpo, sizeof(int64_t) * 2 * count, cudaMemcpyHostToDevice, s);

@@ -47,6 +47,7 @@ constexpr int kCtrChunks = 41;      // its chunks
 constexpr int kCtrClaim = 42;       // [42 + 3 r, 45 + 3 r): trades of each list that retry pass r claimed
 static_assert(24 + 3 * (kRetryPassesMax + 1) <= 40 && 42 + 3 * kRetryPassesMax <= kCounters - 1, "counter layout");
 constexpr int kRowChunk = 2048;      // entries per sample of the entry -> row index
+constexpr int kScratch = 16;         // device words of a handle for creation and export
 constexpr int kDefSegs = 1024;      // most segments of the trades that deferred ones are counted in
 constexpr int kStats = 7 + 2 * kClasses;   // counters cb_stats reports
 constexpr int kTimings = 6 + kClasses;     // values cb_timings reports
@@ -79,8 +80,9 @@ struct Graph {
   uint64_t seed = 0, g = 0;
   // segments (graphs) of the handle
   int nseg = 1;
+  bool batch = false;             // made by cb_create_batch
   Seg* segs = nullptr;            // device table (nseg)
-  int32_t* seg_of = nullptr;      // device: segment of each node id / position (null when nseg == 1)
+  int32_t* seg_of = nullptr;      // device: segment of each node id / position (null for a plain handle)
   Seg* hsegs = nullptr;           // host copy (g not kept current)
   int64_t nbuckets = 1;           // permutation buckets over all segments
   int32_t* pairs = nullptr;       // batch export: every graph's pairs, local ids
@@ -115,14 +117,14 @@ struct Graph {
   int32_t* def_list = nullptr;             // by kind for a retry pass; in index order with the chunks' first ones for the in-order pass
   int64_t* counters = nullptr;             // two sets of kCounters, then the CTAs that ended the step
   int32_t* err = nullptr;                  // latched device error
+  int64_t* scratch = nullptr;              // kScratch words right after it
+  void* arena = nullptr;                   // the allocation that holds the arrays above and below
   // workspaces
   void* ws_global = nullptr;               // global workspace for trades too big for smem
   size_t ws_slice = 0;                     // bytes per CTA slice
   int ws_ctas = 0;                         // number of slices
-  void* sort_ws = nullptr;                 // permutation sort scratch
-  size_t sort_ws_bytes = 0;
-  void* scan_ws = nullptr;
-  size_t scan_ws_bytes = 0;
+  char* sort_ws = nullptr;                 // permutation scratch
+  char* scan_ws = nullptr;
   int64_t* host_counters = nullptr;        // host mirror of counters
   int64_t dev_bytes = 0, dev_bytes_peak = 0;   // device memory held by the handle
 
@@ -211,33 +213,34 @@ int64_t bucket_space(int64_t span, int B);
 // classes (may be null): build the size-class lists of the current step too.
 int compute_permutation(Graph* h, uint32_t dg, int64_t g_abs, int32_t* order_out, int32_t* pos_out, int64_t* rp_out,
                         const ClassArgs* classes);
-int clear_perm_ws(Graph* h);
+size_t perm_zero_bytes(int64_t nbuckets);   // the start of its scratch that has to be zero at first
 
 // rows.cu
 // dst row q <- src row rowmap[q] with values mapped through valmap (identity if null), ascending
 int permute_rows(Graph* h, int64_t nrows, const int64_t* src_rp, const int32_t* src_col,
                  const int32_t* rowmap, const int32_t* valmap, const int64_t* dst_rp, int32_t* dst_col);
-// Validation of the input: scan_rows checks ids and says whether every row is
-// strictly increasing (synchronises); validate_sorted_graph then checks the
-// symmetry of such rows and latches kErrValidate (not synchronising; `grouped`
-// is scratch of row_ptr[n] int32).
+// Validation of the input: scan_rows checks ids and order and counts the
+// entries on each side of the diagonal (synchronises); validate_sorted_graph
+// then checks the symmetry of well formed rows and latches kErrValidate (not
+// synchronising; `grouped` is scratch of row_ptr[n] int32).
 struct Validation {
-  char* ws = nullptr;
+  char* ws = nullptr;          // graphs too large for L2: the partition's scratch
   size_t bytes = 0;
   int sh = 0, nb = 0, ctas = 0;
-  int32_t* flags = nullptr;
   int32_t* counts = nullptr;   // upper entries per (bucket, CTA)
   int64_t* place = nullptr;    // their exclusive scan
   void* scan = nullptr;
+  int32_t err = 0;             // the device error word (kErrValidate: bad offsets)
+  int64_t maxdeg = 0, upper = 0, lower = 0;
+  bool unsorted = false;       // some row is not strictly increasing
   bool bad = false;            // an id out of range or a self loop
 };
-int scan_rows(Graph* h, const int64_t* rp, const int32_t* col, int64_t n, Validation* v, bool* sorted);
+int scan_rows(Graph* h, const int64_t* rp, const int32_t* col, int64_t n, Validation* v);
 int validate_sorted_graph(Graph* h, const int64_t* rp, const int32_t* col, int64_t n, Validation* v, int32_t* grouped);
 void free_validation(Graph* h, Validation* v);
 // like permute_rows without sorting (rows keep their order)
 int relabel_rows(Graph* h, int64_t nrows, const int64_t* src_rp, const int32_t* src_col, const int32_t* rowmap,
                  const int32_t* valmap, const int64_t* dst_rp, int32_t* dst_col);
-int check_row_offsets(Graph* h, const int64_t* rp, int64_t n);
 // canonical pairs (x < y, sorted, local ids) of the current step into `pairs`
 // (2m int32, device); uses the spare adjacency buffer
 int export_sorted_pairs(Graph* h, int32_t* pairs);

@@ -566,7 +566,7 @@ size_t perm_ws_bytes(int64_t nbuckets, int64_t slots) {
 }
 
 // The bucket sort's shared memory for the largest "bucket_cap" (set once,
-// outside any stream capture), and the scratch's zero words.
+// outside any stream capture).
 int init_perm_kernels(Graph* h) {
   CB_CUDA(h, cudaFuncSetAttribute(k_bucket_sort, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                   static_cast<int>(bucket_smem_bytes(kBucketCapMax))));
@@ -574,10 +574,7 @@ int init_perm_kernels(Graph* h) {
                                   static_cast<int>(bucket_smem_bytes(kBucketCapMax))));
   return CB_OK;
 }
-int clear_perm_ws(Graph* h) {
-  CB_CUDA(h, cudaMemsetAsync(h->sort_ws, 0, zero_bytes(h->nbuckets), h->stream));
-  return CB_OK;
-}
+size_t perm_zero_bytes(int64_t nbuckets) { return zero_bytes(nbuckets); }
 
 namespace {
 // Keys a rescan of every bucket would compute.

@@ -91,10 +91,11 @@ def test_dense_cores_through_the_in_order_pass(n, b, options):
 
 
 # rows of 32, 33, 256, 257, 1024, 1025 and more entries above the diagonal
-# (a warp on its tile, a warp on a listed row, 1024 threads, a global slice), a star
+# (a warp on its tile, a warp on a listed row, 128 to 1024 threads, a global slice), a star
 # whose hub is the first or the last node, and an output buffer that is only
 # 4-byte aligned.
-@pytest.mark.parametrize("d", [1, 2, 31, 32, 33, 64, 65, 128, 129, 255, 256, 257, 511, 512, 513, 1023, 1024, 1025, 2049, 5000, 20000])
+@pytest.mark.parametrize("d", [1, 2, 31, 32, 33, 64, 65, 128, 129, 255, 256, 257, 511, 512, 513, 1023, 1024, 1025, 2047, 2048,
+                               2049, 4097, 8192, 8193, 16384, 16385, 20000])
 @pytest.mark.parametrize("hub_last", [False, True])
 def test_export_of_long_rows(d, hub_last):
     import torch
