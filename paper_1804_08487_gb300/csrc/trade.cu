@@ -1384,40 +1384,6 @@ struct LaneCfg {
   static constexpr int kTeams = 32 * kWarpWarps / W;   // teams per CTA
   static constexpr size_t kSmem = Ws::kBytes * kTeams;
 };
-template <int W, bool kOneSeed>
-__global__ void __launch_bounds__(32 * kWarpWarps, 4) k_phase_a_lanes(StepCtx c, const int32_t* __restrict__ lists,
-                                                                   const int64_t* __restrict__ ctr, int cls) {
-  using Cfg = LaneCfg<W>;
-  extern __shared__ __align__(16) char lsm[];
-  const int id = threadIdx.x / W;
-  const typename Cfg::Ws w{lsm + Cfg::Ws::kBytes * id};
-  LaneTeam<W> tm;
-  const ClassList cl = class_list(c, lists, ctr, cls);
-  const int64_t step = static_cast<int64_t>(gridDim.x) * Cfg::kTeams;
-  // a warp's teams run in lockstep, so its loop ends when none has a trade
-  const int first = id & ~(32 / W - 1);
-  for (int64_t q0 = static_cast<int64_t>(blockIdx.x) * Cfg::kTeams + first; q0 < cl.len; q0 += step) {
-    const int64_t q = q0 + (id - first);
-    const bool active = q < cl.len;
-    const int64_t t = cl.list[active ? q : q0];
-    if (!phase_a_reg<LaneTeam<W>, kWarpJ, Cfg::B, true, kOneSeed>(tm, c, t, w, active) && tm.rank == 0) defer_trade(c, t);
-  }
-}
-
-template <bool kOneSeed>
-__global__ void __launch_bounds__(32 * kWarpWarps, 4) k_phase_a_warp(StepCtx c, const int32_t* __restrict__ lists,
-                                                                  const int64_t* __restrict__ ctr, int cls) {
-  extern __shared__ __align__(16) char wsm[];
-  const int wid = threadIdx.x >> 5;
-  const WarpWs w{wsm + WarpWs::kBytes * wid};
-  WarpTeam tm;
-  const ClassList cl = class_list(c, lists, ctr, cls);
-  const int64_t step = static_cast<int64_t>(gridDim.x) * kWarpWarps;
-  for (int64_t q = static_cast<int64_t>(blockIdx.x) * kWarpWarps + wid; q < cl.len; q += step)
-    if (!phase_a_reg<WarpTeam, kWarpJ, kWarpB, true, kOneSeed>(tm, c, cl.list[q], w) && tm.rank == 0)
-      defer_trade(c, cl.list[q]);
-}
-
 // Phase A of larger trades: a CTA of CT threads holds CT / NT teams of NT
 // threads (named barriers), each running one trade at a time with kTeamJ
 // entries per thread in registers (L <= NT kTeamJ).
@@ -1428,25 +1394,136 @@ struct TeamCfg {
   using Ws = RegWs<NT * kTeamJ, B, kCand>;
   static constexpr int kMax = NT * kTeamJ;
 };
+// The first pass of a handle of fewer than kFuseMax trades runs classes 0 to 5
+// in one kernel, and 6 and 7 in another.  A class's trades are cut into CTA
+// rounds (one trade per team), the classes' rounds follow each other, and CTA
+// b takes rounds b, b + G, ...: the classes run side by side on different
+// CTAs, where a launch per class spends its time on the latency of one round
+// each (n=4096, four classes: 53 us -> 18 in one kernel; n=2^17: 153 -> 135).
+// Large graphs keep a kernel per class: CTAs of one SM in different classes
+// share its instruction cache badly (n=2^20: 848 us per class, 947 together).
+constexpr int64_t kFuseMax = int64_t(1) << 17;
+struct Rounds {
+  int64_t at = 0;   // rounds of the classes so far
+  // this CTA's first round of a class of `rounds`
+  __device__ __forceinline__ int64_t first(int64_t rounds) {
+    const int64_t G = gridDim.x;
+    const int64_t i = (static_cast<int64_t>(blockIdx.x) + G - at % G) % G;
+    at += rounds;
+    return i;
+  }
+};
+
+template <int W, bool kOneSeed>
+__device__ void run_lanes(const StepCtx& c, const ClassList& cl, char* smem, Rounds& rs) {
+  using Cfg = LaneCfg<W>;
+  const int id = threadIdx.x / W;
+  const typename Cfg::Ws w{smem + Cfg::Ws::kBytes * id};
+  LaneTeam<W> tm;
+  // a warp's teams run in lockstep, so its loop ends when none has a trade
+  const int lead = id & ~(32 / W - 1);
+  const int64_t step = static_cast<int64_t>(gridDim.x) * Cfg::kTeams;
+  for (int64_t q0 = rs.first((cl.len + Cfg::kTeams - 1) / Cfg::kTeams) * Cfg::kTeams + lead; q0 < cl.len; q0 += step) {
+    const int64_t q = q0 + (id - lead);
+    const bool active = q < cl.len;
+    const int64_t t = cl.list[active ? q : q0];
+    if (!phase_a_reg<LaneTeam<W>, kWarpJ, Cfg::B, true, kOneSeed>(tm, c, t, w, active) && tm.rank == 0) defer_trade(c, t);
+  }
+}
+template <bool kOneSeed>
+__device__ void run_warps(const StepCtx& c, const ClassList& cl, char* smem, Rounds& rs) {
+  const int wid = threadIdx.x >> 5;
+  const WarpWs w{smem + WarpWs::kBytes * wid};
+  WarpTeam tm;
+  const int64_t step = static_cast<int64_t>(gridDim.x) * kWarpWarps;
+  for (int64_t q = rs.first((cl.len + kWarpWarps - 1) / kWarpWarps) * kWarpWarps + wid; q < cl.len; q += step)
+    if (!phase_a_reg<WarpTeam, kWarpJ, kWarpB, true, kOneSeed>(tm, c, cl.list[q], w) && tm.rank == 0)
+      defer_trade(c, cl.list[q]);
+}
 template <int CT, int NT, bool kOneSeed>
-__global__ void __launch_bounds__(CT, CT == 256 ? 4 : 1) k_phase_a_team(StepCtx c, const int32_t* __restrict__ lists,
-                                                                      const int64_t* __restrict__ ctr, int cls) {
+__device__ void run_teams(const StepCtx& c, const ClassList& cl, char* smem, int64_t* red, Rounds& rs) {
   constexpr int kTeams = CT / NT;
   using Ws = typename TeamCfg<NT>::Ws;
-  extern __shared__ __align__(16) char tsm[];
-  __shared__ int64_t red[kTeams * SubTeam<NT>::kRedSlots];
   const int id = threadIdx.x / NT;
   SubTeam<NT> tm(red + id * SubTeam<NT>::kRedSlots, id);
-  const Ws w{tsm + Ws::kBytes * id};
-  const ClassList cl = class_list(c, lists, ctr, cls);
+  const Ws w{smem + Ws::kBytes * id};
   const int64_t step = static_cast<int64_t>(gridDim.x) * kTeams;
-  for (int64_t q = static_cast<int64_t>(blockIdx.x) * kTeams + id; q < cl.len; q += step)
+  for (int64_t q = rs.first((cl.len + kTeams - 1) / kTeams) * kTeams + id; q < cl.len; q += step)
     if (!phase_a_reg<SubTeam<NT>, kTeamJ, TeamCfg<NT>::B, false, kOneSeed>(tm, c, cl.list[q], w) && tm.rank == 0)
       defer_trade(c, cl.list[q]);
 }
-template <int CT, int NT>
-constexpr size_t team_smem() {
-  return TeamCfg<NT>::Ws::kBytes * (CT / NT);
+
+// Class K alone.
+template <int K>
+constexpr size_t class_smem() {
+  return K == 0 ? LaneCfg<8>::kSmem : K == 1 ? LaneCfg<16>::kSmem : K == 2 ? WarpWs::kBytes * kWarpWarps
+         : K == 3 ? TeamCfg<64>::Ws::kBytes * 4 : K == 4 ? TeamCfg<128>::Ws::kBytes * 2
+         : K == 5 ? TeamCfg<256>::Ws::kBytes : K == 6 ? TeamCfg<512>::Ws::kBytes * 2 : TeamCfg<1024>::Ws::kBytes;
+}
+template <int K, bool kOneSeed>
+__global__ void __launch_bounds__(K < 6 ? 256 : kBigThreads, K < 6 ? 4 : 1) k_phase_a_class(StepCtx c,
+                                                                const int32_t* __restrict__ lists,
+                                                                const int64_t* __restrict__ ctr) {
+  extern __shared__ __align__(16) char smem[];
+  __shared__ int64_t red[K < 3 ? 1 : K < 6 ? 4 * SubTeam<64>::kRedSlots : SubTeam<kBigThreads>::kRedSlots];
+  Rounds rs;
+  const ClassList cl = class_list(c, lists, ctr, K);
+  if constexpr (K == 0) run_lanes<8, kOneSeed>(c, cl, smem, rs);
+  else if constexpr (K == 1) run_lanes<16, kOneSeed>(c, cl, smem, rs);
+  else if constexpr (K == 2) run_warps<kOneSeed>(c, cl, smem, rs);
+  else if constexpr (K == 3) run_teams<256, 64, kOneSeed>(c, cl, smem, red, rs);
+  else if constexpr (K == 4) run_teams<256, 128, kOneSeed>(c, cl, smem, red, rs);
+  else if constexpr (K == 5) run_teams<256, 256, kOneSeed>(c, cl, smem, red, rs);
+  else if constexpr (K == 6) run_teams<kBigThreads, 512, kOneSeed>(c, cl, smem, red, rs);
+  else run_teams<kBigThreads, kBigThreads, kOneSeed>(c, cl, smem, red, rs);
+}
+
+// Classes 0 to 5 (without the lane teams or the teams where an option sends
+// their trades elsewhere): 256 threads, the longest trades first.
+constexpr int kRunLanes = 1, kRunTeams = 2;
+constexpr size_t small_smem() {
+  size_t m = LaneCfg<8>::kSmem;
+  for (size_t x : {LaneCfg<16>::kSmem, WarpWs::kBytes * kWarpWarps, TeamCfg<64>::Ws::kBytes * 4,
+                   TeamCfg<128>::Ws::kBytes * 2, TeamCfg<256>::Ws::kBytes})
+    m = x > m ? x : m;
+  return m;
+}
+template <bool kOneSeed>
+__global__ void __launch_bounds__(256, 4) k_phase_a_small(StepCtx c, const int32_t* __restrict__ lists,
+                                                        const int64_t* __restrict__ ctr, int what) {
+  extern __shared__ __align__(16) char smem[];
+  __shared__ int64_t red[4 * SubTeam<64>::kRedSlots];
+  static_assert(4 * SubTeam<64>::kRedSlots >= SubTeam<256>::kRedSlots && 4 * SubTeam<64>::kRedSlots >= 2 * SubTeam<128>::kRedSlots, "");
+  Rounds rs;
+  if (what & kRunTeams) {
+    run_teams<256, 256, kOneSeed>(c, class_list(c, lists, ctr, 5), smem, red, rs);
+    __syncthreads();   // the next class lays the shared memory out anew
+    run_teams<256, 128, kOneSeed>(c, class_list(c, lists, ctr, 4), smem, red, rs);
+    __syncthreads();
+    run_teams<256, 64, kOneSeed>(c, class_list(c, lists, ctr, 3), smem, red, rs);
+    __syncthreads();
+  }
+  run_warps<kOneSeed>(c, class_list(c, lists, ctr, 2), smem, rs);
+  if (what & kRunLanes) {
+    __syncthreads();
+    run_lanes<16, kOneSeed>(c, class_list(c, lists, ctr, 1), smem, rs);
+    __syncthreads();
+    run_lanes<8, kOneSeed>(c, class_list(c, lists, ctr, 0), smem, rs);
+  }
+}
+
+// Classes 7 and 6: 1024 threads.
+constexpr size_t kLargeSmem = 2 * TeamCfg<512>::Ws::kBytes > TeamCfg<kBigThreads>::Ws::kBytes
+                                  ? 2 * TeamCfg<512>::Ws::kBytes : TeamCfg<kBigThreads>::Ws::kBytes;
+template <bool kOneSeed>
+__global__ void __launch_bounds__(kBigThreads, 1) k_phase_a_large(StepCtx c, const int32_t* __restrict__ lists,
+                                                                const int64_t* __restrict__ ctr) {
+  extern __shared__ __align__(16) char smem[];
+  __shared__ int64_t red[SubTeam<kBigThreads>::kRedSlots];
+  Rounds rs;
+  run_teams<kBigThreads, kBigThreads, kOneSeed>(c, class_list(c, lists, ctr, 7), smem, red, rs);
+  __syncthreads();
+  run_teams<kBigThreads, 512, kOneSeed>(c, class_list(c, lists, ctr, 6), smem, red, rs);
 }
 
 // ------------------------------------------------------ rebuild: fix-up
@@ -2005,6 +2082,8 @@ __global__ void __launch_bounds__(NT, NT == 256 ? 4 : 1) k_resolve(StepCtx c, co
 }  // namespace
 
 namespace {
+template <int K>
+using Int = std::integral_constant<int, K>;
 // Attributes of the kernels built in a one-graph and a general version.
 template <bool kOneSeed>
 int init_seed_kernels(Graph* h) {
@@ -2012,26 +2091,26 @@ int init_seed_kernels(Graph* h) {
                                   static_cast<int>(block_smem_bytes(kBlockMaxCap))));
   CB_CUDA(h, cudaFuncSetAttribute(k_phase_a_block<kBigThreads, kOneSeed>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                   static_cast<int>(block_smem_bytes(kSmemMaxCap))));
-  CB_CUDA(h, cudaFuncSetAttribute(k_phase_a_team<kBigThreads, 512, kOneSeed>,
-                                  cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                  static_cast<int>(team_smem<kBigThreads, 512>())));
-  CB_CUDA(h, cudaFuncSetAttribute(k_phase_a_team<kBigThreads, kBigThreads, kOneSeed>,
-                                  cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                  static_cast<int>(team_smem<kBigThreads, kBigThreads>())));
-  CB_CUDA(h, cudaFuncSetAttribute(k_phase_a_lanes<8, kOneSeed>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                  static_cast<int>(LaneCfg<8>::kSmem)));
-  CB_CUDA(h, cudaFuncSetAttribute(k_phase_a_lanes<16, kOneSeed>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                  static_cast<int>(LaneCfg<16>::kSmem)));
-  CB_CUDA(h, cudaFuncSetAttribute(k_phase_a_warp<kOneSeed>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                  static_cast<int>(WarpWs::kBytes * kWarpWarps)));
+  auto of_class = [&](auto k) -> int {
+    constexpr int K = decltype(k)::value;
+    CB_CUDA(h, cudaFuncSetAttribute(k_phase_a_class<K, kOneSeed>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                    static_cast<int>(class_smem<K>())));
+    CB_CUDA(h, cudaFuncSetAttribute(k_phase_a_class<K, kOneSeed>, cudaFuncAttributePreferredSharedMemoryCarveout,
+                                    cudaSharedmemCarveoutMaxShared));
+    return CB_OK;
+  };
+  int rc;
+  if ((rc = of_class(Int<0>{})) || (rc = of_class(Int<1>{})) || (rc = of_class(Int<2>{})) || (rc = of_class(Int<3>{})) ||
+      (rc = of_class(Int<4>{})) || (rc = of_class(Int<5>{})) || (rc = of_class(Int<6>{})) || (rc = of_class(Int<7>{})))
+    return rc;
+  CB_CUDA(h, cudaFuncSetAttribute(k_phase_a_large<kOneSeed>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                  static_cast<int>(kLargeSmem)));
+  CB_CUDA(h, cudaFuncSetAttribute(k_phase_a_small<kOneSeed>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                  static_cast<int>(small_smem())));
   // shared memory, not L1, limits how many CTAs of these kernels an SM holds
   CB_CUDA(h, cudaFuncSetAttribute(k_phase_a_block<kMedThreads, kOneSeed>,
                                   cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared));
-  CB_CUDA(h, cudaFuncSetAttribute(k_phase_a_lanes<8, kOneSeed>, cudaFuncAttributePreferredSharedMemoryCarveout,
-                                  cudaSharedmemCarveoutMaxShared));
-  CB_CUDA(h, cudaFuncSetAttribute(k_phase_a_lanes<16, kOneSeed>, cudaFuncAttributePreferredSharedMemoryCarveout,
-                                  cudaSharedmemCarveoutMaxShared));
-  CB_CUDA(h, cudaFuncSetAttribute(k_phase_a_warp<kOneSeed>, cudaFuncAttributePreferredSharedMemoryCarveout,
+  CB_CUDA(h, cudaFuncSetAttribute(k_phase_a_small<kOneSeed>, cudaFuncAttributePreferredSharedMemoryCarveout,
                                   cudaSharedmemCarveoutMaxShared));
   return CB_OK;
 }
@@ -2171,20 +2250,22 @@ int super_step(Graph* h) {
   const size_t big_smem_st = block_smem_bytes(std::max(h->smem_max, 1));
   const unsigned mgrid = static_cast<unsigned>(h->num_sms * 4);
   const unsigned bgrid = static_cast<unsigned>(std::max(1, std::min(h->num_sms, h->ws_ctas)));
-  const unsigned sgrid = static_cast<unsigned>(h->num_sms);
   const unsigned wgrid = static_cast<unsigned>(h->num_sms * 8);
+  // resident CTAs, at most one per trade
+  const unsigned small_grid = static_cast<unsigned>(std::min<int64_t>(mgrid, ntasks));
+  const unsigned large_grid = static_cast<unsigned>(std::min<int64_t>(h->num_sms, ntasks));
   char* gws = static_cast<char*>(h->ws_global);
   c.cand_max = h->cand_max;
   c.wait_ns = h->wait_ns;
   c.hold_publish = h->hold_publish;
   const int32_t* L = h->lists;
-  // one kernel per size class (no trade is larger than twice the largest
-  // degree: classes above that are not launched); a trade whose dependency
-  // has not published yet is marked deferred.  With "timing" on, the pass
-  // brackets each class's kernel with events ev[4 + k] .. ev[5 + k] (a class
-  // without its own kernel takes none).
+  // the first pass: one kernel for classes 0 to 5 and one for 6 and 7, or one
+  // per class (large graphs), and the largest trades (no trade is larger than
+  // twice the largest degree: classes above that are not launched); a trade
+  // whose dependency has not published yet is deferred.  With "timing" on,
+  // events ev[4] .. ev[13] bracket the classes' kernels.
   const int64_t max_trade = 2 * h->maxdeg;
-  auto has = [&](int k) { return k == 0 || max_trade > th.th[k - 1]; };
+  const bool fused = ntasks < kFuseMax;
   auto mark = [&](int k) -> int {
     if (h->timing) CB_CUDA(h, cudaEventRecord(ev[4 + k], s));
     return CB_OK;
@@ -2194,59 +2275,46 @@ int super_step(Graph* h) {
   auto run_classes_as = [&](auto one_seed) -> int {
     constexpr bool kOne = decltype(one_seed)::value;
     int r;
-    if ((r = mark(0))) return r;
-    if (h->lane_teams) {
-      k_phase_a_lanes<8, kOne><<<wgrid, 32 * kWarpWarps, LaneCfg<8>::kSmem, s>>>(c, L, cnt, 0);
+    auto run_class = [&](auto k) -> int {
+      constexpr int K = decltype(k)::value;
+      int rk;
+      if ((rk = mark(K))) return rk;
+      if ((K > 0 && max_trade <= th.th[K > 0 ? K - 1 : 0]) || (K < 2 && !h->lane_teams)) return CB_OK;
+      const unsigned grid = K < 3 ? wgrid : K < 6 ? mgrid : static_cast<unsigned>(h->num_sms);
+      k_phase_a_class<K, kOne><<<grid, K < 6 ? 256 : kBigThreads, class_smem<K>(), s>>>(c, L, cnt);
+      return launched();
+    };
+    if (fused) {
+      if ((r = mark(0))) return r;
+      k_phase_a_small<kOne><<<small_grid, 256, small_smem(), s>>>(
+          c, L, cnt, (h->lane_teams ? kRunLanes : 0) | (h->cta_paths ? kRunTeams : 0));
       if ((r = launched())) return r;
+      for (int k = 1; k < 6; ++k)
+        if ((r = mark(k))) return r;
+    } else {
+      if ((r = run_class(Int<0>{})) || (r = run_class(Int<1>{})) || (r = run_class(Int<2>{}))) return r;
+      if (h->cta_paths && ((r = run_class(Int<3>{})) || (r = run_class(Int<4>{})) || (r = run_class(Int<5>{})))) return r;
+      for (int k = 3; k < 6 && !h->cta_paths; ++k)
+        if ((r = mark(k))) return r;
     }
-    if ((r = mark(1))) return r;
-    if (h->lane_teams && has(1)) {
-      k_phase_a_lanes<16, kOne><<<wgrid, 32 * kWarpWarps, LaneCfg<16>::kSmem, s>>>(c, L, cnt, 1);
-      if ((r = launched())) return r;
-    }
-    if ((r = mark(2))) return r;
-    if (has(2)) {
-      k_phase_a_warp<kOne><<<wgrid, 32 * kWarpWarps, WarpWs::kBytes * kWarpWarps, s>>>(c, L, cnt, 2);
-      if ((r = launched())) return r;
-    }
-    if ((r = mark(3))) return r;
-    if (h->cta_paths) {
-      if (has(3)) {
-        k_phase_a_team<256, 64, kOne><<<mgrid, 256, team_smem<256, 64>(), s>>>(c, L, cnt, 3);
-        if ((r = launched())) return r;
-      }
-      if ((r = mark(4))) return r;
-      if (has(4)) {
-        k_phase_a_team<256, 128, kOne><<<mgrid, 256, team_smem<256, 128>(), s>>>(c, L, cnt, 4);
-        if ((r = launched())) return r;
-      }
-      if ((r = mark(5))) return r;
-      if (has(5)) {
-        k_phase_a_team<256, 256, kOne><<<mgrid, 256, team_smem<256, 256>(), s>>>(c, L, cnt, 5);
-        if ((r = launched())) return r;
-      }
+    if (!h->cta_paths) {
+      k_phase_a_block<kMedThreads, kOne><<<mgrid, kMedThreads, med_smem_st, s>>>(c, L, cnt, 5, block_max, gws,
+                                                                                h->ws_slice, block_max);
+      if ((r = launched()) || (r = mark(6)) || (r = mark(7))) return r;
+    } else if (fused) {
       if ((r = mark(6))) return r;
-      if (has(6)) {
-        k_phase_a_team<kBigThreads, 512, kOne><<<sgrid, kBigThreads, team_smem<kBigThreads, 512>(), s>>>(c, L, cnt, 6);
+      if (max_trade > th.th[5]) {
+        k_phase_a_large<kOne><<<large_grid, kBigThreads, kLargeSmem, s>>>(c, L, cnt);
         if ((r = launched())) return r;
       }
       if ((r = mark(7))) return r;
-      if (has(7)) {
-        k_phase_a_team<kBigThreads, kBigThreads, kOne>
-            <<<sgrid, kBigThreads, team_smem<kBigThreads, kBigThreads>(), s>>>(c, L, cnt, 7);
-        if ((r = launched())) return r;
-      }
-      if ((r = mark(8))) return r;
-    } else {
-      k_phase_a_block<kMedThreads, kOne><<<mgrid, kMedThreads, med_smem_st, s>>>(c, L, cnt, 5, block_max, gws,
-                                                                                h->ws_slice, block_max);
-      if ((r = launched())) return r;
-      for (int k = 4; k <= 8; ++k)
-        if ((r = mark(k))) return r;
+    } else if ((r = run_class(Int<6>{})) || (r = run_class(Int<7>{}))) {
+      return r;
     }
+    if ((r = mark(8))) return r;
     // the largest trades: 1024 threads, up to smem_max entries in shared
     // memory (staged by a bulk copy), a global-memory slice above
-    if (has(8)) {
+    if (max_trade > th.th[7]) {
       k_phase_a_block<kBigThreads, kOne><<<bgrid, kBigThreads, big_smem_st, s>>>(c, L, cnt, 8, h->smem_max, gws,
                                                                                 h->ws_slice, h->smem_max);
       if ((r = launched())) return r;
