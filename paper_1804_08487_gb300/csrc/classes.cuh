@@ -21,21 +21,19 @@ struct ClassArgs {
   int64_t* ctr;          // zeroed counters: kCtrClsLen, kCtrFirstEnt
 };
 
-constexpr int kClassThreads = 256;
-
 // Chunks of trades a CTA classifies at a time: one trade per thread while
 // that leaves work for every CTA, eight (an eighth of the atomics on the list
 // lengths) for large graphs.
 inline int class_per(int64_t ntasks) { return ntasks > (int64_t(1) << 18) ? 8 : 1; }
-inline int64_t class_chunks(int64_t ntasks) {
-  const int64_t c = int64_t(kClassThreads) * class_per(ntasks);
+inline int64_t class_chunks(int64_t ntasks, int threads) {
+  const int64_t c = int64_t(threads) * class_per(ntasks);
   return (ntasks + c - 1) / c;
 }
 
-// Chunks first, first + stride, ... by a CTA of kClassThreads threads: per
+// Chunks first, first + stride, ... by a CTA of NT threads: per
 // class one reservation of list space per chunk; a chunk's trades stay
 // together, roughly in index order, so their rows are neighbours in memory.
-template <int PER>
+template <int NT, int PER>
 __device__ void classify_chunks(const ClassArgs& a, int64_t first, int64_t stride) {
   __shared__ int cnt[kClasses];
   __shared__ int put[kClasses];
@@ -43,7 +41,7 @@ __device__ void classify_chunks(const ClassArgs& a, int64_t first, int64_t strid
   __shared__ int64_t base[kClasses];
   const int lane = threadIdx.x & 31;
   const unsigned below = (1u << lane) - 1u;
-  constexpr int64_t kChunk = int64_t(kClassThreads) * PER;
+  constexpr int64_t kChunk = int64_t(NT) * PER;
   for (int64_t ch = first; ch * kChunk < a.ntasks; ch += stride) {
     if (threadIdx.x < kClasses) {
       cnt[threadIdx.x] = put[threadIdx.x] = 0;
@@ -53,7 +51,7 @@ __device__ void classify_chunks(const ClassArgs& a, int64_t first, int64_t strid
     int8_t cls[PER];
 #pragma unroll
     for (int j = 0; j < PER; ++j) {
-      const int64_t t = ch * kChunk + j * kClassThreads + threadIdx.x;
+      const int64_t t = ch * kChunk + j * NT + threadIdx.x;
       int k = -1, L = 0;
       if (t < a.ntasks) {
         const int64_t b0 = a.rp[2 * t], b1 = a.rp[2 * t + 1];
@@ -85,7 +83,7 @@ __device__ void classify_chunks(const ClassArgs& a, int64_t first, int64_t strid
     __syncthreads();
 #pragma unroll
     for (int j = 0; j < PER; ++j) {
-      const int64_t t = ch * kChunk + j * kClassThreads + threadIdx.x;
+      const int64_t t = ch * kChunk + j * NT + threadIdx.x;
       const int k = cls[j];
 #pragma unroll
       for (int q = 0; q < kClasses; ++q) {
@@ -101,9 +99,10 @@ __device__ void classify_chunks(const ClassArgs& a, int64_t first, int64_t strid
   }
 }
 
+template <int NT>
 __device__ __forceinline__ void classify(const ClassArgs& a, int64_t first, int64_t stride) {
-  if (a.ntasks > (int64_t(1) << 18)) classify_chunks<8>(a, first, stride);
-  else classify_chunks<1>(a, first, stride);
+  if (a.ntasks > (int64_t(1) << 18)) classify_chunks<NT, 8>(a, first, stride);
+  else classify_chunks<NT, 1>(a, first, stride);
 }
 
 }  // namespace cb

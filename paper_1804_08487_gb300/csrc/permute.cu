@@ -44,7 +44,6 @@ int64_t bucket_space(int64_t span, int B) {
 namespace {
 
 constexpr int kPermThreads = 256;
-static_assert(kPermThreads == kClassThreads, "the permutation kernels classify trades");
 
 __device__ __forceinline__ uint32_t bucket_of(uint64_t key, int B) {
   return B == 0 ? 0u : static_cast<uint32_t>(key >> (64 - B));
@@ -218,7 +217,8 @@ __device__ __forceinline__ BucketWs bucket_ws(void* base, int cap) {
   return w;
 }
 
-// Exclusive prefix sum over the CTA, and the total.
+// Exclusive prefix sum over the CTA of NT threads, and the total.
+template <int NT>
 __device__ __forceinline__ int64_t cta_scan(int64_t v, int64_t* wsum, int64_t* total) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   int64_t incl = v;
@@ -231,7 +231,7 @@ __device__ __forceinline__ int64_t cta_scan(int64_t v, int64_t* wsum, int64_t* t
   __syncthreads();
   int64_t before = 0, all = 0;
 #pragma unroll
-  for (int w = 0; w < kPermThreads / 32; ++w) {
+  for (int w = 0; w < NT / 32; ++w) {
     if (w < warp) before += wsum[w];
     all += wsum[w];
   }
@@ -243,19 +243,20 @@ __device__ __forceinline__ int64_t cta_scan(int64_t v, int64_t* wsum, int64_t* t
 // The s keys of a bucket in shared memory, to positions p0.. and entries
 // e0..: a counting sort on the kSubBits bits below the highest bit where they
 // differ (keys agree above it, so the digit orders them).
+template <int NT>
 __device__ void sort_bucket(const BucketWs& w, int s, int64_t p0, int64_t e0, const PermOut& out) {
   __shared__ unsigned long long s_or, s_and;
-  __shared__ int64_t wsum[kPermThreads / 32];
-  constexpr int kPer = kSubBins / kPermThreads;   // bins per thread in the scan
+  __shared__ int64_t wsum[NT / 32];
+  constexpr int kPer = kSubBins / NT;   // bins per thread in the scan
   const int lane = threadIdx.x & 31;
   if (threadIdx.x == 0) {
     s_or = 0ull;
     s_and = ~0ull;
   }
-  for (int i = threadIdx.x; i < kSubBins; i += kPermThreads) w.bcur[i] = 0;
+  for (int i = threadIdx.x; i < kSubBins; i += NT) w.bcur[i] = 0;
   __syncthreads();
   unsigned long long lor = 0ull, land = ~0ull;
-  for (int i = threadIdx.x; i < s; i += kPermThreads) {
+  for (int i = threadIdx.x; i < s; i += NT) {
     lor |= w.key[i];
     land &= w.key[i];
   }
@@ -272,7 +273,7 @@ __device__ void sort_bucket(const BucketWs& w, int s, int64_t p0, int64_t e0, co
   const uint64_t diff = s_or ^ s_and;            // the bits where the bucket's keys differ
   const int top = diff ? 63 - __clzll(static_cast<long long>(diff)) : 0;
   const int sh = top + 1 > kSubBits ? top + 1 - kSubBits : 0;
-  for (int i = threadIdx.x; i < s; i += kPermThreads)
+  for (int i = threadIdx.x; i < s; i += NT)
     atomicAdd(&w.bcur[static_cast<int>(w.key[i] >> sh) & (kSubBins - 1)], 1);
   __syncthreads();
   // exclusive scan of the bin counts: kPer consecutive bins per thread
@@ -280,7 +281,7 @@ __device__ void sort_bucket(const BucketWs& w, int s, int64_t p0, int64_t e0, co
 #pragma unroll
   for (int q = 0; q < kPer; ++q) local += w.bcur[threadIdx.x * kPer + q];
   int64_t all;
-  int run = static_cast<int>(cta_scan(local, wsum, &all));
+  int run = static_cast<int>(cta_scan<NT>(local, wsum, &all));
 #pragma unroll
   for (int q = 0; q < kPer; ++q) {
     const int bi = threadIdx.x * kPer + q;
@@ -291,11 +292,11 @@ __device__ void sort_bucket(const BucketWs& w, int s, int64_t p0, int64_t e0, co
   }
   if (threadIdx.x == 0) w.bstart[kSubBins] = s;
   __syncthreads();
-  for (int i = threadIdx.x; i < s; i += kPermThreads)
+  for (int i = threadIdx.x; i < s; i += NT)
     w.slot[atomicAdd(&w.bcur[static_cast<int>(w.key[i] >> sh) & (kSubBins - 1)], 1)] = static_cast<uint16_t>(i);
   __syncthreads();
   // rank within the bin: the bin's start plus the smaller (key, id) in it
-  for (int i = threadIdx.x; i < s; i += kPermThreads) {
+  for (int i = threadIdx.x; i < s; i += NT) {
     const uint64_t ki = w.key[i];
     const int32_t ii = w.id[i];
     const int d = static_cast<int>(ki >> sh) & (kSubBins - 1);
@@ -311,11 +312,11 @@ __device__ void sort_bucket(const BucketWs& w, int s, int64_t p0, int64_t e0, co
   }
   __syncthreads();
   if (!out.rp) return;
-  for (int base = 0; base < s; base += kPermThreads) {
+  for (int base = 0; base < s; base += NT) {
     const int r = base + static_cast<int>(threadIdx.x);
     int64_t tot;
     const int64_t d = r < s ? w.sdeg[r] : 0;
-    const int64_t x = cta_scan(d, wsum, &tot);
+    const int64_t x = cta_scan<NT>(d, wsum, &tot);
     if (r < s) put_row(out, p0 + r, e0 + x, d);
     e0 += tot;
   }
@@ -324,10 +325,10 @@ __device__ void sort_bucket(const BucketWs& w, int s, int64_t p0, int64_t e0, co
 // A bucket that does not fit: get(i, &key, &id) enumerates candidates
 // i < count and says which belong to the bucket; each is ranked against all
 // others (keys computed anew each time).
-template <class Get>
+template <int NT, class Get>
 __device__ void rank_bucket(int64_t count, Get get, int64_t s, int64_t p0, int64_t e0, const PermOut& out) {
-  __shared__ int64_t wsum[kPermThreads / 32];
-  for (int64_t i = threadIdx.x; i < count; i += kPermThreads) {
+  __shared__ int64_t wsum[NT / 32];
+  for (int64_t i = threadIdx.x; i < count; i += NT) {
     uint64_t ki, kj;
     int32_t ii, ij;
     if (!get(i, &ki, &ii)) continue;
@@ -339,27 +340,37 @@ __device__ void rank_bucket(int64_t count, Get get, int64_t s, int64_t p0, int64
   }
   __syncthreads();
   if (!out.rp) return;
-  for (int64_t base = 0; base < s; base += kPermThreads) {
+  for (int64_t base = 0; base < s; base += NT) {
     const int64_t r = base + threadIdx.x;
     int64_t tot;
     const int64_t d = r < s ? out.rp[p0 + r] : 0;
-    const int64_t x = cta_scan(d, wsum, &tot);
+    const int64_t x = cta_scan<NT>(d, wsum, &tot);
     if (r < s) put_row(out, p0 + r, e0 + x, d);
     e0 += tot;
   }
 }
 
+// A bucket's word: nodes in it (bits 33..63) and their degrees summed (bits
+// 0..32); n < 2^31 and row_ptr[n] < 2^33, so prefix sums over the words of a
+// handle keep both fields.
+constexpr int kCountShift = 33;
+constexpr uint64_t kDegMask = (uint64_t(1) << kCountShift) - 1;
+
 // Small handles: CTA b computes every key of its bucket's graph.  It costs
-// span x buckets keys per graph, the launch and the memory round trip it saves
-// cost more up to kRescanWork keys.
-__global__ void __launch_bounds__(kPermThreads) k_perm_rescan(int64_t n, int nseg, KeySrc ks, int nb, int cap,
-                                                             PermOut out, const int64_t* __restrict__ rp_id,
-                                                             int64_t nnz, ClassArgs ca) {
+// span x buckets keys per graph; the launch and the memory round trip it saves
+// cost more up to kRescanWork keys.  The latency of a thread's keys bounds it,
+// so 1024 threads share them, degrees are loaded whether needed or not, and
+// the next keys do not wait for the last ones (a permutation of 4096 nodes on
+// its own: 12.3 us per call with 256 threads, 10.2 so).
+constexpr int kRescanThreads = 1024;
+__global__ void __launch_bounds__(kRescanThreads) k_perm_rescan(int64_t n, int nseg, KeySrc ks, int nb, int cap,
+                                                               PermOut out, const int64_t* __restrict__ rp_id,
+                                                               int64_t nnz, ClassArgs ca) {
   extern __shared__ uint64_t shk[];
   __shared__ int cnt;
-  __shared__ int64_t wsum[kPermThreads / 32];
+  __shared__ int64_t wsum[kRescanThreads / 32];
   if (static_cast<int>(blockIdx.x) >= nb) {
-    classify(ca, blockIdx.x - nb, gridDim.x - nb);
+    classify<kRescanThreads>(ca, blockIdx.x - nb, gridDim.x - nb);
     return;
   }
   const int64_t b = blockIdx.x;
@@ -369,15 +380,16 @@ __global__ void __launch_bounds__(kPermThreads) k_perm_rescan(int64_t n, int nse
   if (threadIdx.x == 0) cnt = 0;
   if (b == 0 && threadIdx.x == 0 && out.rp) put_rows_end(out, n, nnz);
   __syncthreads();
+  const int64_t first_entry = out.rp ? rp_id[k.off] : 0;
   int64_t lower = 0, lower_deg = 0;
 #pragma unroll 4
-  for (int64_t x = k.off + threadIdx.x; x < k.off + k.span; x += kPermThreads) {
+  for (int64_t x = k.off + threadIdx.x; x < k.off + k.span; x += kRescanThreads) {
+    const int32_t d = out.rp ? out.deg[x] : 0;
     const uint64_t key = perm_key(k, x);
     const uint32_t bk = bucket_of(key, k.B);
-    if (bk < mine) {
-      ++lower;
-      if (out.rp) lower_deg += out.deg[x];
-    } else if (bk == mine) {
+    lower += bk < mine;
+    lower_deg += bk < mine ? d : 0;
+    if (bk == mine) {
       const int q = atomicAdd(&cnt, 1);
       if (q < cap) {
         w.key[q] = key;
@@ -385,15 +397,17 @@ __global__ void __launch_bounds__(kPermThreads) k_perm_rescan(int64_t n, int nse
       }
     }
   }
-  int64_t before, deg_before;
-  cta_scan(lower, wsum, &before);
-  cta_scan(lower_deg, wsum, &deg_before);
+  // both sums in one scan: nodes below 2^31, entries below 2^33
+  int64_t both;
+  cta_scan<kRescanThreads>(static_cast<int64_t>((static_cast<uint64_t>(lower) << kCountShift) + static_cast<uint64_t>(lower_deg)),
+                           wsum, &both);
   const int s = cnt;
-  const int64_t p0 = k.off + before, e0 = (out.rp ? rp_id[k.off] : 0) + deg_before;
+  const int64_t p0 = k.off + static_cast<int64_t>(static_cast<uint64_t>(both) >> kCountShift);
+  const int64_t e0 = first_entry + static_cast<int64_t>(static_cast<uint64_t>(both) & kDegMask);
   if (s <= cap) {
-    sort_bucket(w, s, p0, e0, out);
+    sort_bucket<kRescanThreads>(w, s, p0, e0, out);
   } else {
-    rank_bucket(
+    rank_bucket<kRescanThreads>(
         k.span,
         [&](int64_t i, uint64_t* key, int32_t* id) {
           *key = perm_key(k, k.off + i);
@@ -407,12 +421,6 @@ __global__ void __launch_bounds__(kPermThreads) k_perm_rescan(int64_t n, int nse
 constexpr int64_t kRescanWork = int64_t(1) << 21;
 constexpr int64_t kRescanBuckets = 4096;   // CTAs
 
-// A bucket's word: nodes in it (bits 33..63) and their degrees summed (bits
-// 0..32); n < 2^31 and row_ptr[n] < 2^33, so prefix sums over the words of a
-// handle keep both fields.
-constexpr int kCountShift = 33;
-constexpr uint64_t kDegMask = (uint64_t(1) << kCountShift) - 1;
-
 // Node ids into their buckets; the last CTA to finish turns the bucket words
 // into their exclusive prefix sums and clears them for the next call.
 __global__ void __launch_bounds__(kPermThreads) k_perm_scatter(int64_t n, KeySrc ks, int nb,
@@ -422,7 +430,7 @@ __global__ void __launch_bounds__(kPermThreads) k_perm_scatter(int64_t n, KeySrc
                                                               int32_t* __restrict__ bid, ClassArgs ca) {
   __shared__ int64_t wsum[kPermThreads / 32];
   __shared__ int last;
-  classify(ca, blockIdx.x, gridDim.x);
+  classify<kPermThreads>(ca, blockIdx.x, gridDim.x);
   SegKey k = seg_key(ks, 0);
   int cur = 0;
   for (int64_t x = blockIdx.x * int64_t(blockDim.x) + threadIdx.x; x < n; x += int64_t(gridDim.x) * blockDim.x) {
@@ -453,7 +461,7 @@ __global__ void __launch_bounds__(kPermThreads) k_perm_scatter(int64_t n, KeySrc
       sum += v[j];
     }
     int64_t tot;
-    uint64_t p = run + static_cast<uint64_t>(cta_scan(static_cast<int64_t>(sum), wsum, &tot));
+    uint64_t p = run + static_cast<uint64_t>(cta_scan<kPermThreads>(static_cast<int64_t>(sum), wsum, &tot));
 #pragma unroll
     for (int j = 0; j < kPer; ++j)
       if (i0 + j < nb) {
@@ -490,9 +498,9 @@ __global__ void __launch_bounds__(kPermThreads) k_bucket_sort(int64_t n, int nse
         w.key[i] = perm_key(k, x);
       }
       __syncthreads();
-      sort_bucket(w, static_cast<int>(s), p0, e0, out);
+      sort_bucket<kPermThreads>(w, static_cast<int>(s), p0, e0, out);
     } else if (s <= k.cap) {   // above the shared-memory cap
-      rank_bucket(
+      rank_bucket<kPermThreads>(
           s,
           [&](int64_t i, uint64_t* key, int32_t* id) {
             *id = ids[i];
@@ -501,7 +509,7 @@ __global__ void __launch_bounds__(kPermThreads) k_bucket_sort(int64_t n, int nse
           },
           s, p0, e0, out);
     } else {                   // the bucket's space did not hold all of it
-      rank_bucket(
+      rank_bucket<kPermThreads>(
           k.span,
           [&](int64_t i, uint64_t* key, int32_t* id) {
             *key = perm_key(k, k.off + i);
@@ -515,7 +523,9 @@ __global__ void __launch_bounds__(kPermThreads) k_bucket_sort(int64_t n, int nse
 }
 
 // Trades of the current step by size class, on its own (relaxed permutations).
-__global__ void __launch_bounds__(kClassThreads) k_classify(ClassArgs ca) { classify(ca, blockIdx.x, gridDim.x); }
+__global__ void __launch_bounds__(kPermThreads) k_classify(ClassArgs ca) {
+  classify<kPermThreads>(ca, blockIdx.x, gridDim.x);
+}
 
 __global__ void k_order_degrees(int64_t n, const int32_t* __restrict__ order, const int32_t* __restrict__ deg_id,
                                 int32_t* __restrict__ out) {
@@ -602,10 +612,10 @@ int compute_permutation(Graph* h, uint32_t dg, int64_t g_abs, int32_t* order_out
   ks.g_abs = static_cast<uint32_t>(g_abs < 0 ? 0 : g_abs);
   ClassArgs ca{};
   if (classes) ca = *classes;
-  const int64_t chunks = class_chunks(ca.ntasks);
+  const int64_t chunks = class_chunks(ca.ntasks, kPermThreads);
   if (h->relaxed) {
     if (ca.ntasks) {
-      k_classify<<<static_cast<unsigned>(std::min<int64_t>(chunks, int64_t(h->num_sms) * 8)), kClassThreads, 0, s>>>(ca);
+      k_classify<<<static_cast<unsigned>(std::min<int64_t>(chunks, int64_t(h->num_sms) * 8)), kPermThreads, 0, s>>>(ca);
       CB_CUDA(h, cudaGetLastError());
       ++h->launches;
     }
@@ -632,9 +642,10 @@ int compute_permutation(Graph* h, uint32_t dg, int64_t g_abs, int32_t* order_out
   const int cap = bucket_cap_of(h);
   const PermOut out{order_out, pos_out, rp_out, h->deg_id, rp_out ? h->chunk_row : nullptr};
   if (nb <= kRescanBuckets && rescan_work(h) <= kRescanWork) {
-    const unsigned grid = static_cast<unsigned>(nb + std::min<int64_t>(chunks, int64_t(h->num_sms) * 4));
-    k_perm_rescan<<<grid, kPermThreads, bucket_smem_bytes(cap), s>>>(n, h->nseg, ks, static_cast<int>(nb), cap, out,
-                                                                    h->rp_id, h->nnz, ca);
+    const unsigned grid = static_cast<unsigned>(
+        nb + std::min<int64_t>(class_chunks(ca.ntasks, kRescanThreads), int64_t(h->num_sms) * 2));
+    k_perm_rescan<<<grid, kRescanThreads, bucket_smem_bytes(cap), s>>>(n, h->nseg, ks, static_cast<int>(nb), cap, out,
+                                                                      h->rp_id, h->nnz, ca);
     CB_CUDA(h, cudaGetLastError());
     ++h->launches;
     return CB_OK;
@@ -718,7 +729,7 @@ extern "C" int cb_permutation_static(int64_t n, uint64_t seed, uint64_t g, int32
   const int cap = static_cast<int>(std::min<int64_t>(space, 2048));
   const ClassArgs none{};
   if (n * nb <= kRescanWork) {   // no scratch at all
-    k_perm_rescan<<<nb, kPermThreads, bucket_smem_bytes(cap), s>>>(n, 1, ks, nb, cap, out, nullptr, 0, none);
+    k_perm_rescan<<<nb, kRescanThreads, bucket_smem_bytes(cap), s>>>(n, 1, ks, nb, cap, out, nullptr, 0, none);
     if ((e = cudaGetLastError()) != cudaSuccess) return cuda_fail(nullptr, e, "k_perm_rescan");
     return CB_OK;
   }
