@@ -195,6 +195,32 @@ int cuda_fail(Graph* g, cudaError_t e, const char* what);
     if (e_ != cudaSuccess) return ::cb::cuda_fail((g), e_, #call); \
   } while (0)
 
+// Overlapped launches (programmatic dependent launch): a kernel launched with
+// overlap = true may be set up while the kernel before it in the stream still
+// runs, so its launch costs no idle time; its first statement has to be
+// after_previous(), which waits until that kernel has finished and its writes
+// are visible.  Kernels that call before_next() let their successor be set up
+// as soon as all their CTAs have started.  Without overlap both do nothing.
+#ifdef __CUDACC__
+__device__ __forceinline__ void after_previous() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void before_next() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+template <class... P, class... A>
+cudaError_t launch(bool overlap, void (*kernel)(P...), unsigned grid, unsigned block, size_t smem, cudaStream_t s,
+                   A... args) {
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = dim3(grid);
+  cfg.blockDim = dim3(block);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = s;
+  cfg.attrs = attr;
+  cfg.numAttrs = overlap ? 1 : 0;
+  return cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);
+}
+#endif
+
 // ---- kernels / host launchers implemented in the .cu files ----
 // scan.cu
 size_t scan_ws_bytes(int64_t n);
@@ -252,6 +278,7 @@ int init_trade_kernels(Graph* h);   // one-time kernel attributes (outside strea
 int init_perm_kernels(Graph* h);
 size_t trade_ws_slice_bytes(int64_t max_trade);
 int retry_passes_of(const Graph* h);   // retry passes a super step launches
+bool small_handle(const Graph* h);     // launch-bound: its super steps use overlapped launches
 
 // api.cu
 // stream-ordered device allocation counted in the handle's device bytes

@@ -366,6 +366,8 @@ constexpr int kRescanThreads = 1024;
 __global__ void __launch_bounds__(kRescanThreads) k_perm_rescan(int64_t n, int nseg, KeySrc ks, int nb, int cap,
                                                                PermOut out, const int64_t* __restrict__ rp_id,
                                                                int64_t nnz, ClassArgs ca) {
+  after_previous();
+  before_next();
   extern __shared__ uint64_t shk[];
   __shared__ int cnt;
   __shared__ int64_t wsum[kRescanThreads / 32];
@@ -428,6 +430,8 @@ __global__ void __launch_bounds__(kPermThreads) k_perm_scatter(int64_t n, KeySrc
                                                               unsigned long long* __restrict__ words,
                                                               uint64_t* __restrict__ prefix, int* __restrict__ ticket,
                                                               int32_t* __restrict__ bid, ClassArgs ca) {
+  after_previous();
+  before_next();
   __shared__ int64_t wsum[kPermThreads / 32];
   __shared__ int last;
   classify<kPermThreads>(ca, blockIdx.x, gridDim.x);
@@ -481,6 +485,8 @@ __global__ void __launch_bounds__(kPermThreads) k_bucket_sort(int64_t n, int nse
                                                              const uint64_t* __restrict__ prefix,
                                                              const int32_t* __restrict__ bid, PermOut out,
                                                              int64_t nnz) {
+  after_previous();
+  before_next();
   extern __shared__ uint64_t shk[];
   const BucketWs w = bucket_ws(shk, cap);
   if (blockIdx.x == 0 && threadIdx.x == 0 && out.rp) put_rows_end(out, n, nnz);
@@ -644,20 +650,17 @@ int compute_permutation(Graph* h, uint32_t dg, int64_t g_abs, int32_t* order_out
   if (nb <= kRescanBuckets && rescan_work(h) <= kRescanWork) {
     const unsigned grid = static_cast<unsigned>(
         nb + std::min<int64_t>(class_chunks(ca.ntasks, kRescanThreads), int64_t(h->num_sms) * 2));
-    k_perm_rescan<<<grid, kRescanThreads, bucket_smem_bytes(cap), s>>>(n, h->nseg, ks, static_cast<int>(nb), cap, out,
-                                                                      h->rp_id, h->nnz, ca);
-    CB_CUDA(h, cudaGetLastError());
+    CB_CUDA(h, launch(small_handle(h), k_perm_rescan, grid, kRescanThreads, bucket_smem_bytes(cap), s, n, h->nseg, ks,
+                      static_cast<int>(nb), cap, out, h->rp_id, h->nnz, ca));
     ++h->launches;
     return CB_OK;
   }
   const PermWs w = carve(h->sort_ws, nb);
-  k_perm_scatter<<<grid_for(n, kPermThreads, h->num_sms), kPermThreads, 0, s>>>(
-      n, ks, static_cast<int>(nb), rp_out ? h->deg_id : nullptr, w.words, w.prefix, w.ticket, w.bid, ca);
-  CB_CUDA(h, cudaGetLastError());
+  CB_CUDA(h, launch(small_handle(h), k_perm_scatter, grid_for(n, kPermThreads, h->num_sms), kPermThreads, 0, s, n, ks,
+                    static_cast<int>(nb), rp_out ? h->deg_id : nullptr, w.words, w.prefix, w.ticket, w.bid, ca));
   const unsigned sgrid = static_cast<unsigned>(nb < h->num_sms * 8 ? nb : h->num_sms * 8);
-  k_bucket_sort<<<sgrid, kPermThreads, bucket_smem_bytes(cap), s>>>(n, h->nseg, ks, static_cast<int>(nb), cap, w.prefix,
-                                                                   w.bid, out, h->nnz);
-  CB_CUDA(h, cudaGetLastError());
+  CB_CUDA(h, launch(small_handle(h), k_bucket_sort, sgrid, kPermThreads, bucket_smem_bytes(cap), s, n, h->nseg, ks,
+                    static_cast<int>(nb), cap, w.prefix, w.bid, out, h->nnz));
   h->launches += 2;
   return CB_OK;
 }

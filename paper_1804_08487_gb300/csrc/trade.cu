@@ -1464,6 +1464,8 @@ template <int K, bool kOneSeed>
 __global__ void __launch_bounds__(K < 6 ? 256 : kBigThreads, K < 6 ? 4 : 1) k_phase_a_class(StepCtx c,
                                                                 const int32_t* __restrict__ lists,
                                                                 const int64_t* __restrict__ ctr) {
+  after_previous();
+  before_next();
   extern __shared__ __align__(16) char smem[];
   __shared__ int64_t red[K < 3 ? 1 : K < 6 ? 4 * SubTeam<64>::kRedSlots : SubTeam<kBigThreads>::kRedSlots];
   Rounds rs;
@@ -1491,6 +1493,8 @@ constexpr size_t small_smem() {
 template <bool kOneSeed>
 __global__ void __launch_bounds__(256, 4) k_phase_a_small(StepCtx c, const int32_t* __restrict__ lists,
                                                         const int64_t* __restrict__ ctr, int what) {
+  after_previous();
+  before_next();
   extern __shared__ __align__(16) char smem[];
   __shared__ int64_t red[4 * SubTeam<64>::kRedSlots];
   static_assert(4 * SubTeam<64>::kRedSlots >= SubTeam<256>::kRedSlots && 4 * SubTeam<64>::kRedSlots >= 2 * SubTeam<128>::kRedSlots, "");
@@ -1518,6 +1522,8 @@ constexpr size_t kLargeSmem = 2 * TeamCfg<512>::Ws::kBytes > TeamCfg<kBigThreads
 template <bool kOneSeed>
 __global__ void __launch_bounds__(kBigThreads, 1) k_phase_a_large(StepCtx c, const int32_t* __restrict__ lists,
                                                                 const int64_t* __restrict__ ctr) {
+  after_previous();
+  before_next();
   extern __shared__ __align__(16) char smem[];
   __shared__ int64_t red[SubTeam<kBigThreads>::kRedSlots];
   Rounds rs;
@@ -1681,6 +1687,8 @@ template <bool kNarrow, bool kLast>
 __global__ void __launch_bounds__(kFixThreads, 4) k_fixup(StepCtx c, int64_t nnz, uint32_t s_lo, uint32_t s_hi,
                                                        int32_t* __restrict__ ph, const uint16_t* __restrict__ fb,
                                                        int32_t* __restrict__ out, StepEnd end) {
+  after_previous();
+  before_next();
   __shared__ int64_t qe[kFixQueue];
   __shared__ int qn;
   if (threadIdx.x == 0) qn = 0;
@@ -1770,6 +1778,8 @@ template <int NT, bool kOneSeed>
 __global__ void __launch_bounds__(NT, NT == 256 ? 4 : 1) k_phase_a_block(StepCtx c, const int32_t* __restrict__ lists,
                                                       const int64_t* __restrict__ ctr, int cls, int smem_max,
                                                       char* gws, size_t slice, int stage_cap) {
+  after_previous();
+  before_next();
   // dynamic shared memory: the workspace, then the staging buffer of a
   // trade's entries (stage_cap + 8 int32, 16-byte aligned)
   extern __shared__ __align__(16) char sbuf[];
@@ -1933,6 +1943,8 @@ __global__ void __launch_bounds__(kDefListThreads) k_def_list(StepCtx c, int64_t
                                                              int32_t* __restrict__ list,
                                                              int32_t* __restrict__ chunk_first,
                                                              unsigned long long* __restrict__ nchunks) {
+  after_previous();
+  before_next();
   __shared__ int64_t red[BlockTeam<kDefListThreads>::kRedSlots];
   const int64_t n0 = static_cast<int64_t>(c.def_n[0]);
   const int64_t total = n0 + static_cast<int64_t>(c.def_n[1] + c.def_n[2]);
@@ -1997,6 +2009,8 @@ __global__ void __launch_bounds__(NT, NT == 256 ? 4 : 1) k_resolve(StepCtx c, co
                                                                 const unsigned long long* __restrict__ nchunks,
                                                                 unsigned long long* claim, int gen_max, char* gws,
                                                                 size_t slice) {
+  after_previous();
+  before_next();
   using Ws256 = typename TeamCfg<256>::Ws;
   constexpr int kWarps = NT / 32, kTeams = NT / 256;
   extern __shared__ __align__(16) char sbuf[];
@@ -2150,6 +2164,11 @@ int fix_passes(const Graph* h) {
 // Retry passes run where many trades are deferred at once; below kRetryMin
 // trades the in-order pass alone is faster.
 constexpr int64_t kRetryMin = int64_t(1) << 20;
+// Overlapped launches: step time without -> with, n=2^12 88 -> 80 us, 2^14 166
+// -> 160, 2^15 187 -> 184, but 2^16 214 -> 219 and 2^18 436 -> 543 (waiting CTAs
+// take the place of running ones).
+constexpr int64_t kOverlapMax = int64_t(1) << 15;
+bool small_handle(const Graph* h) { return h->ntasks < kOverlapMax; }
 int retry_passes_of(const Graph* h) { return h->ntasks >= kRetryMin ? h->retry_passes : 0; }
 
 int super_step(Graph* h) {
@@ -2265,7 +2284,7 @@ int super_step(Graph* h) {
   // whose dependency has not published yet is deferred.  With "timing" on,
   // events ev[4] .. ev[13] bracket the classes' kernels.
   const int64_t max_trade = 2 * h->maxdeg;
-  const bool fused = ntasks < kFuseMax;
+  const bool fused = ntasks < kFuseMax, overlap = small_handle(h);
   auto mark = [&](int k) -> int {
     if (h->timing) CB_CUDA(h, cudaEventRecord(ev[4 + k], s));
     return CB_OK;
@@ -2281,13 +2300,13 @@ int super_step(Graph* h) {
       if ((rk = mark(K))) return rk;
       if ((K > 0 && max_trade <= th.th[K > 0 ? K - 1 : 0]) || (K < 2 && !h->lane_teams)) return CB_OK;
       const unsigned grid = K < 3 ? wgrid : K < 6 ? mgrid : static_cast<unsigned>(h->num_sms);
-      k_phase_a_class<K, kOne><<<grid, K < 6 ? 256 : kBigThreads, class_smem<K>(), s>>>(c, L, cnt);
+      CB_CUDA(h, launch(overlap, k_phase_a_class<K, kOne>, grid, K < 6 ? 256 : kBigThreads, class_smem<K>(), s, c, L, cnt));
       return launched();
     };
     if (fused) {
       if ((r = mark(0))) return r;
-      k_phase_a_small<kOne><<<small_grid, 256, small_smem(), s>>>(
-          c, L, cnt, (h->lane_teams ? kRunLanes : 0) | (h->cta_paths ? kRunTeams : 0));
+      CB_CUDA(h, launch(overlap, k_phase_a_small<kOne>, small_grid, 256, small_smem(), s, c, L, cnt,
+                        (h->lane_teams ? kRunLanes : 0) | (h->cta_paths ? kRunTeams : 0)));
       if ((r = launched())) return r;
       for (int k = 1; k < 6; ++k)
         if ((r = mark(k))) return r;
@@ -2304,7 +2323,7 @@ int super_step(Graph* h) {
     } else if (fused) {
       if ((r = mark(6))) return r;
       if (max_trade > th.th[5]) {
-        k_phase_a_large<kOne><<<large_grid, kBigThreads, kLargeSmem, s>>>(c, L, cnt);
+        CB_CUDA(h, launch(overlap, k_phase_a_large<kOne>, large_grid, kBigThreads, kLargeSmem, s, c, L, cnt));
         if ((r = launched())) return r;
       }
       if ((r = mark(7))) return r;
@@ -2315,8 +2334,8 @@ int super_step(Graph* h) {
     // the largest trades: 1024 threads, up to smem_max entries in shared
     // memory (staged by a bulk copy), a global-memory slice above
     if (max_trade > th.th[7]) {
-      k_phase_a_block<kBigThreads, kOne><<<bgrid, kBigThreads, big_smem_st, s>>>(c, L, cnt, 8, h->smem_max, gws,
-                                                                                h->ws_slice, h->smem_max);
+      CB_CUDA(h, launch(overlap, k_phase_a_block<kBigThreads, kOne>, bgrid, kBigThreads, big_smem_st, s, c, L, cnt, 8,
+                        h->smem_max, gws, h->ws_slice, h->smem_max));
       if ((r = launched())) return r;
     }
     return mark(9);
@@ -2357,15 +2376,15 @@ int super_step(Graph* h) {
     const int nsegs = static_cast<int>((nwords + seg_words - 1) / seg_words);
     int32_t* list = h->def_list;
     int32_t* chunk_first = h->def_list + ntasks;
-    k_def_list<<<nsegs, kDefListThreads, 0, s>>>(c, nwords, nsegs, static_cast<int>(grid), list, chunk_first,
-                                                ucnt + kCtrChunks);
+    CB_CUDA(h, launch(overlap, k_def_list, nsegs, kDefListThreads, 0, s, c, nwords, nsegs, static_cast<int>(grid), list,
+                      chunk_first, ucnt + kCtrChunks));
     if ((rc = launched())) return rc;
     if (big)
-      k_resolve<kBigThreads><<<grid, kBigThreads, resolve_smem<kBigThreads>(h->smem_max), s>>>(
-          c, list, chunk_first, ucnt + kCtrChunks, ucnt + kCtrFinished, h->smem_max, gws, h->ws_slice);
+      CB_CUDA(h, launch(overlap, k_resolve<kBigThreads>, grid, kBigThreads, resolve_smem<kBigThreads>(h->smem_max), s, c,
+                        list, chunk_first, ucnt + kCtrChunks, ucnt + kCtrFinished, h->smem_max, gws, h->ws_slice));
     else
-      k_resolve<kMedThreads><<<grid, kMedThreads, resolve_smem<kMedThreads>(block_max), s>>>(
-          c, list, chunk_first, ucnt + kCtrChunks, ucnt + kCtrFinished, block_max, gws, h->ws_slice);
+      CB_CUDA(h, launch(overlap, k_resolve<kMedThreads>, grid, kMedThreads, resolve_smem<kMedThreads>(block_max), s, c,
+                        list, chunk_first, ucnt + kCtrChunks, ucnt + kCtrFinished, block_max, gws, h->ws_slice));
     if ((rc = launched())) return rc;
   }
   if (h->timing) CB_CUDA(h, cudaEventRecord(ev[2], s));
@@ -2385,7 +2404,7 @@ int super_step(Graph* h) {
       const bool last = q == passes - 1;
       auto fk = c.narrow ? (last ? k_fixup<true, true> : k_fixup<true, false>)
                          : (last ? k_fixup<false, true> : k_fixup<false, false>);
-      fk<<<fgrid, kFixThreads, 0, s>>>(c, nnz, lo, hi, c.ph, c.fb, out, end);
+      CB_CUDA(h, launch(overlap, fk, fgrid, kFixThreads, 0, s, c, nnz, lo, hi, c.ph, c.fb, out, end));
       if ((rc = launched())) return rc;
     }
     std::swap(h->col[0], h->col[1]);   // the step's output is now the other side of the ping-pong
