@@ -2,7 +2,8 @@
 // device, and the successor lists Suc of a trade sequence (Section 4.1).
 //
 // The sequence runs as a dataflow in the manner of EM-CB / IM-CB (Sections
-// 4.1-4.2), in the position space of the handle's current super step:
+// 4.1-4.2) on node ids (a trade's keys are functions of ids); the input rows
+// and the output are in the position space of the handle's current super step:
 //   - Suc gives, for every (trade, endpoint), the endpoint's next trade, and
 //     for every node its first trade.
 //   - Every edge waits in an inbox of the next trade of either endpoint:
@@ -11,7 +12,9 @@
 //     Trade k's inbox for node x has deg(x) slots, reserved by one 64-bit
 //     atomic per entry (both sides' counts packed).
 //   - The reservation that fills the last slot queues the trade.
-//   - Persistent CTAs take queued trades in queue order. Each one:
+//   - Persistent CTAs take queued trades in queue order: trades of at most
+//     128 (or 64) entries one per warp, larger ones on a team of three quarters
+//     of the CTA's threads.  Each trade:
 //       - gathers both inboxes, waiting (bounded) for entries still being
 //         written;
 //       - finds the common and disjoint neighbours through a hash of u's
@@ -38,17 +41,18 @@ namespace cb {
 struct UniBufs {
   int64_t cap_trades = 0;      // trades per chunk the buffers hold
   int64_t n = 0;
-  int32_t* tp = nullptr;       // 2L: positions of u_i (even) and v_i (odd)
-  int32_t* dslot = nullptr;    // 2L: degree of each slot's node (scan input)
+  int32_t* tp = nullptr;       // 2L: u_i (even) and v_i (odd)
+  int32_t* dslot = nullptr;    // 2L: degree of each slot's node
   int64_t* ib = nullptr;       // 2L+1: first inbox entry of each slot
   int32_t* suc = nullptr;      // 2L: slot ids grouped by node, increasing
-  int32_t* nxt = nullptr;      // 2L: next trade of the slot's node after its trade
+  int32_t* nxt = nullptr;      // 2L: next slot of the slot's node
   unsigned long long* fill = nullptr;   // L: inbox counts (side 0 low, side 1 high)
   int32_t* queue = nullptr;    // L: runnable trades; small ones from the front, big ones from the back
   int32_t* occ = nullptr;      // n: occurrences, then fill cursors
+  int32_t* first = nullptr;    // n: first slot of the node at each position
   int64_t* sbeg = nullptr;     // n+1: Suc offsets
   int32_t* ocur = nullptr;     // n: output row cursors
-  unsigned long long* ctr = nullptr;   // run queue head and tail, a cache line apart
+  unsigned long long* ctr = nullptr;   // heads and tails of the two run queues, a cache line apart
   void* scan_ws = nullptr;
   int2* inbox = nullptr;
   int64_t inbox_cap = 0;
@@ -60,12 +64,30 @@ struct UniBufs {
 
 namespace {
 
-constexpr int32_t kInf = 0x7fffffff;            // no further trade
-// Executor CTAs of NT = 256 (two per SM), 512 or 1024 threads (option
-// "uniform_threads"): larger CTAs give a hub trade more threads but keep
-// fewer trades running at once.
+// "Next trade" of a node is its slot there, 2 trade + side, so that a message
+// knows its side without a look at the trade; kInf: no further trade.
+constexpr int32_t kInf = 0x7fffffff;
+__device__ __forceinline__ int32_t trade_of(int32_t slot) { return slot == kInf ? kInf : slot >> 1; }
+// Executor CTAs of NT = 256, 512 or 1024 threads (option "uniform_threads"):
+// three quarters of them are one team for large trades, the other warps take the small trades one each, and so do the
+// team's warps once the large trades are all taken.  Every CTA serves both
+// queues, so whichever CTAs are resident finish the sequence.  A larger team
+// makes the hub trades on the critical chain shorter.
 template <int NT>
-constexpr int uni_smem_elems() { return NT == 1024 ? 4096 : 2048; }   // trades up to this many entries in shared memory
+__host__ __device__ constexpr int uni_team() { return NT / 4 * 3; }
+template <int NT>
+__host__ __device__ constexpr int uni_warps() { return NT / 128; }
+template <int NT>
+__host__ __device__ constexpr int uni_smem_elems() { return NT == 1024 ? 4096 : 2048; }   // trades up to this many entries in shared memory
+// Small trades have at most kUniSmall entries (four per lane of a warp), in
+// chunks of at most kUniFewMax trades half as many: there the chain of
+// dependent trades bounds the time, and a team finishes a trade of 65 to 128
+// entries sooner than a warp; in longer chunks the teams are too few for them.
+// 64 against 128 entries: n=2^14 0.54 and 0.74 ms, 2^17 2.03 and 2.10, 2^20
+// 11.0 and 10.2 (n/2 trades each).
+constexpr int kUniSmall = 128;
+constexpr int64_t kUniFewMax = 65536;
+inline int uni_small(int64_t trades) { return trades <= kUniFewMax ? kUniSmall / 2 : kUniSmall; }
 constexpr int64_t kUniChunkMin = 65536;
 
 __device__ __forceinline__ void latch(int32_t* err, int32_t code) { atomicCAS(err, 0, code); }
@@ -112,23 +134,30 @@ __device__ __forceinline__ void uniform_pair(uint64_t seed, int64_t n, uint64_t 
   *v = static_cast<int32_t>(w + (w >= a));
 }
 
-// pairs of trades first..first+count-1; mapped through pos (node id ->
-// position) when given; with rp, each slot's degree goes to dslot.
-__global__ void k_uni_draw(int64_t count, uint64_t first, uint64_t seed, int64_t n, const int32_t* __restrict__ pos,
-                           const int64_t* __restrict__ rp, int32_t* __restrict__ out, int32_t* __restrict__ dslot) {
+// pairs of trades first..first+count-1; with the nodes' degrees, each slot's
+// goes to dslot, its node's occurrences are counted and *big counts trades of
+// more than small entries.
+__global__ void k_uni_draw(int64_t count, uint64_t first, uint64_t seed, int64_t n, const int32_t* __restrict__ deg,
+                           int32_t* __restrict__ out, int32_t* __restrict__ dslot,
+                           int32_t* __restrict__ occ, int small, unsigned long long* __restrict__ big) {
+  int large = 0;
   for (int64_t i = blockIdx.x * int64_t(blockDim.x) + threadIdx.x; i < count; i += int64_t(gridDim.x) * blockDim.x) {
     int32_t u, v;
     uniform_pair(seed, n, first + static_cast<uint64_t>(i), &u, &v);
-    if (pos) {
-      u = pos[u];
-      v = pos[v];
-    }
     out[2 * i] = u;
     out[2 * i + 1] = v;
     if (dslot) {
-      dslot[2 * i] = static_cast<int32_t>(rp[u + 1] - rp[u]);
-      dslot[2 * i + 1] = static_cast<int32_t>(rp[v + 1] - rp[v]);
+      const int32_t du = deg[u], dv = deg[v];
+      dslot[2 * i] = du;
+      dslot[2 * i + 1] = dv;
+      large += int64_t(du) + dv > small;
+      atomicAdd(&occ[u], 1);
+      atomicAdd(&occ[v], 1);
     }
+  }
+  if (dslot) {
+    large = __reduce_add_sync(kFull, large);
+    if ((threadIdx.x & 31) == 0 && large) atomicAdd(big, static_cast<unsigned long long>(large));
   }
 }
 
@@ -157,9 +186,10 @@ __global__ void k_uni_fill(int64_t slots, const int32_t* __restrict__ tp, const 
 }
 
 // Each node's slot list in increasing order (a node is in a trade at most
-// once, so slot order is trade order); with nxt, every slot's next trade.
+// once, so slot order is trade order); with nxt, every slot's next slot and
+// every node's first one at its position.
 __global__ void k_uni_sort(int64_t n, const int64_t* __restrict__ sbeg, int32_t* __restrict__ suc,
-                           int32_t* __restrict__ nxt) {
+                           int32_t* __restrict__ nxt, const int32_t* __restrict__ pos, int32_t* __restrict__ first) {
   for (int64_t x = blockIdx.x * int64_t(blockDim.x) + threadIdx.x; x < n; x += int64_t(gridDim.x) * blockDim.x) {
     const int64_t b = sbeg[x], e = sbeg[x + 1];
     for (int64_t i = b + 1; i < e; ++i) {   // lists are short: Poisson(2L/n) long
@@ -171,8 +201,10 @@ __global__ void k_uni_sort(int64_t n, const int64_t* __restrict__ sbeg, int32_t*
       }
       suc[j + 1] = key;
     }
-    if (nxt)
-      for (int64_t i = b; i < e; ++i) nxt[suc[i]] = (i + 1 < e) ? (suc[i + 1] >> 1) : kInf;
+    if (nxt) {
+      first[pos[x]] = b < e ? suc[b] : kInf;
+      for (int64_t i = b; i < e; ++i) nxt[suc[i]] = (i + 1 < e) ? suc[i + 1] : kInf;
+    }
   }
 }
 
@@ -188,12 +220,13 @@ struct UniCtx {
   uint64_t first;            // global index of the chunk's first trade
   uint64_t seed;
   const int64_t* rp;         // position-space row offsets (degrees never change)
-  const int32_t* order;      // node id at each position (keys use ids)
+  const int32_t* order;      // node id at each position
+  const int32_t* pos;        // position of each node id
   const int32_t* tp;
+  const int32_t* dslot;
   const int32_t* nxt;
   const int64_t* ib;
-  const int64_t* sbeg;
-  const int32_t* suc;
+  const int32_t* first_slot;   // of the node at each position
   int2* inbox;
   unsigned long long* fill;
   int32_t* queue;
@@ -205,33 +238,48 @@ struct UniCtx {
   int64_t slice_elems;
   unsigned long long* swaps;   // (performed, possible) swap counts, or null
   uint64_t wait_ns;            // longest single wait (run queue, inbox entry)
+  int small;                   // entries of the largest small trade, at most kUniSmall
   int64_t hold_trade;          // test hook: messages to this trade of the chunk are dropped (-1: none)
 };
 
-// The run queue: a ticket (kHead) takes the next slot, a push (kTail)
-// fills the next slot; the two counters sit on different cache lines.
-// Every trade is queued exactly once, so every ticket below L ends.
-constexpr int kHead = 0, kTail = 16, kCtrWords = 32;
+// The two run queues, small trades from the front of the array and large ones
+// from its back: a ticket (kHead) takes the queue's next place, a push (kTail)
+// fills the next place; the counters sit on different cache lines.  Every
+// trade is queued exactly once and kBig says how many are large, so every
+// ticket below a queue's length ends.
+constexpr int kHead = 0, kTail = 16, kQueueCtr = 32, kBig = 64, kCtrWords = 80;
 
-__device__ __forceinline__ void push(const UniCtx& c, int64_t k) {
-  const unsigned long long q = atomicAdd(&c.ctr[kTail], 1ull);
+__device__ __forceinline__ int64_t queue_len(const UniCtx& c, int big) {
+  const int64_t nb = static_cast<int64_t>(c.ctr[kBig]);
+  return big ? nb : c.L - nb;
+}
+
+__device__ __forceinline__ int32_t* queue_at(const UniCtx& c, int big, unsigned long long q) {
+  return c.queue + (big ? c.L - 1 - static_cast<int64_t>(q) : static_cast<int64_t>(q));
+}
+
+__device__ __forceinline__ void push(const UniCtx& c, int64_t k, int64_t entries) {
+  const int big = entries > c.small;
+  const unsigned long long q = atomicAdd(&c.ctr[kQueueCtr * big + kTail], 1ull);
   if (q >= static_cast<unsigned long long>(c.L)) {
     latch(c.err, kErrUniform);
     return;
   }
-  st_relaxed_i32(c.queue + q, static_cast<int32_t>(k));
+  st_relaxed_i32(queue_at(c, big, q), static_cast<int32_t>(k));
 }
 
-// The next queued trade, or -1 when every slot is taken or a wait gave up.
-__device__ int64_t take_ticket(const UniCtx& c) {
-  const unsigned long long q = atomicAdd(&c.ctr[kHead], 1ull);
-  if (q >= static_cast<unsigned long long>(c.L)) return -1;
-  int32_t t = ld_relaxed_i32(c.queue + q);
+// The next queued trade, or -1 when every place of the queue (of len trades)
+// is taken or a wait gave up.
+__device__ int64_t take_ticket(const UniCtx& c, int big, int64_t len) {
+  const unsigned long long q = atomicAdd(&c.ctr[kQueueCtr * big + kHead], 1ull);
+  if (q >= static_cast<unsigned long long>(len)) return -1;
+  const int32_t* place = queue_at(c, big, q);
+  int32_t t = ld_relaxed_i32(place);
   if (t < 0) {
     const uint64_t t0 = globaltimer();
     for (;;) {
       __nanosleep(200);
-      t = ld_relaxed_i32(c.queue + q);
+      t = ld_relaxed_i32(place);
       if (t >= 0) break;
       if (ld_volatile_i32(c.err) != 0) return -1;
       if (globaltimer() - t0 > c.wait_ns) {
@@ -243,56 +291,71 @@ __device__ int64_t take_ticket(const UniCtx& c) {
   return t;
 }
 
-// Append (other, other_tau) to node x's inbox at trade d.
-__device__ void append(const UniCtx& c, int32_t d, int32_t x, int32_t other, int32_t other_tau) {
-  if (d == c.hold_trade) return;   // test hook: the trade never becomes runnable
-  const int32_t a = c.tp[2 * int64_t(d)], b = c.tp[2 * int64_t(d) + 1];
-  const int side = (x == a) ? 0 : 1;
-  if (x != a && x != b) {
+// One message: the edge {a, b} with a's next slot ta and b's next slot tb, to
+// the earlier of the two trades (both inboxes when they are the same trade),
+// or out.  reserve() takes the places (one atomic per message) and loads what
+// deliver(), which writes them, needs of the destination.
+struct Msg {
+  int32_t a, ta, b, tb, d;
+  unsigned long long old;   // previous inbox counts of trade d, or the two row cursors
+  int64_t ib;
+  int2 deg;                 // the destination's degrees, or the positions of a and b
+};
+
+__device__ __forceinline__ unsigned long long msg_inc(const Msg& m) {
+  unsigned long long inc = 0;
+  if (trade_of(m.ta) == m.d) inc += (m.ta & 1) ? (1ull << 32) : 1ull;
+  if (trade_of(m.tb) == m.d) inc += (m.tb & 1) ? (1ull << 32) : 1ull;
+  return inc;
+}
+
+__device__ __forceinline__ void reserve(const UniCtx& c, Msg& m) {
+  m.d = min(trade_of(m.ta), trade_of(m.tb));
+  if (m.d == kInf) {
+    m.deg = make_int2(c.pos[m.a], c.pos[m.b]);
+    const uint32_t sa = static_cast<uint32_t>(atomicAdd(&c.ocur[m.deg.x], 1));
+    const uint32_t sb = static_cast<uint32_t>(atomicAdd(&c.ocur[m.deg.y], 1));
+    m.old = (static_cast<unsigned long long>(sb) << 32) | sa;
+    return;
+  }
+  m.old = atomicAdd(&c.fill[m.d], msg_inc(m));
+  m.ib = c.ib[2 * int64_t(m.d)];
+  m.deg = reinterpret_cast<const int2*>(c.dslot)[m.d];
+}
+
+// places s0, s1: the entry's place on its side of trade d
+__device__ __forceinline__ void put_entry(const UniCtx& c, const Msg& m, int side, int32_t other, int32_t other_tau) {
+  const uint32_t place = static_cast<uint32_t>(side ? m.old >> 32 : m.old);
+  if (place >= static_cast<uint32_t>(side ? m.deg.y : m.deg.x)) {
     latch(c.err, kErrUniform);
     return;
   }
-  const uint64_t du = static_cast<uint64_t>(c.rp[a + 1] - c.rp[a]), dv = static_cast<uint64_t>(c.rp[b + 1] - c.rp[b]);
-  const unsigned long long inc = side ? (1ull << 32) : 1ull;
-  const unsigned long long old = atomicAdd(&c.fill[d], inc);
-  const uint64_t slot = side ? (old >> 32) : (old & 0xffffffffull);
-  if (slot >= (side ? dv : du)) {
-    latch(c.err, kErrUniform);
+  st_relaxed_v2(c.inbox + m.ib + (side ? m.deg.x : 0) + place, other, other_tau);
+}
+
+__device__ __forceinline__ void deliver(const UniCtx& c, const Msg& m) {
+  if (m.d == kInf) {
+    const int32_t pa = m.deg.x, pb = m.deg.y;
+    const int64_t ba = c.rp[pa], bb = c.rp[pb];
+    const uint32_t sa = static_cast<uint32_t>(m.old), sb = static_cast<uint32_t>(m.old >> 32);
+    if (sa < c.rp[pa + 1] - ba) c.col_out[ba + sa] = pb;
+    else latch(c.err, kErrRowLength);
+    if (sb < c.rp[pb + 1] - bb) c.col_out[bb + sb] = pa;
+    else latch(c.err, kErrRowLength);
     return;
   }
-  st_relaxed_v2(c.inbox + c.ib[2 * int64_t(d) + side] + slot, other, other_tau);
-  if (old + inc == ((dv << 32) | du)) push(c, d);
-}
-
-// The edge {a, b} into its rows of the output.
-__device__ void commit(const UniCtx& c, int32_t a, int32_t b) {
-  const int64_t ba = c.rp[a], bb = c.rp[b];
-  const int32_t sa = atomicAdd(&c.ocur[a], 1), sb = atomicAdd(&c.ocur[b], 1);
-  if (sa < c.rp[a + 1] - ba) c.col_out[ba + sa] = b;
-  else latch(c.err, kErrRowLength);
-  if (sb < c.rp[b + 1] - bb) c.col_out[bb + sb] = a;
-  else latch(c.err, kErrRowLength);
-}
-
-// The edge {a, b}, a's next trade ta, b's next trade tb: to the earlier of
-// the two (both inboxes when they are the same trade), or out.
-__device__ void route(const UniCtx& c, int32_t a, int32_t ta, int32_t b, int32_t tb) {
-  const int32_t d = min(ta, tb);
-  if (d == kInf) {
-    commit(c, a, b);
-    return;
-  }
-  if (ta == d) append(c, d, a, b, tb);
-  if (tb == d) append(c, d, b, a, ta);
-}
-
-__device__ __forceinline__ int32_t first_trade(const UniCtx& c, int32_t x) {
-  const int64_t b = c.sbeg[x];
-  return b < c.sbeg[x + 1] ? (c.suc[b] >> 1) : kInf;
+  if (trade_of(m.ta) == m.d) put_entry(c, m, m.ta & 1, m.b, m.tb);
+  if (trade_of(m.tb) == m.d) put_entry(c, m, m.tb & 1, m.a, m.ta);
+  const unsigned long long full =
+      (static_cast<unsigned long long>(static_cast<uint32_t>(m.deg.y)) << 32) | static_cast<uint32_t>(m.deg.x);
+  if (m.old + msg_inc(m) == full) push(c, m.d, int64_t(m.deg.x) + m.deg.y);
 }
 
 // Every edge of the input to the first trade of either endpoint; trades with
-// no entries to wait for are queued here.
+// no entries to wait for are queued here.  The edges of a row that go to the
+// row's own first trade take their places with one atomic per 32 of them.
+// Scattered L2 accesses bound it, about six per edge (24 million edges, n=2^20:
+// 1.05 ms).
 __global__ void k_uni_route(UniCtx c, int64_t n, const int32_t* __restrict__ col) {
   const int lane = threadIdx.x & 31;
   const int64_t gw = (blockIdx.x * int64_t(blockDim.x) + threadIdx.x) >> 5;
@@ -300,16 +363,44 @@ __global__ void k_uni_route(UniCtx c, int64_t n, const int32_t* __restrict__ col
   for (int64_t a = gw; a < n; a += nw) {
     const int64_t b0 = c.rp[a], b1 = c.rp[a + 1];
     if (b0 == b1) continue;
-    const int32_t ta = first_trade(c, static_cast<int32_t>(a));
-    for (int64_t q = b0 + lane; q < b1; q += 32) {
-      const int32_t b = col[q];
-      if (b > a) route(c, static_cast<int32_t>(a), ta, b, first_trade(c, b));
+    const int32_t ta = c.first_slot[a], da = trade_of(ta), ida = c.order[a];
+    int64_t ib = 0;
+    int2 deg = make_int2(0, 0);
+    if (da != kInf) {
+      ib = c.ib[2 * int64_t(da)];
+      deg = reinterpret_cast<const int2*>(c.dslot)[da];
+    }
+    for (int64_t q0 = b0; q0 < b1; q0 += 32) {
+      const int64_t q = q0 + lane;
+      Msg m;
+      m.a = ida;
+      m.ta = ta;
+      const int32_t pb = q < b1 ? col[q] : 0;
+      const bool has = q < b1 && pb > a;
+      m.tb = has ? c.first_slot[pb] : kInf;
+      m.b = has ? c.order[pb] : 0;
+      m.d = min(da, trade_of(m.tb));
+      const bool mine = has && da != kInf && m.d == da && trade_of(m.tb) != da && da != c.hold_trade;
+      const unsigned mm = __ballot_sync(kFull, mine);
+      if (mm) {
+        const unsigned long long one = (ta & 1) ? (1ull << 32) : 1ull;
+        unsigned long long old = 0;
+        if (lane == 0) old = atomicAdd(&c.fill[da], one * static_cast<unsigned>(__popc(mm)));
+        old = __shfl_sync(kFull, old, 0);
+        m.old = old + one * static_cast<unsigned>(__popc(mm & ((1u << lane) - 1u)));
+        m.ib = ib;
+        m.deg = deg;
+        if (mine) deliver(c, m);
+      }
+      // hold_trade is a test hook: messages to that trade are dropped, so it never becomes runnable
+      if (has && !mine && !(m.d == c.hold_trade)) {
+        reserve(c, m);
+        deliver(c, m);
+      }
     }
   }
-  for (int64_t k = blockIdx.x * int64_t(blockDim.x) + threadIdx.x; k < c.L; k += int64_t(gridDim.x) * blockDim.x) {
-    const int32_t a = c.tp[2 * k], b = c.tp[2 * k + 1];
-    if (c.rp[a + 1] == c.rp[a] && c.rp[b + 1] == c.rp[b]) push(c, k);
-  }
+  for (int64_t k = blockIdx.x * int64_t(blockDim.x) + threadIdx.x; k < c.L; k += int64_t(gridDim.x) * blockDim.x)
+    if (c.dslot[2 * k] == 0 && c.dslot[2 * k + 1] == 0) push(c, k, 0);
 }
 
 // Bounded wait for an inbox entry still being written (the cold path).
@@ -368,108 +459,55 @@ __device__ __forceinline__ uint32_t hash_slot(int32_t x, int hbits) {
   return (static_cast<uint32_t>(x) * 0x9E3779B1u) >> (32 - hbits);
 }
 
-// One message: the edge {a, b} with a's next trade ta and b's next trade tb.
-// reserve() takes the slots (one atomic per message), deliver() writes them.
-struct Msg {
-  int32_t a, ta, b, tb, d;
-  unsigned long long old;   // previous inbox counts of trade d, or the two row cursors
-};
-
-__device__ __forceinline__ void reserve(const UniCtx& c, Msg& m) {
-  m.d = min(m.ta, m.tb);
-  if (m.d == kInf) {
-    const uint32_t sa = static_cast<uint32_t>(atomicAdd(&c.ocur[m.a], 1));
-    const uint32_t sb = static_cast<uint32_t>(atomicAdd(&c.ocur[m.b], 1));
-    m.old = (static_cast<unsigned long long>(sb) << 32) | sa;
-    return;
-  }
-  const int32_t x0 = c.tp[2 * int64_t(m.d)];
-  unsigned long long inc = 0;
-  if (m.ta == m.d) inc += (m.a == x0) ? 1ull : (1ull << 32);
-  if (m.tb == m.d) inc += (m.b == x0) ? 1ull : (1ull << 32);
-  m.old = atomicAdd(&c.fill[m.d], inc);
-}
-
-__device__ void deliver_one(const UniCtx& c, int32_t d, int side, uint64_t slot, uint64_t cap, int32_t other,
-                            int32_t other_tau) {
-  if (slot >= cap) {
-    latch(c.err, kErrUniform);
-    return;
-  }
-  st_relaxed_v2(c.inbox + c.ib[2 * int64_t(d) + side] + slot, other, other_tau);
-}
-
-__device__ void deliver(const UniCtx& c, const Msg& m) {
-  if (m.d == kInf) {
-    const int64_t ba = c.rp[m.a], bb = c.rp[m.b];
-    const uint32_t sa = static_cast<uint32_t>(m.old), sb = static_cast<uint32_t>(m.old >> 32);
-    if (sa < c.rp[m.a + 1] - ba) c.col_out[ba + sa] = m.b;
-    else latch(c.err, kErrRowLength);
-    if (sb < c.rp[m.b + 1] - bb) c.col_out[bb + sb] = m.a;
-    else latch(c.err, kErrRowLength);
-    return;
-  }
-  const int64_t d = m.d;
-  const int32_t x0 = c.tp[2 * d], x1 = c.tp[2 * d + 1];
-  const uint64_t du = static_cast<uint64_t>(c.rp[x0 + 1] - c.rp[x0]), dv = static_cast<uint64_t>(c.rp[x1 + 1] - c.rp[x1]);
-  unsigned long long inc = 0;
-  const uint64_t s0 = m.old & 0xffffffffull, s1 = m.old >> 32;
-  if (m.ta == m.d) {
-    if (m.a != x0 && m.a != x1) latch(c.err, kErrUniform);
-    const int side = m.a == x0 ? 0 : 1;
-    deliver_one(c, m.d, side, side ? s1 : s0, side ? dv : du, m.b, m.tb);
-    inc += side ? (1ull << 32) : 1ull;
-  }
-  if (m.tb == m.d) {
-    if (m.b != x0 && m.b != x1) latch(c.err, kErrUniform);
-    const int side = m.b == x0 ? 0 : 1;
-    deliver_one(c, m.d, side, side ? s1 : s0, side ? dv : du, m.a, m.ta);
-    inc += side ? (1ull << 32) : 1ull;
-  }
-  if (m.old + inc == ((dv << 32) | du)) push(c, d);
-}
-
 // Elements of D with the same full key as entry e and a smaller node id
 // (ties of 64-bit keys: practically never, hence the plain loop).
-__device__ __noinline__ int tied_before(const UniCtx& c, const int2* ent, const uint64_t* key, const uint8_t* flag,
+__device__ __noinline__ int tied_before(const int2* ent, const uint64_t* key, const uint8_t* flag,
                                         int E, int e) {
-  const uint32_t id = static_cast<uint32_t>(c.order[ent[e].x]);
+  const int32_t id = ent[e].x;
   int before = 0;
   for (int q = 0; q < E; ++q)
-    if ((flag[q] & 6) == 0 && key[q] == key[e] && static_cast<uint32_t>(c.order[ent[q].x]) < id) ++before;
+    if ((flag[q] & 6) == 0 && key[q] == key[e] && ent[q].x < id) ++before;
   return before;
 }
 
-// messages per thread with their atomics in flight together (one in the
-// 1024-thread executor, whose threads have 64 registers)
-template <int NT>
-constexpr int msg_batch() { return NT == 1024 ? 1 : 2; }
+// Trade k: its nodes, their degrees, their next slots, and its inbox (u's
+// entries, then v's).  Loaded together as soon as k is known.
+struct Trade {
+  int2 uv, deg, next;
+  const int2* in;
+};
 
-// One trade by the whole CTA.  Returns false when a wait gave up.
-template <int NT, class HT>
-__device__ bool uni_trade(BlockTeam<NT>& tm, const UniCtx& c, int64_t k, const TradeWs<HT>& w, int hbits,
-                          int32_t* hist, int64_t* s_sel, int* s_abort) {
-  const int32_t u = c.tp[2 * k], v = c.tp[2 * k + 1];
-  const int du = static_cast<int>(c.rp[u + 1] - c.rp[u]), dv = static_cast<int>(c.rp[v + 1] - c.rp[v]);
-  const int32_t nu = c.nxt[2 * k], nv = c.nxt[2 * k + 1];
-  const int E = du + dv;
+__device__ __forceinline__ Trade load_trade(const UniCtx& c, int64_t k) {
+  return Trade{reinterpret_cast<const int2*>(c.tp)[k], reinterpret_cast<const int2*>(c.dslot)[k],
+               reinterpret_cast<const int2*>(c.nxt)[k], c.inbox + c.ib[2 * k]};
+}
+
+// One trade by a team.  Returns false when a wait gave up.
+template <class Team, class HT>
+__device__ bool uni_trade(Team& tm, const UniCtx& c, int64_t k, const Trade& t, const TradeWs<HT>& w, int hbits, int32_t* hist,
+                          int* s_sel, int* s_abort, unsigned long long& moved, unsigned long long& possible) {
+  constexpr int NT = Team::N;
+  const int32_t u = t.uv.x, v = t.uv.y;
+  const int du = t.deg.x, E = t.deg.x + t.deg.y;
+  const int2 next = t.next;
+  const int2* in = t.in;
   const int H = 1 << hbits;
-  const int2* inu = c.inbox + c.ib[2 * k];
-  const int2* inv = c.inbox + c.ib[2 * k + 1];
+  const uint64_t gi = c.first + static_cast<uint64_t>(k);
   // 1. gather both inboxes: plain L2 loads, and a bounded wait only for an
-  //    entry still in flight; clear the hash
+  //    entry still in flight; trade k's shuffle keys (Philox on (node id, k));
+  //    clear the hash
   bool ok = true;
 #pragma unroll 4
   for (int e = tm.rank; e < E; e += NT) {
-    const int side = e >= du;
-    const int2* p = side ? inv + (e - du) : inu + e;
-    int2 m = __ldcg(p);
-    if (m.x == -1 && !wait_entry(p, c.err, c.wait_ns, &m)) {
+    int2 m = __ldcg(in + e);
+    if (m.x == -1 && !wait_entry(in + e, c.err, c.wait_ns, &m)) {
       ok = false;
       m = make_int2(0, kInf);
     }
+    const Philox4 r = philox4x32_10(static_cast<uint32_t>(m.x), static_cast<uint32_t>(gi), static_cast<uint32_t>(gi >> 32), 6u, c.seed);
     w.ent[e] = m;
-    w.flag[e] = static_cast<uint8_t>(side);
+    w.key[e] = (static_cast<uint64_t>(r.w0) << 32) | r.w1;
+    w.flag[e] = static_cast<uint8_t>(e >= du ? (m.x == u ? 5 : 1) : (m.x == v ? 4 : 0));
   }
   for (int s = tm.rank; s < H; s += NT) w.hash[s] = 0;
   if (!ok) atomicExch(s_abort, 1);
@@ -481,38 +519,27 @@ __device__ bool uni_trade(BlockTeam<NT>& tm, const UniCtx& c, int64_t k, const T
     while (atomicCAS(&w.hash[s], HT(0), static_cast<HT>(e + 1)) != HT(0)) s = (s + 1) & (H - 1);
   }
   tm.sync();
-  // 3. v's neighbours look themselves up: common neighbours and the edge {u, v}
+  // 3. v's neighbours look themselves up: common neighbours
   for (int e = du + tm.rank; e < E; e += NT) {
     const int32_t x = w.ent[e].x;
-    uint8_t f = 1;
-    if (x == u) f |= 4;
     uint32_t s = hash_slot(x, hbits);
     for (;;) {
       const int32_t h = static_cast<int32_t>(w.hash[s]);
       if (h == 0) break;
       if (w.ent[h - 1].x == x) {
-        f |= 2;
+        w.flag[e] = 3;
         w.flag[h - 1] = 2;   // side 0, common
         break;
       }
       s = (s + 1) & (H - 1);
     }
-    w.flag[e] = f;
   }
   tm.sync();
-  // 4. D = the rest, keyed by trade k's shuffle keys (Philox on (node id, k))
-  const uint64_t gi = c.first + static_cast<uint64_t>(k);
+  // 4. D = the rest
   int64_t cnt = 0;
-#pragma unroll 4
   for (int e = tm.rank; e < E; e += NT) {
-    uint8_t f = w.flag[e];
-    if (f == 0 && w.ent[e].x == v) w.flag[e] = f = 4;
-    if ((f & 6) == 0) {
-      const uint32_t id = static_cast<uint32_t>(c.order[w.ent[e].x]);
-      const Philox4 r = philox4x32_10(id, static_cast<uint32_t>(gi), static_cast<uint32_t>(gi >> 32), 6u, c.seed);
-      w.key[e] = (static_cast<uint64_t>(r.w0) << 32) | r.w1;
-      cnt += 1 + ((f & 1) ? 0 : (int64_t(1) << 32));
-    }
+    const uint8_t f = w.flag[e];
+    if ((f & 6) == 0) cnt += 1 + ((f & 1) ? 0 : (int64_t(1) << 32));
   }
   cnt = tm.sum(cnt);
   const int nd = static_cast<int>(cnt & 0xffffffff), na = static_cast<int>(cnt >> 32);
@@ -529,16 +556,19 @@ __device__ bool uni_trade(BlockTeam<NT>& tm, const UniCtx& c, int64_t k, const T
       for (int e = tm.rank; e < E; e += NT)
         if ((w.flag[e] & 6) == 0 && (w.key[e] & mask) == prefix) atomicAdd(&hist[(w.key[e] >> shift) & 255], 1);
       tm.sync();
-      const int hb = tm.rank < 256 ? hist[tm.rank] : 0;
-      const int64_t below = tm.exscan(hb);
-      if (tm.rank < 256 && below < r && r <= below + hb) {
-        s_sel[0] = tm.rank;
-        s_sel[1] = hb;
-        s_sel[2] = below;
+      // two bins to each of the first 128 threads
+      const bool bins = tm.rank < 128;
+      const int h0 = bins ? hist[2 * tm.rank] : 0, h1 = bins ? hist[2 * tm.rank + 1] : 0;
+      const int below = static_cast<int>(tm.exscan32(static_cast<uint32_t>(h0 + h1)));
+      if (bins && below < r && r <= below + h0 + h1) {
+        const int hi = r > below + h0;
+        s_sel[0] = 2 * tm.rank + hi;
+        s_sel[1] = hi ? h1 : h0;
+        s_sel[2] = hi ? below + h0 : below;
       }
       tm.sync();
-      const int b = static_cast<int>(s_sel[0]), size = static_cast<int>(s_sel[1]);
-      r -= static_cast<int>(s_sel[2]);
+      const int b = s_sel[0], size = s_sel[1];
+      r -= s_sel[2];
       prefix |= static_cast<uint64_t>(b) << shift;
       mask |= uint64_t(255) << shift;
       if (size == 1) break;
@@ -548,109 +578,268 @@ __device__ bool uni_trade(BlockTeam<NT>& tm, const UniCtx& c, int64_t k, const T
       }
     }
   }
-  // decision: below the threshold's bucket to u, above to v, within it by rank
-  int moved = 0;
-#pragma unroll 2
+  // 6. every resulting edge goes on: common neighbours and the edge {u, v}
+  //    stay, an element of D below the threshold's bucket goes to u, above it
+  //    to v, within it by rank.  One message at a time: two to four in flight
+  //    cost registers and took 8 to 22 % longer.
   for (int e = tm.rank; e < E; e += NT) {
     const uint8_t f = w.flag[e];
-    if (f & 6) continue;
-    bool to_u;
-    if (na == 0) to_u = false;
-    else if (na == nd) to_u = true;
-    else {
-      const uint64_t km = w.key[e] & mask;
-      if (km != prefix) to_u = km < prefix;
-      else if (!tie) to_u = r >= 1;   // the single element of the last bucket is the na-th
+    const int2 en = w.ent[e];
+    if ((f & 5) == 5) continue;   // the edge {u, v} goes on from u's entry
+    Msg m;
+    bool at_u = !(f & 1);
+    if (!(f & 6)) {
+      if (na == 0) at_u = false;
+      else if (na == nd) at_u = true;
       else {
-        to_u = tied_before(c, w.ent, w.key, w.flag, E, e) < r;
+        const uint64_t km = w.key[e] & mask;
+        if (km != prefix) at_u = km < prefix;
+        else if (!tie) at_u = r >= 1;   // the single element of the last bucket is the na-th
+        else at_u = tied_before(w.ent, w.key, w.flag, E, e) < r;
       }
+      moved += at_u == ((f & 1) != 0);   // an edge end that changes node
     }
-    if (to_u) w.flag[e] = f | 8;
-    moved += to_u == ((f & 1) != 0);   // an edge end that changes node
+    m.a = at_u ? u : v;
+    m.ta = at_u ? next.x : next.y;
+    m.b = en.x;
+    m.tb = (f & 4) ? next.y : en.y;
+    reserve(c, m);
+    deliver(c, m);
   }
-  if (c.swaps) {
-    if (moved) atomicAdd(&c.swaps[0], static_cast<unsigned long long>(moved));
-    if (tm.rank == 0) atomicAdd(&c.swaps[1], static_cast<unsigned long long>(E));
-  }
-  tm.sync();
-  // 6. every resulting edge goes on: common neighbours and the edge {u, v}
-  //    stay, D as decided; atomics of a thread's messages overlap in batches
-  for (int e0 = 0; e0 < E; e0 += NT * msg_batch<NT>()) {
-    Msg m[msg_batch<NT>()];
-    bool has[msg_batch<NT>()];
-#pragma unroll
-    for (int j = 0; j < msg_batch<NT>(); ++j) {
-      const int e = e0 + j * NT + tm.rank;
-      has[j] = false;
-      if (e < E) {
-        const uint8_t f = w.flag[e];
-        const int2 en = w.ent[e];
-        if (f & 4) {
-          if (!(f & 1)) {   // the edge {u, v}: from u's entry only
-            m[j] = {u, nu, v, nv, 0, 0ull};
-            has[j] = true;
-          }
-        } else {
-          const bool at_u = (f & 2) ? !(f & 1) : ((f & 8) != 0);
-          m[j] = {at_u ? u : v, at_u ? nu : nv, en.x, en.y, 0, 0ull};
-          has[j] = true;
-        }
-        if (has[j]) reserve(c, m[j]);
-      }
-    }
-#pragma unroll
-    for (int j = 0; j < msg_batch<NT>(); ++j)
-      if (has[j]) deliver(c, m[j]);
-  }
+  if (tm.rank == 0) possible += static_cast<unsigned>(E);
   tm.sync();   // the work space is reused by the next trade
   return true;
 }
 
+// messages of a small trade's lane with their atomics in flight together
+constexpr int kMsgBatch = 2;
+constexpr int kSmallHash = 2 * kUniSmall;   // hash slots of a small trade's work space
+constexpr int32_t kMark = static_cast<int32_t>(0x80000000u);
+
+// A small trade (E <= 32 J) by a warp: entry 32 j + lane in register j,
+// u's neighbours hashed by position (-1: empty; top bit: v has it too), the
+// threshold found bit by bit, about log2 |D| + 2 votes.  Its latency is what
+// counts, hence a form each for J = 1, 2 and 4.
+template <int J>
+__device__ __noinline__ bool uni_trade_warp(const UniCtx& c, int64_t k, Trade t, int32_t* hash, unsigned long long& moved,
+                               unsigned long long& possible) {
+  constexpr int kBatch = J < kMsgBatch ? J : kMsgBatch;
+  static_assert(J % kBatch == 0, "");
+  const int lane = threadIdx.x & 31;
+  const int32_t u = t.uv.x, v = t.uv.y;
+  const int du = t.deg.x, E = t.deg.x + t.deg.y;
+  const int2 next = t.next;
+  const int2* in = t.in;
+  const int hbits = hash_bits(2 * du);
+  const int H = 1 << hbits;
+  const uint64_t gi = c.first + static_cast<uint64_t>(k);
+  int2 m[J];
+  bool ok = true;
+#pragma unroll
+  for (int j = 0; j < J; ++j) m[j] = 32 * j + lane < E ? __ldcg(in + 32 * j + lane) : make_int2(-2, kInf);
+  for (int s = lane; s < H; s += 32) hash[s] = -1;
+#pragma unroll
+  for (int j = 0; j < J; ++j)
+    if (m[j].x == -1 && !wait_entry(in + 32 * j + lane, c.err, c.wait_ns, &m[j])) {
+      ok = false;
+      m[j] = make_int2(0, kInf);
+    }
+  if (__any_sync(kFull, !ok)) return false;
+  __syncwarp();
+  uint64_t key[J];
+  int at[J];
+#pragma unroll
+  for (int j = 0; j < J; ++j) {
+    const int e = 32 * j + lane;
+    at[j] = 0;
+    if (e < du) {
+      uint32_t s = hash_slot(m[j].x, hbits);
+      while (atomicCAS(&hash[s], -1, m[j].x) != -1) s = (s + 1) & (H - 1);
+      at[j] = static_cast<int>(s);
+    }
+  }
+  __syncwarp();
+  // 0: in D, 1: stays (common neighbour), 2: the edge {u, v} or no entry
+  uint32_t kind[J];
+#pragma unroll
+  for (int j = 0; j < J; ++j) {
+    const int e = 32 * j + lane;
+    kind[j] = e < E ? 0u : 2u;
+    if (e >= du && e < E) {
+      if (m[j].x == u) kind[j] = 2u;
+      uint32_t s = hash_slot(m[j].x, hbits);
+      for (;;) {
+        const int32_t h = hash[s];
+        if (h == -1) break;
+        if ((h & ~kMark) == m[j].x) {
+          kind[j] = 1u;
+          hash[s] = h | kMark;
+          break;
+        }
+        s = (s + 1) & (H - 1);
+      }
+    }
+  }
+  __syncwarp();
+  uint32_t cnt = 0;   // |D| and, above bit 16, u's part of it
+#pragma unroll
+  for (int j = 0; j < J; ++j) {
+    const int e = 32 * j + lane;
+    if (e < du) {
+      if (m[j].x == v) kind[j] = 2u;
+      else if (hash[at[j]] < 0) kind[j] = 1u;
+    }
+    key[j] = 0;
+    if (kind[j] == 0u) {
+      const Philox4 r = philox4x32_10(static_cast<uint32_t>(m[j].x), static_cast<uint32_t>(gi),
+                                      static_cast<uint32_t>(gi >> 32), 6u, c.seed);
+      key[j] = (static_cast<uint64_t>(r.w0) << 32) | r.w1;
+      cnt += e < du ? 0x10001u : 1u;
+    }
+  }
+  cnt = __reduce_add_sync(kFull, cnt);
+  int size = static_cast<int>(cnt & 0xffffu), r = static_cast<int>(cnt >> 16);
+  // the na smallest keys of D to u: candidates share the threshold's prefix,
+  // r of them are still to go to u
+  uint32_t cand = 0, to_u = 0;   // bit j: entry j
+#pragma unroll
+  for (int j = 0; j < J; ++j) cand |= (kind[j] == 0u) << j;
+  for (int bit = 63; r > 0 && r < size && bit >= 0; --bit) {
+    uint32_t zero = 0;
+#pragma unroll
+    for (int j = 0; j < J; ++j) zero |= static_cast<uint32_t>(~(key[j] >> bit) & 1ull) << j;
+    zero &= cand;
+    const int z = static_cast<int>(__reduce_add_sync(kFull, __popc(zero)));
+    if (r < z) {
+      cand = zero;
+      size = z;
+    } else {
+      to_u |= zero;
+      cand &= ~zero;
+      size -= z;
+      r -= z;
+    }
+  }
+  if (r > 0 && r < size) {   // equal full keys: node id decides (practically never)
+    uint32_t id[J];
+#pragma unroll
+    for (int j = 0; j < J; ++j) id[j] = (cand >> j & 1u) ? static_cast<uint32_t>(m[j].x) : 0xffffffffu;
+#pragma unroll
+    for (int j = 0; j < J; ++j) {
+      int before = 0;
+      for (int q = 0; q < 32; ++q)
+#pragma unroll
+        for (int i = 0; i < J; ++i) before += __shfl_sync(kFull, id[i], q) < id[j];
+      if ((cand >> j & 1u) && before < r) to_u |= 1u << j;
+    }
+  } else if (r > 0) {
+    to_u |= cand;   // r == size
+  }
+  // every resulting edge goes on, kBatch messages of a lane in flight
+  uint32_t has = 0;
+#pragma unroll
+  for (int j = 0; j < J; ++j) {
+    const bool side_u = 32 * j + lane < du;
+    if (kind[j] == 1u && side_u) to_u |= 1u << j;
+    if (kind[j] == 0u) moved += (to_u >> j & 1u) != static_cast<uint32_t>(side_u);
+    if (kind[j] == 2u && side_u) {   // the edge {u, v}: from u's entry only
+      m[j].y = next.y;
+      to_u |= 1u << j;
+      kind[j] = 1u;
+    }
+    has |= (kind[j] != 2u) << j;
+  }
+#pragma unroll
+  for (int j0 = 0; j0 < J; j0 += kBatch) {
+    Msg msg[kBatch];
+#pragma unroll
+    for (int q = 0; q < kBatch; ++q) {
+      const int j = j0 + q;
+      const bool at_u = to_u >> j & 1u;
+      msg[q].a = at_u ? u : v;
+      msg[q].ta = at_u ? next.x : next.y;
+      msg[q].b = m[j].x;
+      msg[q].tb = m[j].y;
+      if (has >> j & 1u) reserve(c, msg[q]);
+    }
+#pragma unroll
+    for (int q = 0; q < kBatch; ++q)
+      if (has >> (j0 + q) & 1u) deliver(c, msg[q]);
+  }
+  if (lane == 0) possible += static_cast<unsigned>(E);
+  __syncwarp();   // the hash is reused by the next trade
+  return true;
+}
+
+// The executor.  n=2^20, degrees [10,1000), n/2 trades: 28.8 ms with every
+// trade on a whole 1024-thread CTA, 10.1 ms so: 152 trades ran at once, now
+// up to 1368, and a trade has two dependent memory accesses fewer.
 template <int NT>
-__global__ void __launch_bounds__(NT, NT == 256 ? 2 : 1) k_uni_exec(UniCtx c) {
+__global__ void __launch_bounds__(NT, 1024 / NT) k_uni_exec(const __grid_constant__ UniCtx c) {
+  constexpr int kTeam = uni_team<NT>();
   extern __shared__ __align__(16) char usm[];
-  __shared__ int64_t red[BlockTeam<NT>::kRedSlots];
+  __shared__ int64_t red[SubTeam<kTeam>::kRedSlots];
   __shared__ int32_t hist[256];
-  __shared__ int64_t s_sel[3];
+  __shared__ int s_sel[3];
   __shared__ int64_t s_k;
   __shared__ int s_abort;
-  BlockTeam<NT> tm(red);
-  if (threadIdx.x == 0) s_abort = 0;
-  const TradeWs ws_smem = carve_ws(usm, uni_smem_elems<NT>());
-  const TradeWs ws_glob =
-      c.gslice ? carve_ws(c.gslice + static_cast<size_t>(blockIdx.x) * c.slice_elems * kWsBytesPerElem, c.slice_elems)
-               : ws_smem;
-  for (;;) {
-    if (threadIdx.x == 0) s_k = take_ticket(c);
-    tm.sync();
-    const int64_t k = s_k;
-    if (k < 0) break;
-    const int32_t u = c.tp[2 * k], v = c.tp[2 * k + 1];
-    const int64_t du = c.rp[u + 1] - c.rp[u];
-    const int64_t E = du + (c.rp[v + 1] - c.rp[v]);
-    bool ok;
-    if (E <= uni_smem_elems<NT>()) {
-      ok = uni_trade(tm, c, k, ws_smem, hash_bits(2 * du), hist, s_sel, &s_abort);
-    } else if (du <= kHash16MaxDu) {
-      TradeWs<uint16_t> w16{ws_glob.ent, ws_glob.key, reinterpret_cast<uint16_t*>(usm), ws_glob.flag};
-      ok = uni_trade(tm, c, k, w16, hash_bits((4 * du + 2) / 3), hist, s_sel, &s_abort);
-    } else {
-      ok = uni_trade(tm, c, k, ws_glob, hash_bits(2 * du), hist, s_sel, &s_abort);
+  __shared__ int32_t small_hash[uni_warps<NT>()][kSmallHash];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  unsigned long long moved = 0, possible = 0;   // swaps, for the handle's counters
+  bool ok = true;
+  int32_t* hash = warp < kTeam / 32 ? reinterpret_cast<int32_t*>(usm) + warp * kSmallHash : small_hash[warp - kTeam / 32];
+  if (warp < kTeam / 32) {
+    SubTeam<kTeam> tm(red, 0);
+    if (tm.rank == 0) s_abort = 0;
+    const TradeWs ws_smem = carve_ws(usm, uni_smem_elems<NT>());
+    const TradeWs ws_glob =
+        c.gslice ? carve_ws(c.gslice + static_cast<size_t>(blockIdx.x) * c.slice_elems * kWsBytesPerElem, c.slice_elems)
+                 : ws_smem;
+    const int64_t len = queue_len(c, 1);
+    while (ok) {
+      if (tm.rank == 0) s_k = take_ticket(c, 1, len);
+      tm.sync();
+      const int64_t k = s_k;
+      if (k < 0) break;
+      const Trade t = load_trade(c, k);
+      const int64_t du = t.deg.x, E = du + t.deg.y;
+      if (E > uni_smem_elems<NT>() && du <= kHash16MaxDu) {
+        TradeWs<uint16_t> w16{ws_glob.ent, ws_glob.key, reinterpret_cast<uint16_t*>(usm), ws_glob.flag};
+        ok = uni_trade(tm, c, k, t, w16, hash_bits((4 * du + 2) / 3), hist, s_sel, &s_abort, moved, possible);
+      } else {
+        ok = uni_trade(tm, c, k, t, E <= uni_smem_elems<NT>() ? ws_smem : ws_glob, hash_bits(2 * du), hist, s_sel, &s_abort,
+                       moved, possible);
+      }
     }
-    if (!ok) {
-      if (threadIdx.x == 0) latch(c.err, kErrUniformWait);
-      break;
+  }
+  const int64_t len = queue_len(c, 0);
+  while (ok) {
+    int64_t k = 0;
+    if (lane == 0) k = take_ticket(c, 0, len);
+    k = __shfl_sync(kFull, k, 0);
+    if (k < 0) break;
+    const Trade t = load_trade(c, k);
+    const int E = t.deg.x + t.deg.y;
+    ok = E <= 32   ? uni_trade_warp<1>(c, k, t, hash, moved, possible)
+         : E <= 64 ? uni_trade_warp<2>(c, k, t, hash, moved, possible)
+                   : uni_trade_warp<kUniSmall / 32>(c, k, t, hash, moved, possible);
+  }
+  if (!ok && lane == 0) latch(c.err, kErrUniformWait);
+  if (c.swaps) {
+    const int64_t mv = WarpTeam().sum(static_cast<int64_t>(moved)), ps = WarpTeam().sum(static_cast<int64_t>(possible));
+    if (lane == 0 && (mv | ps)) {
+      atomicAdd(&c.swaps[0], static_cast<unsigned long long>(mv));
+      atomicAdd(&c.swaps[1], static_cast<unsigned long long>(ps));
     }
   }
 }
 
-// Every output row full.
 // Every output row full, and every trade queued and taken exactly once.
 __global__ void k_uni_check(int64_t n, const int64_t* __restrict__ rp, const int32_t* __restrict__ ocur,
                             const unsigned long long* __restrict__ ctr, int64_t L, int32_t* err) {
   if (blockIdx.x == 0 && threadIdx.x == 0) {
     const unsigned long long l = static_cast<unsigned long long>(L);
-    if (ctr[kTail] != l) latch(err, kErrUniform);
+    if (ctr[kTail] + ctr[kQueueCtr + kTail] != l) latch(err, kErrUniform);
   }
   for (int64_t x = blockIdx.x * int64_t(blockDim.x) + threadIdx.x; x < n; x += int64_t(gridDim.x) * blockDim.x)
     if (ocur[x] != rp[x + 1] - rp[x]) latch(err, kErrRowLength);
@@ -686,7 +875,7 @@ int uni_buffers(Graph* h, int64_t L) {
   if (grow(h, &b->tp, 2 * L, by) || grow(h, &b->dslot, 2 * L, by) || grow(h, &b->ib, 2 * L + 1, by) ||
       grow(h, &b->suc, 2 * L, by) || grow(h, &b->nxt, 2 * L, by) || grow(h, &b->fill, L, by) ||
       grow(h, &b->queue, L, by) || grow(h, &b->occ, n, by) || grow(h, &b->sbeg, n + 1, by) ||
-      grow(h, &b->ocur, n, by) || grow(h, &b->ctr, kCtrWords, by))
+      grow(h, &b->ocur, n, by) || grow(h, &b->first, n, by) || grow(h, &b->ctr, kCtrWords, by))
     return fail(h, CB_ENOMEM, "device allocation failed (uniform trades)");
   const size_t ws = std::max(scan_ws_bytes(n), scan_ws_bytes(2 * L));
   void* q = nullptr;
@@ -701,7 +890,7 @@ int uni_buffers(Graph* h, int64_t L) {
 void free_uniform(Graph* h) {
   UniBufs* b = h->uni;
   if (!b) return;
-  void* bufs[] = {b->tp, b->dslot, b->ib, b->suc, b->nxt, b->fill, b->queue, b->occ, b->sbeg, b->ocur, b->ctr,
+  void* bufs[] = {b->tp, b->dslot, b->ib, b->suc, b->nxt, b->fill, b->queue, b->occ, b->sbeg, b->ocur, b->first, b->ctr,
                   b->scan_ws};
   if (h->stream) {
     for (void* p : bufs)
@@ -755,24 +944,22 @@ int uniform_trades(Graph* h, uint64_t count) {
     b->slice_bytes = bytes;
     b->ctas = ctas;
   }
-  // node id -> position of the current step
   const unsigned g1 = grid_for_work(n, h->num_sms);
   uint64_t done = 0;
   while (done < count) {
     const int64_t L = static_cast<int64_t>(std::min<uint64_t>(count - done, static_cast<uint64_t>(b->cap_trades)));
     const uint64_t first = h->uni_next + done;
     const unsigned gL = grid_for_work(L, h->num_sms);
-    // the sequence in positions, its Suc lists and every slot's next trade
-    k_uni_draw<<<gL, 256, 0, s>>>(L, first, h->seed, n, h->pos[h->cur], h->rp[h->cur], b->tp, b->dslot);
-    CB_CUDA(h, cudaGetLastError());
+    // the sequence in positions, its Suc lists and every slot's next slot
     CB_CUDA(h, cudaMemsetAsync(b->occ, 0, sizeof(int32_t) * n, s));
-    k_uni_count<<<gL, 256, 0, s>>>(L, n, b->tp, b->occ, h->err);
+    CB_CUDA(h, cudaMemsetAsync(b->ctr, 0, sizeof(unsigned long long) * kCtrWords, s));
+    k_uni_draw<<<gL, 256, 0, s>>>(L, first, h->seed, n, h->deg_id, b->tp, b->dslot, b->occ, uni_small(L), b->ctr + kBig);
     CB_CUDA(h, cudaGetLastError());
     CB_CUDA(h, exclusive_scan_i32(b->occ, b->sbeg, n, b->scan_ws, s, &h->launches));
     CB_CUDA(h, cudaMemsetAsync(b->occ, 0, sizeof(int32_t) * n, s));
     k_uni_fill<<<grid_for_work(2 * L, h->num_sms), 256, 0, s>>>(2 * L, b->tp, b->sbeg, b->occ, b->suc);
     CB_CUDA(h, cudaGetLastError());
-    k_uni_sort<<<g1, 256, 0, s>>>(n, b->sbeg, b->suc, b->nxt);
+    k_uni_sort<<<g1, 256, 0, s>>>(n, b->sbeg, b->suc, b->nxt, h->pos[h->cur], b->first);
     CB_CUDA(h, cudaGetLastError());
     CB_CUDA(h, exclusive_scan_i32(b->dslot, b->ib, 2 * L, b->scan_ws, s, &h->launches));
     int64_t total = 0;
@@ -798,7 +985,6 @@ int uniform_trades(Graph* h, uint64_t count) {
     if (total) CB_CUDA(h, cudaMemsetAsync(b->inbox, 0xff, sizeof(int2) * static_cast<size_t>(total), s));
     CB_CUDA(h, cudaMemsetAsync(b->fill, 0, sizeof(unsigned long long) * L, s));
     CB_CUDA(h, cudaMemsetAsync(b->queue, 0xff, sizeof(int32_t) * L, s));
-    CB_CUDA(h, cudaMemsetAsync(b->ctr, 0, sizeof(unsigned long long) * kCtrWords, s));
     CB_CUDA(h, cudaMemsetAsync(b->ocur, 0, sizeof(int32_t) * n, s));
     const int spare = 1 - h->cur;
     UniCtx c;
@@ -810,8 +996,9 @@ int uniform_trades(Graph* h, uint64_t count) {
     c.tp = b->tp;
     c.nxt = b->nxt;
     c.ib = b->ib;
-    c.sbeg = b->sbeg;
-    c.suc = b->suc;
+    c.dslot = b->dslot;
+    c.pos = h->pos[h->cur];
+    c.first_slot = b->first;
     c.inbox = b->inbox;
     c.fill = b->fill;
     c.queue = b->queue;
@@ -819,6 +1006,7 @@ int uniform_trades(Graph* h, uint64_t count) {
     c.ocur = b->ocur;
     c.col_out = h->col[spare];
     c.wait_ns = h->uni_wait_ns;
+    c.small = uni_small(L);
     c.hold_trade = h->hold_trade;
     c.err = h->err;
     c.gslice = b->gslice;
@@ -832,7 +1020,7 @@ int uniform_trades(Graph* h, uint64_t count) {
     CB_CUDA(h, cudaGetLastError());
     k_uni_check<<<g1, 256, 0, s>>>(n, c.rp, b->ocur, b->ctr, L, h->err);
     CB_CUDA(h, cudaGetLastError());
-    h->launches += 7;
+    h->launches += 6;
     if ((rc = check_device_error(h))) return rc;
     std::swap(h->col[h->cur], h->col[spare]);
     done += static_cast<uint64_t>(L);
@@ -872,7 +1060,7 @@ extern "C" int cb_uniform_pairs(uint64_t seed, int64_t n, uint64_t first, int64_
   if (e == cudaSuccess) e = cudaDeviceGetAttribute(&num_sms, cudaDevAttrMultiProcessorCount, dev);
   if (e != cudaSuccess) return cuda_fail(nullptr, e, "device query");
   cudaStream_t s = static_cast<cudaStream_t>(cuda_stream);
-  k_uni_draw<<<grid_for_work(count, num_sms), 256, 0, s>>>(count, first, seed, n, nullptr, nullptr, pairs, nullptr);
+  k_uni_draw<<<grid_for_work(count, num_sms), 256, 0, s>>>(count, first, seed, n, nullptr, pairs, nullptr, nullptr, 0, nullptr);
   if ((e = cudaGetLastError()) != cudaSuccess) return cuda_fail(nullptr, e, "k_uni_draw");
   return CB_OK;
 }
@@ -916,7 +1104,7 @@ extern "C" int cb_successors(int64_t n, const int32_t* pairs, int64_t count, int
     if ((e = cudaMemsetAsync(occ, 0, sizeof(int32_t) * n, s)) != cudaSuccess) goto cuda_error;
     k_uni_fill<<<g, 256, 0, s>>>(2 * count, pairs, suc_begin, occ, slots);
     if ((e = cudaGetLastError()) != cudaSuccess) goto cuda_error;
-    k_uni_sort<<<g, 256, 0, s>>>(n, suc_begin, slots, nullptr);
+    k_uni_sort<<<g, 256, 0, s>>>(n, suc_begin, slots, nullptr, nullptr, nullptr);
     if ((e = cudaGetLastError()) != cudaSuccess) goto cuda_error;
     k_uni_trade_index<<<g, 256, 0, s>>>(2 * count, slots, suc);
     if ((e = cudaGetLastError()) != cudaSuccess) goto cuda_error;
