@@ -382,6 +382,41 @@ inline size_t block_smem_bytes(int cap) {
   return ((ws_a_bytes(cap) + 127) & ~size_t(127)) + (static_cast<size_t>(cap) + 8) * 4;
 }
 
+// Trades above the shared-memory cap: the hash, which every member reaches
+// into, stays in shared memory while it has at most 2^kSplitLg slots (at least
+// 1.25 per entry: 26214 entries), with the entries' key prefixes and flags
+// while they fit; slots and far keys, which only their own member reads, go to
+// the CTA's global slice.  One 1024-thread CTA per SM has the room; below, all
+// of it is in the slice.  n=300007 with hubs of 15000 neighbours, everything
+// above 8192 entries in the slice: first pass of the largest class 395 to 428
+// us, in-order pass 1300 to 1730; so, and with the threshold published before
+// the decisions: 240 to 290, and 530 to 720.
+constexpr int kSplitLg = 15;
+constexpr size_t kSplitSmem = size_t(224) * 1024;
+__device__ inline WsA carve_split(char* smem, size_t room, char* slice, int L) {
+  const size_t L16 = (static_cast<size_t>(L) + 15) & ~size_t(15);
+  WsA w;
+  w.lgH = hash_lg(L);
+  if (w.lgH > kSplitLg && 5 * static_cast<int64_t>(L) <= (int64_t(4) << kSplitLg)) w.lgH = kSplitLg;
+  const size_t H = size_t(1) << w.lgH;
+  const size_t hash = H * 4 + ((H + 15) & ~size_t(15)) + kSelBins * 4 + kCand * 20 + 16;
+  char* p = hash <= room ? smem : slice;
+  w.hkey = reinterpret_cast<uint32_t*>(p); p += H * 4;
+  w.hflag = reinterpret_cast<uint8_t*>(p); p += (H + 15) & ~size_t(15);
+  w.hist = reinterpret_cast<uint32_t*>(p); p += kSelBins * 4;
+  w.ck = reinterpret_cast<uint64_t*>(p); p += kCand * 8;
+  w.ctb = reinterpret_cast<uint64_t*>(p); p += kCand * 8;
+  w.cidx = reinterpret_cast<int32_t*>(p); p += kCand * 4;
+  w.ncand = reinterpret_cast<int32_t*>(p); p += 16;
+  if (hash <= room && hash + 3 * L16 > room) p = slice;
+  w.top = reinterpret_cast<uint16_t*>(p); p += L16 * 2;
+  w.meta = reinterpret_cast<uint8_t*>(p); p += L16;
+  if (hash + 3 * L16 <= room) p = slice;
+  w.slot = reinterpret_cast<int32_t*>(p); p += L16 * 4;
+  w.far = reinterpret_cast<uint16_t*>(p);
+  return w;
+}
+
 __device__ inline WsA carve_a(void* base, int L) {
   const size_t L16 = (static_cast<size_t>(L) + 15) & ~size_t(15);
   char* p = static_cast<char*>(base);
@@ -739,68 +774,61 @@ __device__ bool phase_a(Team& tm, const StepCtx& c, int64_t t, const WsA& w, Sel
   }
   uint64_t tk = 0, tt = 0;
   if (cnt <= kCand) {
-    // own decisions: an element below the threshold's bin stays with u, above it
-    // goes to v; in the bin, full keys decide (the only element: the threshold)
-    for (int i = tm.rank; i < L; i += Team::N) {
+    // the threshold first, so that dependent trades go on: the elements of its
+    // bin (the only one, or ranked by full key)
+    for (int i = tm.rank; cnt > 0 && i < L; i += Team::N) {
       const uint8_t m = w.meta[i];
-      if (!(m & kInD)) continue;
-      const int r = m & kR;
-      const int d = static_cast<int>(w.top[i]) >> (16 - kSelBits);
-      bool low;
-      if (no_thr || d > bin) {
-        low = false;
-      } else if (d < bin) {
-        low = true;
-      } else {
-        const int32_t y = entry_y(w, t2, i);
-        const uint32_t lo = lo_of(t2, m, y), hi = hi_of(t2, m, y);
-        const uint64_t ki = own_key(kc, t, lo, hi), tbi = tie_break(lo, hi);
-        if (cnt == 1) {
-          low = true;
-          sel->key = ki;
-          sel->tb = tbi;
-        } else {
-          const int q = atomicAdd(w.ncand, 1);
-          w.ck[q] = ki;
-          w.ctb[q] = tbi;
-          w.cidx[q] = i;
-          continue;
-        }
+      if (!(m & kInD) || (static_cast<int>(w.top[i]) >> (16 - kSelBits)) != bin) continue;
+      const int32_t y = entry_y(w, t2, i);
+      const uint32_t lo = lo_of(t2, m, y), hi = hi_of(t2, m, y);
+      const int q = cnt == 1 ? 0 : atomicAdd(w.ncand, 1);
+      w.ck[q] = own_key(kc, t, lo, hi);
+      w.ctb[q] = tie_break(lo, hi);
+      w.cidx[q] = i;
+    }
+    tm.sync();
+    const int kk = a - below;
+    for (int q = tm.rank; q < cnt; q += Team::N) {
+      int rk = 0;
+      for (int j = 0; j < cnt; ++j) rk += (w.ck[j] < w.ck[q] || (w.ck[j] == w.ck[q] && w.ctb[j] < w.ctb[q]));
+      if (rk == kk - 1) {
+        sel->key = w.ck[q];
+        sel->tb = w.ctb[q];
       }
-      if ((low ? 0 : 1) != r) {
+      const int i = w.cidx[q];
+      const uint8_t m = w.meta[i];
+      const int r = m & kR;
+      if ((rk < kk ? 0 : 1) != r) {
         w.meta[i] = m | kFlip;
         flag_or(w.hflag, w.slot[i], 16u << (2 * r + ((m & kCol) ? 1 : 0)));
       }
     }
     tm.sync();
-    if (cnt > 1) {   // rank the elements of the threshold's bin
-      const int kk = a - below;
-      for (int q = tm.rank; q < cnt; q += Team::N) {
-        int rk = 0;
-        for (int j = 0; j < cnt; ++j) rk += (w.ck[j] < w.ck[q] || (w.ck[j] == w.ck[q] && w.ctb[j] < w.ctb[q]));
-        if (rk == kk - 1) {
-          sel->key = w.ck[q];
-          sel->tb = w.ctb[q];
-        }
-        const int i = w.cidx[q];
-        const uint8_t m = w.meta[i];
-        const int r = m & kR;
-        if ((rk < kk ? 0 : 1) != r) {
-          w.meta[i] = m | kFlip;
-          flag_or(w.hflag, w.slot[i], 16u << (2 * r + ((m & kCol) ? 1 : 0)));
-        }
-      }
-      tm.sync();
-    }
     if (!no_thr) {
       tk = sel->key;
       tt = sel->tb;
     }
+    if (tm.rank == 0) publish(c, kc, t, pu, pv, tk, tt, publish_fence);
+    // own decisions: an element below the threshold's bin stays with u, above
+    // it goes to v
+    for (int i = tm.rank; i < L; i += Team::N) {
+      const uint8_t m = w.meta[i];
+      if (!(m & kInD)) continue;
+      const int r = m & kR;
+      const int d = static_cast<int>(w.top[i]) >> (16 - kSelBits);
+      if (!no_thr && d == bin) continue;
+      if ((no_thr || d > bin ? 1 : 0) != r) {
+        w.meta[i] = m | kFlip;
+        flag_or(w.hflag, w.slot[i], 16u << (2 * r + ((m & kCol) ? 1 : 0)));
+      }
+    }
+    tm.sync();
   } else {
     // crowded bin (|D| in the tens of thousands): the general selection
     select_kth(tm, kc, w, L, t, a, sel);
     tk = sel->key;
     tt = sel->tb;
+    if (tm.rank == 0) publish(c, kc, t, pu, pv, tk, tt, publish_fence);
     const uint32_t tk16 = static_cast<uint32_t>(tk >> 48);
     for (int i = tm.rank; i < L; i += Team::N) {
       const uint8_t m = w.meta[i];
@@ -822,7 +850,6 @@ __device__ bool phase_a(Team& tm, const StepCtx& c, int64_t t, const WsA& w, Sel
     }
     tm.sync();
   }
-  if (tm.rank == 0) publish(c, kc, t, pu, pv, tk, tt, publish_fence);
   // placement: each entry goes into the new row of its node after the trade
   // (u's or v's row of step g+1) at a slot given by a scan over the team
   int n0 = 0, n1 = 0;
@@ -1777,11 +1804,11 @@ __global__ void __launch_bounds__(kFixThreads, 4) k_fixup(StepCtx c, int64_t nnz
 template <int NT, bool kOneSeed>
 __global__ void __launch_bounds__(NT, NT == 256 ? 4 : 1) k_phase_a_block(StepCtx c, const int32_t* __restrict__ lists,
                                                       const int64_t* __restrict__ ctr, int cls, int smem_max,
-                                                      char* gws, size_t slice, int stage_cap) {
+                                                      size_t room, char* gws, size_t slice, int stage_cap) {
   after_previous();
   before_next();
-  // dynamic shared memory: the workspace, then the staging buffer of a
-  // trade's entries (stage_cap + 8 int32, 16-byte aligned)
+  // dynamic shared memory: the workspace (room bytes, a multiple of 128), then
+  // the staging buffer of a trade's entries (stage_cap + 8 int32)
   extern __shared__ __align__(16) char sbuf[];
   __shared__ int64_t red[BlockTeam<NT>::kRedSlots];
   __shared__ SelOut sel;
@@ -1790,7 +1817,7 @@ __global__ void __launch_bounds__(NT, NT == 256 ? 4 : 1) k_phase_a_block(StepCtx
   const ClassList cl = class_list(c, lists, ctr, cls);
   const int32_t* list = cl.list;
   const int64_t len = cl.len;
-  int32_t* stage = reinterpret_cast<int32_t*>(sbuf + ((ws_a_bytes(smem_max) + 127) & ~size_t(127)));
+  int32_t* stage = reinterpret_cast<int32_t*>(sbuf + room);
   if (threadIdx.x == 0) {
     mbar_init(&mbar, 1);
     mbar_fence_init();
@@ -1819,11 +1846,8 @@ __global__ void __launch_bounds__(NT, NT == 256 ? 4 : 1) k_phase_a_block(StepCtx
     const int64_t t = list[q];
     const TradeRows tr = trade_rows(c, t);
     const int L = tr.du + tr.dv;
-    char* base = sbuf;
-    if (L > smem_max) {
-      base = gws + slice * blockIdx.x;
-      if (threadIdx.x == 0) atomicAdd(c.gws_count, 1ull);
-    }
+    if (L > smem_max && threadIdx.x == 0) atomicAdd(c.gws_count, 1ull);
+    const WsA ws = L > smem_max ? carve_split(sbuf, room, gws + slice * blockIdx.x, L) : carve_a(sbuf, L);
     StageNext sn{false, 0, 0, stage, &mbar};
     if (threadIdx.x == 0 && q + gridDim.x < len) {
       range_of(q + gridDim.x, &nb0, &nL);
@@ -1841,7 +1865,7 @@ __global__ void __launch_bounds__(NT, NT == 256 ? 4 : 1) k_phase_a_block(StepCtx
       }
       ys = stage + stage_off(tr.b0);
     }
-    if (!phase_a<BlockTeam<NT>, kOneSeed>(tm, c, t, carve_a(base, L), &sel, ys, sn) && threadIdx.x == 0)
+    if (!phase_a<BlockTeam<NT>, kOneSeed>(tm, c, t, ws, &sel, ys, sn) && threadIdx.x == 0)
       defer_trade(c, t);
   }
   if (failed) {   // a copy did not complete in time: report, let it land, leave
@@ -1856,26 +1880,24 @@ __global__ void __launch_bounds__(NT, NT == 256 ? 4 : 1) k_phase_a_block(StepCtx
 // 1024-thread CTAs the large ones.  (One launch with CTAs shared out over the
 // lists took 1.06 ms per pass at n=2^25 against 0.6 for two such passes.)
 template <int NT>
-size_t resolve_smem(int gen_max) {
-  return std::max(std::max(std::max(TeamCfg<NT>::Ws::kBytes, TeamCfg<256>::Ws::kBytes * (NT / 256)),
-                           ws_a_bytes(std::max(gen_max, 1))),
-                  WarpWs::kBytes * (NT / 32));
+size_t resolve_smem(int gen_max, int64_t max_trade) {
+  const size_t s = std::max(std::max(std::max(TeamCfg<NT>::Ws::kBytes, TeamCfg<256>::Ws::kBytes * (NT / 256)),
+                                     ws_a_bytes(std::max(gen_max, 1))),
+                            WarpWs::kBytes * (NT / 32));
+  return NT == kBigThreads && max_trade > gen_max ? std::max(s, kSplitSmem) : s;
 }
 // A large trade (L > kDefMedium) on the whole CTA.
 template <int NT, bool kWait>
-__device__ bool run_large(BlockTeam<NT>& tm, const StepCtx& c, int64_t t, char* sbuf, SelOut* sel, int gen_max, char* gws,
-                          size_t slice, uint32_t wait_below) {
+__device__ bool run_large(BlockTeam<NT>& tm, const StepCtx& c, int64_t t, char* sbuf, SelOut* sel, int gen_max, size_t room,
+                          char* gws, size_t slice, uint32_t wait_below) {
   using Ws = typename TeamCfg<NT>::Ws;
   const TradeRows tr = trade_rows(c, t);
   const int L = tr.du + tr.dv;
   if (L <= Ws::kLmax)
     return phase_a_reg<BlockTeam<NT>, kTeamJ, TeamCfg<NT>::B, false, false, kWait>(tm, c, t, Ws{sbuf}, true, wait_below);
-  char* wsb = sbuf;
-  if (L > gen_max) {
-    wsb = gws + slice * blockIdx.x;
-    if (threadIdx.x == 0) atomicAdd(c.gws_count, 1ull);
-  }
-  return phase_a(tm, c, t, carve_a(wsb, L), sel, nullptr, StageNext{false, 0, 0, nullptr, nullptr}, wait_below);
+  if (L > gen_max && threadIdx.x == 0) atomicAdd(c.gws_count, 1ull);
+  const WsA ws = L > gen_max ? carve_split(sbuf, room, gws + slice * blockIdx.x, L) : carve_a(sbuf, L);
+  return phase_a(tm, c, t, ws, sel, nullptr, StageNext{false, 0, 0, nullptr, nullptr}, wait_below);
 }
 __global__ void __launch_bounds__(32 * kWarpWarps, 4) k_retry_warp(StepCtx c, const int32_t* __restrict__ list,
                                                                 const unsigned long long* __restrict__ count,
@@ -1896,8 +1918,8 @@ __global__ void __launch_bounds__(32 * kWarpWarps, 4) k_retry_warp(StepCtx c, co
 template <int NT>
 __global__ void __launch_bounds__(NT, NT == 256 ? 4 : 1) k_retry(StepCtx c, const int32_t* __restrict__ list,
                                                               const unsigned long long* __restrict__ count,
-                                                              unsigned long long* claim, int gen_max, char* gws,
-                                                              size_t slice) {
+                                                              unsigned long long* claim, int gen_max, size_t room,
+                                                              char* gws, size_t slice) {
   extern __shared__ __align__(16) char sbuf[];
   __shared__ int64_t red[BlockTeam<NT>::kRedSlots];
   __shared__ SelOut sel;
@@ -1910,7 +1932,7 @@ __global__ void __launch_bounds__(NT, NT == 256 ? 4 : 1) k_retry(StepCtx c, cons
     const int64_t p = pick;
     __syncthreads();
     if (p >= nl) return;
-    if (!run_large<NT, false>(tm, c, list[p], sbuf, &sel, gen_max, gws, slice, 0u) && threadIdx.x == 0)
+    if (!run_large<NT, false>(tm, c, list[p], sbuf, &sel, gen_max, room, gws, slice, 0u) && threadIdx.x == 0)
       defer_trade(c, list[p]);
   }
 }
@@ -2007,8 +2029,8 @@ template <int NT>
 __global__ void __launch_bounds__(NT, NT == 256 ? 4 : 1) k_resolve(StepCtx c, const int32_t* __restrict__ list,
                                                                 const int32_t* __restrict__ chunk_first,
                                                                 const unsigned long long* __restrict__ nchunks,
-                                                                unsigned long long* claim, int gen_max, char* gws,
-                                                                size_t slice) {
+                                                                unsigned long long* claim, int gen_max, size_t room,
+                                                                char* gws, size_t slice) {
   after_previous();
   before_next();
   using Ws256 = typename TeamCfg<256>::Ws;
@@ -2073,7 +2095,7 @@ __global__ void __launch_bounds__(NT, NT == 256 ? 4 : 1) k_resolve(StepCtx c, co
         __syncthreads();
         const int32_t t = trades[2][i];
         if (t < 0) continue;
-        const bool ok = run_large<NT, true>(tm, c, t, sbuf, &sel, gen_max, gws, slice, from);
+        const bool ok = run_large<NT, true>(tm, c, t, sbuf, &sel, gen_max, room, gws, slice, from);
         __syncthreads();
         if (threadIdx.x == 0) {
           if (ok) trades[2][i] = -1;
@@ -2104,7 +2126,7 @@ int init_seed_kernels(Graph* h) {
   CB_CUDA(h, cudaFuncSetAttribute(k_phase_a_block<kMedThreads, kOneSeed>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                   static_cast<int>(block_smem_bytes(kBlockMaxCap))));
   CB_CUDA(h, cudaFuncSetAttribute(k_phase_a_block<kBigThreads, kOneSeed>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                  static_cast<int>(block_smem_bytes(kSmemMaxCap))));
+                                  static_cast<int>(std::max(block_smem_bytes(kSmemMaxCap), kSplitSmem))));
   auto of_class = [&](auto k) -> int {
     constexpr int K = decltype(k)::value;
     CB_CUDA(h, cudaFuncSetAttribute(k_phase_a_class<K, kOneSeed>, cudaFuncAttributeMaxDynamicSharedMemorySize,
@@ -2135,13 +2157,13 @@ int init_trade_kernels(Graph* h) {
   int rc = init_seed_kernels<true>(h);
   if (rc || (rc = init_seed_kernels<false>(h))) return rc;
   CB_CUDA(h, cudaFuncSetAttribute(k_retry<kBigThreads>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                  static_cast<int>(resolve_smem<kBigThreads>(kSmemMaxCap))));
+                                  static_cast<int>(resolve_smem<kBigThreads>(kSmemMaxCap, 2 * int64_t(kSmemMaxCap)))));
   CB_CUDA(h, cudaFuncSetAttribute(k_retry_warp, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                   static_cast<int>(WarpWs::kBytes * kWarpWarps)));
   CB_CUDA(h, cudaFuncSetAttribute(k_resolve<kMedThreads>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                  static_cast<int>(resolve_smem<kMedThreads>(kBlockMaxCap))));
+                                  static_cast<int>(resolve_smem<kMedThreads>(kBlockMaxCap, 0))));
   CB_CUDA(h, cudaFuncSetAttribute(k_resolve<kBigThreads>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                  static_cast<int>(resolve_smem<kBigThreads>(kSmemMaxCap))));
+                                  static_cast<int>(resolve_smem<kBigThreads>(kSmemMaxCap, 2 * int64_t(kSmemMaxCap)))));
   CB_CUDA(h, cudaFuncSetAttribute(k_resolve<kMedThreads>, cudaFuncAttributePreferredSharedMemoryCarveout,
                                   cudaSharedmemCarveoutMaxShared));
   return CB_OK;
@@ -2265,8 +2287,12 @@ int super_step(Graph* h) {
     if ((rc = launched())) return rc;
     return finish();
   }
+  const int64_t max_trade = 2 * h->maxdeg;
   const size_t med_smem_st = block_smem_bytes(std::max(block_max, 1));   // threshold kernels with staging
-  const size_t big_smem_st = block_smem_bytes(std::max(h->smem_max, 1));
+  const size_t big_smem_st =
+      std::max(block_smem_bytes(std::max(h->smem_max, 1)), max_trade > h->smem_max ? kSplitSmem : 0);
+  // the workspace's part of it, before the staging buffer
+  auto room_of = [](size_t smem, int stage) { return (smem - (static_cast<size_t>(stage) + 8) * 4) & ~size_t(127); };
   const unsigned mgrid = static_cast<unsigned>(h->num_sms * 4);
   const unsigned bgrid = static_cast<unsigned>(std::max(1, std::min(h->num_sms, h->ws_ctas)));
   const unsigned wgrid = static_cast<unsigned>(h->num_sms * 8);
@@ -2283,7 +2309,6 @@ int super_step(Graph* h) {
   // twice the largest degree: classes above that are not launched); a trade
   // whose dependency has not published yet is deferred.  With "timing" on,
   // events ev[4] .. ev[13] bracket the classes' kernels.
-  const int64_t max_trade = 2 * h->maxdeg;
   const bool fused = ntasks < kFuseMax, overlap = small_handle(h);
   auto mark = [&](int k) -> int {
     if (h->timing) CB_CUDA(h, cudaEventRecord(ev[4 + k], s));
@@ -2317,7 +2342,8 @@ int super_step(Graph* h) {
         if ((r = mark(k))) return r;
     }
     if (!h->cta_paths) {
-      k_phase_a_block<kMedThreads, kOne><<<mgrid, kMedThreads, med_smem_st, s>>>(c, L, cnt, 5, block_max, gws,
+      k_phase_a_block<kMedThreads, kOne><<<mgrid, kMedThreads, med_smem_st, s>>>(c, L, cnt, 5, block_max,
+                                                                         room_of(med_smem_st, block_max), gws,
                                                                                 h->ws_slice, block_max);
       if ((r = launched()) || (r = mark(6)) || (r = mark(7))) return r;
     } else if (fused) {
@@ -2335,7 +2361,7 @@ int super_step(Graph* h) {
     // memory (staged by a bulk copy), a global-memory slice above
     if (max_trade > th.th[7]) {
       CB_CUDA(h, launch(overlap, k_phase_a_block<kBigThreads, kOne>, bgrid, kBigThreads, big_smem_st, s, c, L, cnt, 8,
-                        h->smem_max, gws, h->ws_slice, h->smem_max));
+                        h->smem_max, room_of(big_smem_st, h->smem_max), gws, h->ws_slice, h->smem_max));
       if ((r = launched())) return r;
     }
     return mark(9);
@@ -2360,12 +2386,13 @@ int super_step(Graph* h) {
     if ((rc = launched())) return rc;
     if (max_trade > kDefSmall) {
       k_retry<kMedThreads><<<lgrid, kMedThreads, TeamCfg<kMedThreads>::Ws::kBytes, s>>>(c, in + ntasks, count + 1,
-                                                                                       claim + 1, 0, nullptr, 0);
+                                                                                       claim + 1, 0, 0, nullptr, 0);
       if ((rc = launched())) return rc;
     }
     if (max_trade > kDefMedium) {
-      k_retry<kBigThreads><<<bgrid, kBigThreads, resolve_smem<kBigThreads>(h->smem_max), s>>>(
-          c, in + 2 * ntasks, count + 2, claim + 2, h->smem_max, gws, h->ws_slice);
+      const size_t sm = resolve_smem<kBigThreads>(h->smem_max, max_trade);
+      k_retry<kBigThreads><<<bgrid, kBigThreads, sm, s>>>(c, in + 2 * ntasks, count + 2, claim + 2, h->smem_max, sm, gws,
+                                                          h->ws_slice);
       if ((rc = launched())) return rc;
     }
   }
@@ -2379,12 +2406,15 @@ int super_step(Graph* h) {
     CB_CUDA(h, launch(overlap, k_def_list, nsegs, kDefListThreads, 0, s, c, nwords, nsegs, static_cast<int>(grid), list,
                       chunk_first, ucnt + kCtrChunks));
     if ((rc = launched())) return rc;
-    if (big)
-      CB_CUDA(h, launch(overlap, k_resolve<kBigThreads>, grid, kBigThreads, resolve_smem<kBigThreads>(h->smem_max), s, c,
-                        list, chunk_first, ucnt + kCtrChunks, ucnt + kCtrFinished, h->smem_max, gws, h->ws_slice));
-    else
-      CB_CUDA(h, launch(overlap, k_resolve<kMedThreads>, grid, kMedThreads, resolve_smem<kMedThreads>(block_max), s, c,
-                        list, chunk_first, ucnt + kCtrChunks, ucnt + kCtrFinished, block_max, gws, h->ws_slice));
+    if (big) {
+      const size_t sm = resolve_smem<kBigThreads>(h->smem_max, max_trade);
+      CB_CUDA(h, launch(overlap, k_resolve<kBigThreads>, grid, kBigThreads, sm, s, c, list, chunk_first,
+                        ucnt + kCtrChunks, ucnt + kCtrFinished, h->smem_max, sm, gws, h->ws_slice));
+    } else {
+      const size_t sm = resolve_smem<kMedThreads>(block_max, max_trade);
+      CB_CUDA(h, launch(overlap, k_resolve<kMedThreads>, grid, kMedThreads, sm, s, c, list, chunk_first,
+                        ucnt + kCtrChunks, ucnt + kCtrFinished, block_max, sm, gws, h->ws_slice));
+    }
     if ((rc = launched())) return rc;
   }
   if (h->timing) CB_CUDA(h, cudaEventRecord(ev[2], s));

@@ -150,3 +150,35 @@ def test_malformed_graphs_are_refused(n, what, shuffled):
     with pytest.raises(CbError) as err:
         Curveball(rp, col, 1)
     assert err.value.code == CB_EINVAL
+
+
+# Trades above smem_max keep their hash in shared memory up to 26214 entries,
+# with key prefixes and flags beside it up to about 18000 (16384 in the first
+# pass's kernel); above, all of it is in global memory.  Hubs on both sides of
+# these limits, adjacent to each other so that their trades depend on one
+# another; smem_max 64 sends every trade above 64 entries the same way.
+@pytest.mark.parametrize("options", [{}, {"inorder_threads": 256}, {"smem_max": 64}, {"smem_max": 2000, "cta_paths": 0}])
+def test_trades_above_shared_memory(options):
+    n = 40000
+    rng = np.random.default_rng(5)
+    g = synth.powerlaw_graph(n, 2, 30, 2.0, 12)
+    rows = np.repeat(np.arange(n, dtype=np.int64), np.diff(g.row_ptr))
+    pairs = [np.stack([rows, g.col.astype(np.int64)], 1)]
+    for hub, d in enumerate([8185, 8300, 12000, 15990, 16400, 17700, 20000, 26190, 26240, 30000]):
+        pairs.append(np.stack([np.full(d, hub), rng.permutation(n)[:d]], 1))
+    e = np.concatenate(pairs)
+    e = e[e[:, 0] != e[:, 1]]
+    e = np.unique(np.sort(e, axis=1), axis=0)
+    both = np.concatenate([e, e[:, ::-1]])
+    both = both[np.lexsort((both[:, 1], both[:, 0]))]
+    rp = np.concatenate([[0], np.cumsum(np.bincount(both[:, 0], minlength=n))]).astype(np.int64)
+    col = both[:, 1].astype(np.int32)
+    c, o = Curveball(rp, col, 3), Oracle(rp, col, 3)
+    for k, v in options.items():
+        c.set_option(k, v)
+    for _ in range(4):
+        c.global_trades(1)
+        o.superstep(1)
+        assert np.array_equal(c.edges(), o.edges())
+    assert c.stats()["global_ws_trades"] > 0
+    c.close()
