@@ -947,12 +947,12 @@ __host__ __device__ constexpr int lg_ceil(int x) {
 // go to table 2 (kH2 >= LMAX slots, cleared per trade), by compare-and-swap.
 // Clearing the single 8-byte-per-slot table this replaces took 16 stores per
 // member; table 2 and the histogram take 3.
-template <int LMAX, int B, int CAND>
+template <int LMAX, int B, int CAND, int SLOTS = 4>
 struct RegWs {
   static_assert(B >= 5, "tables are cleared in 16-byte stores");
   static constexpr int kLmax = LMAX;
   static constexpr int kCandCap = CAND;                 // candidates ranked directly
-  static constexpr int kH = 1 << lg_ceil(4 * LMAX);
+  static constexpr int kH = 1 << lg_ceil(SLOTS * LMAX);
   static constexpr int kH2 = 1 << lg_ceil(LMAX);
   static_assert(kH + kH2 <= int(kMSlot) + 1, "slot field");
   static constexpr size_t kCk = 0;                              // candidate keys
@@ -1033,7 +1033,7 @@ __device__ bool phase_a_reg(Team& tm, const StepCtx& c, int64_t t, const Ws& w, 
                             uint32_t wait_below = 0) {
   constexpr int N = Team::N;
   constexpr bool kWarp = N <= 32;   // the team is a warp or part of one
-  static_assert(J == 4 && (1 << B) == 4 * N, "four entries and four histogram bins per member");
+  static_assert((J == 4 || J == 8) && (1 << B) == 4 * N, "four histogram bins per member");
   static_assert(N * J == Ws::kLmax && N * J < (1 << 16), "16-bit placement counts");
   constexpr int kLgH = lg_ceil(Ws::kH), kLgH2 = lg_ceil(Ws::kH2);
   const TradeRows tr = trade_rows(c, t);
@@ -1052,9 +1052,10 @@ __device__ bool phase_a_reg(Team& tm, const StepCtx& c, int64_t t, const Ws& w, 
   {
     const uint4 z = make_uint4(0u, 0u, 0u, 0u);
     reinterpret_cast<uint4*>(w.hist())[tm.rank] = z;
-    uint4* h4 = reinterpret_cast<uint4*>(hs2);   // kH2 = 4 N slots of 8 bytes
-    h4[tm.rank] = z;
-    h4[tm.rank + N] = z;
+    uint4* h4 = reinterpret_cast<uint4*>(hs2);   // kH2 = J N slots of 8 bytes
+    static_assert(Ws::kH2 == J * N, "");
+#pragma unroll
+    for (int q = 0; q < J / 2; ++q) h4[tm.rank + q * N] = z;
     if (tm.rank == 0) *w.ncand() = 0;
   }
   // entries and their home slots: every entry stores its key there
@@ -1314,7 +1315,7 @@ __device__ bool phase_a_reg(Team& tm, const StepCtx& c, int64_t t, const Ws& w, 
     equal |= (kt[j] == tk32 ? 1u : 0u) << j;
   }
   if (no_thr) {
-    above = 0xfu;
+    above = (1u << J) - 1u;
   } else {
     for (equal &= in_d; equal;) {   // the threshold itself, and keys that share its top half
       const int j = __ffs(equal) - 1;
@@ -1884,21 +1885,59 @@ size_t resolve_smem(int gen_max, int64_t max_trade) {
   const size_t s = std::max(std::max(std::max(TeamCfg<NT>::Ws::kBytes, TeamCfg<256>::Ws::kBytes * (NT / 256)),
                                      ws_a_bytes(std::max(gen_max, 1))),
                             WarpWs::kBytes * (NT / 32));
-  return NT == kBigThreads && max_trade > gen_max ? std::max(s, kSplitSmem) : s;
+  return NT == kBigThreads && max_trade > std::min(gen_max, TeamCfg<NT>::kMax) ? std::max(s, kSplitSmem) : s;
 }
-// A large trade (L > kDefMedium) on the whole CTA.
-template <int NT, bool kWait>
+// A trade of more than kDefMedium entries on the whole CTA.  4097 to 8192
+// entries, which the shared-memory form takes three times as long for, fit
+// eight to a member of 1024 (two hash slots per entry instead of four: table 2
+// takes a fifth of the entries).
+using HugeWs = RegWs<8 * kBigThreads, 12, kCand, 2>;
+static_assert(HugeWs::kBytes <= kSplitSmem, "");
+template <int NT, bool kWait, bool kOneSeed = false>
 __device__ bool run_large(BlockTeam<NT>& tm, const StepCtx& c, int64_t t, char* sbuf, SelOut* sel, int gen_max, size_t room,
                           char* gws, size_t slice, uint32_t wait_below) {
   using Ws = typename TeamCfg<NT>::Ws;
   const TradeRows tr = trade_rows(c, t);
   const int L = tr.du + tr.dv;
   if (L <= Ws::kLmax)
-    return phase_a_reg<BlockTeam<NT>, kTeamJ, TeamCfg<NT>::B, false, false, kWait>(tm, c, t, Ws{sbuf}, true, wait_below);
+    return phase_a_reg<BlockTeam<NT>, kTeamJ, TeamCfg<NT>::B, false, kOneSeed, kWait>(tm, c, t, Ws{sbuf}, true, wait_below);
+  if constexpr (NT == kBigThreads)
+    if (L <= min(HugeWs::kLmax, gen_max) && HugeWs::kBytes <= room)
+      return phase_a_reg<BlockTeam<NT>, 8, 12, false, kOneSeed, kWait>(tm, c, t, HugeWs{sbuf}, true, wait_below);
   if (L > gen_max && threadIdx.x == 0) atomicAdd(c.gws_count, 1ull);
   const WsA ws = L > gen_max ? carve_split(sbuf, room, gws + slice * blockIdx.x, L) : carve_a(sbuf, L);
-  return phase_a(tm, c, t, ws, sel, nullptr, StageNext{false, 0, 0, nullptr, nullptr}, wait_below);
+  return phase_a<BlockTeam<NT>, kOneSeed>(tm, c, t, ws, sel, nullptr, StageNext{false, 0, 0, nullptr, nullptr}, wait_below);
 }
+// The first pass's largest class: more than min(4096, smem_max) entries, up to
+// 8192 of them in registers.  n=2^25, degrees [10,10000): 7.4 ms per step with
+// the shared-memory form (k_phase_a_block) up to 8192 entries, 4.7 so.
+template <bool kOneSeed>
+__global__ void __launch_bounds__(kBigThreads, 1) k_phase_a_huge(StepCtx c, const int32_t* __restrict__ lists,
+                                                               const int64_t* __restrict__ ctr, int gen_max,
+                                                               char* gws, size_t slice) {
+  after_previous();
+  before_next();
+  extern __shared__ __align__(16) char sbuf[];
+  __shared__ int64_t red[BlockTeam<kBigThreads>::kRedSlots];
+  __shared__ SelOut sel;
+  BlockTeam<kBigThreads> tm(red);
+  const ClassList cl = class_list(c, lists, ctr, 8);
+  for (int64_t q = blockIdx.x; q < cl.len; q += gridDim.x) {
+    const int64_t t = cl.list[q];
+    const TradeRows tr = trade_rows(c, t);
+    const int L = tr.du + tr.dv;
+    bool ok;
+    if (L <= min(HugeWs::kLmax, gen_max)) {
+      ok = phase_a_reg<BlockTeam<kBigThreads>, 8, 12, false, kOneSeed>(tm, c, t, HugeWs{sbuf});
+    } else {
+      if (threadIdx.x == 0) atomicAdd(c.gws_count, 1ull);
+      ok = phase_a<BlockTeam<kBigThreads>, kOneSeed>(tm, c, t, carve_split(sbuf, kSplitSmem, gws + slice * blockIdx.x, L),
+                                                    &sel);
+    }
+    if (!ok && threadIdx.x == 0) defer_trade(c, t);
+  }
+}
+
 __global__ void __launch_bounds__(32 * kWarpWarps, 4) k_retry_warp(StepCtx c, const int32_t* __restrict__ list,
                                                                 const unsigned long long* __restrict__ count,
                                                                 unsigned long long* claim) {
@@ -2139,6 +2178,8 @@ int init_seed_kernels(Graph* h) {
   if ((rc = of_class(Int<0>{})) || (rc = of_class(Int<1>{})) || (rc = of_class(Int<2>{})) || (rc = of_class(Int<3>{})) ||
       (rc = of_class(Int<4>{})) || (rc = of_class(Int<5>{})) || (rc = of_class(Int<6>{})) || (rc = of_class(Int<7>{})))
     return rc;
+  CB_CUDA(h, cudaFuncSetAttribute(k_phase_a_huge<kOneSeed>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                  static_cast<int>(kSplitSmem)));
   CB_CUDA(h, cudaFuncSetAttribute(k_phase_a_large<kOneSeed>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                   static_cast<int>(kLargeSmem)));
   CB_CUDA(h, cudaFuncSetAttribute(k_phase_a_small<kOneSeed>, cudaFuncAttributeMaxDynamicSharedMemorySize,
@@ -2357,11 +2398,16 @@ int super_step(Graph* h) {
       return r;
     }
     if ((r = mark(8))) return r;
-    // the largest trades: 1024 threads, up to smem_max entries in shared
-    // memory (staged by a bulk copy), a global-memory slice above
+    // the largest trades: in registers up to 8192 entries, the hash in shared
+    // memory above; without the register kernels up to smem_max entries in
+    // shared memory, staged by a bulk copy
     if (max_trade > th.th[7]) {
-      CB_CUDA(h, launch(overlap, k_phase_a_block<kBigThreads, kOne>, bgrid, kBigThreads, big_smem_st, s, c, L, cnt, 8,
-                        h->smem_max, room_of(big_smem_st, h->smem_max), gws, h->ws_slice, h->smem_max));
+      if (h->cta_paths)
+        CB_CUDA(h, launch(overlap, k_phase_a_huge<kOne>, bgrid, kBigThreads, kSplitSmem, s, c, L, cnt, h->smem_max, gws,
+                          h->ws_slice));
+      else
+        CB_CUDA(h, launch(overlap, k_phase_a_block<kBigThreads, kOne>, bgrid, kBigThreads, big_smem_st, s, c, L, cnt, 8,
+                          h->smem_max, room_of(big_smem_st, h->smem_max), gws, h->ws_slice, h->smem_max));
       if ((r = launched())) return r;
     }
     return mark(9);

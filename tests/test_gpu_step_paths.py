@@ -152,19 +152,20 @@ def test_malformed_graphs_are_refused(n, what, shuffled):
     assert err.value.code == CB_EINVAL
 
 
-# Trades above smem_max keep their hash in shared memory up to 26214 entries,
-# with key prefixes and flags beside it up to about 18000 (16384 in the first
+# Trades of 4097 to 8192 entries run with eight entries per thread; above, or
+# above smem_max, they keep their hash in shared memory up to 26214
+# entries, with key prefixes and flags beside it up to about 18000 (16384 in the first
 # pass's kernel); above, all of it is in global memory.  Hubs on both sides of
 # these limits, adjacent to each other so that their trades depend on one
 # another; smem_max 64 sends every trade above 64 entries the same way.
 @pytest.mark.parametrize("options", [{}, {"inorder_threads": 256}, {"smem_max": 64}, {"smem_max": 2000, "cta_paths": 0}])
-def test_trades_above_shared_memory(options):
+def test_trades_of_the_largest_class(options):
     n = 40000
     rng = np.random.default_rng(5)
     g = synth.powerlaw_graph(n, 2, 30, 2.0, 12)
     rows = np.repeat(np.arange(n, dtype=np.int64), np.diff(g.row_ptr))
     pairs = [np.stack([rows, g.col.astype(np.int64)], 1)]
-    for hub, d in enumerate([8185, 8300, 12000, 15990, 16400, 17700, 20000, 26190, 26240, 30000]):
+    for hub, d in enumerate([4085, 4200, 8185, 8300, 12000, 15990, 16400, 17700, 20000, 26190, 26240, 30000]):
         pairs.append(np.stack([np.full(d, hub), rng.permutation(n)[:d]], 1))
     e = np.concatenate(pairs)
     e = e[e[:, 0] != e[:, 1]]
