@@ -1416,11 +1416,11 @@ struct LaneCfg {
 // threads (named barriers), each running one trade at a time with kTeamJ
 // entries per thread in registers (L <= NT kTeamJ).
 constexpr int kTeamJ = 4;
-template <int NT>
+template <int NT, int J = kTeamJ, int SLOTS = 4>
 struct TeamCfg {
   static constexpr int B = NT == 64 ? 8 : NT == 128 ? 9 : NT == 256 ? 10 : NT == 512 ? 11 : 12;   // ~1 bin per entry
-  using Ws = RegWs<NT * kTeamJ, B, kCand>;
-  static constexpr int kMax = NT * kTeamJ;
+  using Ws = RegWs<NT * J, B, kCand, SLOTS>;
+  static constexpr int kMax = NT * J;
 };
 // The first pass of a handle of fewer than kFuseMax trades runs classes 0 to 5
 // in one kernel, and 6 and 7 in another.  A class's trades are cut into CTA
@@ -1468,44 +1468,55 @@ __device__ void run_warps(const StepCtx& c, const ClassList& cl, char* smem, Rou
     if (!phase_a_reg<WarpTeam, kWarpJ, kWarpB, true, kOneSeed>(tm, c, cl.list[q], w) && tm.rank == 0)
       defer_trade(c, cl.list[q]);
 }
-template <int CT, int NT, bool kOneSeed>
+template <int CT, int NT, bool kOneSeed, int J = kTeamJ, int SLOTS = 4>
 __device__ void run_teams(const StepCtx& c, const ClassList& cl, char* smem, int64_t* red, Rounds& rs) {
   constexpr int kTeams = CT / NT;
-  using Ws = typename TeamCfg<NT>::Ws;
+  using Cfg = TeamCfg<NT, J, SLOTS>;
+  using Ws = typename Cfg::Ws;
   const int id = threadIdx.x / NT;
   SubTeam<NT> tm(red + id * SubTeam<NT>::kRedSlots, id);
   const Ws w{smem + Ws::kBytes * id};
   const int64_t step = static_cast<int64_t>(gridDim.x) * kTeams;
   for (int64_t q = rs.first((cl.len + kTeams - 1) / kTeams) * kTeams + id; q < cl.len; q += step)
-    if (!phase_a_reg<SubTeam<NT>, kTeamJ, TeamCfg<NT>::B, false, kOneSeed>(tm, c, cl.list[q], w) && tm.rank == 0)
+    if (!phase_a_reg<SubTeam<NT>, J, Cfg::B, false, kOneSeed>(tm, c, cl.list[q], w) && tm.rank == 0)
       defer_trade(c, cl.list[q]);
 }
 
-// Class K alone.
+// Class K alone.  Instruction issue bounds these kernels (55 to 64 % of the
+// slots, no memory level above 25 %).  Trades of more than 256 entries run with
+// eight entries per member on teams of half the size, which halves what a
+// trade costs whatever its size (clearing, scans, the threshold search) and its
+// barriers; two hash slots per entry keep four CTAs on an SM.  n=2^25, degrees
+// [10,10000), ms per step with four and eight: 257 to 512 entries 3.90 and
+// 3.65, to 1024 3.74 and 3.14, to 2048 3.56 and 3.05, to 4096 3.65 and 3.13.  On
+// lanes and warps eight cost more than they save (class 0 2.98 and 4.24, 1
+// 4.38 and 5.79, 2 3.98 and 5.33, 3 4.40 and 4.09 to 4.52): the bins are twice as
+// full, and the rolled loops over their elements run in lockstep.
 template <int K>
-constexpr size_t class_smem() {
-  return K == 0 ? LaneCfg<8>::kSmem : K == 1 ? LaneCfg<16>::kSmem : K == 2 ? WarpWs::kBytes * kWarpWarps
-         : K == 3 ? TeamCfg<64>::Ws::kBytes * 4 : K == 4 ? TeamCfg<128>::Ws::kBytes * 2
-         : K == 5 ? TeamCfg<256>::Ws::kBytes : K == 6 ? TeamCfg<512>::Ws::kBytes * 2 : TeamCfg<1024>::Ws::kBytes;
-}
+struct ClassCfg {
+  static constexpr int kJ = K < 4 ? 4 : 8, kSlots = K < 4 ? 4 : 2;
+  static constexpr int kTeam = (32 << K) / kJ;            // threads per trade
+  static constexpr int kThreads = K < 7 ? 256 : 512;      // per CTA
+  static constexpr int kCtas = 4 * 256 / kThreads;        // per SM
+  static constexpr size_t smem() {
+    if constexpr (K < 2) return LaneCfg<kTeam>::kSmem;
+    else if constexpr (K == 2) return WarpWs::kBytes * kWarpWarps;
+    else return TeamCfg<kTeam, kJ, kSlots>::Ws::kBytes * (kThreads / kTeam);
+  }
+};
 template <int K, bool kOneSeed>
-__global__ void __launch_bounds__(K < 6 ? 256 : kBigThreads, K < 6 ? 4 : 1) k_phase_a_class(StepCtx c,
-                                                                const int32_t* __restrict__ lists,
-                                                                const int64_t* __restrict__ ctr) {
+__global__ void __launch_bounds__(ClassCfg<K>::kThreads, ClassCfg<K>::kCtas)
+    k_phase_a_class(StepCtx c, const int32_t* __restrict__ lists, const int64_t* __restrict__ ctr) {
   after_previous();
   before_next();
+  using Cfg = ClassCfg<K>;
   extern __shared__ __align__(16) char smem[];
-  __shared__ int64_t red[K < 3 ? 1 : K < 6 ? 4 * SubTeam<64>::kRedSlots : SubTeam<kBigThreads>::kRedSlots];
+  __shared__ int64_t red[K < 3 ? 1 : Cfg::kThreads / 16];   // two slots per warp
   Rounds rs;
   const ClassList cl = class_list(c, lists, ctr, K);
-  if constexpr (K == 0) run_lanes<8, kOneSeed>(c, cl, smem, rs);
-  else if constexpr (K == 1) run_lanes<16, kOneSeed>(c, cl, smem, rs);
+  if constexpr (K < 2) run_lanes<Cfg::kTeam, kOneSeed>(c, cl, smem, rs);
   else if constexpr (K == 2) run_warps<kOneSeed>(c, cl, smem, rs);
-  else if constexpr (K == 3) run_teams<256, 64, kOneSeed>(c, cl, smem, red, rs);
-  else if constexpr (K == 4) run_teams<256, 128, kOneSeed>(c, cl, smem, red, rs);
-  else if constexpr (K == 5) run_teams<256, 256, kOneSeed>(c, cl, smem, red, rs);
-  else if constexpr (K == 6) run_teams<kBigThreads, 512, kOneSeed>(c, cl, smem, red, rs);
-  else run_teams<kBigThreads, kBigThreads, kOneSeed>(c, cl, smem, red, rs);
+  else run_teams<Cfg::kThreads, Cfg::kTeam, kOneSeed, Cfg::kJ, Cfg::kSlots>(c, cl, smem, red, rs);
 }
 
 // Classes 0 to 5 (without the lane teams or the teams where an option sends
@@ -2169,7 +2180,7 @@ int init_seed_kernels(Graph* h) {
   auto of_class = [&](auto k) -> int {
     constexpr int K = decltype(k)::value;
     CB_CUDA(h, cudaFuncSetAttribute(k_phase_a_class<K, kOneSeed>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                    static_cast<int>(class_smem<K>())));
+                                    static_cast<int>(ClassCfg<K>::smem())));
     CB_CUDA(h, cudaFuncSetAttribute(k_phase_a_class<K, kOneSeed>, cudaFuncAttributePreferredSharedMemoryCarveout,
                                     cudaSharedmemCarveoutMaxShared));
     return CB_OK;
@@ -2365,8 +2376,9 @@ int super_step(Graph* h) {
       int rk;
       if ((rk = mark(K))) return rk;
       if ((K > 0 && max_trade <= th.th[K > 0 ? K - 1 : 0]) || (K < 2 && !h->lane_teams)) return CB_OK;
-      const unsigned grid = K < 3 ? wgrid : K < 6 ? mgrid : static_cast<unsigned>(h->num_sms);
-      CB_CUDA(h, launch(overlap, k_phase_a_class<K, kOne>, grid, K < 6 ? 256 : kBigThreads, class_smem<K>(), s, c, L, cnt));
+      using Cfg = ClassCfg<K>;
+      const unsigned grid = static_cast<unsigned>(h->num_sms * (K < 3 ? 8 : Cfg::kCtas));
+      CB_CUDA(h, launch(overlap, k_phase_a_class<K, kOne>, grid, Cfg::kThreads, Cfg::smem(), s, c, L, cnt));
       return launched();
     };
     if (fused) {
