@@ -265,6 +265,12 @@ int alloc_arrays(Graph* h) {
     take(&h->far_pack, h->ntasks);
     take(&h->lists, kClasses * h->ntasks);
     take(&h->def_list, 3 * h->ntasks + 2);
+    if (small_permutation(h)) {
+      take(&h->order2, n);
+      take(&h->pos2, n);
+      take(&h->rp2, n + 1);
+      take(&h->chunk_row2, nnz / kRowChunk + 2);
+    }
   };
   layout();
   if (dmalloc(h, reinterpret_cast<void**>(&base), used)) return fail(h, CB_ENOMEM, "device allocation failed");
@@ -379,6 +385,34 @@ int capture_step_graphs(Graph* h) {
   return rc;
 }
 
+// The slots of the current, the next and the third set, put back: a and b first.
+template <class T>
+void settle(T** cur_slot, T** next_slot, T** third, T* a, T* b) {
+  T* const all[3] = {*cur_slot, *next_slot, *third};
+  T* rest = nullptr;
+  for (T* p : all)
+    if (p != a && p != b) rest = p;
+  *cur_slot = a;
+  *next_slot = b;
+  *third = rest;
+}
+
+// After steps that ran ahead: the current step's order, positions and offsets
+// where the same number of plain steps leaves them, so that recorded steps
+// stay valid.
+int settle_sets(Graph* h, int32_t* const orders[2], int32_t* const poss[2], int64_t* const rps[2]) {
+  const int cur = h->cur;
+  if (h->order[cur] != orders[cur]) {   // into a set that holds nothing any more
+    CB_CUDA(h, cudaMemcpyAsync(orders[cur], h->order[cur], sizeof(int32_t) * h->n, cudaMemcpyDeviceToDevice, h->stream));
+    CB_CUDA(h, cudaMemcpyAsync(poss[cur], h->pos[cur], sizeof(int32_t) * h->n, cudaMemcpyDeviceToDevice, h->stream));
+    CB_CUDA(h, cudaMemcpyAsync(rps[cur], h->rp[cur], sizeof(int64_t) * (h->n + 1), cudaMemcpyDeviceToDevice, h->stream));
+  }
+  settle(&h->order[cur], &h->order[1 - cur], &h->order2, orders[cur], orders[1 - cur]);
+  settle(&h->pos[cur], &h->pos[1 - cur], &h->pos2, poss[cur], poss[1 - cur]);
+  settle(&h->rp[cur], &h->rp[1 - cur], &h->rp2, rps[cur], rps[1 - cur]);
+  return CB_OK;
+}
+
 // Every graph's canonical pairs (local ids) of the current step in h->pairs.
 int ensure_pairs(Graph* h) {
   if (h->pairs && h->pairs_step == h->g) return CB_OK;
@@ -459,6 +493,7 @@ int64_t estimate_handle_bytes(int64_t n, int64_t nnz, int64_t maxdeg, int num_sm
   b += sizeof(Seg) + 8 * (n + 1) + 4 * n + 2 * 4 * (nnz + kColPad) + 32 + 8 * (2 * kCounters + 1 + kScratch);   // cb_create
   b += 2 * 4 * n + 2 * 8 * (n + 1) + 2 * 4 * n + 2 * nnz + 4 * (nnz / kRowChunk + 2);                                 // per node, side words
   b += ntasks * (8 + 8 + 4 + 16 + 4 * kClasses + 4 * 3) + ntasks / 8 + 4 * 3 * kDefSegs + 16;                                  // per trade
+  if (ntasks < kOverlapMax) b += 2 * 4 * n + 8 * (n + 1) + 4 * (nnz / kRowChunk + 2);
   b += static_cast<int64_t>(perm_ws_bytes(nb, nb * bucket_space(n, bucket_bits(n))) + scan_ws_bytes(n + 1));
   const int64_t max_trade = 2 * maxdeg;
   if (max_trade > kBlockMaxDefault || maxdeg > 16384) {   // default block_max
@@ -690,10 +725,21 @@ int cb_global_trades(cb_handle h, uint32_t supersteps) {
       h->launches += h->step_launches;
     }
   } else {
+    const bool ahead = supersteps > 1 && runs_ahead(h);
+    int32_t* const orders[2] = {h->order[0], h->order[1]};
+    int32_t* const poss[2] = {h->pos[0], h->pos[1]};
+    int64_t* const rps[2] = {h->rp[0], h->rp[1]};
     for (uint32_t i = 0; i < supersteps; ++i) {
-      int rc = super_step(h);
+      int rc = super_step(h, ahead && i + 1 < supersteps);
       if (!rc && h->swap_stats) rc = count_swaps(h);
       if (!rc && h->pres) rc = record_presence(h);
+      if (rc) {
+        if (ahead) h->latched = rc;   // the sets are where recorded steps do not look for them
+        return rc;
+      }
+    }
+    if (ahead) {
+      const int rc = settle_sets(h, orders, poss, rps);
       if (rc) return rc;
     }
   }

@@ -106,6 +106,11 @@ struct Graph {
   int32_t* chunk_row = nullptr;            // row of every kRowChunk-th entry of the offsets last computed
   int32_t* col[2] = {nullptr, nullptr};    // position-space rows, ascending
   int32_t* pos[2] = {nullptr, nullptr};    // position of each node (pos[1 - cur] is scratch between steps)
+  int32_t* order2 = nullptr;               // third set (small handles; else null): the step after next's, when
+  int32_t* pos2 = nullptr;                 // computed ahead; then set 1 - cur is the next step's between steps
+  int64_t* rp2 = nullptr;
+  int32_t* chunk_row2 = nullptr;
+  bool ahead = false;                      // set 1 - cur and the class lists are computed
   uint16_t* stash = nullptr;               // per placed entry (step g+1 layout): bit0 own flip, bits 1.. far key prefix
   uint64_t* thr_key = nullptr;             // per trade: threshold key
   uint64_t* thr_tb = nullptr;              // per trade: threshold tie-break (lo<<32|hi)
@@ -195,6 +200,11 @@ int cuda_fail(Graph* g, cudaError_t e, const char* what);
     if (e_ != cudaSuccess) return ::cb::cuda_fail((g), e_, #call); \
   } while (0)
 
+// Overlapped launches: step time without -> with, n=2^12 88 -> 80 us, 2^14 166
+// -> 160, 2^15 187 -> 184, but 2^16 214 -> 219 and 2^18 436 -> 543 (waiting CTAs
+// take the place of running ones).
+constexpr int64_t kOverlapMax = int64_t(1) << 15;
+
 // Overlapped launches (programmatic dependent launch): a kernel launched with
 // overlap = true may be set up while the kernel before it in the stream still
 // runs, so its launch costs no idle time; its first statement has to be
@@ -238,7 +248,8 @@ int64_t bucket_space(int64_t span, int B);
 // its device step counter + dg, or the step g_abs for all when g_abs >= 0.
 // classes (may be null): build the size-class lists of the current step too.
 int compute_permutation(Graph* h, uint32_t dg, int64_t g_abs, int32_t* order_out, int32_t* pos_out, int64_t* rp_out,
-                        const ClassArgs* classes);
+                        const ClassArgs* classes, bool beside = false);   // beside: see k_perm_rescan
+bool small_permutation(const Graph* h);   // one kernel, overlapped launches
 size_t perm_zero_bytes(int64_t nbuckets);   // the start of its scratch that has to be zero at first
 
 // rows.cu
@@ -272,7 +283,10 @@ int relabel_rows(Graph* h, int64_t nrows, const int64_t* src_rp, const int32_t* 
 int export_sorted_pairs(Graph* h, int32_t* pairs);
 
 // trade.cu
-int super_step(Graph* h);
+// ahead: another step of the same call follows and compute its permutation
+// beside this step's in-order pass (handles that runs_ahead() allows)
+int super_step(Graph* h, bool ahead = false);
+bool runs_ahead(const Graph* h);
 int flush_timing(Graph* h, int set, bool add);   // wait for a recorded event set; add it to phase_ms
 int init_trade_kernels(Graph* h);   // one-time kernel attributes (outside stream capture)
 int init_perm_kernels(Graph* h);

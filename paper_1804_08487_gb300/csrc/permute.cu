@@ -363,11 +363,8 @@ constexpr uint64_t kDegMask = (uint64_t(1) << kCountShift) - 1;
 // the next keys do not wait for the last ones (a permutation of 4096 nodes on
 // its own: 12.3 us per call with 256 threads, 10.2 so).
 constexpr int kRescanThreads = 1024;
-__global__ void __launch_bounds__(kRescanThreads) k_perm_rescan(int64_t n, int nseg, KeySrc ks, int nb, int cap,
-                                                               PermOut out, const int64_t* __restrict__ rp_id,
-                                                               int64_t nnz, ClassArgs ca) {
-  after_previous();
-  before_next();
+__device__ void perm_rescan(int64_t n, int nseg, const KeySrc& ks, int nb, int cap, const PermOut& out,
+                            const int64_t* __restrict__ rp_id, int64_t nnz, const ClassArgs& ca) {
   extern __shared__ uint64_t shk[];
   __shared__ int cnt;
   __shared__ int64_t wsum[kRescanThreads / 32];
@@ -418,6 +415,17 @@ __global__ void __launch_bounds__(kRescanThreads) k_perm_rescan(int64_t n, int n
         },
         s, p0, e0, out);
   }
+}
+// beside: the kernel before it, the in-order pass, has started but may still
+// run (it uses few SMs, and nothing that this kernel writes); the kernel after
+// has to find both complete, so the wait comes last.
+__global__ void __launch_bounds__(kRescanThreads) k_perm_rescan(int64_t n, int nseg, KeySrc ks, int nb, int cap,
+                                                               PermOut out, const int64_t* __restrict__ rp_id,
+                                                               int64_t nnz, ClassArgs ca, bool beside) {
+  if (!beside) after_previous();
+  before_next();
+  perm_rescan(n, nseg, ks, nb, cap, out, rp_id, nnz, ca);
+  if (beside) after_previous();
 }
 // 2^21 keys are 64 buckets of a 2^15-node graph: 128 keys per thread.
 constexpr int64_t kRescanWork = int64_t(1) << 21;
@@ -606,8 +614,12 @@ int bucket_cap_of(const Graph* h) {
 }
 }  // namespace
 
+bool small_permutation(const Graph* h) {
+  return h->n > 0 && h->nnz > 0 && small_handle(h) && h->nbuckets <= kRescanBuckets && rescan_work(h) <= kRescanWork;
+}
+
 int compute_permutation(Graph* h, uint32_t dg, int64_t g_abs, int32_t* order_out, int32_t* pos_out, int64_t* rp_out,
-                        const ClassArgs* classes) {
+                        const ClassArgs* classes, bool beside) {
   const int64_t n = h->n;
   if (n == 0) return CB_OK;
   cudaStream_t s = h->stream;
@@ -646,12 +658,12 @@ int compute_permutation(Graph* h, uint32_t dg, int64_t g_abs, int32_t* order_out
   ks.seg_of = h->seg_of;
   const int64_t nb = h->nbuckets;
   const int cap = bucket_cap_of(h);
-  const PermOut out{order_out, pos_out, rp_out, h->deg_id, rp_out ? h->chunk_row : nullptr};
+  const PermOut out{order_out, pos_out, rp_out, h->deg_id, !rp_out ? nullptr : beside ? h->chunk_row2 : h->chunk_row};
   if (nb <= kRescanBuckets && rescan_work(h) <= kRescanWork) {
     const unsigned grid = static_cast<unsigned>(
         nb + std::min<int64_t>(class_chunks(ca.ntasks, kRescanThreads), int64_t(h->num_sms) * 2));
     CB_CUDA(h, launch(small_handle(h), k_perm_rescan, grid, kRescanThreads, bucket_smem_bytes(cap), s, n, h->nseg, ks,
-                      static_cast<int>(nb), cap, out, h->rp_id, h->nnz, ca));
+                      static_cast<int>(nb), cap, out, h->rp_id, h->nnz, ca, beside));
     ++h->launches;
     return CB_OK;
   }
@@ -732,7 +744,7 @@ extern "C" int cb_permutation_static(int64_t n, uint64_t seed, uint64_t g, int32
   const int cap = static_cast<int>(std::min<int64_t>(space, 2048));
   const ClassArgs none{};
   if (n * nb <= kRescanWork) {   // no scratch at all
-    k_perm_rescan<<<nb, kRescanThreads, bucket_smem_bytes(cap), s>>>(n, 1, ks, nb, cap, out, nullptr, 0, none);
+    k_perm_rescan<<<nb, kRescanThreads, bucket_smem_bytes(cap), s>>>(n, 1, ks, nb, cap, out, nullptr, 0, none, false);
     if ((e = cudaGetLastError()) != cudaSuccess) return cuda_fail(nullptr, e, "k_perm_rescan");
     return CB_OK;
   }

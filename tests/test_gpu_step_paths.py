@@ -183,3 +183,58 @@ def test_trades_of_the_largest_class(options):
         assert np.array_equal(c.edges(), o.edges())
     assert c.stats()["global_ws_trades"] > 0
     c.close()
+
+
+# Steps of one call on small handles compute the next permutation beside the
+# in-order pass, in a third set of arrays: calls of different lengths, single
+# steps, recorded steps and other uses of the handle between them.
+@pytest.mark.parametrize("n,b", [(9, 5), (1025, 60), (4096, 200), (5001, 2000), (32769, 30), (65534, 12)])
+def test_calls_of_several_steps(n, b):
+    g = synth.powerlaw_graph(n, 1, max(2, b), 2.0, 23)
+    c, o = Curveball(g.row_ptr, g.col, 7), Oracle(g.row_ptr, g.col, 7)
+    for i, k in enumerate([1, 2, 3, 1, 4, 5, 6, 2, 2, 7]):
+        if i == 4:
+            c.set_option("cuda_graph", 1)
+        if i == 6:
+            c.set_option("cuda_graph", 0)
+        if i == 8:
+            c.set_option("relaxed", 1)
+            o.set_relaxed(True)
+        if i == 9:
+            c.set_option("relaxed", 0)
+            o.set_relaxed(False)
+        c.global_trades(k)
+        o.superstep(k)
+        assert np.array_equal(c.edges(), o.edges()), f"after call {i} of {k} steps"
+        if i % 3 == 0 and n > 1:
+            c.uniform_trades(n)
+            o.uniform_trades(n)
+        if i == 5:
+            c.set_option("cuda_graph", 1)
+            c.global_trades(1)
+            o.superstep(1)
+            c.set_option("cuda_graph", 0)
+            c.global_trades(4)
+            o.superstep(4)
+            c.set_option("cuda_graph", 1)
+            c.global_trades(3)
+            o.superstep(3)
+            assert np.array_equal(c.edges(), o.edges())
+    c.close()
+
+
+@pytest.mark.parametrize("sizes", [(3, 1, 0, 2), (1023, 1024, 1025, 9), (9000, 12001, 700)])
+def test_batch_calls_of_several_steps(sizes):
+    graphs = []
+    for n in sizes:
+        g = synth.powerlaw_graph(n, 2, min(n // 2, 60), 2.0, n) if n >= 4 else None
+        graphs.append((g.row_ptr, g.col) if g else (np.zeros(n + 1, np.int64), np.zeros(0, np.int32)))
+    seeds = [5 + i for i in range(len(graphs))]
+    e = Ensemble(graphs, seeds)
+    oracles = [Oracle(rp, col, s) for (rp, col), s in zip(graphs, seeds)]
+    for k in (2, 3, 1, 5):
+        e.global_trades(k)
+        for i, o in enumerate(oracles):
+            o.superstep(k)
+            assert np.array_equal(e.graph_edges(i), o.edges())
+    e.close()
