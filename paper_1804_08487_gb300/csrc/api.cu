@@ -265,7 +265,7 @@ int alloc_arrays(Graph* h) {
     take(&h->far_pack, h->ntasks);
     take(&h->lists, kClasses * h->ntasks);
     take(&h->def_list, 3 * h->ntasks + 2);
-    if (small_permutation(h)) {
+    if (may_run_ahead(h->ntasks, nnz)) {
       take(&h->order2, n);
       take(&h->pos2, n);
       take(&h->rp2, n + 1);
@@ -493,7 +493,7 @@ int64_t estimate_handle_bytes(int64_t n, int64_t nnz, int64_t maxdeg, int num_sm
   b += sizeof(Seg) + 8 * (n + 1) + 4 * n + 2 * 4 * (nnz + kColPad) + 32 + 8 * (2 * kCounters + 1 + kScratch);   // cb_create
   b += 2 * 4 * n + 2 * 8 * (n + 1) + 2 * 4 * n + 2 * nnz + 4 * (nnz / kRowChunk + 2);                                 // per node, side words
   b += ntasks * (8 + 8 + 4 + 16 + 4 * kClasses + 4 * 3) + ntasks / 8 + 4 * 3 * kDefSegs + 16;                                  // per trade
-  if (ntasks < kOverlapMax) b += 2 * 4 * n + 8 * (n + 1) + 4 * (nnz / kRowChunk + 2);
+  if (may_run_ahead(ntasks, nnz)) b += 2 * 4 * n + 8 * (n + 1) + 4 * (nnz / kRowChunk + 2);
   b += static_cast<int64_t>(perm_ws_bytes(nb, nb * bucket_space(n, bucket_bits(n))) + scan_ws_bytes(n + 1));
   const int64_t max_trade = 2 * maxdeg;
   if (max_trade > kBlockMaxDefault || maxdeg > 16384) {   // default block_max
@@ -712,7 +712,10 @@ int cb_global_trades(cb_handle h, uint32_t supersteps) {
     if (rc) return rc;
   }
   for (double& v : h->phase_ms) v = 0;
-  if (h->use_graph && !h->timing && !h->swap_stats && !h->pres && supersteps > 0) {
+  // recorded steps save small handles host time; larger ones gain more from
+  // running ahead, which a recorded single step cannot
+  const bool ahead = supersteps > 1 && runs_ahead(h);
+  if (h->use_graph && !h->timing && !h->swap_stats && !h->pres && supersteps > 0 && !(ahead && !small_handle(h))) {
     if (!h->step_exec[0]) {
       const int rc = capture_step_graphs(h);
       if (rc) return rc;
@@ -725,7 +728,6 @@ int cb_global_trades(cb_handle h, uint32_t supersteps) {
       h->launches += h->step_launches;
     }
   } else {
-    const bool ahead = supersteps > 1 && runs_ahead(h);
     int32_t* const orders[2] = {h->order[0], h->order[1]};
     int32_t* const poss[2] = {h->pos[0], h->pos[1]};
     int64_t* const rps[2] = {h->rp[0], h->rp[1]};

@@ -106,7 +106,7 @@ struct Graph {
   int32_t* chunk_row = nullptr;            // row of every kRowChunk-th entry of the offsets last computed
   int32_t* col[2] = {nullptr, nullptr};    // position-space rows, ascending
   int32_t* pos[2] = {nullptr, nullptr};    // position of each node (pos[1 - cur] is scratch between steps)
-  int32_t* order2 = nullptr;               // third set (small handles; else null): the step after next's, when
+  int32_t* order2 = nullptr;               // third set (may_run_ahead(); else null): the step after next's, when
   int32_t* pos2 = nullptr;                 // computed ahead; then set 1 - cur is the next step's between steps
   int64_t* rp2 = nullptr;
   int32_t* chunk_row2 = nullptr;
@@ -249,7 +249,6 @@ int64_t bucket_space(int64_t span, int B);
 // classes (may be null): build the size-class lists of the current step too.
 int compute_permutation(Graph* h, uint32_t dg, int64_t g_abs, int32_t* order_out, int32_t* pos_out, int64_t* rp_out,
                         const ClassArgs* classes, bool beside = false);   // beside: see k_perm_rescan
-bool small_permutation(const Graph* h);   // one kernel, overlapped launches
 size_t perm_zero_bytes(int64_t nbuckets);   // the start of its scratch that has to be zero at first
 
 // rows.cu
@@ -286,6 +285,7 @@ int export_sorted_pairs(Graph* h, int32_t* pairs);
 // ahead: another step of the same call follows and compute its permutation
 // beside this step's in-order pass (handles that runs_ahead() allows)
 int super_step(Graph* h, bool ahead = false);
+bool may_run_ahead(int64_t ntasks, int64_t nnz);
 bool runs_ahead(const Graph* h);
 int flush_timing(Graph* h, int set, bool add);   // wait for a recorded event set; add it to phase_ms
 int init_trade_kernels(Graph* h);   // one-time kernel attributes (outside stream capture)

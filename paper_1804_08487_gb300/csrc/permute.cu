@@ -431,14 +431,14 @@ __global__ void __launch_bounds__(kRescanThreads) k_perm_rescan(int64_t n, int n
 constexpr int64_t kRescanWork = int64_t(1) << 21;
 constexpr int64_t kRescanBuckets = 4096;   // CTAs
 
-// Node ids into their buckets; the last CTA to finish turns the bucket words
+// Node ids into their buckets (beside: as k_perm_rescan); the last CTA to finish turns the bucket words
 // into their exclusive prefix sums and clears them for the next call.
 __global__ void __launch_bounds__(kPermThreads) k_perm_scatter(int64_t n, KeySrc ks, int nb,
                                                               const int32_t* __restrict__ deg,
                                                               unsigned long long* __restrict__ words,
                                                               uint64_t* __restrict__ prefix, int* __restrict__ ticket,
-                                                              int32_t* __restrict__ bid, ClassArgs ca) {
-  after_previous();
+                                                              int32_t* __restrict__ bid, ClassArgs ca, bool beside) {
+  if (!beside) after_previous();
   before_next();
   __shared__ int64_t wsum[kPermThreads / 32];
   __shared__ int last;
@@ -487,6 +487,7 @@ __global__ void __launch_bounds__(kPermThreads) k_perm_scatter(int64_t n, KeySrc
     prefix[nb] = run;
     *ticket = 0;
   }
+  if (beside) after_previous();   // (the other CTAs need not stay)
 }
 
 __global__ void __launch_bounds__(kPermThreads) k_bucket_sort(int64_t n, int nseg, KeySrc ks, int nb, int cap,
@@ -614,10 +615,6 @@ int bucket_cap_of(const Graph* h) {
 }
 }  // namespace
 
-bool small_permutation(const Graph* h) {
-  return h->n > 0 && h->nnz > 0 && small_handle(h) && h->nbuckets <= kRescanBuckets && rescan_work(h) <= kRescanWork;
-}
-
 int compute_permutation(Graph* h, uint32_t dg, int64_t g_abs, int32_t* order_out, int32_t* pos_out, int64_t* rp_out,
                         const ClassArgs* classes, bool beside) {
   const int64_t n = h->n;
@@ -662,14 +659,14 @@ int compute_permutation(Graph* h, uint32_t dg, int64_t g_abs, int32_t* order_out
   if (nb <= kRescanBuckets && rescan_work(h) <= kRescanWork) {
     const unsigned grid = static_cast<unsigned>(
         nb + std::min<int64_t>(class_chunks(ca.ntasks, kRescanThreads), int64_t(h->num_sms) * 2));
-    CB_CUDA(h, launch(small_handle(h), k_perm_rescan, grid, kRescanThreads, bucket_smem_bytes(cap), s, n, h->nseg, ks,
+    CB_CUDA(h, launch(beside || small_handle(h), k_perm_rescan, grid, kRescanThreads, bucket_smem_bytes(cap), s, n, h->nseg, ks,
                       static_cast<int>(nb), cap, out, h->rp_id, h->nnz, ca, beside));
     ++h->launches;
     return CB_OK;
   }
   const PermWs w = carve(h->sort_ws, nb);
-  CB_CUDA(h, launch(small_handle(h), k_perm_scatter, grid_for(n, kPermThreads, h->num_sms), kPermThreads, 0, s, n, ks,
-                    static_cast<int>(nb), rp_out ? h->deg_id : nullptr, w.words, w.prefix, w.ticket, w.bid, ca));
+  CB_CUDA(h, launch(beside || small_handle(h), k_perm_scatter, grid_for(n, kPermThreads, h->num_sms), kPermThreads, 0, s, n, ks,
+                    static_cast<int>(nb), rp_out ? h->deg_id : nullptr, w.words, w.prefix, w.ticket, w.bid, ca, beside));
   const unsigned sgrid = static_cast<unsigned>(nb < h->num_sms * 8 ? nb : h->num_sms * 8);
   CB_CUDA(h, launch(small_handle(h), k_bucket_sort, sgrid, kPermThreads, bucket_smem_bytes(cap), s, n, h->nseg, ks,
                     static_cast<int>(nb), cap, w.prefix, w.bid, out, h->nnz));
@@ -752,7 +749,7 @@ extern "C" int cb_permutation_static(int64_t n, uint64_t seed, uint64_t g, int32
   const PermWs w = carve(base, nb);
   if ((e = cudaMemsetAsync(base, 0, zero_bytes(nb), s)) != cudaSuccess) return cuda_fail(nullptr, e, "cudaMemsetAsync");
   k_perm_scatter<<<grid_for(n, kPermThreads, num_sms), kPermThreads, 0, s>>>(n, ks, nb, nullptr, w.words, w.prefix,
-                                                                            w.ticket, w.bid, none);
+                                                                            w.ticket, w.bid, none, false);
   if ((e = cudaGetLastError()) != cudaSuccess) return cuda_fail(nullptr, e, "k_perm_scatter");
   const unsigned sgrid = static_cast<unsigned>(nb < num_sms * 8 ? nb : num_sms * 8);
   k_bucket_sort<<<sgrid, kPermThreads, bucket_smem_bytes(cap), s>>>(n, 1, ks, nb, cap, w.prefix, w.bid, out, 0);

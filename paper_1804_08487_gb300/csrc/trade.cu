@@ -2245,9 +2245,13 @@ bool small_handle(const Graph* h) { return h->ntasks < kOverlapMax; }
 int retry_passes_of(const Graph* h) { return h->ntasks >= kRetryMin ? h->retry_passes : 0; }
 
 // The next step's permutation and class lists need nothing of this step's
-// trades, so a small handle with another step to come computes them beside the
-// in-order pass, which leaves most SMs idle: step time n=2^12 71.6 -> 63.3 us,
-// 2^14 141 -> 123, 2^15 182 -> 169.
+// trades.  With another step to come they are computed beside the in-order
+// pass, which leaves most SMs idle: the whole permutation of a small handle, of
+// others its first kernel.  Step time n=2^12 71.6 -> 63.3 us, 2^14 141 -> 123,
+// 2^15 182 -> 169, 2^16 211 -> 195, 2^17 286 -> 268, 2^18 442 -> 430, 2^20 1273
+// -> 1265; at 2^21 (2^20 trades) both take 2386.
+constexpr int64_t kAheadMax = int64_t(1) << 20;
+bool may_run_ahead(int64_t ntasks, int64_t nnz) { return nnz > 0 && ntasks < kAheadMax; }
 bool runs_ahead(const Graph* h) { return h->order2 && !h->relaxed && !h->timing && !h->swap_stats; }
 
 int super_step(Graph* h, bool ahead) {

@@ -185,10 +185,10 @@ def test_trades_of_the_largest_class(options):
     c.close()
 
 
-# Steps of one call on small handles compute the next permutation beside the
-# in-order pass, in a third set of arrays: calls of different lengths, single
+# Steps of one call compute the next permutation (of larger handles the first
+# of its kernels) beside the in-order pass, in a third set of arrays: calls of different lengths, single
 # steps, recorded steps and other uses of the handle between them.
-@pytest.mark.parametrize("n,b", [(9, 5), (1025, 60), (4096, 200), (5001, 2000), (32769, 30), (65534, 12)])
+@pytest.mark.parametrize("n,b", [(9, 5), (1025, 60), (4096, 200), (5001, 2000), (32769, 30), (65534, 12), (150001, 9)])
 def test_calls_of_several_steps(n, b):
     g = synth.powerlaw_graph(n, 1, max(2, b), 2.0, 23)
     c, o = Curveball(g.row_ptr, g.col, 7), Oracle(g.row_ptr, g.col, 7)
@@ -223,7 +223,7 @@ def test_calls_of_several_steps(n, b):
     c.close()
 
 
-@pytest.mark.parametrize("sizes", [(3, 1, 0, 2), (1023, 1024, 1025, 9), (9000, 12001, 700)])
+@pytest.mark.parametrize("sizes", [(3, 1, 0, 2), (1023, 1024, 1025, 9), (9000, 12001, 700), (40001, 30, 90000)])
 def test_batch_calls_of_several_steps(sizes):
     graphs = []
     for n in sizes:
