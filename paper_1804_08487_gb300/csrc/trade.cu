@@ -625,45 +625,58 @@ __device__ bool phase_a(Team& tm, const StepCtx& c, int64_t t, const WsA& w, Sel
   // + 1 as key: a plain store into an empty home slot, read back after a
   // barrier; an entry whose home slot another key won claims a further slot
   // with a compare-and-swap), then the presence bit (row, column) in the
-  // slot's flags
-  for (int i = tm.rank; i < L; i += Team::N) {
-    const int r = i >= du;
-    const int32_t yy = ystage ? ystage[i] : __ldcg(c.col + tr.b0 + i);
-    const int64_t s = yy >> 1;
-    uint8_t m = static_cast<uint8_t>(r | ((yy & 1) ? kCol : 0));
-    if (s == t) {
-      m |= kUV;
-      w.slot[i] = -1;
-    } else {
-      m |= kPend;
-      w.slot[i] = static_cast<int32_t>(hslot(static_cast<uint32_t>(s), w.lgH));
+  // slot's flags.  All passes take kBatch entries of a member at a time, loads
+  // first: parts of the work space may be in global memory.
+  constexpr int N = Team::N, kBatch = 4;
+  const uint32_t hmask = (1u << w.lgH) - 1u;
+  auto entry = [&](int i) { return ystage ? ystage[i] : __ldcg(c.col + tr.b0 + i); };
+  for (int i0 = tm.rank; i0 < L; i0 += N * kBatch) {
+    int32_t yy[kBatch];
+#pragma unroll
+    for (int q = 0; q < kBatch; ++q) yy[q] = i0 + q * N < L ? entry(i0 + q * N) : 0;
+#pragma unroll
+    for (int q = 0; q < kBatch; ++q) {
+      const int i = i0 + q * N;
+      if (i >= L) break;
+      const int r = i >= du;
+      const int64_t s = yy[q] >> 1;
+      uint8_t m = static_cast<uint8_t>(r | ((yy[q] & 1) ? kCol : 0));
+      int32_t sl = -1;
+      if (s == t) {
+        m |= kUV;
+      } else {
+        sl = static_cast<int32_t>(hslot(static_cast<uint32_t>(s), w.lgH));
+        if (w.hkey[sl] == 0u) w.hkey[sl] = static_cast<uint32_t>(s) + 1u;
+      }
+      w.slot[i] = sl;
+      w.meta[i] = m;
     }
-    w.meta[i] = m;
   }
-  {
-    const uint32_t hmask = (1u << w.lgH) - 1u;
-    for (int i = tm.rank; i < L; i += Team::N) {
-      if (!(w.meta[i] & kPend)) continue;
-      const int32_t yy = ystage ? ystage[i] : __ldcg(c.col + tr.b0 + i);
-      const int sl = w.slot[i];
-      if (w.hkey[sl] == 0u) w.hkey[sl] = (static_cast<uint32_t>(yy) >> 1) + 1u;
+  tm.sync();
+  for (int i0 = tm.rank; i0 < L; i0 += N * kBatch) {
+    uint32_t key[kBatch], col[kBatch], at[kBatch], won[kBatch];
+#pragma unroll
+    for (int q = 0; q < kBatch; ++q) {
+      const int i = i0 + q * N;
+      const uint32_t yy = i < L ? static_cast<uint32_t>(entry(i)) : 2u * static_cast<uint32_t>(t);
+      key[q] = (yy >> 1) + 1u;
+      col[q] = yy & 1u;
     }
-    tm.sync();
-    for (int i = tm.rank; i < L; i += Team::N) {
-      const uint8_t m = w.meta[i];
-      if (!(m & kPend)) continue;
-      const int32_t yy = ystage ? ystage[i] : __ldcg(c.col + tr.b0 + i);
-      const uint32_t sl = static_cast<uint32_t>(w.slot[i]);
-      const uint32_t key = (static_cast<uint32_t>(yy) >> 1) + 1u;
-      if (w.hkey[sl] != key)   // lost the slot to another key: claim one further on
-        w.slot[i] = static_cast<int32_t>(h_claim(w.hkey, hmask, key, (sl + 1u) & hmask));
-      w.meta[i] = m & ~kPend;
+#pragma unroll
+    for (int q = 0; q < kBatch; ++q) {
+      at[q] = hslot(key[q] - 1u, w.lgH);
+      won[q] = key[q] == static_cast<uint32_t>(t) + 1u ? key[q] : w.hkey[at[q]];   // the edge {u, v} has no slot
     }
-    tm.sync();
-    for (int i = tm.rank; i < L; i += Team::N) {
-      const uint8_t m = w.meta[i];
-      if (m & kUV) continue;
-      flag_or(w.hflag, w.slot[i], 1u << (2 * (m & kR) + ((m & kCol) ? 1 : 0)));
+#pragma unroll
+    for (int q = 0; q < kBatch; ++q) {
+      const int i = i0 + q * N;
+      if (i >= L || key[q] == static_cast<uint32_t>(t) + 1u) continue;
+      uint32_t sl = at[q];
+      if (won[q] != key[q]) {   // lost the slot to another key: claim one further on
+        sl = h_claim(w.hkey, hmask, key[q], (sl + 1u) & hmask);
+        w.slot[i] = static_cast<int32_t>(sl);
+      }
+      flag_or(w.hflag, static_cast<int>(sl), 1u << (2 * (i >= du ? 1 : 0) + col[q]));
     }
   }
   tm.sync();
@@ -677,30 +690,44 @@ __device__ bool phase_a(Team& tm, const StepCtx& c, int64_t t, const WsA& w, Sel
   int cnt_a = 0;
   // both trades' keys of every edge; entries of blocks of several edges are
   // for the second loop
-  for (int i = tm.rank; i < L; i += Team::N) {
-    uint8_t m = w.meta[i];
-    w.far[i] = 0;
-    w.top[i] = 0;
-    if (m & kUV) continue;
-    const int r = m & kR;
-    const uint32_t colb = (m & kCol) ? 1u : 0u;
-    const int sl = w.slot[i];
-    const uint32_t s = w.hkey[sl] - 1u;
-    const uint32_t f = w.hflag[sl] & 15u;
-    const uint32_t x = t2u + r, y = 2u * s + colb;
-    const EdgeKeys ek = edge_keys<kOneSeed>(c, kc, min(x, y), max(x, y));
-    const bool lo_mine = x < y;
-    const uint32_t top = static_cast<uint32_t>((lo_mine ? ek.lo_side : ek.hi_side) >> 48);
-    w.top[i] = static_cast<uint16_t>(top);
-    w.far[i] = static_cast<uint16_t>((lo_mine ? ek.hi_side : ek.lo_side) >> (64 - kFarBits));
-    if (f & (f - 1u)) {
-      m |= kPend;
-    } else if (!tr.single) {
-      m |= kInD;
-      cnt_a += (r == 0);
-      atomicAdd(&w.hist[top >> (16 - kSelBits)], 1u);
+  for (int i0 = tm.rank; i0 < L; i0 += N * kBatch) {
+    int32_t sl[kBatch];
+    uint8_t mq[kBatch];
+#pragma unroll
+    for (int q = 0; q < kBatch; ++q) {
+      const int i = i0 + q * N;
+      mq[q] = i < L ? w.meta[i] : kUV;
+      sl[q] = i < L ? w.slot[i] : -1;
     }
-    w.meta[i] = m;
+#pragma unroll
+    for (int q = 0; q < kBatch; ++q) {
+      const int i = i0 + q * N;
+      if (i >= L) break;
+      uint8_t m = mq[q];
+      if (m & kUV) {
+        w.far[i] = 0;
+        w.top[i] = 0;
+        continue;
+      }
+      const int r = m & kR;
+      const uint32_t colb = (m & kCol) ? 1u : 0u;
+      const uint32_t s = w.hkey[sl[q]] - 1u;
+      const uint32_t f = w.hflag[sl[q]] & 15u;
+      const uint32_t x = t2u + r, y = 2u * s + colb;
+      const EdgeKeys ek = edge_keys<kOneSeed>(c, kc, min(x, y), max(x, y));
+      const bool lo_mine = x < y;
+      const uint32_t top = static_cast<uint32_t>((lo_mine ? ek.lo_side : ek.hi_side) >> 48);
+      w.top[i] = static_cast<uint16_t>(top);
+      w.far[i] = static_cast<uint16_t>((lo_mine ? ek.hi_side : ek.lo_side) >> (64 - kFarBits));
+      if (f & (f - 1u)) {
+        m |= kPend;
+      } else if (!tr.single) {
+        m |= kInD;
+        cnt_a += (r == 0);
+        atomicAdd(&w.hist[top >> (16 - kSelBits)], 1u);
+      }
+      w.meta[i] = m;
+    }
   }
   // blocks of two or more edges: common neighbours and dependencies
   for (int i = tm.rank; i < L; i += Team::N) {
@@ -776,15 +803,23 @@ __device__ bool phase_a(Team& tm, const StepCtx& c, int64_t t, const WsA& w, Sel
   if (cnt <= kCand) {
     // the threshold first, so that dependent trades go on: the elements of its
     // bin (the only one, or ranked by full key)
-    for (int i = tm.rank; cnt > 0 && i < L; i += Team::N) {
-      const uint8_t m = w.meta[i];
-      if (!(m & kInD) || (static_cast<int>(w.top[i]) >> (16 - kSelBits)) != bin) continue;
-      const int32_t y = entry_y(w, t2, i);
-      const uint32_t lo = lo_of(t2, m, y), hi = hi_of(t2, m, y);
-      const int q = cnt == 1 ? 0 : atomicAdd(w.ncand, 1);
-      w.ck[q] = own_key(kc, t, lo, hi);
-      w.ctb[q] = tie_break(lo, hi);
-      w.cidx[q] = i;
+    for (int i0 = tm.rank; cnt > 0 && i0 < L; i0 += N * kBatch) {
+      uint32_t mine = 0;
+#pragma unroll
+      for (int q = 0; q < kBatch; ++q) {
+        const int i = i0 + q * N;
+        if (i < L && (w.meta[i] & kInD) && (static_cast<int>(w.top[i]) >> (16 - kSelBits)) == bin) mine |= 1u << q;
+      }
+      for (; mine; mine &= mine - 1u) {
+        const int i = i0 + (__ffs(mine) - 1) * N;
+        const uint8_t m = w.meta[i];
+        const int32_t y = entry_y(w, t2, i);
+        const uint32_t lo = lo_of(t2, m, y), hi = hi_of(t2, m, y);
+        const int q = cnt == 1 ? 0 : atomicAdd(w.ncand, 1);
+        w.ck[q] = own_key(kc, t, lo, hi);
+        w.ctb[q] = tie_break(lo, hi);
+        w.cidx[q] = i;
+      }
     }
     tm.sync();
     const int kk = a - below;
@@ -811,15 +846,24 @@ __device__ bool phase_a(Team& tm, const StepCtx& c, int64_t t, const WsA& w, Sel
     if (tm.rank == 0) publish(c, kc, t, pu, pv, tk, tt, publish_fence);
     // own decisions: an element below the threshold's bin stays with u, above
     // it goes to v
-    for (int i = tm.rank; i < L; i += Team::N) {
-      const uint8_t m = w.meta[i];
-      if (!(m & kInD)) continue;
-      const int r = m & kR;
-      const int d = static_cast<int>(w.top[i]) >> (16 - kSelBits);
-      if (!no_thr && d == bin) continue;
-      if ((no_thr || d > bin ? 1 : 0) != r) {
-        w.meta[i] = m | kFlip;
-        flag_or(w.hflag, w.slot[i], 16u << (2 * r + ((m & kCol) ? 1 : 0)));
+    for (int i0 = tm.rank; i0 < L; i0 += N * kBatch) {
+      uint8_t mq[kBatch];
+      int d[kBatch];
+      int32_t sl[kBatch];
+#pragma unroll
+      for (int q = 0; q < kBatch; ++q) {
+        const int i = i0 + q * N;
+        mq[q] = i < L ? w.meta[i] : 0;
+        d[q] = i < L ? static_cast<int>(w.top[i]) >> (16 - kSelBits) : 0;
+        sl[q] = i < L ? w.slot[i] : 0;
+      }
+#pragma unroll
+      for (int q = 0; q < kBatch; ++q) {
+        const uint8_t m = mq[q];
+        const int r = m & kR;
+        if (!(m & kInD) || (!no_thr && d[q] == bin) || (no_thr || d[q] > bin ? 1 : 0) == r) continue;
+        w.meta[i0 + q * N] = m | kFlip;
+        flag_or(w.hflag, sl[q], 16u << (2 * r + ((m & kCol) ? 1 : 0)));
       }
     }
     tm.sync();
@@ -864,40 +908,58 @@ __device__ bool phase_a(Team& tm, const StepCtx& c, int64_t t, const WsA& w, Sel
   if (tm.rank == Team::N - 1 && (s0 + n0 != du || s1 + n1 != dv)) latch(c.err, kErrRowLength);
   const int64_t ou = c.rp_next[pu];
   const int64_t ov = tr.single ? 0 : c.rp_next[pv];
-  for (int i = tm.rank; i < L; i += Team::N) {
-    const uint8_t m = w.meta[i];
-    const int f = (m & kFlip) ? 1 : 0;
-    int in_far = 0;
-    if (!(m & kUV)) {   // will the far trade decide this edge?
-      const int r = m & kR;
-      const int sl = w.slot[i];
-      const uint32_t s = w.hkey[sl] - 1u;
-      const uint32_t fl = w.hflag[sl];
-      const int u0 = fl & 1, u1 = (fl >> 1) & 1, v0 = (fl >> 2) & 1, v1 = (fl >> 3) & 1;
-      const int cr = r ? (v0 + v1) : (u0 + u1);
-      if (tr.single || s < t32) {
-        in_far = (cr == 1);                 // trade s acted before t: initial block
-      } else if (s < T32) {
-        if (u0 + u1 + v0 + v1 == 1) {
-          in_far = 1;
-        } else {                            // block after t's own decisions: presence bits 0..3, flips 4..7
-          const int myrow = r ^ f;
-          int same = 0;
+  for (int i0 = tm.rank; i0 < L; i0 += N * kBatch) {
+    uint8_t mq[kBatch];
+    int32_t slq[kBatch];
+    uint16_t far[kBatch];
+    uint32_t sq[kBatch], flq[kBatch];
 #pragma unroll
-          for (int q = 0; q < 4; ++q) {
-            if (!((fl >> q) & 1)) continue;
-            same += (((q >> 1) ^ ((fl >> (4 + q)) & 1)) == myrow);
+    for (int q = 0; q < kBatch; ++q) {
+      const int i = i0 + q * N;
+      mq[q] = i < L ? w.meta[i] : kUV;
+      slq[q] = i < L ? w.slot[i] : -1;
+      far[q] = i < L ? w.far[i] : 0;
+    }
+#pragma unroll
+    for (int q = 0; q < kBatch; ++q) {
+      const bool uv = (mq[q] & kUV) != 0;
+      sq[q] = uv ? 0u : w.hkey[slq[q]] - 1u;
+      flq[q] = uv ? 0u : w.hflag[slq[q]];
+    }
+#pragma unroll
+    for (int q = 0; q < kBatch; ++q) {
+      if (i0 + q * N >= L) break;
+      const uint8_t m = mq[q];
+      const int f = (m & kFlip) ? 1 : 0, r = m & kR;
+      const uint32_t s = sq[q], fl = flq[q];
+      int in_far = 0;
+      if (!(m & kUV)) {   // will the far trade decide this edge?
+        const int u0 = fl & 1, u1 = (fl >> 1) & 1, v0 = (fl >> 2) & 1, v1 = (fl >> 3) & 1;
+        const int cr = r ? (v0 + v1) : (u0 + u1);
+        if (tr.single || s < t32) {
+          in_far = (cr == 1);                 // trade s acted before t: initial block
+        } else if (s < T32) {
+          if (u0 + u1 + v0 + v1 == 1) {
+            in_far = 1;
+          } else {                            // block after t's own decisions: presence bits 0..3, flips 4..7
+            const int myrow = r ^ f;
+            int same = 0;
+#pragma unroll
+            for (int b = 0; b < 4; ++b) {
+              if (!((fl >> b) & 1)) continue;
+              same += (((b >> 1) ^ ((fl >> (4 + b)) & 1)) == myrow);
+            }
+            in_far = (same == 1);
           }
-          in_far = (same == 1);
         }
       }
+      const int side = r ^ f;
+      const int k = side ? s1++ : s0++;
+      if (k >= (side ? dv : du)) continue;   // counts checked above: never write outside the row
+      const int64_t slot = (side ? ov : ou) + k;
+      c.ph[slot] = m & kUV ? static_cast<int32_t>(t2 + 1 - r) : static_cast<int32_t>(2 * s + ((m & kCol) ? 1 : 0));
+      c.fb[slot] = static_cast<uint16_t>(f | (in_far ? ((static_cast<uint32_t>(far[q]) << 1) | kFbInFar) : 0u));
     }
-    const int side = (m & kR) ^ f;
-    const int k = side ? s1++ : s0++;
-    if (k >= (side ? dv : du)) continue;   // counts checked above: never write outside the row
-    const int64_t slot = (side ? ov : ou) + k;
-    c.ph[slot] = entry_y(w, t2, i);
-    c.fb[slot] = static_cast<uint16_t>(f | (in_far ? ((w.far[i] << 1) | kFbInFar) : 0u));
   }
   tm.sync();
   return true;
