@@ -167,7 +167,7 @@ def workload(name):
 # code changed since reports no traffic.  profiles/ holds the captures.
 MEASURED_TRAFFIC = {
     # profiles/rebuild_traffic_n2p25.md: mean of four super steps
-    ("rebuild phase (k_far_pack, k_chunk_rows, k_fixup passes)", "n2^25"): {
+    ("rebuild phase (k_fixup passes)", "n2^25"): {
         "bytes": 92497908608,
         "trade_cu_sha256": "048fcb563ef234b9ff0c1de074ee5f6ff6650e8c2293f61419123590ebc5da4b",
     },
@@ -188,9 +188,8 @@ def measured_traffic(unit, workload):
 
 
 # the threshold phase's kernel of each size class (cb_timings ms[4 + k])
-CLASS_KERNELS = ["k_phase_a_lanes<8>", "k_phase_a_lanes<16>", "k_phase_a_warp", "k_phase_a_team<256,64>",
-                 "k_phase_a_team<256,128>", "k_phase_a_team<256,256>", "k_phase_a_team<1024,512>",
-                 "k_phase_a_team<1024,1024>", "k_phase_a_block<1024>"]
+# (below 2^17 trades the classes share k_phase_a_small and k_phase_a_large)
+CLASS_KERNELS = [f"k_phase_a_class<{k}>" for k in range(8)] + ["k_phase_a_huge"]
 # algorithmic bytes: a threshold kernel reads each directed entry of its
 # trades (4 B) and writes it into the new row with its side word (4 + 2 B),
 # plus per trade its two rows' offsets, positions, threshold and done flag
@@ -203,9 +202,9 @@ FIXUP_BYTES_PER_ENTRY = 10
 FIXUP_BYTES_PER_TRADE = 16
 
 
-# the rebuild is timed as one unit per super step: the far-trade records,
-# each chunk's first row, and the fix-up passes over slices of the far trades
-REBUILD_UNIT = "rebuild phase (k_far_pack, k_chunk_rows, k_fixup passes)"
+# the rebuild is timed as one unit per super step: the fix-up passes over
+# slices of the far trades
+REBUILD_UNIT = "rebuild phase (k_fixup passes)"
 
 
 def dominant_kernel(stats, phases, m, ntasks, K):

@@ -202,9 +202,10 @@ int cb_stats(cb_handle h, int64_t* out, int count);
  * threshold phase (every trade's |A_{u-v}|-th smallest key, including the
  * passes that resolve dependent trades), ms[2] = the rebuild phase (new rows
  * for the next step), ms[3] = whole super steps, ms[4 + k], k < 9 = the
- * first threshold pass's kernel of size class k (0 where the class shares
- * another class's kernel), ms[13] = the retry passes over deferred trades,
- * ms[14] = the in-order pass.  Returns the number of values written
+ * first threshold pass's kernel of size class k (below 2^17 trades classes 0
+ * to 5 share class 0's kernel and 6 and 7 class 6's; the others' entries are
+ * then near 0), ms[13] = the retry passes over deferred trades, ms[14] = the
+ * in-order pass.  Returns the number of values written
  * (<= count, at most 15).  Waits for the events still outstanding.
  */
 int cb_timings(cb_handle h, double* ms, int count);
@@ -217,6 +218,10 @@ int cb_timings(cb_handle h, double* ms, int count);
  *               graph launch per super step [0].  Not while "timing" is on.
  *               The handle's stream must support capture (not the legacy
  *               default stream).  Changing any other option re-records.
+ *               Calls of several steps on handles of 2^15 to 2^20 trades
+ *               launch directly all the same: each step's permutation then
+ *               starts beside the step before, which one recorded step
+ *               cannot do.
  *   "tile_max"  trades up to this size run on warps or parts of a warp
  *               [128]; 0..128.
  *   "tile_paths" 1: trades up to tile_max entries run on warps or parts of
@@ -224,11 +229,12 @@ int cb_timings(cb_handle h, double* ms, int count);
  *   "block_max" trades up to this size run on a 256-thread CTA [1024];
  *               0..2048 (values below tile_max act as tile_max).
  *   "smem_max"  larger trades run on a 1024-thread CTA; with "cta_paths" 1
- *               up to min(4096, smem_max) entries in registers, with 0 up
- *               to smem_max entries in shared memory; more in a
+ *               up to min(8192, smem_max) entries in registers, with 0 up
+ *               to smem_max entries in shared memory; more with their hash in
+ *               shared memory (up to 26214 entries) and the rest in a
  *               global-memory workspace [8192]; 64..8192.
- *   "cta_paths" 1: threshold phase of the 256- and 1024-thread classes with
- *               the entries in registers (4 per thread); 0: in shared
+ *   "cta_paths" 1: threshold phase of the classes above a warp's with the
+ *               entries in registers (4 or 8 per thread); 0: in shared
  *               memory [1].
  *   "cand_max"  register paths: when at most this many elements share the
  *               threshold's leading key bits they are ranked directly,
@@ -238,9 +244,9 @@ int cb_timings(cb_handle h, double* ms, int count);
  *               or 256 (four CTAs per SM; trades above 1024 entries in
  *               shared memory up to block_max, from global memory above)
  *               [1024; 256 for cb_create_batch].
- *   "uniform_threads" CTA size of the executor of cb_uniform_trades: 256
- *               (two CTAs per SM), 512 or 1024 (more threads per hub trade,
- *               fewer trades at once) [1024].
+ *   "uniform_threads" CTA size of the executor of cb_uniform_trades: 256,
+ *               512 or 1024; three quarters of a CTA are the team of one
+ *               large trade, its other warps run a small trade each [1024].
  *   "lane_teams" 1: trades of at most 32 / 64 entries run on teams of 8 /
  *               16 lanes, several per warp; 0: on whole warps [1].
  *   "retry_passes" parallel passes over the deferred trades between the

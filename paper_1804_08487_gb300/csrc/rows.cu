@@ -249,7 +249,7 @@ __global__ void __launch_bounds__(kVThreads) k_vpart(int64_t n, const int64_t* _
       for (int j = 0; j < kTileLoads; ++j) {
         const int64_t e = e0 + 32 * j + lane;
         const int64_t x = tile.r0 + tile.row_of(e);
-        if (y[j] <= x || y[j] >= n) continue;   // as k_vcount counted
+        if (y[j] <= x || y[j] >= n) continue;   // as k_scan_rows counted
         const int64_t slot = static_cast<int64_t>(atomicAdd(&cur[y[j] >> sh], 1ull));
         if (slot < cap) part[slot] = make_int2(static_cast<int32_t>(x), y[j]);
         else latch(err, kErrValidate);

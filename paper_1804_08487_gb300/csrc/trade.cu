@@ -24,9 +24,9 @@
 //     and a 16-bit side word (bit 0 the own trade's flip, bits 1..11 the top
 //     11 bits of the far trade's key for the edge, bit 12 set when the far
 //     trade decides the edge).  The first pass runs every trade by size
-//     class; a trade whose dependency has not published is deferred and
-//     listed, retry passes run the lists, and one in-order pass completes
-//     what is left, waiting (bounded) for its dependencies.
+//     class; a trade whose dependency has not published is deferred, retry
+//     passes (large handles) run lists of them, and one in-order pass
+//     completes what is left, waiting (bounded) for its dependencies.
 //  B. Rebuild (fix-up).  Every placeholder becomes the step-(g+1) position
 //     of the far end: per far trade one packed record (the new positions of
 //     its two nodes, the top 8 bits of its threshold), read in slices small
@@ -36,8 +36,8 @@
 // Phase A by trade size L = deg u + deg v (nine classes): lane teams of 8 or
 // 16 threads (several trades per warp) and whole warps up to `tile_max`
 // entries, teams of 64 to 1024 threads with the entries in registers up to
-// min(4096, `smem_max`), and a 1024-thread CTA with the entries in shared
-// memory (a global-memory slice above `smem_max`) for the largest.  The team
+// min(8192, `smem_max`), and a 1024-thread CTA with the hash in shared memory
+// and the rest in a global-memory slice for the largest.  The team
 // and shared-memory kernels come in a version for handles of one graph,
 // whose seed's Philox round keys are kernel parameters, and a general one.
 #include <algorithm>
@@ -2364,11 +2364,9 @@ int super_step(Graph* h, bool ahead) {
   const int64_t ntasks = h->ntasks;
   const int tile_max = h->tile_paths ? std::min(h->tile_max, kTileMaxCap) : 0;
   const int block_max = std::max(h->block_max, tile_max);
-  // size classes: lane teams of 8 / 16 (L <= 32 / 64), a warp (L <=
-  // tile_max), teams of 64 / 128 / 256 threads (up to 256 / 512 / block_max
-  // <= 1024 entries), of 512 / 1024 threads in a 1024-thread CTA (up to 2048
-  // / min(4096, smem_max)), and the largest trades on the shared-memory
-  // kernel; "cta_paths" 0 sends everything above the warp class to the
+  // size classes (L up to 32, 64, tile_max, 256, 512, block_max <= 1024, 2048,
+  // min(4096, smem_max), larger); "cta_paths" 0 sends everything above the
+  // warp class to the
   // shared-memory kernels (256 threads up to block_max, 1024 above)
   ClassArgs ca;
   ca.n = h->n;
