@@ -238,6 +238,11 @@ size_t scan_ws_bytes(int64_t n);
 cudaError_t exclusive_scan_i32(const int32_t* in, int64_t* out, int64_t n, void* ws, cudaStream_t s,
                                int64_t* launches = nullptr);
 
+// Parts of a permutation: all of it, or, ahead of time, its scatter beside the
+// end of the first pass (nothing where one kernel does it all) and the rest,
+// with the class lists, beside the in-order pass.
+enum class PermPart { kWhole, kScatterAhead, kRestAhead };
+
 // permute.cu
 struct ClassArgs;
 size_t perm_ws_bytes(int64_t nbuckets, int64_t slots);
@@ -248,7 +253,7 @@ int64_t bucket_space(int64_t span, int B);
 // its device step counter + dg, or the step g_abs for all when g_abs >= 0.
 // classes (may be null): build the size-class lists of the current step too.
 int compute_permutation(Graph* h, uint32_t dg, int64_t g_abs, int32_t* order_out, int32_t* pos_out, int64_t* rp_out,
-                        const ClassArgs* classes, bool beside = false);   // beside: see k_perm_rescan
+                        const ClassArgs* classes, PermPart part = PermPart::kWhole);
 size_t perm_zero_bytes(int64_t nbuckets);   // the start of its scratch that has to be zero at first
 
 // rows.cu

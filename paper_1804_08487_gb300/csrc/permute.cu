@@ -493,10 +493,11 @@ __global__ void __launch_bounds__(kPermThreads) k_perm_scatter(int64_t n, KeySrc
 __global__ void __launch_bounds__(kPermThreads) k_bucket_sort(int64_t n, int nseg, KeySrc ks, int nb, int cap,
                                                              const uint64_t* __restrict__ prefix,
                                                              const int32_t* __restrict__ bid, PermOut out,
-                                                             int64_t nnz) {
-  after_previous();
+                                                             int64_t nnz, ClassArgs ca, bool beside) {
+  if (!beside) after_previous();
   before_next();
   extern __shared__ uint64_t shk[];
+  classify<kPermThreads>(ca, blockIdx.x, gridDim.x);
   const BucketWs w = bucket_ws(shk, cap);
   if (blockIdx.x == 0 && threadIdx.x == 0 && out.rp) put_rows_end(out, n, nnz);
   for (int64_t b = blockIdx.x; b < nb; b += gridDim.x) {
@@ -535,6 +536,7 @@ __global__ void __launch_bounds__(kPermThreads) k_bucket_sort(int64_t n, int nse
     }
     __syncthreads();
   }
+  if (beside && blockIdx.x == 0) after_previous();
 }
 
 // Trades of the current step by size class, on its own (relaxed permutations).
@@ -616,7 +618,7 @@ int bucket_cap_of(const Graph* h) {
 }  // namespace
 
 int compute_permutation(Graph* h, uint32_t dg, int64_t g_abs, int32_t* order_out, int32_t* pos_out, int64_t* rp_out,
-                        const ClassArgs* classes, bool beside) {
+                        const ClassArgs* classes, PermPart part) {
   const int64_t n = h->n;
   if (n == 0) return CB_OK;
   cudaStream_t s = h->stream;
@@ -627,6 +629,7 @@ int compute_permutation(Graph* h, uint32_t dg, int64_t g_abs, int32_t* order_out
   ks.g_abs = static_cast<uint32_t>(g_abs < 0 ? 0 : g_abs);
   ClassArgs ca{};
   if (classes) ca = *classes;
+  const bool beside = part != PermPart::kWhole;
   const int64_t chunks = class_chunks(ca.ntasks, kPermThreads);
   if (h->relaxed) {
     if (ca.ntasks) {
@@ -657,20 +660,28 @@ int compute_permutation(Graph* h, uint32_t dg, int64_t g_abs, int32_t* order_out
   const int cap = bucket_cap_of(h);
   const PermOut out{order_out, pos_out, rp_out, h->deg_id, !rp_out ? nullptr : beside ? h->chunk_row2 : h->chunk_row};
   if (nb <= kRescanBuckets && rescan_work(h) <= kRescanWork) {
+    if (part == PermPart::kScatterAhead) return CB_OK;
     const unsigned grid = static_cast<unsigned>(
         nb + std::min<int64_t>(class_chunks(ca.ntasks, kRescanThreads), int64_t(h->num_sms) * 2));
-    CB_CUDA(h, launch(beside || small_handle(h), k_perm_rescan, grid, kRescanThreads, bucket_smem_bytes(cap), s, n, h->nseg, ks,
-                      static_cast<int>(nb), cap, out, h->rp_id, h->nnz, ca, beside));
+    CB_CUDA(h, launch(beside || small_handle(h), k_perm_rescan, grid, kRescanThreads, bucket_smem_bytes(cap), s, n, h->nseg,
+                      ks, static_cast<int>(nb), cap, out, h->rp_id, h->nnz, ca, beside));
     ++h->launches;
     return CB_OK;
   }
   const PermWs w = carve(h->sort_ws, nb);
-  CB_CUDA(h, launch(beside || small_handle(h), k_perm_scatter, grid_for(n, kPermThreads, h->num_sms), kPermThreads, 0, s, n, ks,
-                    static_cast<int>(nb), rp_out ? h->deg_id : nullptr, w.words, w.prefix, w.ticket, w.bid, ca, beside));
-  const unsigned sgrid = static_cast<unsigned>(nb < h->num_sms * 8 ? nb : h->num_sms * 8);
-  CB_CUDA(h, launch(small_handle(h), k_bucket_sort, sgrid, kPermThreads, bucket_smem_bytes(cap), s, n, h->nseg, ks,
-                    static_cast<int>(nb), cap, w.prefix, w.bid, out, h->nnz));
-  h->launches += 2;
+  const ClassArgs none{};
+  if (part != PermPart::kRestAhead) {
+    CB_CUDA(h, launch(beside || small_handle(h), k_perm_scatter, grid_for(n, kPermThreads, h->num_sms), kPermThreads, 0, s,
+                      n, ks, static_cast<int>(nb), rp_out ? h->deg_id : nullptr, w.words, w.prefix, w.ticket, w.bid, ca,
+                      beside));
+    ++h->launches;
+  }
+  if (part != PermPart::kScatterAhead) {
+    const unsigned sgrid = static_cast<unsigned>(nb < h->num_sms * 8 ? nb : h->num_sms * 8);
+    CB_CUDA(h, launch(beside || small_handle(h), k_bucket_sort, sgrid, kPermThreads, bucket_smem_bytes(cap), s, n, h->nseg,
+                      ks, static_cast<int>(nb), cap, w.prefix, w.bid, out, h->nnz, beside ? ca : none, beside));
+    ++h->launches;
+  }
   return CB_OK;
 }
 
@@ -752,7 +763,7 @@ extern "C" int cb_permutation_static(int64_t n, uint64_t seed, uint64_t g, int32
                                                                             w.ticket, w.bid, none, false);
   if ((e = cudaGetLastError()) != cudaSuccess) return cuda_fail(nullptr, e, "k_perm_scatter");
   const unsigned sgrid = static_cast<unsigned>(nb < num_sms * 8 ? nb : num_sms * 8);
-  k_bucket_sort<<<sgrid, kPermThreads, bucket_smem_bytes(cap), s>>>(n, 1, ks, nb, cap, w.prefix, w.bid, out, 0);
+  k_bucket_sort<<<sgrid, kPermThreads, bucket_smem_bytes(cap), s>>>(n, 1, ks, nb, cap, w.prefix, w.bid, out, 0, none, false);
   if ((e = cudaGetLastError()) != cudaSuccess) return cuda_fail(nullptr, e, "k_bucket_sort");
   return CB_OK;
 }

@@ -972,8 +972,7 @@ __device__ bool phase_a(Team& tm, const StepCtx& c, int64_t t, const WsA& w, Sel
 // i mod N): each member keeps its entries' neighbour positions, key bits and
 // flags in registers across the passes, so the only shared-memory traffic is
 // the far-trade hash, one histogram and the few candidates of the threshold's
-// bin.  Used by the first pass only: a trade whose dependency has not
-// published yet is deferred to the in-order pass.
+// bin.
 
 // Per entry a member keeps the neighbour position y, the top 32 bits of its
 // own key, and a word of the far trade's hash slot (bits 0..14) and the far
@@ -1002,7 +1001,7 @@ __host__ __device__ constexpr int lg_ceil(int x) {
 // of at most LMAX entries and 2^B histogram bins (four per member).
 //
 // The far-trade hash has two tables of (key, block word) pairs.  Table 1
-// (kH slots, at least 4 per entry) is never cleared: in one round every entry
+// (kH slots, SLOTS per entry) is never cleared: in one round every entry
 // stores its key and a zero block word into its home slot, whatever is there,
 // so after a barrier each home slot holds a key of this trade.  Only the
 // entries that find another key there (about 8 % at 4 to 8 slots per entry)
@@ -2308,10 +2307,10 @@ int retry_passes_of(const Graph* h) { return h->ntasks >= kRetryMin ? h->retry_p
 
 // The next step's permutation and class lists need nothing of this step's
 // trades.  With another step to come they are computed beside the in-order
-// pass, which leaves most SMs idle: the whole permutation of a small handle, of
-// others its first kernel.  Step time n=2^12 71.6 -> 63.3 us, 2^14 141 -> 123,
-// 2^15 182 -> 169, 2^16 211 -> 195, 2^17 286 -> 268, 2^18 442 -> 430, 2^20 1273
-// -> 1265; at 2^21 (2^20 trades) both take 2386.
+// pass, which leaves most SMs idle (of handles above the one-kernel form, the
+// scatter beside the end of the first pass).  Step time n=2^12 71.6 -> 63.3 us,
+// 2^14 141 -> 123, 2^15 182 -> 168, 2^16 211 -> 191, 2^17 286 -> 260, 2^18 442 ->
+// 423, 2^20 1273 -> 1258; from 2^20 trades on nothing is left of it.
 constexpr int64_t kAheadMax = int64_t(1) << 20;
 bool may_run_ahead(int64_t ntasks, int64_t nnz) { return nnz > 0 && ntasks < kAheadMax; }
 bool runs_ahead(const Graph* h) { return h->order2 && !h->relaxed && !h->timing && !h->swap_stats; }
@@ -2531,6 +2530,7 @@ int super_step(Graph* h, bool ahead) {
       if ((rc = launched())) return rc;
     }
   }
+  if (ahead && (rc = compute_permutation(h, 2, -1, h->order2, h->pos2, h->rp2, nullptr, PermPart::kScatterAhead))) return rc;
   if (h->timing) CB_CUDA(h, cudaEventRecord(ev[5 + kClasses], s));
   {
     const bool big = h->inorder_threads == kBigThreads;
@@ -2556,7 +2556,7 @@ int super_step(Graph* h, bool ahead) {
     ClassArgs next = ca;
     next.rp = h->rp[nxt];
     next.ctr = h->counters + nxt * kCounters;
-    if ((rc = compute_permutation(h, 2, -1, h->order2, h->pos2, h->rp2, &next, true))) return rc;
+    if ((rc = compute_permutation(h, 2, -1, h->order2, h->pos2, h->rp2, &next, PermPart::kRestAhead))) return rc;
   }
   if (h->timing) CB_CUDA(h, cudaEventRecord(ev[2], s));
   // rebuild: the fix-up in passes over slices of the far trades; its output
