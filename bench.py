@@ -168,8 +168,8 @@ def workload(name):
 MEASURED_TRAFFIC = {
     # profiles/rebuild_traffic_n2p25.md: mean of four super steps
     ("rebuild phase (k_fixup passes)", "n2^25"): {
-        "bytes": 92497908608,
-        "trade_cu_sha256": "048fcb563ef234b9ff0c1de074ee5f6ff6650e8c2293f61419123590ebc5da4b",
+        "bytes": 94235662720,
+        "trade_cu_sha256": "dda02c42b60800db265c37075008e5b8d8520221dfbd464117ee477b449d96da",
     },
 }
 
