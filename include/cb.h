@@ -276,6 +276,9 @@ int cb_timings(cb_handle h, double* ms, int count);
  *   "hold_publish" 1: trades never publish that their threshold is ready,
  *               so a trade that depends on another waits until "wait_ms"
  *               runs out (a test of the timeout path) [0].
+ *   "inorder_ctas" CTAs of the in-order pass that take part, the others leave
+ *               at once (a test that the pass completes on any part of its
+ *               grid); 0: all [0]; 0..65535.
  *   "hold_trade" uniform trades: messages to this trade (index within the
  *               call) are dropped, so it never runs and the executor's
  *               waits run out (a test of the timeout path); -1: none [-1].

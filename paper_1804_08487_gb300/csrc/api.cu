@@ -925,6 +925,11 @@ int cb_set_option(cb_handle h, const char* key, int64_t value) {
     h->hold_publish = static_cast<int>(value);
     return CB_OK;
   }
+  if (!std::strcmp(key, "inorder_ctas")) {
+    if (value < 0 || value > 65535) return fail(h, CB_EINVAL, "inorder_ctas out of range [0, 65535]");
+    h->inorder_ctas = static_cast<int>(value);
+    return CB_OK;
+  }
   if (!std::strcmp(key, "hold_trade")) {
     if (value < -1) return fail(h, CB_EINVAL, "hold_trade is -1 or a trade index");
     h->hold_trade = value;

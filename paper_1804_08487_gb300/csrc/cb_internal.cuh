@@ -142,6 +142,7 @@ struct Graph {
   uint64_t wait_ns = 1000000000ull;       // longest single wait of a super step (dependency, bulk copy)
   uint64_t uni_wait_ns = 20000000000ull;  // longest single wait of the uniform-trade executor
   int hold_publish = 0;                   // test hook: trades never publish their done flags
+  int inorder_ctas = 0;                   // test hook: CTAs of the in-order pass that take part (0: all)
   int64_t hold_trade = -1;                // test hook: uniform trade whose messages are dropped
   int block_max = kBlockMaxDefault;
   int smem_max = kSmemMaxCap;

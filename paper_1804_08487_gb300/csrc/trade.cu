@@ -90,6 +90,7 @@ struct StepCtx {
   int cand_max;                    // register paths: most candidates ranked directly (else more radix digits)
   uint64_t wait_ns;                // longest single wait on dependencies or a bulk copy
   int hold_publish;                // test hook: no trade publishes its done flag (waits run out)
+  unsigned inorder_ctas;           // CTAs of the in-order pass that take part (a test hook; default: all)
   uint32_t ks[20];                 // one graph (seg_of null): the Philox round keys of its seed
 };
 
@@ -2056,12 +2057,16 @@ __global__ void __launch_bounds__(NT, NT == 256 ? 4 : 1) k_retry(StepCtx c, cons
 // trade waits for an unpublished dependency of an earlier chunk, and is tried
 // again when the dependency is in its own.
 //
-// Every wait ends: chunks are claimed in index order, so the smallest
-// unfinished trade is in a claimed chunk (or the CTAs come to it), everything
-// its CTA waits for is finished, and the CTA comes to it; by induction on the
-// index all trades are run, whatever the residency of the grid.  Chains of
-// dependent trades advance at the pace of the published thresholds.  A wait
-// that runs out latches kErrResolve; after any error all leave.
+// Every wait ends: every chunk, a CTA's first one too, is claimed from one
+// counter in index order, so the chunks before a claimed one are finished or
+// held by CTAs that run.  The smallest unfinished trade is then in a claimed
+// chunk (or the CTAs come to it), everything its CTA waits for is finished,
+// and the CTA comes to it; by induction on the index all trades are run,
+// whichever CTAs of the grid are resident.  (A first chunk by block index would
+// be held by a CTA that may not have started, while the running ones wait for
+// its trades: with other streams' kernels on the SMs it may never start.)
+// Chains of dependent trades advance at the pace of the published thresholds.
+// A wait that runs out latches kErrResolve; after any error all leave.
 constexpr int kChunkWork = 32, kWorkMedium = 8;   // work of a chunk (= a large trade), of a medium trade
 
 // Work of a small and of a medium trade: 1 and 8 when there are many, up to
@@ -2163,7 +2168,14 @@ __global__ void __launch_bounds__(NT, NT == 256 ? 4 : 1) k_resolve(StepCtx c, co
   WarpTeam wt;
   const WarpWs ww{sbuf + WarpWs::kBytes * warp};
   const Ws256 w256{sbuf + Ws256::kBytes * id};
-  for (int64_t ch = blockIdx.x; ch < chunks;) {
+  if (chunks == 0 || blockIdx.x >= c.inorder_ctas) return;
+  for (;;) {
+    // (claimed only now: a chunk held while the one before it waits would hold up others)
+    if (threadIdx.x == 0) pick = static_cast<int64_t>(atomicAdd(claim, 1ull));
+    __syncthreads();
+    const int64_t ch = pick;
+    __syncthreads();
+    if (ch >= chunks) return;
     const int32_t first = chunk_first[ch], count = chunk_first[ch + 1] - first;
     const uint32_t from = static_cast<uint32_t>(list[first]);   // trades before it are in earlier chunks
     if (warp == 0) {
@@ -2221,11 +2233,6 @@ __global__ void __launch_bounds__(NT, NT == 256 ? 4 : 1) k_resolve(StepCtx c, co
       if (__syncthreads_or(threadIdx.x == 0 && ld_volatile_i32(c.err) != 0)) return;
       if (!more) break;
     }
-    // (claimed only now: a chunk held while this one waits would hold up others)
-    if (threadIdx.x == 0) pick = gridDim.x + static_cast<int64_t>(atomicAdd(claim, 1ull));
-    __syncthreads();
-    ch = pick;
-    __syncthreads();
   }
 }
 
@@ -2431,6 +2438,7 @@ int super_step(Graph* h, bool ahead) {
   c.cand_max = h->cand_max;
   c.wait_ns = h->wait_ns;
   c.hold_publish = h->hold_publish;
+  c.inorder_ctas = h->inorder_ctas ? static_cast<unsigned>(h->inorder_ctas) : ~0u;
   const int32_t* L = h->lists;
   // the first pass: one kernel for classes 0 to 5 and one for 6 and 7, or one
   // per class (large graphs), and the largest trades (no trade is larger than
