@@ -212,6 +212,11 @@ constexpr int64_t kOverlapMax = int64_t(1) << 15;
 // after_previous(), which waits until that kernel has finished and its writes
 // are visible.  Kernels that call before_next() let their successor be set up
 // as soon as all their CTAs have started.  Without overlap both do nothing.
+// A kernel with after_previous() is resident while the one before it still
+// writes.  So it takes no __restrict__ pointers, and reads what earlier kernels
+// write by plain loads or __ldcg, never __ldg: __restrict__ and __ldg both
+// promise data that does not change while the kernel lives, and would let the
+// compiler move a load above the wait.
 #ifdef __CUDACC__
 __device__ __forceinline__ void after_previous() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void before_next() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }

@@ -61,7 +61,8 @@ struct KeySrc {
   uint32_t g_abs;
 };
 
-// One graph's part of it.
+// One graph's part of it.  (__ldg for what creation fixed; the step counter is
+// written by the end of each step, see after_previous().)
 struct SegKey {
   uint64_t seed;
   int64_t off, n, span, base, slot_base;
@@ -77,7 +78,7 @@ __device__ __forceinline__ SegKey seg_key(const KeySrc& ks, int i) {
   k.span = S ? __ldg(&S->span) : ks.s0.span;
   k.base = S ? __ldg(&S->bucket_base) : ks.s0.bucket_base;
   k.slot_base = S ? __ldg(&S->slot_base) : ks.s0.slot_base;
-  k.g = ks.use_abs ? ks.g_abs : (S ? __ldg(&S->g) : ks.s0.g) + ks.dg;
+  k.g = ks.use_abs ? ks.g_abs : (S ? S->g : ks.s0.g) + ks.dg;
   k.B = S ? __ldg(&S->B) : ks.s0.B;
   k.cap = S ? __ldg(&S->cap) : ks.s0.cap;
   return k;
@@ -364,7 +365,7 @@ constexpr uint64_t kDegMask = (uint64_t(1) << kCountShift) - 1;
 // its own: 12.3 us per call with 256 threads, 10.2 so).
 constexpr int kRescanThreads = 1024;
 __device__ void perm_rescan(int64_t n, int nseg, const KeySrc& ks, int nb, int cap, const PermOut& out,
-                            const int64_t* __restrict__ rp_id, int64_t nnz, const ClassArgs& ca) {
+                            const int64_t* rp_id, int64_t nnz, const ClassArgs& ca) {
   extern __shared__ uint64_t shk[];
   __shared__ int cnt;
   __shared__ int64_t wsum[kRescanThreads / 32];
@@ -420,7 +421,7 @@ __device__ void perm_rescan(int64_t n, int nseg, const KeySrc& ks, int nb, int c
 // run (it uses few SMs, and nothing that this kernel writes); the kernel after
 // has to find both complete, so the wait comes last.
 __global__ void __launch_bounds__(kRescanThreads) k_perm_rescan(int64_t n, int nseg, KeySrc ks, int nb, int cap,
-                                                               PermOut out, const int64_t* __restrict__ rp_id,
+                                                               PermOut out, const int64_t* rp_id,
                                                                int64_t nnz, ClassArgs ca, bool beside) {
   if (!beside) after_previous();
   before_next();
@@ -434,10 +435,9 @@ constexpr int64_t kRescanBuckets = 4096;   // CTAs
 // Node ids into their buckets (beside: as k_perm_rescan); the last CTA to finish turns the bucket words
 // into their exclusive prefix sums and clears them for the next call.
 __global__ void __launch_bounds__(kPermThreads) k_perm_scatter(int64_t n, KeySrc ks, int nb,
-                                                              const int32_t* __restrict__ deg,
-                                                              unsigned long long* __restrict__ words,
-                                                              uint64_t* __restrict__ prefix, int* __restrict__ ticket,
-                                                              int32_t* __restrict__ bid, ClassArgs ca, bool beside) {
+                                                              const int32_t* deg, unsigned long long* words,
+                                                              uint64_t* prefix, int* ticket, int32_t* bid,
+                                                              ClassArgs ca, bool beside) {
   if (!beside) after_previous();
   before_next();
   __shared__ int64_t wsum[kPermThreads / 32];
@@ -452,7 +452,7 @@ __global__ void __launch_bounds__(kPermThreads) k_perm_scatter(int64_t n, KeySrc
     }
     const uint32_t lb = bucket_of(perm_key(k, x), k.B);
     const unsigned long long inc =
-        (1ull << kCountShift) + (deg ? static_cast<unsigned long long>(deg[x]) : 0ull);
+        (1ull << kCountShift) + (deg ? static_cast<unsigned long long>(__ldg(deg + x)) : 0ull);
     const int64_t q = static_cast<int64_t>(atomicAdd(words + k.base + lb, inc) >> kCountShift);
     if (q < k.cap) bid[k.slot_base + int64_t(lb) * k.cap + q] = static_cast<int32_t>(x);
   }
@@ -491,9 +491,8 @@ __global__ void __launch_bounds__(kPermThreads) k_perm_scatter(int64_t n, KeySrc
 }
 
 __global__ void __launch_bounds__(kPermThreads) k_bucket_sort(int64_t n, int nseg, KeySrc ks, int nb, int cap,
-                                                             const uint64_t* __restrict__ prefix,
-                                                             const int32_t* __restrict__ bid, PermOut out,
-                                                             int64_t nnz, ClassArgs ca, bool beside) {
+                                                             const uint64_t* prefix, const int32_t* bid,
+                                                             PermOut out, int64_t nnz, ClassArgs ca, bool beside) {
   if (!beside) after_previous();
   before_next();
   extern __shared__ uint64_t shk[];

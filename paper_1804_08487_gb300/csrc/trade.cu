@@ -249,8 +249,8 @@ struct KeyCtx {
   uint32_t g, off;
 };
 __device__ __forceinline__ KeyCtx key_ctx(const StepCtx& c, int64_t t) {
-  const Seg* S = c.segs + (c.seg_of ? __ldg(c.seg_of + 2 * t) : 0);
-  return {__ldg(&S->seed), __ldg(&S->g), static_cast<uint32_t>(__ldg(&S->off))};
+  const Seg* S = c.segs + (c.seg_of ? c.seg_of[2 * t] : 0);
+  return {S->seed, S->g, static_cast<uint32_t>(S->off)};
 }
 
 // Both trades' keys of the edge whose step-start positions are lo < hi.
@@ -1103,8 +1103,8 @@ __device__ bool phase_a_reg(Team& tm, const StepCtx& c, int64_t t, const Ws& w, 
   const int du = tr.du, L = active ? tr.du + tr.dv : 0;
   // the nodes' positions in step g+1, loaded now so that their dependent
   // loads overlap the trade's work
-  const uint32_t pu = static_cast<uint32_t>(__ldg(c.pos_next + __ldg(c.order + 2 * t)));
-  const uint32_t pv = tr.single ? 0u : static_cast<uint32_t>(__ldg(c.pos_next + __ldg(c.order + 2 * t + 1)));
+  const uint32_t pu = static_cast<uint32_t>(c.pos_next[c.order[2 * t]]);
+  const uint32_t pv = tr.single ? 0u : static_cast<uint32_t>(c.pos_next[c.order[2 * t + 1]]);
   const uint32_t t32 = static_cast<uint32_t>(t), T32 = static_cast<uint32_t>(c.T);
   const uint32_t t2u = 2u * t32;
   const unsigned lanes = tm.lanes();
@@ -1568,7 +1568,7 @@ struct ClassCfg {
 };
 template <int K, bool kOneSeed>
 __global__ void __launch_bounds__(ClassCfg<K>::kThreads, ClassCfg<K>::kCtas)
-    k_phase_a_class(StepCtx c, const int32_t* __restrict__ lists, const int64_t* __restrict__ ctr) {
+    k_phase_a_class(StepCtx c, const int32_t* lists, const int64_t* ctr) {
   after_previous();
   before_next();
   using Cfg = ClassCfg<K>;
@@ -1592,8 +1592,8 @@ constexpr size_t small_smem() {
   return m;
 }
 template <bool kOneSeed>
-__global__ void __launch_bounds__(256, 4) k_phase_a_small(StepCtx c, const int32_t* __restrict__ lists,
-                                                        const int64_t* __restrict__ ctr, int what) {
+__global__ void __launch_bounds__(256, 4) k_phase_a_small(StepCtx c, const int32_t* lists,
+                                                        const int64_t* ctr, int what) {
   after_previous();
   before_next();
   extern __shared__ __align__(16) char smem[];
@@ -1621,8 +1621,8 @@ __global__ void __launch_bounds__(256, 4) k_phase_a_small(StepCtx c, const int32
 constexpr size_t kLargeSmem = 2 * TeamCfg<512>::Ws::kBytes > TeamCfg<kBigThreads>::Ws::kBytes
                                   ? 2 * TeamCfg<512>::Ws::kBytes : TeamCfg<kBigThreads>::Ws::kBytes;
 template <bool kOneSeed>
-__global__ void __launch_bounds__(kBigThreads, 1) k_phase_a_large(StepCtx c, const int32_t* __restrict__ lists,
-                                                                const int64_t* __restrict__ ctr) {
+__global__ void __launch_bounds__(kBigThreads, 1) k_phase_a_large(StepCtx c, const int32_t* lists,
+                                                                const int64_t* ctr) {
   after_previous();
   before_next();
   extern __shared__ __align__(16) char smem[];
@@ -1670,8 +1670,8 @@ struct FarRaw<false> {
 };
 template <bool kNarrow>
 __device__ __forceinline__ FarRaw<kNarrow> far_raw(const void* pack, uint32_t s) {
-  if constexpr (kNarrow) return {__ldg(static_cast<const unsigned long long*>(pack) + s)};
-  else return {__ldg(static_cast<const int4*>(pack) + s)};
+  if constexpr (kNarrow) return {static_cast<const unsigned long long*>(pack)[s]};
+  else return {static_cast<const int4*>(pack)[s]};
 }
 template <bool kNarrow>
 __device__ __forceinline__ FarTrade far_decode(const FarRaw<kNarrow>& r) {
@@ -1686,11 +1686,11 @@ __device__ __forceinline__ FarTrade far_decode(const FarRaw<kNarrow>& r) {
 template <bool kNarrow>
 __device__ __forceinline__ FarTrade far_trade(const void* pack, uint32_t s) {
   if constexpr (kNarrow) {
-    const uint64_t v = __ldg(static_cast<const unsigned long long*>(pack) + s);
+    const uint64_t v = static_cast<const unsigned long long*>(pack)[s];
     return {static_cast<int32_t>(v & 0x0FFFFFFFu), static_cast<int32_t>((v >> 28) & 0x0FFFFFFFu),
             static_cast<uint32_t>(v >> 56)};
   } else {
-    const int4 v = __ldg(static_cast<const int4*>(pack) + s);
+    const int4 v = static_cast<const int4*>(pack)[s];
     return {v.x, v.y, static_cast<uint32_t>(v.z)};
   }
 }
@@ -1786,8 +1786,8 @@ __global__ void k_step_end(StepEnd e) { end_step(e); }
 // together, so that their extra loads hold up no warp.
 template <bool kNarrow, bool kLast>
 __global__ void __launch_bounds__(kFixThreads, 4) k_fixup(StepCtx c, int64_t nnz, uint32_t s_lo, uint32_t s_hi,
-                                                       int32_t* __restrict__ ph, const uint16_t* __restrict__ fb,
-                                                       int32_t* __restrict__ out, StepEnd end) {
+                                                       int32_t* ph, const uint16_t* fb,
+                                                       int32_t* out, StepEnd end) {
   after_previous();
   before_next();
   __shared__ int64_t qe[kFixQueue];
@@ -1822,16 +1822,18 @@ __global__ void __launch_bounds__(kFixThreads, 4) k_fixup(StepCtx c, int64_t nnz
     uint32_t res[kFixPer];
     FarRaw<kNarrow> ftv[kFixPer];
     uint32_t todo = 0;   // bit j: entry j is this pass's
+    bool unfilled = false;
 #pragma unroll
     for (int j = 0; j < kFixPer; ++j) {
       const uint32_t p = pv[j];
       res[j] = (p & kPhDone) && p != 0xFFFFFFFFu ? (p & ~kPhDone) : 0u;   // an earlier pass resolved it
       const uint32_t s = p >> 1;
       const bool mine = !(p & kPhDone) && s >= s_lo && s < s_hi && p < static_cast<uint32_t>(c.n);
-      if (!(p & kPhDone) && p >= static_cast<uint32_t>(c.n)) latch(c.err, kErrRowLength);   // a slot phase A did not fill
+      unfilled |= !(p & kPhDone) && p >= static_cast<uint32_t>(c.n);
       if (mine) ftv[j] = far_raw<kNarrow>(c.far_pack, s);
       todo |= static_cast<uint32_t>(mine) << j;
     }
+    if (unfilled) latch(c.err, kErrRowLength);   // a slot phase A did not fill
 #pragma unroll
     for (int j = 0; j < kFixPer; ++j) {
       if (!((todo >> j) & 1u)) continue;
@@ -1876,8 +1878,8 @@ __global__ void __launch_bounds__(kFixThreads, 4) k_fixup(StepCtx c, int64_t nnz
 // ---------------------------------------------------------------- team paths
 
 template <int NT, bool kOneSeed>
-__global__ void __launch_bounds__(NT, NT == 256 ? 4 : 1) k_phase_a_block(StepCtx c, const int32_t* __restrict__ lists,
-                                                      const int64_t* __restrict__ ctr, int cls, int smem_max,
+__global__ void __launch_bounds__(NT, NT == 256 ? 4 : 1) k_phase_a_block(StepCtx c, const int32_t* lists,
+                                                      const int64_t* ctr, int cls, int smem_max,
                                                       size_t room, char* gws, size_t slice, int stage_cap) {
   after_previous();
   before_next();
@@ -1985,8 +1987,8 @@ __device__ bool run_large(BlockTeam<NT>& tm, const StepCtx& c, int64_t t, char* 
 // 8192 of them in registers.  n=2^25, degrees [10,10000): 7.4 ms per step with
 // the shared-memory form (k_phase_a_block) up to 8192 entries, 4.7 so.
 template <bool kOneSeed>
-__global__ void __launch_bounds__(kBigThreads, 1) k_phase_a_huge(StepCtx c, const int32_t* __restrict__ lists,
-                                                               const int64_t* __restrict__ ctr, int gen_max,
+__global__ void __launch_bounds__(kBigThreads, 1) k_phase_a_huge(StepCtx c, const int32_t* lists,
+                                                               const int64_t* ctr, int gen_max,
                                                                char* gws, size_t slice) {
   after_previous();
   before_next();
@@ -2011,8 +2013,8 @@ __global__ void __launch_bounds__(kBigThreads, 1) k_phase_a_huge(StepCtx c, cons
   }
 }
 
-__global__ void __launch_bounds__(32 * kWarpWarps, 4) k_retry_warp(StepCtx c, const int32_t* __restrict__ list,
-                                                                const unsigned long long* __restrict__ count,
+__global__ void __launch_bounds__(32 * kWarpWarps, 4) k_retry_warp(StepCtx c, const int32_t* list,
+                                                                const unsigned long long* count,
                                                                 unsigned long long* claim) {
   extern __shared__ __align__(16) char wsm[];
   const int wid = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -2028,8 +2030,8 @@ __global__ void __launch_bounds__(32 * kWarpWarps, 4) k_retry_warp(StepCtx c, co
   }
 }
 template <int NT>
-__global__ void __launch_bounds__(NT, NT == 256 ? 4 : 1) k_retry(StepCtx c, const int32_t* __restrict__ list,
-                                                              const unsigned long long* __restrict__ count,
+__global__ void __launch_bounds__(NT, NT == 256 ? 4 : 1) k_retry(StepCtx c, const int32_t* list,
+                                                              const unsigned long long* count,
                                                               unsigned long long* claim, int gen_max, size_t room,
                                                               char* gws, size_t slice) {
   extern __shared__ __align__(16) char sbuf[];
@@ -2078,10 +2080,10 @@ __device__ __forceinline__ int chunk_work(int64_t n, int ctas, int least) {
 
 constexpr int kDefListThreads = 256;
 __global__ void __launch_bounds__(kDefListThreads) k_def_list(StepCtx c, int64_t nwords, int nsegs, int ctas,
-                                                             int32_t* __restrict__ list,
-                                                             int32_t* __restrict__ chunk_first,
-                                                             unsigned long long* __restrict__ nchunks,
-                                                             int64_t* __restrict__ clear) {
+                                                             int32_t* list,
+                                                             int32_t* chunk_first,
+                                                             unsigned long long* nchunks,
+                                                             int64_t* clear) {
   after_previous();
   before_next();
   if (clear && blockIdx.x == 0)   // the next step's counters
@@ -2145,9 +2147,9 @@ __global__ void __launch_bounds__(kDefListThreads) k_def_list(StepCtx c, int64_t
 }
 
 template <int NT>
-__global__ void __launch_bounds__(NT, NT == 256 ? 4 : 1) k_resolve(StepCtx c, const int32_t* __restrict__ list,
-                                                                const int32_t* __restrict__ chunk_first,
-                                                                const unsigned long long* __restrict__ nchunks,
+__global__ void __launch_bounds__(NT, NT == 256 ? 4 : 1) k_resolve(StepCtx c, const int32_t* list,
+                                                                const int32_t* chunk_first,
+                                                                const unsigned long long* nchunks,
                                                                 unsigned long long* claim, int gen_max, size_t room,
                                                                 char* gws, size_t slice) {
   after_previous();
