@@ -290,6 +290,9 @@ int cb_timings(cb_handle h, double* ms, int count);
  *               starts a new record; 0 stops and frees it [0].
  *   "fix_passes" passes of the rebuild over slices of the far trades (0:
  *               as many as keep one slice's records in L2) [0]; 0..64.
+ *   "fix_ctas"  CTAs of the rebuild (a test of its queue of ties, which one
+ *               of many CTAs fills only in the largest graphs); 0: four per
+ *               SM [0]; 0..65535.
  *   "swap_stats" 1: count neighbourhood swaps (see cb_swap_counts) from zero
  *               in every later super step and uniform trade; super steps
  *               then run without the recorded CUDA graphs, plus one counting

@@ -940,6 +940,11 @@ int cb_set_option(cb_handle h, const char* key, int64_t value) {
     h->fix_passes = static_cast<int>(value);
     return CB_OK;
   }
+  if (!std::strcmp(key, "fix_ctas")) {
+    if (value < 0 || value > 65535) return fail(h, CB_EINVAL, "fix_ctas out of range [0, 65535]");
+    h->fix_ctas = static_cast<int>(value);
+    return CB_OK;
+  }
   if (!std::strcmp(key, "cta_paths")) {
     if (value < 0 || value > 1) return fail(h, CB_EINVAL, "cta_paths is 0 or 1");
     h->cta_paths = static_cast<int>(value);

@@ -137,6 +137,7 @@ struct Graph {
   int tile_max = kTileMaxCap;
   int tile_paths = 1;   // threshold phase of small trades: 1 one warp per trade, 0 256-thread CTAs
   int fix_passes = 0;   // passes of the rebuild's fix-up over slices of the far trades (0: sized for L2)
+  int fix_ctas = 0;             // test hook: CTAs of the rebuild (0: four per SM)
   int cta_paths = 1;    // threshold phase of larger trades: 1 register-resident CTA kernels, 0 shared-memory ones
   int cand_max = 32;    // register paths: candidates ranked directly (tests lower it to force radix digits)
   uint64_t wait_ns = 1000000000ull;       // longest single wait of a super step (dependency, bulk copy)

@@ -1819,6 +1819,7 @@ __global__ void __launch_bounds__(kFixThreads, 4) k_fixup(StepCtx c, int64_t nnz
     const int64_t nxt = ch + gridDim.x;
     if (nxt < nchunks) fix_load<kLast>(ph, fb, nxt * kFixChunk + tofs, nnz, pn, bn);
     // first every gather of the thread's entries in this slice, then the decisions
+    bool full = false;   // this thread took a place that leaves no room for a chunk more
     uint32_t res[kFixPer];
     FarRaw<kNarrow> ftv[kFixPer];
     uint32_t todo = 0;   // bit j: entry j is this pass's
@@ -1844,7 +1845,9 @@ __global__ void __launch_bounds__(kFixThreads, 4) k_fixup(StepCtx c, int64_t nnz
       if (b & kFbInFar) {   // the far trade decides: key prefixes first
         const uint32_t f8 = ((b >> 1) & ((1u << kFarBits) - 1u)) >> (kFarBits - 8);
         if (f8 == ft.top) {   // 1 in 256: resolved with the queue
-          qe[atomicAdd(&qn, 1)] = base + j;
+          const int at = atomicAdd(&qn, 1);
+          qe[at] = base + j;
+          full |= at >= kFixQueue - kFixChunk;
           continue;
         }
         side = f8 < ft.top ? 0 : 1;
@@ -1863,8 +1866,10 @@ __global__ void __launch_bounds__(kFixThreads, 4) k_fixup(StepCtx c, int64_t nnz
           if (base + j < nnz) out[base + j] = static_cast<int32_t>(res[j]);
       }
     }
-    __syncthreads();   // queued entries (and, on the last pass, their vector stores) are in place
-    if (qn > kFixQueue - kFixChunk) flush();   // room for a whole chunk more
+    // queued entries (and, on the last pass, their vector stores) are in place.
+    // The barrier carries the decision to flush: a look at qn after it could
+    // see the next chunk's entries of a faster warp, and differ between warps.
+    if (__syncthreads_or(full)) flush();
 #pragma unroll
     for (int j = 0; j < kFixPer; ++j) pv[j] = pn[j];
 #pragma unroll
@@ -2577,7 +2582,7 @@ int super_step(Graph* h, bool ahead) {
     const int64_t nchunks = (nnz + kFixChunk - 1) / kFixChunk;
     const int passes = fix_passes(h);
     const int64_t per = (ntasks + passes - 1) / passes;
-    const unsigned fgrid = static_cast<unsigned>(std::min<int64_t>(nchunks, int64_t(h->num_sms) * 4));
+    const unsigned fgrid = static_cast<unsigned>(std::min<int64_t>(nchunks, h->fix_ctas ? h->fix_ctas : h->num_sms * 4));
     int32_t* out = h->col[cur];
     for (int q = 0; q < passes; ++q) {
       const uint32_t lo = static_cast<uint32_t>(std::min<int64_t>(ntasks, q * per));
