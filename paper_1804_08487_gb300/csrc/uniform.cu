@@ -34,6 +34,7 @@
 
 #include "cb_internal.cuh"
 #include "philox.cuh"
+#include "run_queues.cuh"
 #include "team.cuh"
 
 namespace cb {
@@ -242,38 +243,32 @@ struct UniCtx {
   int64_t hold_trade;          // test hook: messages to this trade of the chunk are dropped (-1: none)
 };
 
-// The two run queues, small trades from the front of the array and large ones
-// from its back: a ticket (kHead) takes the queue's next place, a push (kTail)
-// fills the next place; the counters sit on different cache lines.  Every
-// trade is queued exactly once and kBig says how many are large, so every
-// ticket below a queue's length ends.
+// The two run queues (run_queues.cuh): a ticket (kHead) takes the queue's next
+// place, a push (kTail) fills the next place; the counters sit on different
+// cache lines.  Every trade is queued exactly once and kBig says how many are
+// large, so every ticket below a queue's length ends; a push past it latches
+// the error and touches no place.
 constexpr int kHead = 0, kTail = 16, kQueueCtr = 32, kBig = 64, kCtrWords = 80;
 
-__device__ __forceinline__ int64_t queue_len(const UniCtx& c, int big) {
-  const int64_t nb = static_cast<int64_t>(c.ctr[kBig]);
-  return big ? nb : c.L - nb;
-}
-
-__device__ __forceinline__ int32_t* queue_at(const UniCtx& c, int big, unsigned long long q) {
-  return c.queue + (big ? c.L - 1 - static_cast<int64_t>(q) : static_cast<int64_t>(q));
-}
+__device__ __forceinline__ RunQueues queues(const UniCtx& c) { return {c.L, static_cast<int64_t>(c.ctr[kBig])}; }
 
 __device__ __forceinline__ void push(const UniCtx& c, int64_t k, int64_t entries) {
   const int big = entries > c.small;
+  const RunQueues rq = queues(c);
   const unsigned long long q = atomicAdd(&c.ctr[kQueueCtr * big + kTail], 1ull);
-  if (q >= static_cast<unsigned long long>(c.L)) {
+  if (!rq.holds(big, q)) {
     latch(c.err, kErrUniform);
     return;
   }
-  st_relaxed_i32(queue_at(c, big, q), static_cast<int32_t>(k));
+  st_relaxed_i32(c.queue + rq.place(big, q), static_cast<int32_t>(k));
 }
 
-// The next queued trade, or -1 when every place of the queue (of len trades)
-// is taken or a wait gave up.
-__device__ int64_t take_ticket(const UniCtx& c, int big, int64_t len) {
+// The next queued trade, or -1 when every place of the queue is taken or a
+// wait gave up.
+__device__ int64_t take_ticket(const UniCtx& c, int big, const RunQueues& rq) {
   const unsigned long long q = atomicAdd(&c.ctr[kQueueCtr * big + kHead], 1ull);
-  if (q >= static_cast<unsigned long long>(len)) return -1;
-  const int32_t* place = queue_at(c, big, q);
+  if (!rq.holds(big, q)) return -1;
+  const int32_t* place = c.queue + rq.place(big, q);
   int32_t t = ld_relaxed_i32(place);
   if (t < 0) {
     const uint64_t t0 = globaltimer();
@@ -786,6 +781,7 @@ __global__ void __launch_bounds__(NT, 1024 / NT) k_uni_exec(const __grid_constan
   __shared__ int32_t small_hash[uni_warps<NT>()][kSmallHash];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   unsigned long long moved = 0, possible = 0;   // swaps, for the handle's counters
+  const RunQueues rq = queues(c);
   bool ok = true;
   int32_t* hash = warp < kTeam / 32 ? reinterpret_cast<int32_t*>(usm) + warp * kSmallHash : small_hash[warp - kTeam / 32];
   if (warp < kTeam / 32) {
@@ -795,9 +791,8 @@ __global__ void __launch_bounds__(NT, 1024 / NT) k_uni_exec(const __grid_constan
     const TradeWs ws_glob =
         c.gslice ? carve_ws(c.gslice + static_cast<size_t>(blockIdx.x) * c.slice_elems * kWsBytesPerElem, c.slice_elems)
                  : ws_smem;
-    const int64_t len = queue_len(c, 1);
     while (ok) {
-      if (tm.rank == 0) s_k = take_ticket(c, 1, len);
+      if (tm.rank == 0) s_k = take_ticket(c, 1, rq);
       tm.sync();
       const int64_t k = s_k;
       if (k < 0) break;
@@ -812,10 +807,9 @@ __global__ void __launch_bounds__(NT, 1024 / NT) k_uni_exec(const __grid_constan
       }
     }
   }
-  const int64_t len = queue_len(c, 0);
   while (ok) {
     int64_t k = 0;
-    if (lane == 0) k = take_ticket(c, 0, len);
+    if (lane == 0) k = take_ticket(c, 0, rq);
     k = __shfl_sync(kFull, k, 0);
     if (k < 0) break;
     const Trade t = load_trade(c, k);
@@ -834,12 +828,16 @@ __global__ void __launch_bounds__(NT, 1024 / NT) k_uni_exec(const __grid_constan
   }
 }
 
-// Every output row full, and every trade queued and taken exactly once.
+// Every output row full, and every place of both queues filled once and taken.
 __global__ void k_uni_check(int64_t n, const int64_t* __restrict__ rp, const int32_t* __restrict__ ocur,
                             const unsigned long long* __restrict__ ctr, int64_t L, int32_t* err) {
   if (blockIdx.x == 0 && threadIdx.x == 0) {
-    const unsigned long long l = static_cast<unsigned long long>(L);
-    if (ctr[kTail] + ctr[kQueueCtr + kTail] != l) latch(err, kErrUniform);
+    const RunQueues rq{L, static_cast<int64_t>(ctr[kBig])};
+    for (int big = 0; big < 2; ++big) {
+      const int64_t len = rq.length(big);
+      if (static_cast<int64_t>(ctr[kQueueCtr * big + kTail]) != len || static_cast<int64_t>(ctr[kQueueCtr * big + kHead]) < len)
+        latch(err, kErrUniform);
+    }
   }
   for (int64_t x = blockIdx.x * int64_t(blockDim.x) + threadIdx.x; x < n; x += int64_t(gridDim.x) * blockDim.x)
     if (ocur[x] != rp[x + 1] - rp[x]) latch(err, kErrRowLength);
