@@ -370,9 +370,11 @@ int cb_permutation_static(int64_t n, uint64_t seed, uint64_t g, int32_t* order_o
  * Pick the fastest work split for this handle: runs up to max_steps real
  * super steps (they advance the chain; the result does not depend on the
  * options): one to load the kernels, then the rest shared evenly by the
- * current settings and the candidate settings, one knob at a time, of
- * "tile_max", "block_max", "smem_max", "inorder_threads" and
- * "retry_passes", timed with CUDA events; a candidate replaces the best
+ * current settings (which also get what is left over) and the candidate
+ * settings, one knob at a time, of "tile_max", "block_max", "smem_max",
+ * "inorder_threads" and, where the handle runs retry passes, "retry_passes".
+ * Each setting's steps are launched as one call of cb_global_trades launches
+ * them and timed with CUDA events; a candidate replaces the best
  * setting so far only when it is at least 2 % faster.  chosen (may be NULL) receives up to
  * `count` values: tile_max, block_max, smem_max, inorder_threads, super
  * steps used, retry_passes.  Returns the number of values written.

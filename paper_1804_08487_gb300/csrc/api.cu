@@ -413,6 +413,25 @@ int settle_sets(Graph* h, int32_t* const orders[2], int32_t* const poss[2], int6
   return CB_OK;
 }
 
+// `steps` super steps launched directly, each step's permutation beside the
+// step before where the handle allows it; with swap counts and the presence
+// record when `record`.
+int direct_steps(Graph* h, uint32_t steps, bool record) {
+  const bool ahead = steps > 1 && runs_ahead(h);
+  int32_t* const orders[2] = {h->order[0], h->order[1]};
+  int32_t* const poss[2] = {h->pos[0], h->pos[1]};
+  int64_t* const rps[2] = {h->rp[0], h->rp[1]};
+  int rc = CB_OK;
+  for (uint32_t i = 0; i < steps && !rc; ++i) {
+    rc = super_step(h, ahead && i + 1 < steps);
+    if (!rc && record && h->swap_stats) rc = count_swaps(h);
+    if (!rc && record && h->pres) rc = record_presence(h);
+  }
+  if (!rc && ahead) rc = settle_sets(h, orders, poss, rps);
+  if (rc && ahead) h->latched = rc;   // the sets are where recorded steps do not look for them
+  return rc;
+}
+
 // Every graph's canonical pairs (local ids) of the current step in h->pairs.
 int ensure_pairs(Graph* h) {
   if (h->pairs && h->pairs_step == h->g) return CB_OK;
@@ -728,22 +747,8 @@ int cb_global_trades(cb_handle h, uint32_t supersteps) {
       h->launches += h->step_launches;
     }
   } else {
-    int32_t* const orders[2] = {h->order[0], h->order[1]};
-    int32_t* const poss[2] = {h->pos[0], h->pos[1]};
-    int64_t* const rps[2] = {h->rp[0], h->rp[1]};
-    for (uint32_t i = 0; i < supersteps; ++i) {
-      int rc = super_step(h, ahead && i + 1 < supersteps);
-      if (!rc && h->swap_stats) rc = count_swaps(h);
-      if (!rc && h->pres) rc = record_presence(h);
-      if (rc) {
-        if (ahead) h->latched = rc;   // the sets are where recorded steps do not look for them
-        return rc;
-      }
-    }
-    if (ahead) {
-      const int rc = settle_sets(h, orders, poss, rps);
-      if (rc) return rc;
-    }
+    const int rc = direct_steps(h, supersteps, true);
+    if (rc) return rc;
   }
   h->stats[5] = h->launches - launches0;
   return CB_OK;
@@ -1027,18 +1032,18 @@ int cb_autotune(cb_handle h, uint32_t max_steps, int64_t* chosen, int count) {
   drop_step_graphs(h);
   const bool timing = h->timing;
   h->timing = false;
+  const uint64_t g0 = h->g;
   uint32_t used = 0;
   int rc = CB_OK;
-  // `per` super steps under the current options (fewer if the budget ends);
-  // ms = their device time per step
-  uint32_t per = 1;
-  auto trial = [&](float* ms) -> int {
+  // `steps` super steps under the current options (fewer if the budget ends),
+  // launched as one call of that many steps launches them; ms = their device
+  // time per step
+  auto trial = [&](uint32_t steps, float* ms) -> int {
     if (cudaEventRecord(e0, h->stream) != cudaSuccess) return fail(h, CB_ECUDA, "cudaEventRecord failed");
-    uint32_t k = 0;
-    for (; k < per && used < max_steps; ++k, ++used) {
-      const int r = super_step(h);
-      if (r) return r;
-    }
+    const uint32_t k = std::min(steps, max_steps - used);
+    const int r = direct_steps(h, k, false);
+    used = static_cast<uint32_t>(h->g - g0);
+    if (r) return r;
     if (cudaEventRecord(e1, h->stream) != cudaSuccess || cudaEventSynchronize(e1) != cudaSuccess ||
         cudaEventElapsedTime(ms, e0, e1) != cudaSuccess)
       return fail(h, CB_ECUDA, "event timing failed");
@@ -1051,35 +1056,40 @@ int cb_autotune(cb_handle h, uint32_t max_steps, int64_t* chosen, int count) {
     int ncand;
   };
   constexpr int kKnobs = 5;
+  const int nknobs = runs_retries(h) ? kKnobs : kKnobs - 1;   // elsewhere retry_passes launches nothing
   Knob knobs[kKnobs] = {{&h->tile_max, {32, 64, 128, 0}, 3},
                         {&h->block_max, {512, 1024, 2048, 0}, 3},
                         {&h->smem_max, {4096, 8192, 0, 0}, 2},
                         {&h->inorder_threads, {256, 1024, 0, 0}, 2},
                         {&h->retry_passes, {1, 2, 3, 0}, 3}};
   float ms = 0;
-  if (used < max_steps) rc = trial(&ms);   // first launches load the kernels: not timed as a candidate
+  if (used < max_steps) rc = trial(1, &ms);   // first launches load the kernels: not timed as a candidate
+  // the current settings, then every other candidate: super steps shared
+  // evenly, at least one each; the current settings get what is left over
+  uint32_t per = 1, first = 1;
   {
-    // the current settings, then every other candidate: super steps shared
-    // evenly, at least one each
-    int total = 1;
-    for (const Knob& kn : knobs) total += kn.ncand;
-    if (max_steps > used) per = std::max<uint32_t>(1, (max_steps - used) / static_cast<uint32_t>(total));
+    uint32_t others = 0;
+    for (int k = 0; k < nknobs; ++k)
+      for (int j = 0; j < knobs[k].ncand; ++j) others += knobs[k].cand[j] != *knobs[k].field;
+    const uint32_t left = max_steps - used;
+    per = std::max<uint32_t>(1, left / (1 + others));
+    first = left > per * others ? left - per * others : per;
   }
   float best_ms = 3.4e38f;
   if (rc == CB_OK && used < max_steps) {
-    rc = trial(&ms);
+    rc = trial(first, &ms);
     if (rc == CB_OK) best_ms = ms;
   }
   // one knob at a time; a setting replaces the best one so far only when it
   // is at least 2 % faster (a step's time varies with its deferred trades)
-  for (int k = 0; k < kKnobs && rc == CB_OK; ++k) {
+  for (int k = 0; k < nknobs && rc == CB_OK; ++k) {
     const int cur = *knobs[k].field;
     int best = cur;
     for (int j = 0; j < knobs[k].ncand && used < max_steps && rc == CB_OK; ++j) {
       if (knobs[k].cand[j] == cur) continue;
       *knobs[k].field = knobs[k].cand[j];
       rc = size_trade_workspace(h);   // the global workspace follows block_max and smem_max
-      if (rc == CB_OK) rc = trial(&ms);
+      if (rc == CB_OK) rc = trial(per, &ms);
       if (rc == CB_OK && ms < 0.98f * best_ms) {
         best_ms = ms;
         best = knobs[k].cand[j];

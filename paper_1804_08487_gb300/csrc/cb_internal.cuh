@@ -303,6 +303,7 @@ int flush_timing(Graph* h, int set, bool add);   // wait for a recorded event se
 int init_trade_kernels(Graph* h);   // one-time kernel attributes (outside stream capture)
 int init_perm_kernels(Graph* h);
 size_t trade_ws_slice_bytes(int64_t max_trade);
+bool runs_retries(const Graph* h);     // large enough for retry passes
 int retry_passes_of(const Graph* h);   // retry passes a super step launches
 bool small_handle(const Graph* h);     // launch-bound: its super steps use overlapped launches
 

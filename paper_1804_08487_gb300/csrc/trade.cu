@@ -2317,7 +2317,8 @@ int fix_passes(const Graph* h) {
 // trades the in-order pass alone is faster.
 constexpr int64_t kRetryMin = int64_t(1) << 20;
 bool small_handle(const Graph* h) { return h->ntasks < kOverlapMax; }
-int retry_passes_of(const Graph* h) { return h->ntasks >= kRetryMin ? h->retry_passes : 0; }
+bool runs_retries(const Graph* h) { return h->ntasks >= kRetryMin; }
+int retry_passes_of(const Graph* h) { return runs_retries(h) ? h->retry_passes : 0; }
 
 // The next step's permutation and class lists need nothing of this step's
 // trades.  With another step to come they are computed beside the in-order
