@@ -202,7 +202,7 @@ int cb_stats(cb_handle h, int64_t* out, int count);
  * threshold phase (every trade's |A_{u-v}|-th smallest key, including the
  * passes that resolve dependent trades), ms[2] = the rebuild phase (new rows
  * for the next step), ms[3] = whole super steps, ms[4 + k], k < 9 = the
- * first threshold pass's kernel of size class k (below 2^17 trades classes 0
+ * first threshold pass's kernel of size class k (below "fuse_max" trades classes 0
  * to 5 share class 0's kernel and 6 and 7 class 6's; the others' entries are
  * then near 0), ms[13] = the retry passes over deferred trades, ms[14] = the
  * in-order pass.  Returns the number of values written
@@ -252,8 +252,14 @@ int cb_timings(cb_handle h, double* ms, int count);
  *   "retry_passes" parallel passes over the deferred trades between the
  *               first pass and the in-order pass, each running every deferred
  *               trade whose dependencies have published by then [2]; 0..4.
- *               Handles of fewer than 2^20 trades go straight to the in-order
- *               pass, which is faster there.
+ *               Handles of fewer than "retry_min" trades go straight to the
+ *               in-order pass, which is faster there.
+ *   "retry_min" trades from which a handle runs retry passes [2^20]; 0..2^31
+ *               (a test knob: any value on any handle).
+ *   "fuse_max"  trades from which the first pass has a kernel per size class
+ *               of eight entries per thread above 256 entries, instead of
+ *               two kernels of four [2^17]; 0..2^31 (a test knob: any value
+ *               on any handle).
  *   "relaxed"   1: relaxed global trades (Def. "Relaxed global trade",
  *               Appendix EM-GCB): super step g orders the nodes by
  *               h(x) = (a x + b) mod p, p the smallest prime >= n, with

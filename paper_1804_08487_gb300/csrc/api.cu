@@ -945,6 +945,11 @@ int cb_set_option(cb_handle h, const char* key, int64_t value) {
     h->fix_passes = static_cast<int>(value);
     return CB_OK;
   }
+  if (!std::strcmp(key, "fuse_max") || !std::strcmp(key, "retry_min")) {
+    if (value < 0 || value > (int64_t(1) << 31)) return fail(h, CB_EINVAL, std::string(key) + " out of range [0, 2^31]");
+    (key[0] == 'f' ? h->fuse_max : h->retry_min) = value;
+    return CB_OK;
+  }
   if (!std::strcmp(key, "fix_ctas")) {
     if (value < 0 || value > 65535) return fail(h, CB_EINVAL, "fix_ctas out of range [0, 65535]");
     h->fix_ctas = static_cast<int>(value);

@@ -46,6 +46,8 @@ constexpr int kCtrFinished = 40;    // chunks of the in-order pass claimed
 constexpr int kCtrChunks = 41;      // its chunks
 constexpr int kCtrClaim = 42;       // [42 + 3 r, 45 + 3 r): trades of each list that retry pass r claimed
 static_assert(24 + 3 * (kRetryPassesMax + 1) <= 40 && 42 + 3 * kRetryPassesMax <= kCounters - 1, "counter layout");
+constexpr int64_t kFuseMax = int64_t(1) << 17;    // trades from which the first pass has a kernel per class
+constexpr int64_t kRetryMin = int64_t(1) << 20;   // trades from which retry passes run
 constexpr int kRowChunk = 2048;      // entries per sample of the entry -> row index
 constexpr int kScratch = 16;         // device words of a handle for creation and export
 constexpr int kDefSegs = 1024;      // most segments of the trades that deferred ones are counted in
@@ -137,6 +139,7 @@ struct Graph {
   int tile_max = kTileMaxCap;
   int tile_paths = 1;   // threshold phase of small trades: 1 one warp per trade, 0 256-thread CTAs
   int fix_passes = 0;   // passes of the rebuild's fix-up over slices of the far trades (0: sized for L2)
+  int64_t fuse_max = kFuseMax, retry_min = kRetryMin;   // options, to test both sides on small graphs
   int fix_ctas = 0;             // test hook: CTAs of the rebuild (0: four per SM)
   int cta_paths = 1;    // threshold phase of larger trades: 1 register-resident CTA kernels, 0 shared-memory ones
   int cand_max = 32;    // register paths: candidates ranked directly (tests lower it to force radix digits)

@@ -1492,7 +1492,7 @@ struct TeamCfg {
 // each (n=4096, four classes: 53 us -> 18 in one kernel; n=2^17: 153 -> 135).
 // Large graphs keep a kernel per class: CTAs of one SM in different classes
 // share its instruction cache badly (n=2^20: 848 us per class, 947 together).
-constexpr int64_t kFuseMax = int64_t(1) << 17;
+// (kFuseMax in cb_internal.cuh.)
 struct Rounds {
   int64_t at = 0;   // rounds of the classes so far
   // this CTA's first round of a class of `rounds`
@@ -2314,10 +2314,9 @@ int fix_passes(const Graph* h) {
 }
 
 // Retry passes run where many trades are deferred at once; below kRetryMin
-// trades the in-order pass alone is faster.
-constexpr int64_t kRetryMin = int64_t(1) << 20;
+// trades (cb_internal.cuh) the in-order pass alone is faster.
 bool small_handle(const Graph* h) { return h->ntasks < kOverlapMax; }
-bool runs_retries(const Graph* h) { return h->ntasks >= kRetryMin; }
+bool runs_retries(const Graph* h) { return h->ntasks >= h->retry_min; }
 int retry_passes_of(const Graph* h) { return runs_retries(h) ? h->retry_passes : 0; }
 
 // The next step's permutation and class lists need nothing of this step's
@@ -2453,7 +2452,7 @@ int super_step(Graph* h, bool ahead) {
   // twice the largest degree: classes above that are not launched); a trade
   // whose dependency has not published yet is deferred.  With "timing" on,
   // events ev[4] .. ev[13] bracket the classes' kernels.
-  const bool fused = ntasks < kFuseMax, overlap = small_handle(h);
+  const bool fused = ntasks < h->fuse_max, overlap = small_handle(h);
   auto mark = [&](int k) -> int {
     if (h->timing) CB_CUDA(h, cudaEventRecord(ev[4 + k], s));
     return CB_OK;
