@@ -119,9 +119,11 @@ __global__ void k_autocorr(int64_t npairs, int64_t first, int64_t W, int64_t sta
 //     (1,1) as series & (series >> k);
 //   - every term of G^2 is i ln i for a count i <= N, read from a table in
 //     fixed point (rounded from long double), so G^2 is a sum of integers.
-//     The scale keeps the largest value below 2^61: G^2 - ln N is then within
-//     1.2e-13 of its exact value at 8192 states and 1e-14 at 301, where the
-//     FP64 formula is off by up to 4.5e-12 and 1.9e-13.
+//     The scale keeps the largest value below 2^61.  Nine terms, rounded by up
+//     to half a unit and doubled, and ln N leave G^2 - ln N within 9.5 units of
+//     its exact value: 5.4e-13 at 8192 states, 8.4e-15 at 301.  The largest
+//     errors over 200000 random tables are 4.3e-13 and 6.3e-15; the FP64
+//     formula's on the same tables are 5.3e-12 and 2.2e-13.
 // 8 graphs of 2000 nodes, 301 states, kmax 32: the whole pass (300 super
 // steps, record, classification) went from 212 to 69 ms, all but 5 ms of it
 // here.
