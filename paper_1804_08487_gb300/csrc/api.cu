@@ -62,12 +62,21 @@ void dfree(Graph* h, void* p) {
   if (p) cudaFreeAsync(p, h->stream);
 }
 
+// The 16-byte records of the "wide_pack" option.
+size_t wide_bytes(const Graph* h) { return 16 * static_cast<size_t>(std::max<int64_t>(h->ntasks, 1)); }
+void free_wide(Graph* h) {
+  if (!h->far_wide) return;
+  dfree(h, h->far_wide);
+  h->dev_bytes -= static_cast<int64_t>(wide_bytes(h));
+  h->far_wide = nullptr;
+}
+
 void release(Graph* h) {
   if (!h) return;
   if (h->stream) cudaStreamSynchronize(h->stream);
   free_uniform(h);
   free_presence(h);
-  void* bufs[] = {h->arena, h->ws_global, h->pairs, h->lcg_ab, h->lcg_gaps, h->swaps};
+  void* bufs[] = {h->arena, h->far_wide, h->ws_global, h->pairs, h->lcg_ab, h->lcg_gaps, h->swaps};
   if (h->stream)
     for (void* b : bufs) dfree(h, b);
   for (auto& x : h->step_exec)
@@ -225,9 +234,12 @@ int alloc_arrays(Graph* h) {
   h->m = nnz / 2;
   h->T = n / 2;
   h->ntasks = h->T + (n & 1);
-  int64_t slots = 0;
-  for (int i = 0; i < h->nseg; ++i) slots += int64_t(h->hsegs[i].cap) << h->hsegs[i].B;
-  const size_t sort_bytes = perm_ws_bytes(h->nbuckets, std::max<int64_t>(slots, 1));
+  int64_t slots = 0, keys = 0;
+  for (int i = 0; i < h->nseg; ++i) {
+    slots += int64_t(h->hsegs[i].cap) << h->hsegs[i].B;
+    keys += h->hsegs[i].span << h->hsegs[i].B;
+  }
+  const size_t sort_bytes = perm_ws_bytes(h->nbuckets, perm_rescans(h->nbuckets, keys) ? 0 : slots);
   const size_t scan_bytes = scan_ws_bytes(std::max<int64_t>(n + 1, h->nbuckets + 1));
   size_t used = 0, zeroed = 0;
   char* base = nullptr;
@@ -262,9 +274,9 @@ int alloc_arrays(Graph* h) {
     take(&h->stash, nnz);
     take(&h->thr_key, h->ntasks);
     take(&h->thr_tb, h->ntasks);
-    take(&h->far_pack, h->ntasks);
-    take(&h->lists, kClasses * h->ntasks);
-    take(&h->def_list, 3 * h->ntasks + 2);
+    take(&h->far_pack, h->ntasks * (n <= kNarrowPackMax ? 1 : 2));
+    take(&h->lists, kClassLists * h->ntasks);
+    take(&h->def_list, 2 * h->ntasks + 2);
     if (may_run_ahead(h->ntasks, nnz)) {
       take(&h->order2, n);
       take(&h->pos2, n);
@@ -511,9 +523,10 @@ int64_t estimate_handle_bytes(int64_t n, int64_t nnz, int64_t maxdeg, int num_sm
   int64_t b = 0;
   b += sizeof(Seg) + 8 * (n + 1) + 4 * n + 2 * 4 * (nnz + kColPad) + 32 + 8 * (2 * kCounters + 1 + kScratch);   // cb_create
   b += 2 * 4 * n + 2 * 8 * (n + 1) + 2 * 4 * n + 2 * nnz + 4 * (nnz / kRowChunk + 2);                                 // per node, side words
-  b += ntasks * (8 + 8 + 4 + 16 + 4 * kClasses + 4 * 3) + ntasks / 8 + 4 * 3 * kDefSegs + 16;                                  // per trade
+  b += ntasks * (8 + 8 + 4 + (n <= kNarrowPackMax ? 8 : 16) + 4 * kClassLists + 4 * 2) + ntasks / 8 + 4 * 3 * kDefSegs + 16;                                  // per trade
   if (may_run_ahead(ntasks, nnz)) b += 2 * 4 * n + 8 * (n + 1) + 4 * (nnz / kRowChunk + 2);
-  b += static_cast<int64_t>(perm_ws_bytes(nb, nb * bucket_space(n, bucket_bits(n))) + scan_ws_bytes(n + 1));
+  b += static_cast<int64_t>(perm_ws_bytes(nb, perm_rescans(nb, n * nb) ? 0 : nb * bucket_space(n, bucket_bits(n))) +
+                            scan_ws_bytes(n + 1));
   const int64_t max_trade = 2 * maxdeg;
   if (max_trade > kBlockMaxDefault || maxdeg > 16384) {   // default block_max
     const size_t slice = trade_ws_slice_bytes(std::max<int64_t>(max_trade, 1));
@@ -1013,7 +1026,13 @@ int cb_set_option(cb_handle h, const char* key, int64_t value) {
   }
   if (!std::strcmp(key, "wide_pack")) {
     if (value < 0 || value > 1) return fail(h, CB_EINVAL, "wide_pack is 0 or 1");
-    h->wide_pack = value != 0;
+    if (!value) {
+      free_wide(h);
+    } else if (!h->far_wide) {
+      void* p = nullptr;
+      CB_CUDA(h, dmalloc(h, &p, wide_bytes(h)));
+      h->far_wide = p;
+    }
     return CB_OK;
   }
   if (!std::strcmp(key, "bucket_cap")) {

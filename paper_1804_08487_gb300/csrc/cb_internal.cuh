@@ -37,6 +37,7 @@ constexpr int kCounters = 64;       // device counters of one super step (two se
 // Trade size classes of the threshold phase (one team size each) and the
 // device counters of a super step.
 constexpr int kClasses = 9;
+constexpr int kClassLists = (kClasses + 1) / 2;   // arrays of their lists, two classes to each
 constexpr int kWarpClasses = 3;     // classes 0..2 run on warps or parts of a warp
 constexpr int kCtrClsLen = 0;       // [0, kClasses): trades per class
 constexpr int kCtrFirstEnt = 10;    // [10, 10 + kClasses): their directed entries
@@ -48,6 +49,7 @@ constexpr int kCtrClaim = 42;       // [42 + 3 r, 45 + 3 r): trades of each list
 static_assert(24 + 3 * (kRetryPassesMax + 1) <= 40 && 42 + 3 * kRetryPassesMax <= kCounters - 1, "counter layout");
 constexpr int64_t kFuseMax = int64_t(1) << 17;    // trades from which the first pass has a kernel per class
 constexpr int64_t kRetryMin = int64_t(1) << 20;   // trades from which retry passes run
+constexpr int64_t kNarrowPackMax = int64_t(1) << 28;   // nodes up to which a far-trade record fits 8 bytes
 constexpr int kRowChunk = 2048;      // entries per sample of the entry -> row index
 constexpr int kScratch = 16;         // device words of a handle for creation and export
 constexpr int kDefSegs = 1024;      // most segments of the trades that deferred ones are counted in
@@ -117,8 +119,9 @@ struct Graph {
   uint64_t* thr_key = nullptr;             // per trade: threshold key
   uint64_t* thr_tb = nullptr;              // per trade: threshold tie-break (lo<<32|hi)
   uint32_t* done = nullptr;                // per trade: the step + 1 once its threshold is published
-  int4* far_pack = nullptr;                // per trade: new positions of its nodes, threshold prefix (rebuild)
-  int32_t* lists = nullptr;                // kClasses x ntasks: the trades of each size class
+  uint64_t* far_pack = nullptr;            // per trade, 8 or (above kNarrowPackMax) 16 bytes: new positions of its nodes, threshold prefix (rebuild)
+  void* far_wide = nullptr;                // 16-byte records in its place, where 8 would do ("wide_pack", tests)
+  int32_t* lists = nullptr;                // kClassLists x ntasks: the trades of each size class (pair_lists.cuh)
   uint32_t* def_bits = nullptr;            // deferred trades, one bit each (zero between steps)
   int32_t* def_seg = nullptr;              // their counts per kind and segment (zero between steps)
   int32_t* def_list = nullptr;             // by kind for a retry pass; in index order with the chunks' first ones for the in-order pass
@@ -155,7 +158,6 @@ struct Graph {
   int retry_passes = 2;         // parallel passes over the deferred trades before the in-order pass
   int lane_teams = 1;           // trades up to 32 / 64 entries on teams of 8 / 16 lanes
   int uni_threads = 1024;       // CTA size of the uniform-trade executor (256, 512 or 1024)
-  bool wide_pack = false;       // 16-byte far-trade records even when 8 bytes would do (tests)
   // relaxed global trade: permutations from h(x) = (a x + b) mod p
   bool relaxed = false;
   uint64_t lcg_p = 0;           // smallest prime >= n
@@ -258,6 +260,9 @@ struct ClassArgs;
 size_t perm_ws_bytes(int64_t nbuckets, int64_t slots);
 int bucket_bits(int64_t n);
 int64_t bucket_space(int64_t span, int B);
+// Does a handle of so many buckets, with so many keys to compute for all of
+// them, take the one-kernel form?  (It needs no bucket space.)
+bool perm_rescans(int64_t nbuckets, int64_t keys);
 // order_out[p] = node at position p; pos_out[x] = position of x, rp_out[p] =
 // row offsets of that order (n + 1; either may be null).  Each segment uses
 // its device step counter + dg, or the step g_abs for all when g_abs >= 0.

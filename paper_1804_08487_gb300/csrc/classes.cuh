@@ -5,6 +5,7 @@
 // step's keys, so neither waits for the other and no launch is spent on them.
 #pragma once
 #include "cb_internal.cuh"
+#include "pair_lists.cuh"
 #include "team.cuh"
 
 namespace cb {
@@ -17,7 +18,7 @@ struct ClassArgs {
   int64_t n, ntasks;     // ntasks 0: nothing to classify
   const int64_t* rp;     // row offsets of the current step
   ClassTh th;
-  int32_t* lists;        // class k's trades from lists + k ntasks
+  int32_t* lists;        // two classes to an array of ntasks (pair_lists.cuh)
   int64_t* ctr;          // zeroed counters: kCtrClsLen, kCtrFirstEnt
 };
 
@@ -92,7 +93,7 @@ __device__ void classify_chunks(const ClassArgs& a, int64_t first, int64_t strid
         int p = 0;
         if (lane == 0) p = atomicAdd(&put[q], __popc(b));
         p = __shfl_sync(kFull, p, 0);
-        if (k == q) a.lists[q * a.ntasks + base[q] + p + __popc(b & below)] = static_cast<int32_t>(t);
+        if (k == q) a.lists[pair_place(q, base[q] + p + __popc(b & below), a.ntasks)] = static_cast<int32_t>(t);
       }
     }
     __syncthreads();

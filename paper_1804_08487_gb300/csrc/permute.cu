@@ -586,6 +586,8 @@ unsigned grid_for(int64_t work, int threads, int num_sms) {
 
 }  // namespace
 
+bool perm_rescans(int64_t nbuckets, int64_t keys) { return nbuckets <= kRescanBuckets && keys <= kRescanWork; }
+
 // Scratch of a handle: bucket words, prefixes, and `slots` ids of bucket space.
 size_t perm_ws_bytes(int64_t nbuckets, int64_t slots) {
   return zero_bytes(nbuckets) + align_up(sizeof(uint64_t) * (nbuckets + 1)) + align_up(sizeof(int32_t) * slots);
@@ -643,7 +645,7 @@ int compute_permutation(Graph* h, uint32_t dg, int64_t g_abs, int32_t* order_out
     CB_CUDA(h, cudaGetLastError());
     h->launches += 2;
     if (rp_out) {
-      int32_t* deg = carve(h->sort_ws, h->nbuckets).bid;   // bucket space: at least n
+      int32_t* deg = reinterpret_cast<int32_t*>(h->thr_key);   // 8 bytes per trade, free until the first pass
       k_order_degrees<<<grid_for(n, kPermThreads, h->num_sms), kPermThreads, 0, s>>>(n, order_out, h->deg_id, deg);
       CB_CUDA(h, cudaGetLastError());
       ++h->launches;
@@ -658,7 +660,7 @@ int compute_permutation(Graph* h, uint32_t dg, int64_t g_abs, int32_t* order_out
   const int64_t nb = h->nbuckets;
   const int cap = bucket_cap_of(h);
   const PermOut out{order_out, pos_out, rp_out, h->deg_id, !rp_out ? nullptr : beside ? h->chunk_row2 : h->chunk_row};
-  if (nb <= kRescanBuckets && rescan_work(h) <= kRescanWork) {
+  if (perm_rescans(nb, rescan_work(h))) {
     if (part == PermPart::kScatterAhead) return CB_OK;
     const unsigned grid = static_cast<unsigned>(
         nb + std::min<int64_t>(class_chunks(ca.ntasks, kRescanThreads), int64_t(h->num_sms) * 2));

@@ -5,6 +5,7 @@
 #include <algorithm>
 
 #include "cb_internal.cuh"
+#include "pair_lists.cuh"
 #include "team.cuh"
 
 namespace cb {
@@ -410,7 +411,7 @@ struct AboveArgs {
   const int32_t* seg_of;
   int32_t* pairs;
   bool wide;                // pairs is 8-byte aligned: a pair per store (a caller's buffer may not be)
-  int32_t* list[kSortLists];   // rows with more than kSortWarp entries, by size
+  int32_t* lists;           // rows with more than kSortWarp entries, by size (pair_lists.cuh, n places)
   unsigned long long* list_n;
 };
 
@@ -426,7 +427,7 @@ __device__ __forceinline__ void above_done(const AboveArgs& a, int64_t x, int c)
   a.cnt[x] = c;
   if (c > kSortWarp) {
     const int k = c <= kSortMid ? 0 : c <= 128 * kSortKeys ? 1 : c <= 512 * kSortKeys ? 2 : 3;
-    a.list[k][atomicAdd(a.list_n + k, 1ull)] = static_cast<int32_t>(x);
+    a.lists[pair_place(k, static_cast<int64_t>(atomicAdd(a.list_n + k, 1ull)), a.n)] = static_cast<int32_t>(x);
   }
 }
 
@@ -547,7 +548,7 @@ __global__ void __launch_bounds__(256) k_above_warp(AboveArgs a, int per) {
 __global__ void __launch_bounds__(256) k_above_listed(AboveArgs a) {
   const int64_t rows = static_cast<int64_t>(a.list_n[0]), nw = int64_t(gridDim.x) * (blockDim.x >> 5);
   for (int64_t i = (blockIdx.x * int64_t(blockDim.x) + threadIdx.x) >> 5; i < rows; i += nw) {
-    const int32_t x = a.list[0][i];
+    const int32_t x = a.lists[pair_place(0, i, a.n)];
     const int c = a.cnt[x];
     const int32_t sb = a.seg_of ? static_cast<int32_t>(a.segs[a.seg_of[x]].off) : 0;
     if (c <= 512) write_sorted<16>(a, x, a.rp[x], c, a.off[x], sb);
@@ -613,7 +614,7 @@ __global__ void __launch_bounds__(NT, NT == 1024 ? 1 : 1024 / NT) k_above_block(
   const int lane = threadIdx.x & 31, at = (threadIdx.x >> 5) * 32 * kSortKeys + lane;
   const int64_t rows = static_cast<int64_t>(a.list_n[which]);
   for (int64_t i = blockIdx.x; i < rows; i += gridDim.x) {
-    const int32_t x = a.list[which][i];
+    const int32_t x = a.lists[pair_place(which, i, a.n)];
     const int c = a.cnt[x];
     const int64_t b = a.rp[x], o = a.off[x];
     const int32_t sb = a.seg_of ? static_cast<int32_t>(a.segs[a.seg_of[x]].off) : 0;
@@ -789,7 +790,8 @@ int export_sorted_pairs(Graph* h, int32_t* pairs) {
   a.seg_of = h->seg_of;
   a.pairs = pairs;
   a.wide = reinterpret_cast<uintptr_t>(pairs) % 8 == 0;
-  for (int k = 0; k < kSortLists; ++k) a.list[k] = h->lists + k * n;   // 4.5 n entries
+  a.lists = h->lists;   // kClassLists n / 2 places
+  static_assert((kSortLists + 1) / 2 * 2 <= kClassLists, "");
   a.list_n = reinterpret_cast<unsigned long long*>(h->scratch);
   const bool lists = h->maxdeg > kSortWarp;
   if (lists) CB_CUDA(h, cudaMemsetAsync(a.list_n, 0, kSortLists * sizeof(unsigned long long), s));

@@ -82,7 +82,7 @@ struct StepCtx {
   int32_t* err;
   uint32_t* def_bits;              // bit t: trade t is deferred
   unsigned long long* def_n;       // trades this pass deferred, by kind
-  int32_t* def_list;               // kDefKinds x ntasks: their lists, or null: in def_bits and def_seg
+  int32_t* def_list;               // their lists by kind (pair_lists.cuh), or null: in def_bits and def_seg
   int32_t* def_seg;                // and per segment of the trades (kDefKinds x kDefSegs)
   int64_t def_seg_trades;          // trades of a segment
   int narrow;                      // 8-byte far-trade records
@@ -99,13 +99,15 @@ struct SelOut {
   int32_t bin, below, cnt, pad;
 };
 
-// The trades of class k: (list, length).
+// The trades of class k.
 struct ClassList {
-  const int32_t* list;
+  const int32_t* first;
   int64_t len;
+  int step;   // lists of odd classes run backwards (pair_lists.cuh)
+  __device__ __forceinline__ int32_t operator[](int64_t q) const { return first[step * q]; }
 };
 __device__ __forceinline__ ClassList class_list(const StepCtx& c, const int32_t* lists, const int64_t* ctr, int k) {
-  return {lists + k * c.ntasks, ctr[kCtrClsLen + k]};
+  return {lists + pair_place(k, 0, c.ntasks), ctr[kCtrClsLen + k], (k & 1) ? -1 : 1};
 }
 
 struct TradeRows {
@@ -154,7 +156,7 @@ __device__ __forceinline__ void defer_trade(const StepCtx& c, int64_t t) {
   const int k = def_kind(tr.du + tr.dv);
   const int64_t at = static_cast<int64_t>(atomicAdd(c.def_n + k, 1ull));
   if (c.def_list) {
-    c.def_list[k * c.ntasks + at] = static_cast<int32_t>(t);
+    c.def_list[pair_place(k, at, c.ntasks)] = static_cast<int32_t>(t);
   } else {
     atomicOr(c.def_bits + (t >> 5), 1u << (t & 31));
     atomicAdd(c.def_seg + k * kDefSegs + t / c.def_seg_trades, 1);
@@ -280,9 +282,8 @@ __device__ __forceinline__ bool far_keeps_low(const StepCtx& c, const KeyCtx& kc
 }
 
 // What the rebuild needs of a far trade s: the new positions of its two nodes
-// and the top 8 bits of its threshold key.  Up to 2^28 positions it fits 8
-// bytes (28 + 28 + 8 bits), else 16.
-constexpr int64_t kNarrowPackMax = int64_t(1) << 28;
+// and the top 8 bits of its threshold key.  Up to 2^28 positions
+// (kNarrowPackMax) it fits 8 bytes (28 + 28 + 8 bits), else 16.
 
 // Trade t's threshold, its record, and (when a later trade may wait for it)
 // its done flag: by one member, as soon as the threshold is known, so that
@@ -1516,7 +1517,7 @@ __device__ void run_lanes(const StepCtx& c, const ClassList& cl, char* smem, Rou
   for (int64_t q0 = rs.first((cl.len + Cfg::kTeams - 1) / Cfg::kTeams) * Cfg::kTeams + lead; q0 < cl.len; q0 += step) {
     const int64_t q = q0 + (id - lead);
     const bool active = q < cl.len;
-    const int64_t t = cl.list[active ? q : q0];
+    const int64_t t = cl[active ? q : q0];
     if (!phase_a_reg<LaneTeam<W>, kWarpJ, Cfg::B, true, kOneSeed>(tm, c, t, w, active) && tm.rank == 0) defer_trade(c, t);
   }
 }
@@ -1527,8 +1528,8 @@ __device__ void run_warps(const StepCtx& c, const ClassList& cl, char* smem, Rou
   WarpTeam tm;
   const int64_t step = static_cast<int64_t>(gridDim.x) * kWarpWarps;
   for (int64_t q = rs.first((cl.len + kWarpWarps - 1) / kWarpWarps) * kWarpWarps + wid; q < cl.len; q += step)
-    if (!phase_a_reg<WarpTeam, kWarpJ, kWarpB, true, kOneSeed>(tm, c, cl.list[q], w) && tm.rank == 0)
-      defer_trade(c, cl.list[q]);
+    if (!phase_a_reg<WarpTeam, kWarpJ, kWarpB, true, kOneSeed>(tm, c, cl[q], w) && tm.rank == 0)
+      defer_trade(c, cl[q]);
 }
 template <int CT, int NT, bool kOneSeed, int J = kTeamJ, int SLOTS = 4>
 __device__ void run_teams(const StepCtx& c, const ClassList& cl, char* smem, int64_t* red, Rounds& rs) {
@@ -1540,8 +1541,8 @@ __device__ void run_teams(const StepCtx& c, const ClassList& cl, char* smem, int
   const Ws w{smem + Ws::kBytes * id};
   const int64_t step = static_cast<int64_t>(gridDim.x) * kTeams;
   for (int64_t q = rs.first((cl.len + kTeams - 1) / kTeams) * kTeams + id; q < cl.len; q += step)
-    if (!phase_a_reg<SubTeam<NT>, J, Cfg::B, false, kOneSeed>(tm, c, cl.list[q], w) && tm.rank == 0)
-      defer_trade(c, cl.list[q]);
+    if (!phase_a_reg<SubTeam<NT>, J, Cfg::B, false, kOneSeed>(tm, c, cl[q], w) && tm.rank == 0)
+      defer_trade(c, cl[q]);
 }
 
 // Class K alone.  Instruction issue bounds these kernels (55 to 64 % of the
@@ -1896,7 +1897,6 @@ __global__ void __launch_bounds__(NT, NT == 256 ? 4 : 1) k_phase_a_block(StepCtx
   __shared__ uint64_t mbar;
   BlockTeam<NT> tm(red);
   const ClassList cl = class_list(c, lists, ctr, cls);
-  const int32_t* list = cl.list;
   const int64_t len = cl.len;
   int32_t* stage = reinterpret_cast<int32_t*>(sbuf + room);
   if (threadIdx.x == 0) {
@@ -1908,7 +1908,7 @@ __global__ void __launch_bounds__(NT, NT == 256 ? 4 : 1) k_phase_a_block(StepCtx
   // member 0 reads the next trade's row range at the start of each trade; the
   // copy goes out once the current trade has read its staged entries
   auto range_of = [&](int64_t q, int64_t* b0, int* L) {
-    const int64_t t = list[q];
+    const int64_t t = cl[q];
     const TradeRows tr = trade_rows(c, t);
     *b0 = tr.b0;
     *L = tr.du + tr.dv;
@@ -1924,7 +1924,7 @@ __global__ void __launch_bounds__(NT, NT == 256 ? 4 : 1) k_phase_a_block(StepCtx
   }
   bool failed = false;
   for (int64_t q = blockIdx.x; q < len; q += gridDim.x) {
-    const int64_t t = list[q];
+    const int64_t t = cl[q];
     const TradeRows tr = trade_rows(c, t);
     const int L = tr.du + tr.dv;
     if (L > smem_max && threadIdx.x == 0) atomicAdd(c.gws_count, 1ull);
@@ -2003,7 +2003,7 @@ __global__ void __launch_bounds__(kBigThreads, 1) k_phase_a_huge(StepCtx c, cons
   BlockTeam<kBigThreads> tm(red);
   const ClassList cl = class_list(c, lists, ctr, 8);
   for (int64_t q = blockIdx.x; q < cl.len; q += gridDim.x) {
-    const int64_t t = cl.list[q];
+    const int64_t t = cl[q];
     const TradeRows tr = trade_rows(c, t);
     const int L = tr.du + tr.dv;
     bool ok;
@@ -2051,8 +2051,8 @@ __global__ void __launch_bounds__(NT, NT == 256 ? 4 : 1) k_retry(StepCtx c, cons
     const int64_t p = pick;
     __syncthreads();
     if (p >= nl) return;
-    if (!run_large<NT, false>(tm, c, list[p], sbuf, &sel, gen_max, room, gws, slice, 0u) && threadIdx.x == 0)
-      defer_trade(c, list[p]);
+    const int32_t t = list[NT == kMedThreads ? -p : p];   // the medium trades' list runs backwards (pair_lists.cuh)
+    if (!run_large<NT, false>(tm, c, t, sbuf, &sel, gen_max, room, gws, slice, 0u) && threadIdx.x == 0) defer_trade(c, t);
   }
 }
 
@@ -2306,10 +2306,11 @@ size_t trade_smem_bytes(int entries) { return ws_a_bytes(entries); }
 
 // Passes of the fix-up: enough that one pass's far-trade records (8 or 16
 // bytes per trade) stay below kFixSliceBytes, or the "fix_passes" option.
+bool narrow_pack(const Graph* h) { return h->n <= kNarrowPackMax && !h->far_wide; }
 constexpr int64_t kFixSliceBytes = int64_t(72) << 20;
 int fix_passes(const Graph* h) {
   if (h->fix_passes > 0) return h->fix_passes;
-  const int64_t rec = (h->n <= kNarrowPackMax && !h->wide_pack) ? 8 : 16;
+  const int64_t rec = narrow_pack(h) ? 8 : 16;
   return static_cast<int>(std::max<int64_t>(1, (h->ntasks * rec + kFixSliceBytes - 1) / kFixSliceBytes));
 }
 
@@ -2357,7 +2358,7 @@ int super_step(Graph* h, bool ahead) {
   c.chunk_row = h->chunk_row;
   c.thr_key = h->thr_key;
   c.thr_tb = h->thr_tb;
-  c.far_pack = h->far_pack;
+  c.far_pack = h->far_wide ? h->far_wide : h->far_pack;
   c.done = h->done;
   c.err = h->err;
   c.def_bits = h->def_bits;
@@ -2365,7 +2366,7 @@ int super_step(Graph* h, bool ahead) {
   const int64_t nwords = (h->ntasks + 31) / 32;
   const int64_t seg_words = std::max<int64_t>(1, (nwords + kDefSegs - 1) / kDefSegs);
   c.def_seg_trades = 32 * seg_words;
-  c.narrow = h->n <= kNarrowPackMax && !h->wide_pack;
+  c.narrow = narrow_pack(h);
   philox_round_keys(h->hsegs[0].seed, c.ks);   // used only when the handle holds one graph
   // counters (kCtr* in cb_internal.cuh), zero at the start of the step: class
   // lists, deferrals per pass, ranges claimed, global-workspace trades
@@ -2534,13 +2535,13 @@ int super_step(Graph* h, bool ahead) {
     k_retry_warp<<<wgrid, 32 * kWarpWarps, WarpWs::kBytes * kWarpWarps, s>>>(c, in, count, claim);
     if ((rc = launched())) return rc;
     if (max_trade > kDefSmall) {
-      k_retry<kMedThreads><<<lgrid, kMedThreads, TeamCfg<kMedThreads>::Ws::kBytes, s>>>(c, in + ntasks, count + 1,
+      k_retry<kMedThreads><<<lgrid, kMedThreads, TeamCfg<kMedThreads>::Ws::kBytes, s>>>(c, in + pair_place(1, 0, ntasks), count + 1,
                                                                                        claim + 1, 0, 0, nullptr, 0);
       if ((rc = launched())) return rc;
     }
     if (max_trade > kDefMedium) {
       const size_t sm = resolve_smem<kBigThreads>(h->smem_max, max_trade);
-      k_retry<kBigThreads><<<bgrid, kBigThreads, sm, s>>>(c, in + 2 * ntasks, count + 2, claim + 2, h->smem_max, sm, gws,
+      k_retry<kBigThreads><<<bgrid, kBigThreads, sm, s>>>(c, in + pair_place(2, 0, ntasks), count + 2, claim + 2, h->smem_max, sm, gws,
                                                           h->ws_slice);
       if ((rc = launched())) return rc;
     }
