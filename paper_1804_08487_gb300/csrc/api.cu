@@ -485,7 +485,6 @@ int set_relaxed(Graph* h, bool on) {
   if (h->nseg != 1) return fail(h, CB_EINVAL, "relaxed permutations are for handles of one graph");
   if (on == h->relaxed) return CB_OK;
   const int64_t n = h->n;
-  cudaStream_t s = h->stream;
   int rc;
   if (on && !h->lcg_ab) {
     h->lcg_p = next_prime_host(static_cast<uint64_t>(std::max<int64_t>(n, 2)));

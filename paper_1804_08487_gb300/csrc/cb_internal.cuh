@@ -13,9 +13,7 @@ namespace cb {
 enum DevErr : int32_t {
   kErrNone = 0,
   kErrRowLength = 1,     // a rebuilt row does not match the degree
-  kErrRowSide = 2,       // entry written to the wrong row of a trade
   kErrValidate = 3,      // input graph not simple / symmetric / in range
-  kErrBucket = 4,        // permutation bucket bookkeeping failed
   kErrResolve = 5,       // a dependency wait of the in-order pass gave up
   kErrStage = 6,         // a bulk copy into shared memory did not complete in time
   kErrUniform = 7,       // uniform trades: an inbox or the run queue overflowed, or a message missed its trade
@@ -32,7 +30,6 @@ constexpr int kTileMaxCap = 128;    // largest trade (deg u + deg v) on the flat
 constexpr int kBlockMaxCap = 2048;  // largest trade on the 256-thread path
 constexpr int kBlockMaxDefault = 1024;   // default of the "block_max" option
 constexpr int kSmemMaxCap = 8192;   // largest trade kept in shared memory on the 1024-thread path
-constexpr int kBlockThreads = 256;  // CTA size of the block path
 constexpr int kCounters = 64;       // device counters of one super step (two sets per handle, used in turn)
 // Trade size classes of the threshold phase (one team size each) and the
 // device counters of a super step.

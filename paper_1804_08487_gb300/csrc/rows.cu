@@ -1,6 +1,6 @@
 // Row-level utilities outside the super step: relabelling a CSR into another
-// row order and node numbering (with each row sorted), input validation, the
-// inverse of a permutation and the canonical edge export (Section 2: ordered
+// row order and node numbering (with each row sorted), input validation and
+// the canonical edge export (Section 2: ordered
 // edges [a,b], a<b).
 #include <algorithm>
 

@@ -1,4 +1,4 @@
-// Cooperative "teams" working on one trade or one row: part of a warp (4 to
+// Cooperative "teams" working on one trade or one row: part of a warp (8 or
 // 16 lanes, LaneTeam), a warp (WarpTeam), part of a CTA (64 to 512 threads
 // with a named barrier, SubTeam) or a whole CTA (BlockTeam).
 // The trade and row algorithms are written once against this interface; all
@@ -15,23 +15,12 @@ struct WarpTeam {
   int rank;
   __device__ __forceinline__ WarpTeam() : rank(threadIdx.x & 31) {}
   __device__ __forceinline__ void sync() const { __syncwarp(); }
-  __device__ __forceinline__ bool any(bool p) const { return __any_sync(kFull, p); }
   // does any team of this warp need a branch? (p is the same in every member)
   __device__ __forceinline__ bool warp_any(bool p) const { return p; }
   __device__ __forceinline__ int64_t sum(int64_t v) const {
 #pragma unroll
     for (int o = 16; o; o >>= 1) v += __shfl_xor_sync(kFull, v, o);
     return v;
-  }
-  // exclusive prefix sum over ranks
-  __device__ __forceinline__ int64_t exscan(int64_t v) const {
-    int64_t x = v;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-      const int64_t y = __shfl_up_sync(kFull, x, o);
-      if (rank >= o) x += y;
-    }
-    return x - v;
   }
   // value held by member `src`
   __device__ __forceinline__ uint64_t bcast(uint64_t v, int src) const { return __shfl_sync(kFull, v, src); }
@@ -54,7 +43,7 @@ struct WarpTeam {
   __device__ __forceinline__ uint32_t warps_before(uint32_t) const { return 0u; }
 };
 
-// W consecutive lanes of a warp (W = 4, 8 or 16): a warp holds 32 / W such
+// W consecutive lanes of a warp (W = 8 or 16): a warp holds 32 / W such
 // teams, each on its own trade, in lockstep.  Every call names the whole
 // warp, so all teams must reach every call together (warp-uniform control
 // flow: a branch around a call is taken when any team needs it, see
@@ -64,7 +53,7 @@ struct WarpTeam {
 // against 1257 of a whole warp on one.
 template <int W>
 struct LaneTeam {
-  static_assert(W == 4 || W == 8 || W == 16, "lane teams of 4, 8 or 16 lanes");
+  static_assert(W == 8 || W == 16, "lane teams of 8 or 16 lanes");
   static constexpr int N = W;
   int rank;
   unsigned mask;
@@ -109,7 +98,6 @@ struct BlockTeam {
   int64_t* red;
   __device__ __forceinline__ BlockTeam(int64_t* r) : rank(threadIdx.x), buf(0), red(r) {}
   __device__ __forceinline__ void sync() const { __syncthreads(); }
-  __device__ __forceinline__ bool any(bool p) const { return __syncthreads_or(p); }
   __device__ int64_t sum(int64_t v) {
     const int lane = rank & 31;
 #pragma unroll
@@ -174,17 +162,6 @@ struct BlockTeam {
   }
 };
 
-// First index i in [0, len) with a[i] >= v (len if none).
-template <class T>
-__device__ __forceinline__ int lower_bound(const T* a, int len, T v) {
-  int lo = 0, hi = len;
-  while (lo < hi) {
-    const int mid = (lo + hi) >> 1;
-    if (a[mid] < v) lo = mid + 1; else hi = mid;
-  }
-  return lo;
-}
-
 // In-place ascending bitonic sort of a[0..P), P a power of two.
 template <class Team, class T>
 __device__ void team_bitonic_sort(Team& tm, T* a, int P) {
@@ -229,15 +206,6 @@ struct SubTeam {
   int64_t* red;
   __device__ __forceinline__ SubTeam(int64_t* r, int id) : rank(threadIdx.x % NT), bar(id + 1), buf(0), red(r) {}
   __device__ __forceinline__ void sync() const { asm volatile("bar.sync %0, %1;" ::"r"(bar), "n"(NT) : "memory"); }
-  __device__ __forceinline__ bool any(bool p) const {
-    int r;
-    asm volatile(
-        "{\n .reg .pred q, o;\n setp.ne.s32 q, %1, 0;\n bar.red.or.pred o, %2, %3, q;\n selp.s32 %0, 1, 0, o;\n}"
-        : "=r"(r)
-        : "r"(p ? 1 : 0), "r"(bar), "n"(NT)
-        : "memory");
-    return r != 0;
-  }
   __device__ int64_t sum(int64_t v) {
     const int lane = rank & 31;
 #pragma unroll
@@ -250,23 +218,6 @@ struct SubTeam {
 #pragma unroll
     for (int o = 16; o; o >>= 1) x += __shfl_xor_sync(kFull, x, o);
     return x;
-  }
-  __device__ int64_t exscan(int64_t v) {
-    const int lane = rank & 31, w = rank >> 5;
-    int64_t x = v;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-      const int64_t y = __shfl_up_sync(kFull, x, o);
-      if (lane >= o) x += y;
-    }
-    int64_t* part = red + buf * NW;
-    if (lane == 31) part[w] = x;
-    sync();
-    buf ^= 1;
-    int64_t before = lane < w ? part[lane] : 0;
-#pragma unroll
-    for (int o = 16; o; o >>= 1) before += __shfl_xor_sync(kFull, before, o);
-    return x - v + before;
   }
   __device__ __forceinline__ bool warp_any(bool p) const { return p; }
   // see WarpTeam; one barrier each, through the same two buffers

@@ -2302,7 +2302,6 @@ int init_trade_kernels(Graph* h) {
 size_t trade_ws_slice_bytes(int64_t max_trade) {
   return (ws_a_bytes(static_cast<int>(max_trade)) + 255) & ~size_t(255);
 }
-size_t trade_smem_bytes(int entries) { return ws_a_bytes(entries); }
 
 // Passes of the fix-up: enough that one pass's far-trade records (8 or 16
 // bytes per trade) stay below kFixSliceBytes, or the "fix_passes" option.
