@@ -91,7 +91,8 @@ struct StepCtx {
   uint64_t wait_ns;                // longest single wait on dependencies or a bulk copy
   int hold_publish;                // test hook: no trade publishes its done flag (waits run out)
   unsigned inorder_ctas;           // CTAs of the in-order pass that take part (a test hook; default: all)
-  uint32_t ks[20];                 // one graph (seg_of null): the Philox round keys of its seed
+  uint64_t seed;                   // one graph (seg_of null): its seed
+  uint32_t ks[20];                 // and the seed's Philox round keys
 };
 
 struct SelOut {
@@ -245,12 +246,18 @@ __device__ __forceinline__ bool at_or_below(uint64_t key, uint64_t tb, uint64_t 
 
 // Key parameters of a trade's graph: its seed, its step and its first
 // position (keys count positions from the start of the graph).  Both ends of
-// an edge are in the same graph.
+// an edge are in the same graph.  kOneSeed (a handle of one graph, which starts
+// at position 0): only the step is loaded, and two subtractions per edge fall
+// away.  (Plain loads stay in the loop over the trades, see after_previous():
+// with all three loaded per trade the in-order pass took 65.6 us at n=2^17 and
+// 80 at n=2^20, n=4096 stepped ten times 597; so, 58.7, 72 and 581.)
 struct KeyCtx {
   uint64_t seed;
   uint32_t g, off;
 };
+template <bool kOneSeed>
 __device__ __forceinline__ KeyCtx key_ctx(const StepCtx& c, int64_t t) {
+  if constexpr (kOneSeed) return {c.seed, c.segs->g, 0u};
   const Seg* S = c.segs + (c.seg_of ? c.seg_of[2 * t] : 0);
   return {S->seed, S->g, static_cast<uint32_t>(S->off)};
 }
@@ -614,7 +621,7 @@ __device__ bool phase_a(Team& tm, const StepCtx& c, int64_t t, const WsA& w, Sel
                         const int32_t* ystage = nullptr, StageNext sn = StageNext{false, 0, 0, nullptr, nullptr},
                         uint32_t wait_below = 0) {
   const TradeRows tr = trade_rows(c, t);
-  const KeyCtx kc = key_ctx(c, t);
+  const KeyCtx kc = key_ctx<kOneSeed>(c, t);
   const int du = tr.du, dv = tr.dv, L = du + dv;
   const int H = 1 << w.lgH;
   const int64_t t2 = 2 * t;
@@ -1100,7 +1107,7 @@ __device__ bool phase_a_reg(Team& tm, const StepCtx& c, int64_t t, const Ws& w, 
   static_assert(N * J == Ws::kLmax && N * J < (1 << 16), "16-bit placement counts");
   constexpr int kLgH = lg_ceil(Ws::kH), kLgH2 = lg_ceil(Ws::kH2);
   const TradeRows tr = trade_rows(c, t);
-  const KeyCtx kc = key_ctx(c, t);
+  const KeyCtx kc = key_ctx<kOneSeed>(c, t);
   const int du = tr.du, L = active ? tr.du + tr.dv : 0;
   // the nodes' positions in step g+1, loaded now so that their dependent
   // loads overlap the trade's work
@@ -1546,8 +1553,8 @@ __device__ void run_teams(const StepCtx& c, const ClassList& cl, char* smem, int
 }
 
 // Class K alone.  Instruction issue bounds these kernels (55 to 64 % of the
-// slots, no memory level above 25 %).  Trades of more than 256 entries run with
-// eight entries per member on teams of half the size, which halves what a
+// slots; L1 at 40 %, L2 and DRAM below 25).  Trades of more than 256 entries run
+// with eight entries per member on teams of half the size, which halves what a
 // trade costs whatever its size (clearing, scans, the threshold search) and its
 // barriers; two hash slots per entry keep four CTAs on an SM.  n=2^25, degrees
 // [10,10000), ms per step with four and eight: 257 to 512 entries 3.90 and
@@ -1749,7 +1756,7 @@ __device__ uint32_t fix_tie(const StepCtx& c, int64_t e, uint32_t y, uint32_t b)
     low = fp < tp;
   } else {
     const uint32_t xr = static_cast<uint32_t>(c.pos[c.order_next[fix_row(c, e)]]) ^ (b & 1u);
-    low = far_keeps_low(c, key_ctx(c, s), s, min(xr, y), max(xr, y));
+    low = far_keeps_low(c, key_ctx<false>(c, s), s, min(xr, y), max(xr, y));
   }
   return static_cast<uint32_t>(low ? ft.x : ft.y);
 }
@@ -1824,18 +1831,16 @@ __global__ void __launch_bounds__(kFixThreads, 4) k_fixup(StepCtx c, int64_t nnz
     uint32_t res[kFixPer];
     FarRaw<kNarrow> ftv[kFixPer];
     uint32_t todo = 0;   // bit j: entry j is this pass's
-    bool unfilled = false;
 #pragma unroll
     for (int j = 0; j < kFixPer; ++j) {
       const uint32_t p = pv[j];
       res[j] = (p & kPhDone) && p != 0xFFFFFFFFu ? (p & ~kPhDone) : 0u;   // an earlier pass resolved it
       const uint32_t s = p >> 1;
       const bool mine = !(p & kPhDone) && s >= s_lo && s < s_hi && p < static_cast<uint32_t>(c.n);
-      unfilled |= !(p & kPhDone) && p >= static_cast<uint32_t>(c.n);
+      if (!(p & kPhDone) && p >= static_cast<uint32_t>(c.n)) latch(c.err, kErrRowLength);
       if (mine) ftv[j] = far_raw<kNarrow>(c.far_pack, s);
       todo |= static_cast<uint32_t>(mine) << j;
     }
-    if (unfilled) latch(c.err, kErrRowLength);   // a slot phase A did not fill
 #pragma unroll
     for (int j = 0; j < kFixPer; ++j) {
       if (!((todo >> j) & 1u)) continue;
@@ -2151,9 +2156,8 @@ __global__ void __launch_bounds__(kDefListThreads) k_def_list(StepCtx c, int64_t
   }
 }
 
-template <int NT>
-__global__ void __launch_bounds__(NT, NT == 256 ? 4 : 1) k_resolve(StepCtx c, const int32_t* list,
-                                                                const int32_t* chunk_first,
+template <int NT, bool kOneSeed>
+__global__ void __launch_bounds__(NT, NT == 256 ? 4 : 1) k_resolve(StepCtx c, const int32_t* list, const int32_t* chunk_first,
                                                                 const unsigned long long* nchunks,
                                                                 unsigned long long* claim, int gen_max, size_t room,
                                                                 char* gws, size_t slice) {
@@ -2175,13 +2179,13 @@ __global__ void __launch_bounds__(NT, NT == 256 ? 4 : 1) k_resolve(StepCtx c, co
   WarpTeam wt;
   const WarpWs ww{sbuf + WarpWs::kBytes * warp};
   const Ws256 w256{sbuf + Ws256::kBytes * id};
-  if (chunks == 0 || blockIdx.x >= c.inorder_ctas) return;
+  if (blockIdx.x >= c.inorder_ctas) return;
   for (;;) {
-    // (claimed only now: a chunk held while the one before it waits would hold up others)
+    // (claimed only now: a chunk held while the one before it waits would hold
+    // up others; the first claim and the load of *nchunks go out together)
     if (threadIdx.x == 0) pick = static_cast<int64_t>(atomicAdd(claim, 1ull));
     __syncthreads();
-    const int64_t ch = pick;
-    __syncthreads();
+    const int64_t ch = pick;   // written again only after the barriers of this chunk
     if (ch >= chunks) return;
     const int32_t first = chunk_first[ch], count = chunk_first[ch + 1] - first;
     const uint32_t from = static_cast<uint32_t>(list[first]);   // trades before it are in earlier chunks
@@ -2206,7 +2210,7 @@ __global__ void __launch_bounds__(NT, NT == 256 ? 4 : 1) k_resolve(StepCtx c, co
       for (int i = warp; i < n[0]; i += kWarps) {
         const int32_t t = trades[0][i];
         if (t < 0) continue;
-        const bool ok = phase_a_reg<WarpTeam, kWarpJ, kWarpB, true, false, true>(wt, c, t, ww, true, from);
+        const bool ok = phase_a_reg<WarpTeam, kWarpJ, kWarpB, true, kOneSeed, true>(wt, c, t, ww, true, from);
         if (lane == 0) {
           if (ok) trades[0][i] = -1;
           else atomicAdd(&left, 1);
@@ -2217,7 +2221,7 @@ __global__ void __launch_bounds__(NT, NT == 256 ? 4 : 1) k_resolve(StepCtx c, co
         for (int i = id; i < n[1]; i += kTeams) {
           const int32_t t = trades[1][i];
           if (t < 0) continue;
-          const bool ok = phase_a_reg<SubTeam<256>, kTeamJ, TeamCfg<256>::B, false, false, true>(st, c, t, w256, true, from);
+          const bool ok = phase_a_reg<SubTeam<256>, kTeamJ, TeamCfg<256>::B, false, kOneSeed, true>(st, c, t, w256, true, from);
           if (st.rank == 0) {
             if (ok) trades[1][i] = -1;
             else atomicAdd(&left, 1);
@@ -2228,7 +2232,7 @@ __global__ void __launch_bounds__(NT, NT == 256 ? 4 : 1) k_resolve(StepCtx c, co
         __syncthreads();
         const int32_t t = trades[2][i];
         if (t < 0) continue;
-        const bool ok = run_large<NT, true>(tm, c, t, sbuf, &sel, gen_max, room, gws, slice, from);
+        const bool ok = run_large<NT, true, kOneSeed>(tm, c, t, sbuf, &sel, gen_max, room, gws, slice, from);
         __syncthreads();
         if (threadIdx.x == 0) {
           if (ok) trades[2][i] = -1;
@@ -2273,6 +2277,12 @@ int init_seed_kernels(Graph* h) {
                                   static_cast<int>(kLargeSmem)));
   CB_CUDA(h, cudaFuncSetAttribute(k_phase_a_small<kOneSeed>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                   static_cast<int>(small_smem())));
+  CB_CUDA(h, cudaFuncSetAttribute(k_resolve<kMedThreads, kOneSeed>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                  static_cast<int>(resolve_smem<kMedThreads>(kBlockMaxCap, 0))));
+  CB_CUDA(h, cudaFuncSetAttribute(k_resolve<kBigThreads, kOneSeed>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                  static_cast<int>(resolve_smem<kBigThreads>(kSmemMaxCap, 2 * int64_t(kSmemMaxCap)))));
+  CB_CUDA(h, cudaFuncSetAttribute(k_resolve<kMedThreads, kOneSeed>, cudaFuncAttributePreferredSharedMemoryCarveout,
+                                  cudaSharedmemCarveoutMaxShared));
   // shared memory, not L1, limits how many CTAs of these kernels an SM holds
   CB_CUDA(h, cudaFuncSetAttribute(k_phase_a_block<kMedThreads, kOneSeed>,
                                   cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared));
@@ -2290,12 +2300,6 @@ int init_trade_kernels(Graph* h) {
                                   static_cast<int>(resolve_smem<kBigThreads>(kSmemMaxCap, 2 * int64_t(kSmemMaxCap)))));
   CB_CUDA(h, cudaFuncSetAttribute(k_retry_warp, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                   static_cast<int>(WarpWs::kBytes * kWarpWarps)));
-  CB_CUDA(h, cudaFuncSetAttribute(k_resolve<kMedThreads>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                  static_cast<int>(resolve_smem<kMedThreads>(kBlockMaxCap, 0))));
-  CB_CUDA(h, cudaFuncSetAttribute(k_resolve<kBigThreads>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                  static_cast<int>(resolve_smem<kBigThreads>(kSmemMaxCap, 2 * int64_t(kSmemMaxCap)))));
-  CB_CUDA(h, cudaFuncSetAttribute(k_resolve<kMedThreads>, cudaFuncAttributePreferredSharedMemoryCarveout,
-                                  cudaSharedmemCarveoutMaxShared));
   return CB_OK;
 }
 
@@ -2366,7 +2370,8 @@ int super_step(Graph* h, bool ahead) {
   const int64_t seg_words = std::max<int64_t>(1, (nwords + kDefSegs - 1) / kDefSegs);
   c.def_seg_trades = 32 * seg_words;
   c.narrow = narrow_pack(h);
-  philox_round_keys(h->hsegs[0].seed, c.ks);   // used only when the handle holds one graph
+  c.seed = h->hsegs[0].seed;   // both used only when the handle holds one graph
+  philox_round_keys(c.seed, c.ks);
   // counters (kCtr* in cb_internal.cuh), zero at the start of the step: class
   // lists, deferrals per pass, ranges claimed, global-workspace trades
   int64_t* cnt = h->counters + cur * kCounters;
@@ -2558,11 +2563,11 @@ int super_step(Graph* h, bool ahead) {
     if ((rc = launched())) return rc;
     if (big) {
       const size_t sm = resolve_smem<kBigThreads>(h->smem_max, max_trade);
-      CB_CUDA(h, launch(overlap, k_resolve<kBigThreads>, grid, kBigThreads, sm, s, c, list, chunk_first,
+      CB_CUDA(h, launch(overlap, c.seg_of ? k_resolve<kBigThreads, false> : k_resolve<kBigThreads, true>, grid, kBigThreads, sm, s, c, list, chunk_first,
                         ucnt + kCtrChunks, ucnt + kCtrFinished, h->smem_max, sm, gws, h->ws_slice));
     } else {
       const size_t sm = resolve_smem<kMedThreads>(block_max, max_trade);
-      CB_CUDA(h, launch(overlap, k_resolve<kMedThreads>, grid, kMedThreads, sm, s, c, list, chunk_first,
+      CB_CUDA(h, launch(overlap, c.seg_of ? k_resolve<kMedThreads, false> : k_resolve<kMedThreads, true>, grid, kMedThreads, sm, s, c, list, chunk_first,
                         ucnt + kCtrChunks, ucnt + kCtrFinished, block_max, sm, gws, h->ws_slice));
     }
     if ((rc = launched())) return rc;
