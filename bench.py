@@ -168,8 +168,8 @@ def workload(name):
 MEASURED_TRAFFIC = {
     # profiles/rebuild_traffic_n2p25.md: mean of four super steps
     ("rebuild phase (k_fixup passes)", "n2^25"): {
-        "bytes": 94235662720,
-        "trade_cu_sha256": "dda02c42b60800db265c37075008e5b8d8520221dfbd464117ee477b449d96da",
+        "bytes": 93936838272,
+        "trade_cu_sha256": "a9e42776c98207277b4da6690c6030e44d9c882b52fba3dd8c223e8427d69df1",
     },
 }
 
@@ -668,7 +668,7 @@ def run_uniform(args):
         "roofline": {"bound": "hbm", "kernel": "uniform trades (whole step)", "achieved": gbs, "peak": peak,
                      "unit": "GB/s", "frac": gbs / peak, "traffic": None,
                      "peak_source": f"{peak_kind} hbm_gbs",
-                     "note": "B_min = 16m + 24n per step; the dataflow is bound by its chain of dependent trades"},
+                     "note": "B_min = 16m + 24n per step; the dataflow is bound by its large trades' teams and its chain of dependent trades"},
         "cpu_baseline": {"value": cpu_v, "unit": UNIT, "cores": 1, "kind": "oracle", "sample": cpu_desc},
         "e2e": {"value": job_rate(world, g.m * K, e2e_s), "unit": UNIT,
                 "h2d_bytes_per_step": (g.row_ptr.nbytes + g.col.nbytes) / K, "d2h_bytes_per_step": 2 * g.m * 4 / K},

@@ -2157,7 +2157,8 @@ __global__ void __launch_bounds__(kDefListThreads) k_def_list(StepCtx c, int64_t
 }
 
 template <int NT, bool kOneSeed>
-__global__ void __launch_bounds__(NT, NT == 256 ? 4 : 1) k_resolve(StepCtx c, const int32_t* list, const int32_t* chunk_first,
+__global__ void __launch_bounds__(NT, NT == 256 ? 4 : 1) k_resolve(StepCtx c, const int32_t* list,
+                                                                const int32_t* chunk_first,
                                                                 const unsigned long long* nchunks,
                                                                 unsigned long long* claim, int gen_max, size_t room,
                                                                 char* gws, size_t slice) {
@@ -2221,7 +2222,8 @@ __global__ void __launch_bounds__(NT, NT == 256 ? 4 : 1) k_resolve(StepCtx c, co
         for (int i = id; i < n[1]; i += kTeams) {
           const int32_t t = trades[1][i];
           if (t < 0) continue;
-          const bool ok = phase_a_reg<SubTeam<256>, kTeamJ, TeamCfg<256>::B, false, kOneSeed, true>(st, c, t, w256, true, from);
+          const bool ok =
+              phase_a_reg<SubTeam<256>, kTeamJ, TeamCfg<256>::B, false, kOneSeed, true>(st, c, t, w256, true, from);
           if (st.rank == 0) {
             if (ok) trades[1][i] = -1;
             else atomicAdd(&left, 1);
@@ -2563,11 +2565,13 @@ int super_step(Graph* h, bool ahead) {
     if ((rc = launched())) return rc;
     if (big) {
       const size_t sm = resolve_smem<kBigThreads>(h->smem_max, max_trade);
-      CB_CUDA(h, launch(overlap, c.seg_of ? k_resolve<kBigThreads, false> : k_resolve<kBigThreads, true>, grid, kBigThreads, sm, s, c, list, chunk_first,
+      CB_CUDA(h, launch(overlap, c.seg_of ? k_resolve<kBigThreads, false> : k_resolve<kBigThreads, true>, grid,
+                        kBigThreads, sm, s, c, list, chunk_first,
                         ucnt + kCtrChunks, ucnt + kCtrFinished, h->smem_max, sm, gws, h->ws_slice));
     } else {
       const size_t sm = resolve_smem<kMedThreads>(block_max, max_trade);
-      CB_CUDA(h, launch(overlap, c.seg_of ? k_resolve<kMedThreads, false> : k_resolve<kMedThreads, true>, grid, kMedThreads, sm, s, c, list, chunk_first,
+      CB_CUDA(h, launch(overlap, c.seg_of ? k_resolve<kMedThreads, false> : k_resolve<kMedThreads, true>, grid,
+                        kMedThreads, sm, s, c, list, chunk_first,
                         ucnt + kCtrChunks, ucnt + kCtrFinished, block_max, sm, gws, h->ws_slice));
     }
     if ((rc = launched())) return rc;
