@@ -1030,7 +1030,7 @@ int cb_set_option(cb_handle h, const char* key, int64_t value) {
     if (value < 0 || value > 1) return fail(h, CB_EINVAL, "wide_pack is 0 or 1");
     if (!value) {
       free_wide(h);
-    } else if (!h->far_wide) {
+    } else if (!h->far_wide && h->n <= kNarrowPackMax) {   // (above, all records are wide)
       void* p = nullptr;
       CB_CUDA(h, dmalloc(h, &p, wide_bytes(h)));
       h->far_wide = p;
